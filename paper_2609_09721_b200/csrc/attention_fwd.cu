@@ -28,13 +28,14 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <mutex>
-
 #include <vector>
 
 #include "efq_common.cuh"
 #include "efq_internal.cuh"
 #include "efq_producers.cuh"
+#include "mxfp4.cuh"
 #include "sm100_ptx.cuh"
 
 namespace efq {
@@ -134,11 +135,6 @@ __device__ __forceinline__ bool wait_all(uint64_t* bar, uint32_t parity, Smem* s
     if (ptx::mbar_try_wait(bar, parity)) return true;
     const bool ok = wait1(bar, parity, sm, status);
     return __all_sync(__activemask(), ok);
-}
-
-__device__ __forceinline__ uint32_t p_swizzled_offset(uint32_t row, uint32_t chunk)
-{
-    return (row >> 3) * 512u + (row & 7u) * 64u + ((chunk ^ ((row >> 1) & 3u)) << 4);
 }
 
 template <int PRODUCER, bool DEBUG, bool FIX8>
@@ -488,7 +484,7 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                 if (g == 0 && !have_p) {      // P~V of tile j-2 must have finished: it reads the group's P buffer
                     if (!wait_all(&sm->p_empty[sb], ph2 ^ 1u, sm, P.status)) { ok = false; break; }
                 }
-                *reinterpret_cast<uint4*>(sm->p[sb] + p_swizzled_offset(row, g)) = codes;
+                *reinterpret_cast<uint4*>(sm->p[sb] + code_tile_offset(row, g)) = codes;
                 sfword |= byte << (8 * g);
                 if (DEBUG && dbg_row) {
                     const int64_t blk = j * 4 + g;
@@ -652,6 +648,9 @@ struct Workspace {
 
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
+bool use_few(int Hq, int Hkv, int64_t Sq);
+int64_t few_chunks(int64_t Sk);
+
 Workspace plan_workspace(int B, int Hq, int Hkv, int64_t Sq, int64_t Sk)
 {
     Workspace w;
@@ -667,6 +666,19 @@ Workspace plan_workspace(int B, int Hq, int Hkv, int64_t Sq, int64_t Sk)
     w.vsf = off; off = align_up(off + static_cast<size_t>(B) * Hkv * (w.Sk_pad / kTile) * kSfBytes, 1024);
     w.total = off;
     return w;
+}
+
+// what a call needs: the few-row path has a layout of its own in the same workspace
+size_t workspace_bytes_for(int B, int Hq, int Hkv, int64_t Sq, int64_t Sk)
+{
+    size_t total = plan_workspace(B, Hq, Hkv, Sq, Sk).total;
+    if (use_few(Hq, Hkv, Sq)) {
+        const int64_t heads = static_cast<int64_t>(B) * Hkv;
+        const size_t few = 1024 + plan_few(heads * few_chunks(Sk), heads, heads * ((Sk + kTile - 1) / kTile * kTile),
+                                           static_cast<int>(Hq / Hkv * Sq)).total;
+        if (few > total) total = few;
+    }
+    return total;
 }
 
 bool shape_ok(int B, int Hq, int Hkv, int64_t Sq, int64_t Sk, int d)
@@ -719,6 +731,13 @@ cudaError_t launch_main(bool debug, bool fix8, dim3 grid, size_t smem, cudaStrea
 // the unpacked one bit for bit.
 bool use_packed_tile(int Hq, int Hkv, int64_t Sq) { return Hq / Hkv > 1 && static_cast<int64_t>(Hq / Hkv) * Sq <= kTile; }
 
+// At most kFewMaxRows query rows per KV group: K and V are read once whatever the kernel does, so the path that quantises
+// them on the way to the tensor core takes over (attention_few.cu).  Depends on the sequence's own shape alone, so that a
+// sequence takes the same path by itself and in a packed batch.
+bool use_few(int Hq, int Hkv, int64_t Sq) { return static_cast<int64_t>(Hq / Hkv) * Sq <= kFewMaxRows; }
+
+int64_t few_chunks(int64_t Sk) { return ((Sk + kTile - 1) / kTile + kFewChunkTiles - 1) / kFewChunkTiles; }
+
 cudaError_t launch_forward(int producer, bool debug, bool fix8, int64_t items, cudaStream_t stream, const CUtensorMap& mq,
                            const CUtensorMap& mk, const CUtensorMap& mv, const FwdParams& P)
 {
@@ -765,14 +784,36 @@ efq_status_t attention_impl(const void* q, const void* k, const void* v, float* 
     auto mis = [](const void* p, uintptr_t a) { return (reinterpret_cast<uintptr_t>(p) & (a - 1)) != 0; };
     if (mis(q, 16) || mis(k, 16) || mis(v, 16) || mis(o, 16)) return EFQ_ERR_ALIGNMENT;
     const Workspace w = plan_workspace(B, Hq, Hkv, Sq, Sk);
-    if (!workspace || workspace_bytes < w.total) return EFQ_ERR_WORKSPACE;
+    if (!workspace || workspace_bytes < workspace_bytes_for(B, Hq, Hkv, Sq, Sk)) return EFQ_ERR_WORKSPACE;
     if (mis(workspace, 256)) return EFQ_ERR_ALIGNMENT;
     const efq_status_t dev_st = check_device();
     if (dev_st != EFQ_OK) return dev_st;
 
     uint8_t* ws = static_cast<uint8_t*>(workspace);
-    const bool packed = use_packed_tile(Hq, Hkv, Sq);
     const int G = Hq / Hkv;
+    if (do_quantize && do_forward && !inject_skip_loads && use_few(Hq, Hkv, Sq)) {
+        FewParams F{};
+        F.q = static_cast<const __nv_bfloat16*>(q); F.k = static_cast<const __nv_bfloat16*>(k); F.v = static_cast<const __nv_bfloat16*>(v);
+        F.o = o;
+        F.Hkv = Hkv; F.G = G; F.causal = causal ? 1 : 0;
+        F.Sq = static_cast<int32_t>(Sq); F.Sk = static_cast<int32_t>(Sk); F.Sk_pad = static_cast<int32_t>(w.Sk_pad);
+        F.dense_chunks = static_cast<int32_t>(few_chunks(Sk));
+        F.q_row = 128; F.q_head = Sq * 128; F.q_seq = Hq * F.q_head;
+        F.k_row = 128; F.k_head = Sk * 128; F.k_seq = Hkv * F.k_head;
+        F.row_cap = static_cast<int32_t>(G * Sq);
+        F.n_counters = B * Hkv;
+        F.rescale_threshold = rescale_threshold;
+        F.K = producer == 3 ? make_producer_consts_lut(softmax_scale) : make_producer_consts(softmax_scale, tau, h);
+        const int64_t units = static_cast<int64_t>(B) * Hkv * F.dense_chunks;
+        const FewPlan fp = plan_few(units, F.n_counters, static_cast<int64_t>(B) * Hkv * w.Sk_pad, F.row_cap);
+        F.scores = reinterpret_cast<float*>(ws + 1024 + fp.scores); F.block_max = reinterpret_cast<float*>(ws + 1024 + fp.block_max);
+        F.partials = reinterpret_cast<float*>(ws + 1024 + fp.partials); F.counters = reinterpret_cast<uint32_t*>(ws + 1024 + fp.counters);
+        F.status = reinterpret_cast<uint32_t*>(ws);
+        F.has_dbg = debug != nullptr ? 1 : 0;
+        if (debug != nullptr) F.dbg = *debug;
+        return launch_few(producer, units, F, stream) == cudaSuccess ? EFQ_OK : EFQ_ERR_CUDA;
+    }
+    const bool packed = use_packed_tile(Hq, Hkv, Sq);
     const int64_t q_rows = packed ? static_cast<int64_t>(B) * Hkv * kTile : static_cast<int64_t>(B) * Hq * w.Sq_pad;
     if (do_quantize) {
         QuantSeg sq{}, sk{}, sv{};
@@ -829,10 +870,12 @@ efq_status_t attention_impl(const void* q, const void* k, const void* v, float* 
 // Q codes [rows of all sequences, 64 B] | Q scale tiles | K codes | K scale tiles |
 // V^T codes [Hkv * 128, sum of Sk_pad / 2 B] (the sequences side by side along the keys) | V scale tiles.
 struct VarlenPlan {
-    int n_active;                    // sequences with query and key tokens
+    int n_active;                    // sequences with query and key tokens that take the general path
+    int n_few, few_rows;             // ... and the few-row path (attention_few.cu); the most query rows of one of them
+    int64_t few_units, few_keys;     // their chunks times KV heads; their keys, padded to 128
     int64_t q_rows, k_rows, k_cols;  // rows of the Q and K code matrices, keys along V^T (all padded to 128)
     int64_t items, quant_ctas;
-    size_t tables, seqs_off, items_off, jobs_off, prefix_off, qc, qsf, kc, ksf, vt, vsf, total;
+    size_t tables, seqs_off, items_off, jobs_off, prefix_off, qc, qsf, kc, ksf, vt, vsf, few_table, few, total;
 };
 
 // checks the two prefix arrays and lays the workspace out; false with st set on bad input
@@ -847,6 +890,13 @@ bool plan_varlen(const int64_t* cu_q, const int64_t* cu_k, int n_seqs, int Hq, i
         const int64_t lq = cu_q[s + 1] - cu_q[s], lk = cu_k[s + 1] - cu_k[s];
         if (lq < 0 || lk < 0) { st = EFQ_ERR_INVALID_ARG; return false; }
         if (lq == 0 || lk == 0) continue;
+        if (use_few(Hq, Hkv, lq)) {
+            ++p.n_few;
+            p.few_rows = std::max(p.few_rows, static_cast<int>(Hq / Hkv * lq));
+            p.few_units += few_chunks(lk) * Hkv;
+            p.few_keys += (lk + kTile - 1) / kTile * kTile;
+            continue;
+        }
         const bool packed = use_packed_tile(Hq, Hkv, lq);
         const int64_t lq_pad = packed ? kTile : (lq + kTile - 1) / kTile * kTile, lk_pad = (lk + kTile - 1) / kTile * kTile;
         ++p.n_active;
@@ -858,7 +908,7 @@ bool plan_varlen(const int64_t* cu_q, const int64_t* cu_k, int n_seqs, int Hq, i
     }
     // 32-bit tile coordinates and grid sizes
     if (p.q_rows >= (1ll << 31) || p.k_rows >= (1ll << 31) || p.k_cols >= (1ll << 31) || p.items >= (1ll << 31) ||
-        p.quant_ctas >= (1ll << 31)) { st = EFQ_ERR_UNSUPPORTED; return false; }
+        p.quant_ctas >= (1ll << 31) || p.few_units >= (1ll << 31) || p.few_keys >= (1ll << 31)) { st = EFQ_ERR_UNSUPPORTED; return false; }
     size_t off = 1024;
     p.seqs_off = off;   off = align_up(off + sizeof(SeqDesc) * p.n_active, 256);
     p.items_off = off;  off = align_up(off + sizeof(ItemDesc) * static_cast<size_t>(p.items), 256);
@@ -871,6 +921,10 @@ bool plan_varlen(const int64_t* cu_q, const int64_t* cu_k, int n_seqs, int Hq, i
     p.ksf = off; off = align_up(off + static_cast<size_t>(p.k_rows / kTile) * kSfBytes, 1024);
     p.vt = off;  off = align_up(off + static_cast<size_t>(Hkv) * 128 * (p.k_cols / 2), 1024);
     p.vsf = off; off = align_up(off + static_cast<size_t>(Hkv) * (p.k_cols / kTile) * kSfBytes, 1024);
+    p.few_table = off;
+    if (p.n_few > kFewInlineSeqs) off = align_up(off + sizeof(FewSeq) * p.n_few, 1024);
+    p.few = off;
+    if (p.n_few > 0) off += plan_few(p.few_units, static_cast<int64_t>(p.n_few) * Hkv, p.few_keys * Hkv, p.few_rows).total;
     p.total = off;
     return true;
 }
@@ -881,7 +935,7 @@ bool plan_varlen(const int64_t* cu_q, const int64_t* cu_k, int n_seqs, int Hq, i
 extern "C" size_t efq_attention_workspace_bytes(int B, int Hq, int Hkv, int64_t Sq, int64_t Sk, int d)
 {
     if (!efq::shape_ok(B, Hq, Hkv, Sq, Sk, d)) return 0;
-    return efq::plan_workspace(B, Hq, Hkv, Sq, Sk).total;
+    return efq::workspace_bytes_for(B, Hq, Hkv, Sq, Sk);
 }
 
 // Producer ids inside the library: 0 = EFQ (affine rule), 1 / 2 = exp-then-quantize scale4 / scale6, 3 = EFQ-LUT,
@@ -1029,7 +1083,7 @@ extern "C" efq_status_t efq_attention_fwd_host_pipelined(const void* q_host, con
                                       causal, softmax_scale, producer == 3 ? 0 : producer, params, workspace,
                                       workspace_bytes, stream_compute);
     if (!efq::shape_ok(1, heads_per_chunk * group, heads_per_chunk, Sq, Sk, d)) return EFQ_ERR_UNSUPPORTED;
-    const size_t slot = efq::plan_workspace(1, heads_per_chunk * group, heads_per_chunk, Sq, Sk).total;
+    const size_t slot = efq::workspace_bytes_for(1, heads_per_chunk * group, heads_per_chunk, Sq, Sk);
     if (workspace_bytes < slot + 256) return EFQ_ERR_WORKSPACE;
     uint8_t* ws = static_cast<uint8_t*>(workspace);
     uint32_t* agg = reinterpret_cast<uint32_t*>(ws + slot);          // first problem seen by any chunk
@@ -1142,14 +1196,25 @@ extern "C" efq_status_t efq_attention_fwd_varlen(const void* q, const void* k, c
     const __nv_bfloat16* qb = static_cast<const __nv_bfloat16*>(q);
     const __nv_bfloat16* kb = static_cast<const __nv_bfloat16*>(k);
     const __nv_bfloat16* vb = static_cast<const __nv_bfloat16*>(v);
-    int64_t q_row = 0, k_row = 0, k_col = 0, n_items = 0, ctas = 0;
-    int a = 0;
+    int64_t q_row = 0, k_row = 0, k_col = 0, n_items = 0, ctas = 0, few_unit = 0, few_key = 0;
+    int a = 0, f = 0;
+    FewParams F{};
+    std::vector<FewSeq> few_long;            // more sequences than the kernel parameters hold
+    if (p.n_few > kFewInlineSeqs) few_long.resize(p.n_few);
+    FewSeq* const few_seqs = few_long.empty() ? F.inline_seqs : few_long.data();
     for (int i = 0; i < n_seqs; ++i) {
         const int64_t q0 = cu_seqlens_q[i], k0 = cu_seqlens_k[i];
         const int64_t lq = cu_seqlens_q[i + 1] - q0, lk = cu_seqlens_k[i + 1] - k0;
         if (lq == 0) continue;
         if (lk == 0) {               // no key at all: the rows are zero, as for a causal row that sees nothing
             if (cudaMemsetAsync(o + q0 * Hq * 128, 0, static_cast<size_t>(lq) * Hq * 128 * sizeof(float), s) != cudaSuccess) return EFQ_ERR_CUDA;
+            continue;
+        }
+        if (use_few(Hq, Hkv, lq)) {
+            few_seqs[f++] = FewSeq{static_cast<int32_t>(lq), static_cast<int32_t>(lk), static_cast<int32_t>(q0), static_cast<int32_t>(k0),
+                                   static_cast<int32_t>(few_key), static_cast<int32_t>(few_unit)};
+            few_key += (lk + kTile - 1) / kTile * kTile;
+            few_unit += few_chunks(lk) * Hkv;
             continue;
         }
         const bool packed = use_packed_tile(Hq, Hkv, lq);
@@ -1194,6 +1259,28 @@ extern "C" efq_status_t efq_attention_fwd_varlen(const void* q, const void* k, c
         k_col += lk_pad;
         ++a;
     }
+    if (p.n_few > 0) {
+        F.q = qb; F.k = kb; F.v = vb; F.o = o;
+        F.Hkv = Hkv; F.G = G; F.causal = causal ? 1 : 0;
+        F.n_seqs = p.n_few;
+        F.q_head = 128; F.q_row = static_cast<int64_t>(Hq) * 128;
+        F.k_head = 128; F.k_row = static_cast<int64_t>(Hkv) * 128;
+        F.row_cap = p.few_rows;
+        F.n_counters = p.n_few * Hkv;
+        F.rescale_threshold = threshold;
+        F.K = producer == 3 ? make_producer_consts_lut(softmax_scale) : make_producer_consts(softmax_scale, tau, h);
+        const FewPlan fp = plan_few(p.few_units, F.n_counters, p.few_keys * Hkv, p.few_rows);
+        uint8_t* const fw = ws + p.few;
+        F.scores = reinterpret_cast<float*>(fw + fp.scores); F.block_max = reinterpret_cast<float*>(fw + fp.block_max);
+        F.partials = reinterpret_cast<float*>(fw + fp.partials); F.counters = reinterpret_cast<uint32_t*>(fw + fp.counters);
+        F.status = reinterpret_cast<uint32_t*>(ws);
+        if (!few_long.empty()) {
+            if (cudaMemcpyAsync(ws + p.few_table, few_long.data(), sizeof(FewSeq) * few_long.size(), cudaMemcpyHostToDevice, s) != cudaSuccess) return EFQ_ERR_CUDA;
+            F.seqs = reinterpret_cast<const FewSeq*>(ws + p.few_table);
+        }
+        if (launch_few(producer, p.few_units, F, s) != cudaSuccess) return EFQ_ERR_CUDA;
+        if (p.n_active == 0) return EFQ_OK;
+    }
     if (p.n_active == 0)             // nothing to launch: the status word still has to read "no problem"
         return cudaMemsetAsync(ws, 0, 4, s) == cudaSuccess ? EFQ_OK : EFQ_ERR_CUDA;
     prefix[3 * p.n_active] = static_cast<int32_t>(ctas);
@@ -1201,7 +1288,7 @@ extern "C" efq_status_t efq_attention_fwd_varlen(const void* q, const void* k, c
     // Pageable host memory: the call returns once the bytes sit in the driver's staging area, so the vector may go.
     if (cudaMemcpyAsync(ws + 1024, tables.data(), p.tables, cudaMemcpyHostToDevice, s) != cudaSuccess) return EFQ_ERR_CUDA;
     if (launch_quantize_jobs(reinterpret_cast<const QuantJob*>(ws + p.jobs_off), reinterpret_cast<const int32_t*>(ws + p.prefix_off),
-                             3 * p.n_active, ctas, reinterpret_cast<uint32_t*>(ws), s) != cudaSuccess)
+                             3 * p.n_active, ctas, p.n_few > 0 ? nullptr : reinterpret_cast<uint32_t*>(ws), s) != cudaSuccess)
         return EFQ_ERR_CUDA;
 
     CUtensorMap mq, mk, mv;

@@ -6,6 +6,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "efq_common.cuh"
+
 namespace efq {
 
 // One operand of one sequence for the quantiser.  Rows of Q and K are quantised along d (blocks of 32), V along
@@ -35,6 +37,7 @@ struct QuantJob {
 // Q, K and V of one [B, H, S, d] problem (or one sequence) in one launch; also clears the 256 status words.
 cudaError_t launch_quantize_qkv(const QuantSeg& q, const QuantSeg& k, const QuantSeg& v, uint32_t* status, cudaStream_t stream);
 // The jobs of a packed batch in one launch: jobs and first_cta (n_jobs + 1 prefix sums of CTAs) live in device memory.
+// status: the words to clear, null if an earlier launch of the call has cleared them.
 cudaError_t launch_quantize_jobs(const QuantJob* jobs, const int32_t* first_cta, int n_jobs, int64_t total_ctas, uint32_t* status,
                                  cudaStream_t stream);
 // CTAs a job needs (256 threads each)
@@ -57,5 +60,46 @@ struct ItemDesc {
     int32_t head;            // query head, or KV head when packed
     int32_t pad;
 };
+
+// ------------------------------------------------------------------------------------------------
+// Few query rows (attention_few.cu): the query rows of a KV group, Hq / Hkv * Sq of them, are at most kFewMaxRows
+// ------------------------------------------------------------------------------------------------
+// 24 rows keep the scores in the workspace below the size of the MXFP4 copies that the general path would need there.
+constexpr int kFewMaxRows = 24;
+// Keys of a chunk: 4 tiles are 256 KB of K and V, enough to hide a CTA's start behind its neighbours, and small enough
+// that a single 8 K context spreads over the whole chip.
+constexpr int kFewChunkTiles = 4;
+constexpr int kFewInlineSeqs = 128;      // sequence tables up to this size travel as kernel parameters
+
+struct FewSeq {
+    int32_t Sq, Sk;          // tokens of the sequence
+    int32_t q0, k0;          // its first query and key token
+    int32_t k_pad0;          // keys of the sequences before it, each padded to 128
+    int32_t first_unit;      // chunks times KV heads of the sequences before it
+};
+
+struct FewParams {
+    const __nv_bfloat16 *q, *k, *v;
+    float* o;                                  // strides as q
+    int32_t Hkv, G, causal;
+    int32_t n_seqs;                            // packed batch: sequences in the table; 0: dense [B, H, S, d]
+    int32_t Sq, Sk, Sk_pad, dense_chunks;      // dense only
+    int64_t q_seq, q_head, q_row, k_seq, k_head, k_row;    // strides in elements
+    int32_t row_cap;                           // query rows the workspace holds per KV head (the most of any sequence)
+    int32_t n_counters;
+    float rescale_threshold;
+    ProducerConsts K;
+    float *scores, *block_max, *partials;      // workspace
+    uint32_t *counters, *status;
+    int32_t has_dbg;
+    efq_debug_t dbg;
+    const FewSeq* seqs;                        // device table; null: inline_seqs
+    FewSeq inline_seqs[kFewInlineSeqs];
+};
+
+struct FewPlan { size_t scores, block_max, partials, counters, total; };   // offsets from a 1024-byte aligned base
+FewPlan plan_few(int64_t units, int64_t heads, int64_t keys_padded_all_heads, int rows);
+// units: chunks times KV heads of all sequences.  Clears the status words.
+cudaError_t launch_few(int producer, int64_t units, const FewParams& P, cudaStream_t stream);
 
 }  // namespace efq

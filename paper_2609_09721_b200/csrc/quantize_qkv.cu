@@ -18,46 +18,9 @@
 
 #include "efq_common.cuh"
 #include "efq_internal.cuh"
+#include "mxfp4.cuh"
 
 namespace efq {
-
-__device__ __forceinline__ float bf16_bits_to_float(uint32_t b) { return __uint_as_float(b << 16); }
-
-// 32 bf16 values (as 16 packed 32-bit words, element 2u in the low half) -> 16 bytes of codes + scale byte
-__device__ __forceinline__ void mxfp4_block(const uint32_t (&w)[16], uint4& codes, uint32_t& byte)
-{
-    uint32_t amax = 0;   // bf16 magnitudes compare like unsigned integers
-#pragma unroll
-    for (int i = 0; i < 16; ++i) {
-        amax = max(amax, w[i] & 0x7fffu);
-        amax = max(amax, (w[i] >> 16) & 0x7fffu);
-    }
-    if (amax == 0) {
-        codes = make_uint4(0, 0, 0, 0);
-        byte = 0;
-        return;
-    }
-    int e = static_cast<int>(amax >> 7) - 127 - 2;   // exponent field of the largest magnitude, minus 2
-    e = max(e, -127);
-    const float s = __uint_as_float(static_cast<uint32_t>(127 - e) << 23);   // 2^-e, field in [2, 254]
-    uint32_t out[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        uint32_t word = 0;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            uint32_t v = w[q * 4 + i];
-            float lo = bf16_bits_to_float(v & 0xffffu) * s;
-            float hi = bf16_bits_to_float(v >> 16) * s;
-            word |= (cvt_e2m1x2(lo, hi) & 0xffu) << (8 * i);
-        }
-        out[q] = word;
-    }
-    codes = make_uint4(out[0], out[1], out[2], out[3]);
-    byte = static_cast<uint32_t>(e + 127);
-}
-
-__device__ __forceinline__ uint32_t sf_tile_offset(uint32_t r, uint32_t b) { return (r & 31u) * 16u + (r >> 5) * 4u + b; }
 
 // One thread per (row, 32-wide block along d); d = 128.  t counts (padded row, block) pairs of the job.  The four
 // scale bytes of a row are gathered by shuffles and stored as one word by the thread of block 0.
@@ -156,7 +119,7 @@ __global__ void __launch_bounds__(256) quantize_jobs_kernel(const QuantJob* __re
                                                             int n_jobs, uint32_t* status)
 {
     const int cta = blockIdx.x;
-    if (cta == 0) status[threadIdx.x] = 0u;
+    if (cta == 0 && status != nullptr) status[threadIdx.x] = 0u;
     int lo = 0, hi = n_jobs;                  // first_cta[lo] <= cta < first_cta[hi]
     while (hi - lo > 1) {
         const int mid = (lo + hi) >> 1;
