@@ -7,11 +7,16 @@
 //                       maxima of the 32-key blocks go to the workspace (4 bytes per row and key against 256 of K)
 //   few_values_kernel   the running maximum of every row before the chunk from the block maxima; Algorithm 1 with
 //                       thread = key (a microscaling block is a warp); V tile -> MXFP4 operand, transposed;
-//                       O^T[channel, row] += V^^T P~; the last chunk of a head to finish adds the chunks up
+//                       O^T[channel, row] += V^^T P~; partial sums of a chunk to the workspace
+//   few_merge_kernel    the chunks of a row added up
 //
-// The KV range is cut into chunks of kChunkTiles tiles whatever the batch, so the result of a sequence does not depend on
+// The KV range is cut into chunks by a rule on the sequence's own shape, so the result of a sequence does not depend on
 // its neighbours.  The shifted scores use the running maximum over all keys up to the tile (Algorithm 2), which the first
 // kernel makes available to every chunk: the codes are those of the one-pass forward, bit for bit.
+//
+// A block takes one chunk; several blocks per SM hide the latencies of one another's tiles (load, quantise, MMA,
+// accumulator).  Loads by TMA with a role per warp (two blocks of 16 warps) were built too and are no faster: the short
+// dependent sequences of the code warps then wait behind the quantisers of their scheduler.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -26,35 +31,37 @@ namespace {
 
 constexpr int kTile = 128;
 constexpr int kFewThreads = 256;
-constexpr int kChunkTiles = kFewChunkTiles;
+constexpr int kStateRing = 4;
 constexpr uint32_t kFewTmemCols = 128;      // four CTAs per SM share the 512 columns
 constexpr uint32_t kColD = 0;               // 2 x 32
 constexpr uint32_t kColSfA = 64;            // 2 x 4
 constexpr uint32_t kColSfB = 72;            // 2 x 4
 
+// The A operand (K or V^T codes of a tile) without swizzle: 8 rows x 16 bytes (a 32-element block) form a core matrix of
+// 128 bytes.  Strides that are no multiple of 128 keep the stores free of bank conflicts: lanes that write one row of
+// eight row groups (V^T) or eight rows of one block (K) meet 32 different banks.
+constexpr uint32_t kARowGroup = 144, kABlock = 16 * kARowGroup + 32;
+__device__ __forceinline__ uint32_t a_offset(uint32_t row, uint32_t blk) { return blk * kABlock + (row >> 3) * kARowGroup + (row & 7u) * 16u; }
+
 // One (sequence, KV head, chunk) of the grid.  Heads run fastest: the CTAs in flight read neighbouring heads of the same
 // tokens, which lie side by side in a token-major cache.
 struct Unit {
     int seq, head, chunk, n_chunks;
-    int Sq, Sk, n_tiles;       // n_tiles: tiles that any row sees
+    int Sq, Sk, Sk_pad, j0, j1;
     const __nv_bfloat16 *q, *k, *v;
     float* o;
     int64_t s_off;             // first score of the (sequence, head) in the workspace, rows Sk_pad apart
-    int Sk_pad;
 };
 
-__device__ __forceinline__ Unit find_unit(const FewParams& P)
+__device__ __forceinline__ Unit find_unit(const FewParams& P, int id)
 {
     Unit u;
-    int id = static_cast<int>(blockIdx.x);
     int64_t kp;
     if (P.n_seqs == 0) {                    // [B, H, S, d]
-        const int n_chunks = P.dense_chunks;
         u.head = id % P.Hkv;
         id /= P.Hkv;
-        u.chunk = id % n_chunks;
-        u.seq = id / n_chunks;
-        u.n_chunks = n_chunks;
+        u.chunk = id % P.dense_chunks;
+        u.seq = id / P.dense_chunks;
         u.Sq = P.Sq; u.Sk = P.Sk;
         kp = static_cast<int64_t>(u.seq) * P.Sk_pad;
         u.q = P.q + u.seq * P.q_seq; u.k = P.k + u.seq * P.k_seq; u.v = P.v + u.seq * P.k_seq; u.o = P.o + u.seq * P.q_seq;
@@ -71,12 +78,14 @@ __device__ __forceinline__ Unit find_unit(const FewParams& P)
         u.head = id % P.Hkv;
         u.chunk = id / P.Hkv;
         u.Sq = s.Sq; u.Sk = s.Sk;
-        u.n_chunks = ((s.Sk + kTile - 1) / kTile + kChunkTiles - 1) / kChunkTiles;
-        kp = static_cast<int64_t>(s.k_pad0) ;
+        kp = s.k_pad0;
         u.q = P.q + s.q0 * P.q_row; u.k = P.k + s.k0 * P.k_row; u.v = P.v + s.k0 * P.k_row; u.o = P.o + s.q0 * P.q_row;
     }
-    u.Sk_pad = (u.Sk + kTile - 1) / kTile * kTile;
-    u.n_tiles = u.Sk_pad / kTile;
+    const int n_tiles = (u.Sk + kTile - 1) / kTile, per = few_chunk_tiles(n_tiles, P.G * u.Sq);
+    u.n_chunks = (n_tiles + per - 1) / per;
+    u.j0 = u.chunk * per;
+    u.j1 = min(u.j0 + per, n_tiles);
+    u.Sk_pad = n_tiles * kTile;
     u.q += static_cast<int64_t>(u.head) * P.G * P.q_head;
     u.o += static_cast<int64_t>(u.head) * P.G * P.q_head;
     u.k += u.head * P.k_head;
@@ -87,7 +96,7 @@ __device__ __forceinline__ Unit find_unit(const FewParams& P)
 
 // Bounded wait for a completion of this CTA's own MMAs.  On expiry the status word takes the error; the CTA carries on
 // with whatever the accumulator holds, so that every thread still meets the block's barriers.
-__device__ __forceinline__ void wait_mma(uint64_t* bar, uint32_t parity, uint32_t* status)
+__device__ __forceinline__ void wait_done(uint64_t* bar, uint32_t parity, uint32_t* status)
 {
     for (int i = 0; i < 20000; ++i)
         if (ptx::mbar_try_wait_suspend(bar, parity, 50000u)) return;
@@ -101,30 +110,33 @@ __device__ __forceinline__ float warp_max(float x)
     return m;
 }
 
-// N consecutive columns (a multiple of 4) of this thread's TMEM lane
+// N consecutive columns (a multiple of 8) of this thread's TMEM lane
 template <int N>
-__device__ __forceinline__ void tmem_ld_cols(uint32_t addr, float (&d)[N])
+__device__ __forceinline__ void tmem_ld_cols(uint32_t addr, float (&r)[N])
 {
 #pragma unroll
-    for (int i = 0; i < N; i += 4)
-        asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
-                     : "=f"(d[i]), "=f"(d[i + 1]), "=f"(d[i + 2]), "=f"(d[i + 3]) : "r"(addr + i) : "memory");
+    for (int o = 0; o < N; o += 8)
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                     : "=f"(r[o]), "=f"(r[o + 1]), "=f"(r[o + 2]), "=f"(r[o + 3]), "=f"(r[o + 4]), "=f"(r[o + 5]), "=f"(r[o + 6]), "=f"(r[o + 7])
+                     : "r"(addr + o) : "memory");
 }
 
 struct __align__(1024) FewSmem {
-    uint8_t a[2][kTile * 64];       // K or V^T codes of a tile
     uint8_t b[2][32 * 64];          // Q codes ([0] only), or the probability operand of a tile
+    uint8_t a[2][4 * kABlock];      // K or V^T codes of a tile
     uint8_t sf_a[2][512];
     uint8_t sf_b[2][512];
-    float alpha[4][32];             // [tile mod 4][row]: a warp may be a tile ahead of one that still reads the tile before
-    float m_start[32];
-    float lsum[4][32];              // [key block of the tile][row]
-    float bmax[kChunkTiles * 4][32];
+    // row state of a tile [tile mod 4][row]: raw running maximum, the same in scaled units, the rescale factor, and per key
+    // block the additive term of the code rule and the scale byte
+    float m_raw[kStateRing][32], m_s[kStateRing][32], alpha[kStateRing][32];
+    float par[kStateRing][4][32];
+    uint32_t byte[kStateRing][4][32];
+    float4 bmax[kFewMaxChunk][32];  // [tile of the chunk][row]: its block maxima
     uint64_t mma_done[2];
     uint32_t tmem_base;
-    uint32_t is_last;
 };
 
+// Operand rows past the last query row are never written: they only reach accumulator columns that nobody reads.
 __device__ __forceinline__ void few_setup(FewSmem* sm, int warp)
 {
     if (warp == 0) ptx::tmem_alloc(&sm->tmem_base, kFewTmemCols);
@@ -133,9 +145,6 @@ __device__ __forceinline__ void few_setup(FewSmem* sm, int warp)
         ptx::mbar_init(&sm->mma_done[1], 1);
         ptx::mbar_init_fence();
     }
-    // rows and blocks that nobody writes: zero codes, byte 0
-    for (int i = threadIdx.x; i < static_cast<int>(sizeof(sm->b) / 16); i += kFewThreads) reinterpret_cast<uint4*>(sm->b)[i] = make_uint4(0, 0, 0, 0);
-    if (threadIdx.x < 64) reinterpret_cast<uint4*>(sm->sf_b)[threadIdx.x] = make_uint4(0, 0, 0, 0);
 }
 
 // D[128, N] = A B^T of one tile: two K = 64 steps, a fresh accumulator
@@ -146,110 +155,121 @@ __device__ __forceinline__ void few_mma(FewSmem* sm, uint32_t tmem, int buf, int
     const uint32_t sfa = tmem + kColSfA + 4 * buf, sfb = tmem + kColSfB + 4 * b_buf, d = tmem + kColD + 32 * buf;
     ptx::tmem_cp_sf(sfa, d_sf + (ptx::smem_u32(sm->sf_a[buf]) >> 4));
     ptx::tmem_cp_sf(sfb, d_sf + (ptx::smem_u32(sm->sf_b[b_buf]) >> 4));
-    const uint64_t da = d_sw64 + (ptx::smem_u32(sm->a[buf]) >> 4), db = d_sw64 + (ptx::smem_u32(sm->b[b_buf]) >> 4);
+    const uint64_t da = ptx::smem_desc(ptx::smem_u32(sm->a[buf]), kABlock, kARowGroup, ptx::kLayoutNone), db = d_sw64 + (ptx::smem_u32(sm->b[b_buf]) >> 4);
     ptx::mma_mxf4(d, da, db, ptx::mxf4_idesc(n, 0), sfa, sfb, 0u);
-    ptx::mma_mxf4(d, da + 2, db + 2, ptx::mxf4_idesc(n, 2), sfa | (2u << 30), sfb | (2u << 30), 1u);
+    ptx::mma_mxf4(d, da + (2 * kABlock >> 4), db + 2, ptx::mxf4_idesc(n, 2), sfa | (2u << 30), sfb | (2u << 30), 1u);
     ptx::mma_commit(&sm->mma_done[buf]);
 }
 
 // N: query rows rounded up to a multiple of 8 (the N of the MMA)
 template <int N>
-__global__ void __launch_bounds__(kFewThreads, 4) few_scores_kernel(const __grid_constant__ FewParams P)
+__global__ void __launch_bounds__(kFewThreads, N <= 8 ? 4 : 3) few_scores_kernel(const __grid_constant__ FewParams P)
 {
     __shared__ FewSmem smem;
     FewSmem* const sm = &smem;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const Unit u = find_unit(P);
-    const int R = P.G * u.Sq;
-    if (blockIdx.x == 0) {                   // the status words, and the counters of the chunks that have finished
-        P.status[tid] = 0u;
-        for (int i = tid; i < P.n_counters; i += kFewThreads) P.counters[i] = 0u;
-    }
     few_setup(sm, warp);
-    __syncthreads();
-    // Q: one thread per (row, block)
-    if (tid < 4 * N) {
-        const int row = tid >> 2, blk = tid & 3;
-        uint32_t byte = 0;
-        if (row < R) {
-            const int g = row / u.Sq, tok = row - g * u.Sq;
-            const uint4* src = reinterpret_cast<const uint4*>(u.q + g * P.q_head + tok * P.q_row + blk * 32);
-            uint32_t w[16];
+    asm volatile("griddepcontrol.wait;" ::: "memory");                // the kernels before: inputs, and the workspace of an earlier call
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const Unit u = find_unit(P, static_cast<int>(blockIdx.x));
+    const int R = P.G * u.Sq;
+    if (blockIdx.x == 0) P.status[tid] = 0u;
+    // K: a quad of lanes takes a key, a lane every fourth 16-byte piece of it - a load instruction reads 64 contiguous
+    // bytes of every key - and so a quarter of each of the four blocks
+    const int quad = tid & 3, key_in_tile = tid >> 2;
+    uint4 kk[2][4];
+    auto load_k = [&](int j) {
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const uint4 x = __ldg(src + i);
-                w[4 * i] = x.x; w[4 * i + 1] = x.y; w[4 * i + 2] = x.z; w[4 * i + 3] = x.w;
-            }
-            uint4 c;
-            mxfp4_block(w, c, byte);
-            *reinterpret_cast<uint4*>(sm->b[0] + code_tile_offset(row, blk)) = c;
-            sm->sf_b[0][sf_tile_offset(row, blk)] = static_cast<uint8_t>(byte);
+        for (int h = 0; h < 2; ++h) {
+            const int key = j * kTile + key_in_tile + 64 * h;
+            const uint4* src = reinterpret_cast<const uint4*>(u.k + key * P.k_row) + quad;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) kk[h][i] = key < u.Sk ? __ldcs(src + 4 * i) : make_uint4(0, 0, 0, 0);
         }
+    };
+    load_k(u.j0);
+    // Q: one thread per (row, block)
+    for (int t = tid; t < 4 * R; t += kFewThreads) {
+        const int row = t >> 2, blk = t & 3, g = row / u.Sq;
+        const uint4* src = reinterpret_cast<const uint4*>(u.q + g * P.q_head + (row - g * u.Sq) * P.q_row + blk * 32);
+        uint32_t w[16];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const uint4 x = __ldg(src + i);
+            w[4 * i] = x.x; w[4 * i + 1] = x.y; w[4 * i + 2] = x.z; w[4 * i + 3] = x.w;
+        }
+        uint4 c;
+        uint32_t byte;
+        mxfp4_block(w, c, byte);
+        *reinterpret_cast<uint4*>(sm->b[0] + code_tile_offset(row, blk)) = c;
+        sm->sf_b[0][sf_tile_offset(row, blk)] = static_cast<uint8_t>(byte);
     }
     ptx::tc_fence_before_sync();
     __syncthreads();
     ptx::tc_fence_after_sync();
     const uint32_t tmem = sm->tmem_base;
-    const int j0 = u.chunk * kChunkTiles, j1 = min(j0 + kChunkTiles, u.n_tiles);
-    float* const S = P.scores + u.s_off;
-    float* const bm = P.block_max + u.s_off / 32;
     const int nblk = u.Sk_pad / 32;
-    constexpr int NH = N / 2;                // rows per half of the CTA; each half has one warp per 32 keys
-    const int quarter = warp & 3, r_first = (warp >> 2) * NH;
+    const int quarter = warp & 3, half = warp >> 2;      // 32 keys of the tile; rows 2 i + half
+    const int shift = P.causal ? u.Sk - u.Sq : u.Sk;     // key <= token + shift; without a mask every key of the sequence
 
-    // raw scores of a finished tile: thread = key
+    // raw scores of a finished tile: thread = key, two rows of the half side by side
     auto put_scores = [&](int j) {
-        const int buf = j & 1;
-        wait_mma(&sm->mma_done[buf], static_cast<uint32_t>((j - j0) >> 1) & 1u, P.status);
+        const int buf = (j - u.j0) & 1;
+        wait_done(&sm->mma_done[buf], static_cast<uint32_t>(j - u.j0) >> 1 & 1u, P.status);
         ptx::tc_fence_after_sync();
-        float s[NH];
-        tmem_ld_cols<NH>(tmem + (static_cast<uint32_t>(quarter * 32) << 16) + kColD + 32 * buf + r_first, s);
+        float s[N];
+        tmem_ld_cols<N>(tmem + (static_cast<uint32_t>(quarter * 32) << 16) + kColD + 32 * buf, s);
         ptx::tmem_wait_ld();
         ptx::tc_fence_before_sync();
         const int key = j * kTile + quarter * 32 + lane;
+        float* const dst = P.scores + u.s_off + key;
+        float* const dst_max = P.block_max + u.s_off / 32 + (key >> 5);
 #pragma unroll
-        for (int i = 0; i < NH; ++i) {
-            const int row = r_first + i;
+        for (int i = 0; i < N; i += 4) {
+            const int row = i + half;
             if (row < R) {
-                const int tok = row % u.Sq;
-                const int limit = P.causal ? min(tok + u.Sk - u.Sq, u.Sk - 1) : u.Sk - 1;
-                const float x = key <= limit ? s[i] : -INFINITY;
-                S[static_cast<int64_t>(row) * u.Sk_pad + key] = x;
-                const float m = warp_max(x);
-                if (lane == 0) bm[static_cast<int64_t>(row) * nblk + (key >> 5)] = m;
+                const float x0 = key < u.Sk && key <= row % u.Sq + shift ? (half ? s[i + 1] : s[i]) : -INFINITY;
+                const float x1 = key < u.Sk && key <= (row + 2) % u.Sq + shift ? (half ? s[i + 3] : s[i + 2]) : -INFINITY;
+                const float m0 = warp_max(x0), m1 = warp_max(x1);
+                dst[row * u.Sk_pad] = x0;
+                if (lane == 0) dst_max[row * nblk] = m0;
+                if (row + 2 < R) {
+                    dst[(row + 2) * u.Sk_pad] = x1;
+                    if (lane == 0) dst_max[(row + 2) * nblk] = m1;
+                }
             }
         }
     };
 
-    for (int j = j0; j < j1; ++j) {
-        const int buf = j & 1;
-        // two (key, block) pairs per thread; both loads set out before the tile before is finished with
-        uint32_t w[2][16];
+    for (int j = u.j0; j < u.j1; ++j) {
+        const int buf = (j - u.j0) & 1;
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-            const int key = j * kTile + (tid >> 2) + 64 * h;
-            const uint4* src = reinterpret_cast<const uint4*>(u.k + key * P.k_row + (tid & 3) * 32);
+            const int row = key_in_tile + 64 * h;
+            uint32_t m[4];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const uint4 x = key < u.Sk ? __ldcs(src + i) : make_uint4(0, 0, 0, 0);
-                w[h][4 * i] = x.x; w[h][4 * i + 1] = x.y; w[h][4 * i + 2] = x.z; w[h][4 * i + 3] = x.w;
+            for (int b = 0; b < 4; ++b)
+                m[b] = bf16x2_absmax(bf16x2_absmax(kk[h][b].x, kk[h][b].y), bf16x2_absmax(kk[h][b].z, kk[h][b].w));
+            // two blocks in one register (low half, high half), then over the quad
+            uint32_t t0 = bf16x2_absmax(__byte_perm(m[0], m[1], 0x5410), __byte_perm(m[0], m[1], 0x7632));
+            uint32_t t1 = bf16x2_absmax(__byte_perm(m[2], m[3], 0x5410), __byte_perm(m[2], m[3], 0x7632));
+            t0 = bf16x2_absmax(t0, __shfl_xor_sync(0xffffffffu, t0, 1));
+            t1 = bf16x2_absmax(t1, __shfl_xor_sync(0xffffffffu, t1, 1));
+            t0 = mxfp4_fields(bf16x2_absmax(t0, __shfl_xor_sync(0xffffffffu, t0, 2)));
+            t1 = mxfp4_fields(bf16x2_absmax(t1, __shfl_xor_sync(0xffffffffu, t1, 2)));
+            const uint32_t s01 = mxfp4_scales(t0), s23 = mxfp4_scales(t1);
+#pragma unroll
+            for (int b = 0; b < 4; ++b) {
+                const uint32_t s2 = __byte_perm(b < 2 ? s01 : s23, 0u, (b & 1) ? 0x3232 : 0x1010);
+                const uint32_t w0 = bf16x2_mul(kk[h][b].x, s2), w1 = bf16x2_mul(kk[h][b].y, s2), w2 = bf16x2_mul(kk[h][b].z, s2), w3 = bf16x2_mul(kk[h][b].w, s2);
+                *reinterpret_cast<uint32_t*>(sm->a[buf] + a_offset(row, b) + quad * 4) =
+                    e2m1_word(bf16_lo(w0), bf16_hi(w0), bf16_lo(w1), bf16_hi(w1), bf16_lo(w2), bf16_hi(w2), bf16_lo(w3), bf16_hi(w3));
             }
+            if (quad == 0)
+                *reinterpret_cast<uint32_t*>(sm->sf_a[buf] + sf_tile_offset(row, 0)) =
+                    mxfp4_byte_lo(t0) | mxfp4_byte_hi(t0) << 8 | mxfp4_byte_lo(t1) << 16 | mxfp4_byte_hi(t1) << 24;
         }
-        if (j > j0) put_scores(j - 1);
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const uint32_t row = static_cast<uint32_t>(tid >> 2) + 64u * h;
-            uint4 c;
-            uint32_t byte;
-            mxfp4_block(w[h], c, byte);
-            *reinterpret_cast<uint4*>(sm->a[buf] + code_tile_offset(row, tid & 3)) = c;
-            uint32_t word = byte;
-            word |= __shfl_down_sync(0xffffffffu, byte, 1) << 8;
-            word |= __shfl_down_sync(0xffffffffu, byte, 2) << 16;
-            word |= __shfl_down_sync(0xffffffffu, byte, 3) << 24;
-            if ((tid & 3) == 0) *reinterpret_cast<uint32_t*>(sm->sf_a[buf] + sf_tile_offset(row, 0)) = word;
-        }
+        if (j + 1 < u.j1) load_k(j + 1);
         ptx::fence_proxy_async_smem();
         ptx::tc_fence_before_sync();
         __syncthreads();
@@ -258,8 +278,9 @@ __global__ void __launch_bounds__(kFewThreads, 4) few_scores_kernel(const __grid
             if (ptx::elect_one()) few_mma(sm, tmem, buf, 0, N);
             __syncwarp();
         }
+        if (j > u.j0) put_scores(j - 1);
     }
-    put_scores(j1 - 1);
+    put_scores(u.j1 - 1);
     ptx::tc_fence_before_sync();
     __syncthreads();
     if (warp == 0) ptx::tmem_dealloc(tmem, kFewTmemCols);
@@ -293,173 +314,228 @@ __device__ __forceinline__ uint32_t key_code(float r, float par, const ProducerC
     }
 }
 
+// Optional dump of one query head (all lanes): the row's score and code of this lane's key, the block's byte, the tile's maximum.
+__device__ __forceinline__ void few_dump(const FewParams& P, const Unit& u, int j, int quarter, int lane, int row, float score, uint32_t word,
+                                         float m_s, uint32_t byte)
+{
+    const int g = row / u.Sq, tok = row - g * u.Sq, blk = j * 4 + quarter, key = blk * 32 + lane;
+    if (u.head * P.G + g != P.dbg.head || tok < P.dbg.q_begin || tok >= P.dbg.q_end) return;
+    const int64_t drow = tok - P.dbg.q_begin, blocks = (u.Sk + 31) / 32;
+    if (P.dbg.raw_scores != nullptr && key < u.Sk) P.dbg.raw_scores[drow * u.Sk + key] = score;
+    if (P.dbg.row_max != nullptr && quarter == 0 && lane == 0) P.dbg.row_max[drow * (u.Sk_pad / kTile) + j] = m_s;
+    if (blk >= blocks) return;
+    if (P.dbg.codes != nullptr && (lane & 7) == 0) reinterpret_cast<uint32_t*>(P.dbg.codes + (drow * blocks + blk) * 16)[lane >> 3] = word;
+    if (P.dbg.scales != nullptr && lane == 0) P.dbg.scales[drow * blocks + blk] = static_cast<uint8_t>(byte);
+}
+
+// Row state of one tile, lane = row (one warp): the running maximum (Eq. rowmax-update), the factor its growth asks for
+// (Eq. alpha) and the scale rule of the four key blocks.
+template <int PRODUCER>
+__device__ __forceinline__ void few_row_state(FewSmem* sm, const FewParams& P, int t, int slot, float m_run, int lane)
+{
+    const float4 b4 = sm->bmax[t][lane];
+    const float bmax[4] = {b4.x, b4.y, b4.z, b4.w};
+    float m_new = fmaxf(m_run, fmaxf(fmaxf(bmax[0], bmax[1]), fmaxf(bmax[2], bmax[3])));
+    if (P.rescale_threshold > 0.0f && m_run != -INFINITY &&
+        !(__fsub_rn(__fmul_rn(P.K.sigma, m_new), __fmul_rn(P.K.sigma, m_run)) > P.rescale_threshold))
+        m_new = m_run;
+    const float m_s = __fmul_rn(P.K.sigma, m_new);
+    const bool grew = m_new > m_run && m_run != -INFINITY;
+    sm->m_raw[slot][lane] = m_new;
+    sm->m_s[slot][lane] = m_s;
+    sm->alpha[slot][lane] = grew ? ex2_approx(__fmul_rn(__fsub_rn(__fmul_rn(P.K.sigma, m_run), m_s), P.K.LOG2E)) : 1.0f;
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+        float par = m_s;
+        uint32_t byte = 0u;
+        if (PRODUCER == 0 || PRODUCER == 3) {
+            const BlockScale s = efq_block_scale(bmax[b], m_s, P.K);
+            par = s.Bb; byte = s.byte;
+        } else if (PRODUCER == 4 || PRODUCER == 5) {
+            const FoldedScale f = etq_folded_scale(bmax[b], m_s, P.K);
+            par = f.live ? f.c0e : -INFINITY;    // a block without a finite score: 2^-inf = 0 everywhere
+            byte = f.byte;
+        }
+        sm->par[slot][b][lane] = par;
+        sm->byte[slot][b][lane] = byte;
+    }
+}
+
 template <int N, int PRODUCER>
 __global__ void __launch_bounds__(kFewThreads, 3) few_values_kernel(const __grid_constant__ FewParams P)
 {
     __shared__ FewSmem smem;
     FewSmem* const sm = &smem;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const Unit u = find_unit(P);
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const Unit u = find_unit(P, static_cast<int>(blockIdx.x));
     const int R = P.G * u.Sq;
     few_setup(sm, warp);
-    const int j0 = u.chunk * kChunkTiles, j1 = min(j0 + kChunkTiles, u.n_tiles);
-    constexpr int NH = N / 2;
-    const int half = warp >> 2, quarter = warp & 3;
-    // V: a thread takes two channels of a 32-key block, a warp 128 contiguous bytes of every key
-    const int ch = (tid & 63) * 2, kb = tid >> 6;
-    uint32_t vv[32];
+    // V: a lane takes eight channels of eight neighbouring keys, a warp 64 channels of a 32-key block: full 128-byte lines
+    const int oct = lane & 7, kg = lane >> 3, v_half = warp & 1, v_blk = warp >> 1;
+    uint4 vv[8];
     auto load_v = [&](int j) {
-        const int key0 = j * kTile + kb * 32;
-        const uint32_t* src = reinterpret_cast<const uint32_t*>(u.v + key0 * P.k_row + ch);
-        const int64_t step = P.k_row / 2;
+        const int key0 = j * kTile + v_blk * 32 + kg * 8;
+        const uint4* src = reinterpret_cast<const uint4*>(u.v + key0 * P.k_row + v_half * 64 + oct * 8);
+        const int64_t step = P.k_row / 8;
+        if ((j + 1) * kTile <= u.Sk) {
 #pragma unroll
-        for (int i = 0; i < 32; ++i) vv[i] = key0 + i < u.Sk ? __ldcs(src + i * step) : 0u;
+            for (int i = 0; i < 8; ++i) vv[i] = __ldcs(src + i * step);
+        } else {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) vv[i] = key0 + i < u.Sk ? __ldcs(src + i * step) : make_uint4(0, 0, 0, 0);
+        }
     };
-    load_v(j0);                              // an input: needs nothing of the scores kernel
+    load_v(u.j0);       // an input: whatever produced it had finished before the scores kernel allowed this one to start
     asm volatile("griddepcontrol.wait;" ::: "memory");
 
-    // running maximum of every row before the chunk, and the chunk's own block maxima
-    const float* bm = P.block_max + u.s_off / 32;
+    // the chunk's block maxima and the running maximum of every row before the chunk
+    const float* const bm = P.block_max + u.s_off / 32;
     const int nblk = u.Sk_pad / 32;
+    for (int i = tid; i < R * (u.j1 - u.j0); i += kFewThreads) {
+        const int t = i / R, row = i - t * R;
+        sm->bmax[t][row] = __ldcg(reinterpret_cast<const float4*>(bm + row * nblk) + u.j0 + t);
+    }
     if (!(P.rescale_threshold > 0.0f)) {
         for (int row = warp; row < R; row += 8) {
             float m = -INFINITY;
-            for (int b = lane; b < j0 * 4; b += 32) m = fmaxf(m, __ldcg(bm + static_cast<int64_t>(row) * nblk + b));
+            for (int b = lane; b < u.j0; b += 32) {
+                const float4 x = __ldcg(reinterpret_cast<const float4*>(bm + row * nblk) + b);
+                m = fmaxf(fmaxf(m, fmaxf(x.x, x.y)), fmaxf(x.z, x.w));
+            }
             m = warp_max(m);
-            if (lane == 0) sm->m_start[row] = m;
+            if (lane == 0) sm->m_raw[kStateRing - 1][row] = m;
         }
     } else if (tid < R) {                    // optional policy: the kept maximum depends on the order of the tiles
         float m = -INFINITY;
-        for (int j = 0; j < j0; ++j) {
-            const float4 b = __ldcg(reinterpret_cast<const float4*>(bm + static_cast<int64_t>(tid) * nblk + 4 * j));
+        for (int j = 0; j < u.j0; ++j) {
+            const float4 b = __ldcg(reinterpret_cast<const float4*>(bm + tid * nblk) + j);
             const float c = fmaxf(m, fmaxf(fmaxf(b.x, b.y), fmaxf(b.z, b.w)));
             if (m == -INFINITY || __fsub_rn(__fmul_rn(P.K.sigma, c), __fmul_rn(P.K.sigma, m)) > P.rescale_threshold) m = c;
         }
-        sm->m_start[tid] = m;
+        sm->m_raw[kStateRing - 1][tid] = m;
     }
-    for (int i = tid; i < R * kChunkTiles * 4; i += kFewThreads) {
-        const int row = i / (kChunkTiles * 4), b = i % (kChunkTiles * 4);
-        if (j0 * 4 + b < nblk) sm->bmax[b][row] = __ldcg(bm + static_cast<int64_t>(row) * nblk + j0 * 4 + b);
-    }
+    // Codes: thread = key of block `quarter`; the warps of a half take the rows 2 i + half.  O^T: thread = channel.
+    constexpr int NH = N / 2;
+    const int quarter = warp & 3, half = warp >> 2;
+    const float* const S = P.scores + u.s_off + half * u.Sk_pad + quarter * 32 + lane;
+    float x[NH];
+    auto load_scores = [&](int j) {
+#pragma unroll
+        for (int i = 0; i < NH; ++i) x[i] = 2 * i + half < R ? __ldcg(S + j * kTile + 2 * i * u.Sk_pad) : -INFINITY;
+    };
+    load_scores(u.j0);
     ptx::tc_fence_before_sync();
     __syncthreads();
     ptx::tc_fence_after_sync();
     const uint32_t tmem = sm->tmem_base;
-    const float* const S = P.scores + u.s_off;
+    if (warp == 0 && lane < R) few_row_state<PRODUCER>(sm, P, 0, 0, sm->m_raw[kStateRing - 1][lane], lane);
+    __syncthreads();
 
-    // lane-parallel row state: lane i keeps the maximum and the denominator (this warp's key blocks) of row 2 i + half
-    const int my_row = 2 * lane + half;
-    const bool has_row = lane < NH && my_row < R;
-    float m_run = has_row ? sm->m_start[my_row] : -INFINITY;
+    const int my_row = 2 * lane + half;      // lane i keeps the denominator (of this block position) of row 2 i + half
+    const bool has_row = my_row < R;
     float l_run = 0.0f;
-    float acc[NH];                           // O^T: channel = TMEM lane of this thread, rows half * NH + i
+    float acc[NH];
 #pragma unroll
     for (int i = 0; i < NH; ++i) acc[i] = 0.0f;
-
-    auto add_tile = [&](int j) {
-        const int buf = j & 1;
-        wait_mma(&sm->mma_done[buf], static_cast<uint32_t>((j - j0) >> 1) & 1u, P.status);
+    auto add_tile = [&](int t) {
+        const int buf = t & 1;
+        wait_done(&sm->mma_done[buf], static_cast<uint32_t>(t >> 1) & 1u, P.status);
         ptx::tc_fence_after_sync();
-        float d[NH];
-        tmem_ld_cols<NH>(tmem + (static_cast<uint32_t>(quarter * 32) << 16) + kColD + 32 * buf + half * NH, d);
+        float d[N];
+        tmem_ld_cols<N>(tmem + (static_cast<uint32_t>(quarter * 32) << 16) + kColD + 32 * buf, d);
         ptx::tmem_wait_ld();
         ptx::tc_fence_before_sync();
 #pragma unroll
-        for (int i = 0; i < NH; ++i) acc[i] = fmaf(acc[i], sm->alpha[j & 3][half * NH + i], d[i]);
+        for (int i = 0; i < NH; ++i) acc[i] = fmaf(acc[i], sm->alpha[t % kStateRing][2 * i + half], half ? d[2 * i + 1] : d[2 * i]);
     };
-
-    // optional dump of one query head (all lanes; byte and m_s are the block's and the tile's)
     const bool dump = P.has_dbg && u.seq == P.dbg.batch && u.head == P.dbg.head / P.G;
-    auto dump_row = [&](int j, int row, float score, uint32_t word, float m_s, uint32_t byte) {
-        const int g = row / u.Sq, tok = row - g * u.Sq, blk = j * 4 + quarter, key = blk * 32 + lane;
-        if (u.head * P.G + g != P.dbg.head || tok < P.dbg.q_begin || tok >= P.dbg.q_end) return;
-        const int64_t drow = tok - P.dbg.q_begin, blocks = (u.Sk + 31) / 32;
-        if (P.dbg.raw_scores != nullptr && key < u.Sk) P.dbg.raw_scores[drow * u.Sk + key] = score;
-        if (P.dbg.row_max != nullptr && quarter == 0 && lane == 0) P.dbg.row_max[drow * u.n_tiles + j] = m_s;
-        if (blk >= blocks) return;
-        if (P.dbg.codes != nullptr && (lane & 7) == 0) reinterpret_cast<uint32_t*>(P.dbg.codes + (drow * blocks + blk) * 16)[lane >> 3] = word;
-        if (P.dbg.scales != nullptr && lane == 0) P.dbg.scales[drow * blocks + blk] = static_cast<uint8_t>(byte);
-    };
-
-    for (int j = j0; j < j1; ++j) {
-        const int buf = j & 1;
-        // ---- row state of the tile (Eq. rowmax-update, Eq. alpha) and the row's part of the scale rule, one row per lane
-        float par = 0.0f, bmax = -INFINITY, m_s = -INFINITY;
-        uint32_t byte = 0u;
-        bool live = false;
-        if (has_row) {
-            const float* b4 = &sm->bmax[(j - j0) * 4][my_row];
-            bmax = b4[32 * quarter];
-            float m_new = fmaxf(m_run, fmaxf(fmaxf(b4[0], b4[32]), fmaxf(b4[64], b4[96])));
-            if (P.rescale_threshold > 0.0f && m_run != -INFINITY &&
-                !(__fsub_rn(__fmul_rn(P.K.sigma, m_new), __fmul_rn(P.K.sigma, m_run)) > P.rescale_threshold))
-                m_new = m_run;
-            m_s = __fmul_rn(P.K.sigma, m_new);
-            const bool grew = m_new > m_run && m_run != -INFINITY;
-            const float alpha = grew ? ex2_approx(__fmul_rn(__fsub_rn(__fmul_rn(P.K.sigma, m_run), m_s), P.K.LOG2E)) : 1.0f;
-            m_run = m_new;
-            l_run *= alpha;
-            if (quarter == 0) sm->alpha[j & 3][my_row] = alpha;
-            live = bmax != -INFINITY;
-            if (PRODUCER == 0 || PRODUCER == 3) {
-                const BlockScale s = efq_block_scale(bmax, m_s, P.K);
-                par = s.Bb; byte = s.byte;
-            } else if (PRODUCER == 4 || PRODUCER == 5) {
-                const FoldedScale f = etq_folded_scale(bmax, m_s, P.K);
-                par = f.c0e; byte = f.byte;
-            } else {
-                par = m_s;
-            }
-        } else if (quarter == 0 && lane < NH) {
-            sm->alpha[j & 3][my_row] = 1.0f;
-        }
-        // ---- Algorithm 1, thread = key: codes of the rows of this half
-        const float* s_tile = S + j * kTile + quarter * 32 + lane;
-        float x[NH];
-#pragma unroll
-        for (int i = 0; i < NH; ++i) x[i] = 2 * i + half < R ? __ldcg(s_tile + static_cast<int64_t>(2 * i + half) * u.Sk_pad) : -INFINITY;
+    for (int j = u.j0; j < u.j1; ++j) {
+        const int t = j - u.j0, buf = t & 1, slot = t % kStateRing;
+        // ---- Algorithm 1, two rows side by side so that their chains of shuffles overlap
+        uint32_t byte = has_row ? sm->byte[slot][quarter][my_row] : 0u;
         int count = 0;                       // of lane i: twice the sum of its row's E2M1 values in this block
         float psum = 0.0f;
 #pragma unroll
-        for (int i = 0; i < NH; ++i) {
-            const int row = 2 * i + half;
-            if (row < R) {
-                uint32_t b = 0u;
-                float p = 0.0f;
-                uint32_t c = key_code<PRODUCER>(x[i], __shfl_sync(0xffffffffu, par, i), P.K, lane, b, p);
-                if (PRODUCER == 4 || PRODUCER == 5) c = __shfl_sync(0xffffffffu, live, i) ? c : 0u;
-                const int n = __reduce_add_sync(0xffffffffu, static_cast<int>((0xC8643210u >> (4u * c)) & 15u));
+        for (int i0 = 0; i0 < NH; i0 += 2) {
+            if (2 * i0 + half < R) {
+                uint32_t c[2], b[2] = {0u, 0u};
+                float p[2] = {0.0f, 0.0f};
+                int n[2];
+#pragma unroll
+                for (int i = 0; i < 2; ++i) c[i] = key_code<PRODUCER>(x[i0 + i], sm->par[slot][quarter][2 * (i0 + i) + half], P.K, lane, b[i], p[i]);
+#pragma unroll
+                for (int i = 0; i < 2; ++i) n[i] = __reduce_add_sync(0xffffffffu, static_cast<int>((0xC8643210u >> (4u * c[i])) & 15u));
                 if (PRODUCER == 6)
-                    for (int o = 16; o > 0; o >>= 1) p += __shfl_xor_sync(0xffffffffu, p, o);
-                if (lane == i) {
-                    count = n;
-                    psum = p;
-                    if (PRODUCER == 1 || PRODUCER == 2 || PRODUCER == 6) byte = b;
+                    for (int o = 16; o > 0; o >>= 1) {
+                        p[0] += __shfl_xor_sync(0xffffffffu, p[0], o);
+                        p[1] += __shfl_xor_sync(0xffffffffu, p[1], o);
+                    }
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    if (lane == i0 + i) {
+                        count = n[i];
+                        psum = p[i];
+                        if (PRODUCER == 1 || PRODUCER == 2 || PRODUCER == 6) byte = b[i];
+                    }
+                    c[i] |= __shfl_down_sync(0xffffffffu, c[i], 1) << 4;
                 }
-                c |= __shfl_down_sync(0xffffffffu, c, 1) << 4;
-                c |= __shfl_down_sync(0xffffffffu, c, 2) << 8;
-                c |= __shfl_down_sync(0xffffffffu, c, 4) << 16;
-                if (dump) dump_row(j, row, x[i], c, __shfl_sync(0xffffffffu, m_s, i), __shfl_sync(0xffffffffu, byte, i));
-                if ((lane & 7) == 0) *reinterpret_cast<uint32_t*>(sm->b[buf] + code_tile_offset(row, quarter) + (lane >> 1)) = c;
+                c[0] |= __shfl_down_sync(0xffffffffu, c[0], 2) << 8;
+                c[1] |= __shfl_down_sync(0xffffffffu, c[1], 2) << 8;
+                c[0] |= __shfl_down_sync(0xffffffffu, c[0], 4) << 16;
+                c[1] |= __shfl_down_sync(0xffffffffu, c[1], 4) << 16;
+                const int row = 2 * i0 + half;
+                if ((lane & 7) == 0) {
+                    *reinterpret_cast<uint32_t*>(sm->b[buf] + code_tile_offset(row, quarter) + (lane >> 1)) = c[0];
+                    *reinterpret_cast<uint32_t*>(sm->b[buf] + code_tile_offset(row + 2, quarter) + (lane >> 1)) = c[1];
+                }
+                if (dump) {
+                    few_dump(P, u, j, quarter, lane, row, x[i0], c[0], sm->m_s[slot][row], __shfl_sync(0xffffffffu, byte, i0));
+                    if (row + 2 < R) few_dump(P, u, j, quarter, lane, row + 2, x[i0 + 1], c[1], sm->m_s[slot][row + 2], __shfl_sync(0xffffffffu, byte, i0 + 1));
+                }
             }
         }
         if (has_row) {
             sm->sf_b[buf][sf_tile_offset(my_row, quarter)] = static_cast<uint8_t>(byte);
-            l_run += PRODUCER == 6 ? psum : static_cast<float>(count) * 0.5f * (byte != 0u ? __uint_as_float(byte << 23) : __uint_as_float(0x00400000u));
+            const float unit = byte != 0u ? __uint_as_float(byte << 23) : __uint_as_float(0x00400000u);
+            l_run = l_run * sm->alpha[slot][my_row] + (PRODUCER == 6 ? psum : static_cast<float>(count) * 0.5f * unit);
         }
-        // ---- V^T operand of the tile
+        if (j + 1 < u.j1) load_scores(j + 1);
+        // ---- V^T operand of the tile: a channel pair per word, its block maximum over the four lanes of a channel group
+        uint32_t w[8][4];
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            uint32_t w[16];
+        for (int i = 0; i < 8; ++i) { w[i][0] = vv[i].x; w[i][1] = vv[i].y; w[i][2] = vv[i].z; w[i][3] = vv[i].w; }
+        uint32_t fields[4];
 #pragma unroll
-            for (int i = 0; i < 16; ++i) w[i] = __byte_perm(vv[2 * i], vv[2 * i + 1], h == 0 ? 0x5410 : 0x7632);
-            uint4 c;
-            uint32_t vb;
-            mxfp4_block(w, c, vb);
-            *reinterpret_cast<uint4*>(sm->a[buf] + code_tile_offset(ch + h, kb)) = c;
-            sm->sf_a[buf][sf_tile_offset(ch + h, kb)] = static_cast<uint8_t>(vb);
+        for (int p = 0; p < 4; ++p) {
+            fields[p] = bf16x2_absmax(bf16x2_absmax(bf16x2_absmax(w[0][p], w[1][p]), bf16x2_absmax(w[2][p], w[3][p])),
+                                      bf16x2_absmax(bf16x2_absmax(w[4][p], w[5][p]), bf16x2_absmax(w[6][p], w[7][p])));
         }
-        if (j + 1 < j1) load_v(j + 1);
+#pragma unroll
+        for (int p = 0; p < 4; ++p) fields[p] = bf16x2_absmax(fields[p], __shfl_xor_sync(0xffffffffu, fields[p], 8));
+#pragma unroll
+        for (int p = 0; p < 4; ++p) fields[p] = mxfp4_fields(bf16x2_absmax(fields[p], __shfl_xor_sync(0xffffffffu, fields[p], 16)));
+        uint8_t* const a_dst = sm->a[buf] + a_offset(v_half * 64 + oct * 8, v_blk) + kg * 4;
+#pragma unroll
+        for (int p = 0; p < 4; ++p) {
+            const uint32_t s2 = mxfp4_scales(fields[p]);
+            uint32_t e[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) e[i] = bf16x2_mul(w[i][p], s2);
+            *reinterpret_cast<uint32_t*>(a_dst + 32 * p) = e2m1_word(bf16_lo(e[0]), bf16_lo(e[1]), bf16_lo(e[2]), bf16_lo(e[3]),
+                                                                     bf16_lo(e[4]), bf16_lo(e[5]), bf16_lo(e[6]), bf16_lo(e[7]));
+            *reinterpret_cast<uint32_t*>(a_dst + 32 * p + 16) = e2m1_word(bf16_hi(e[0]), bf16_hi(e[1]), bf16_hi(e[2]), bf16_hi(e[3]),
+                                                                          bf16_hi(e[4]), bf16_hi(e[5]), bf16_hi(e[6]), bf16_hi(e[7]));
+        }
+        if (j + 1 < u.j1) load_v(j + 1);
+        {   // scale bytes: lane group kg writes channel pair kg
+            const uint32_t f = kg < 2 ? (kg == 0 ? fields[0] : fields[1]) : (kg == 2 ? fields[2] : fields[3]);
+            uint8_t* const d = sm->sf_a[buf] + sf_tile_offset(v_half * 64 + oct * 8 + 2 * kg, v_blk);
+            d[0] = static_cast<uint8_t>(mxfp4_byte_lo(f));
+            d[16] = static_cast<uint8_t>(mxfp4_byte_hi(f));
+        }
+        if (warp == ((t + 1) & 7) && j + 1 < u.j1 && lane < R)
+            few_row_state<PRODUCER>(sm, P, t + 1, (t + 1) % kStateRing, sm->m_raw[slot][lane], lane);
         ptx::fence_proxy_async_smem();
         ptx::tc_fence_before_sync();
         __syncthreads();
@@ -468,119 +544,116 @@ __global__ void __launch_bounds__(kFewThreads, 3) few_values_kernel(const __grid
             if (ptx::elect_one()) few_mma(sm, tmem, buf, buf, N);
             __syncwarp();
         }
-        if (j > j0) add_tile(j - 1);
+        if (t > 0) add_tile(t - 1);
     }
-    add_tile(j1 - 1);
-    if (has_row) sm->lsum[quarter][my_row] = l_run;
-    if (quarter == 0 && has_row) sm->m_start[my_row] = __fmul_rn(P.K.sigma, m_run);   // scaled maximum the chunk refers to
+    add_tile(u.j1 - u.j0 - 1);
+
+    // ---- partial result of the chunk: [row][128] O^T | maximum [row] | denominator [key block][row]
+    float* const part = P.partials + blockIdx.x * (static_cast<size_t>(P.row_cap) * kFewPartFloats);
+#pragma unroll
+    for (int i = 0; i < NH; ++i)
+        if (2 * i + half < R) part[(2 * i + half) * 128 + quarter * 32 + lane] = acc[i];
+    if (has_row) {
+        if (quarter == 0) part[P.row_cap * 128 + my_row] = sm->m_s[(u.j1 - u.j0 - 1) % kStateRing][my_row];
+        part[P.row_cap * (129 + quarter) + my_row] = l_run;
+    }
     ptx::tc_fence_before_sync();
     __syncthreads();
     if (warp == 0) ptx::tmem_dealloc(tmem, kFewTmemCols);
-
-    const int channel = quarter * 32 + lane;
-    auto l_of = [&](int row) { return (sm->lsum[0][row] + sm->lsum[1][row]) + (sm->lsum[2][row] + sm->lsum[3][row]); };
-    auto out_row = [&](int row) { const int g = row / u.Sq; return u.o + g * P.q_head + (row - g * u.Sq) * P.q_row; };
-    if (u.n_chunks == 1) {
-#pragma unroll
-        for (int i = 0; i < NH; ++i) {
-            const int row = half * NH + i;
-            if (row < R) {
-                const float l = l_of(row);
-                out_row(row)[channel] = acc[i] * (l > 0.0f ? 1.0f / l : 0.0f);
-            }
-        }
-        return;
-    }
-    // ---- partial result of the chunk; the last chunk of the head to arrive adds them up
-    const size_t part_floats = static_cast<size_t>(P.row_cap) * 130;     // [row][128] | maximum [row] | denominator [row]
-    float* const part = P.partials + blockIdx.x * part_floats;
-#pragma unroll
-    for (int i = 0; i < NH; ++i) {
-        const int row = half * NH + i;
-        if (row < R) part[row * 128 + channel] = acc[i];
-    }
-    if (tid < R) {
-        part[P.row_cap * 128 + tid] = sm->m_start[tid];
-        part[P.row_cap * 129 + tid] = l_of(tid);
-    }
-    __threadfence();
-    __syncthreads();
-    if (tid == 0) sm->is_last = atomicAdd(P.counters + (u.seq * P.Hkv + u.head), 1u) == static_cast<uint32_t>(u.n_chunks - 1);
-    __syncthreads();
-    if (sm->is_last == 0u) return;
-    __threadfence();
-    const float* const first = P.partials + (blockIdx.x - static_cast<size_t>(u.chunk) * P.Hkv) * part_floats;
-    const size_t step = part_floats * P.Hkv;
-    for (int row = tid >> 7; row < R; row += 2) {
-        const int c_ch = tid & 127;
-        const float m_last = __ldcg(first + (u.n_chunks - 1) * step + P.row_cap * 128 + row);
-        float a = 0.0f, l = 0.0f;
-#pragma unroll 4
-        for (int c = 0; c < u.n_chunks; ++c) {
-            const float* p = first + c * step;
-            const float m = __ldcg(p + P.row_cap * 128 + row);
-            const float w = m == -INFINITY ? 0.0f : ex2_approx(__fmul_rn(__fsub_rn(m, m_last), P.K.LOG2E));
-            l = fmaf(__ldcg(p + P.row_cap * 129 + row), w, l);
-            a = fmaf(__ldcg(p + row * 128 + c_ch), w, a);
-        }
-        out_row(row)[c_ch] = a * (l > 0.0f ? 1.0f / l : 0.0f);
-    }
 }
 
-template <int N, int PRODUCER>
-cudaError_t launch_values(unsigned units, const FewParams& P, cudaStream_t stream)
+// Adds up the chunks of one row (a block per sequence, KV head and row): a warp takes every fourth chunk, a lane four
+// channels, so that all loads of a short list of chunks are in flight together.
+__global__ void __launch_bounds__(128) few_merge_kernel(const __grid_constant__ FewParams P)
 {
-    // may start while the last scores CTAs still run: its first V tile does not depend on them
+    __shared__ float4 sum[4][32];
+    __shared__ float den[4];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int row = static_cast<int>(blockIdx.y);
+    const int head = static_cast<int>(blockIdx.x) % P.Hkv, seq = static_cast<int>(blockIdx.x) / P.Hkv;
+    const int first_id = head + (P.n_seqs == 0 ? seq * P.dense_chunks * P.Hkv : (P.seqs != nullptr ? P.seqs : P.inline_seqs)[seq].first_unit);
+    const Unit u = find_unit(P, first_id);
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (row >= P.G * u.Sq) return;
+    const size_t part_floats = static_cast<size_t>(P.row_cap) * kFewPartFloats, step = part_floats * P.Hkv;
+    const float* const first = P.partials + first_id * part_floats;
+    const float m_last = __ldcg(first + (u.n_chunks - 1) * step + P.row_cap * 128 + row);
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+    float l = 0.0f;
+#pragma unroll 4
+    for (int c = warp; c < u.n_chunks; c += 4) {
+        const float* p = first + c * step;
+        const float m = __ldcg(p + P.row_cap * 128 + row);
+        const float4 x = __ldcg(reinterpret_cast<const float4*>(p + row * 128) + lane);
+        const float lc = (__ldcg(p + P.row_cap * 129 + row) + __ldcg(p + P.row_cap * 130 + row)) +
+                         (__ldcg(p + P.row_cap * 131 + row) + __ldcg(p + P.row_cap * 132 + row));
+        const float w = m == -INFINITY ? 0.0f : ex2_approx(__fmul_rn(__fsub_rn(m, m_last), P.K.LOG2E));
+        l = fmaf(lc, w, l);
+        a.x = fmaf(x.x, w, a.x); a.y = fmaf(x.y, w, a.y); a.z = fmaf(x.z, w, a.z); a.w = fmaf(x.w, w, a.w);
+    }
+    sum[warp][lane] = a;
+    if (lane == 0) den[warp] = l;
+    __syncthreads();
+    const float* s = reinterpret_cast<const float*>(sum) + threadIdx.x;
+    const float t = (s[0] + s[128]) + (s[256] + s[384]), d = (den[0] + den[1]) + (den[2] + den[3]);
+    const int g = row / u.Sq;
+    u.o[g * P.q_head + (row - g * u.Sq) * P.q_row + threadIdx.x] = t * (d > 0.0f ? 1.0f / d : 0.0f);
+}
+
+// Each kernel may start while the one before it still runs; what it needs of that one it waits for itself.
+template <typename Kernel>
+cudaError_t launch_overlapped(Kernel kernel, dim3 grid, int threads, cudaStream_t stream, const FewParams& P)
+{
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(units);
-    cfg.blockDim = dim3(kFewThreads);
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
     cfg.stream = stream;
     cudaLaunchAttribute at{};
     at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, few_values_kernel<N, PRODUCER>, P);
+    return cudaLaunchKernelEx(&cfg, kernel, P);
 }
 
 template <int N>
-cudaError_t launch_n(int producer, unsigned units, const FewParams& P, cudaStream_t stream)
+cudaError_t launch_n(int producer, const FewParams& P, cudaStream_t stream)
 {
-    few_scores_kernel<N><<<units, kFewThreads, 0, stream>>>(P);
-    cudaError_t e = cudaGetLastError();
+    const dim3 grid(static_cast<unsigned>(P.n_units));
+    cudaError_t e = launch_overlapped(few_scores_kernel<N>, grid, kFewThreads, stream, P);
     if (e != cudaSuccess) return e;
     switch (producer) {
-        case 0: return launch_values<N, 0>(units, P, stream);
-        case 1: return launch_values<N, 1>(units, P, stream);
-        case 2: return launch_values<N, 2>(units, P, stream);
-        case 3: return launch_values<N, 3>(units, P, stream);
-        case 4: return launch_values<N, 4>(units, P, stream);
-        case 5: return launch_values<N, 5>(units, P, stream);
-        case 6: return launch_values<N, 6>(units, P, stream);
+        case 0: e = launch_overlapped(few_values_kernel<N, 0>, grid, kFewThreads, stream, P); break;
+        case 1: e = launch_overlapped(few_values_kernel<N, 1>, grid, kFewThreads, stream, P); break;
+        case 2: e = launch_overlapped(few_values_kernel<N, 2>, grid, kFewThreads, stream, P); break;
+        case 3: e = launch_overlapped(few_values_kernel<N, 3>, grid, kFewThreads, stream, P); break;
+        case 4: e = launch_overlapped(few_values_kernel<N, 4>, grid, kFewThreads, stream, P); break;
+        case 5: e = launch_overlapped(few_values_kernel<N, 5>, grid, kFewThreads, stream, P); break;
+        case 6: e = launch_overlapped(few_values_kernel<N, 6>, grid, kFewThreads, stream, P); break;
         default: return cudaErrorInvalidValue;
     }
+    if (e != cudaSuccess) return e;
+    return launch_overlapped(few_merge_kernel, dim3(static_cast<unsigned>(P.n_heads), static_cast<unsigned>(P.row_cap)), 128, stream, P);
 }
 
 }  // namespace
 
-cudaError_t launch_few(int producer, int64_t units, const FewParams& P, cudaStream_t stream)
+cudaError_t launch_few(int producer, const FewParams& P, cudaStream_t stream)
 {
-    if (units <= 0 || units > 0x7fffffffll) return cudaErrorInvalidValue;
-    const unsigned n = static_cast<unsigned>(units);
-    if (P.row_cap <= 8) return launch_n<8>(producer, n, P, stream);
-    if (P.row_cap <= 16) return launch_n<16>(producer, n, P, stream);
-    return launch_n<24>(producer, n, P, stream);
+    if (P.n_units <= 0) return cudaErrorInvalidValue;
+    if (P.row_cap <= 8) return launch_n<8>(producer, P, stream);
+    if (P.row_cap <= 16) return launch_n<16>(producer, P, stream);
+    return launch_n<24>(producer, P, stream);
 }
 
-FewPlan plan_few(int64_t units, int64_t heads, int64_t keys_padded_all_heads, int rows)
+FewPlan plan_few(int64_t units, int64_t keys_padded_all_heads, int rows)
 {
     FewPlan w;
     size_t off = 0;
     auto take = [&](size_t bytes) { const size_t at = off; off = (off + bytes + 1023) / 1024 * 1024; return at; };
     w.scores = take(static_cast<size_t>(keys_padded_all_heads) * rows * sizeof(float));
     w.block_max = take(static_cast<size_t>(keys_padded_all_heads / 32) * rows * sizeof(float));
-    w.partials = take(static_cast<size_t>(units) * rows * 130 * sizeof(float));
-    w.counters = take(static_cast<size_t>(heads) * sizeof(uint32_t));
+    w.partials = take(static_cast<size_t>(units) * rows * kFewPartFloats * sizeof(float));
     w.total = off;
     return w;
 }

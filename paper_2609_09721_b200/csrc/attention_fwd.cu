@@ -649,7 +649,7 @@ struct Workspace {
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 bool use_few(int Hq, int Hkv, int64_t Sq);
-int64_t few_chunks(int64_t Sk);
+int64_t few_chunks(int64_t Sk, int64_t rows);
 
 Workspace plan_workspace(int B, int Hq, int Hkv, int64_t Sq, int64_t Sk)
 {
@@ -674,7 +674,7 @@ size_t workspace_bytes_for(int B, int Hq, int Hkv, int64_t Sq, int64_t Sk)
     size_t total = plan_workspace(B, Hq, Hkv, Sq, Sk).total;
     if (use_few(Hq, Hkv, Sq)) {
         const int64_t heads = static_cast<int64_t>(B) * Hkv;
-        const size_t few = 1024 + plan_few(heads * few_chunks(Sk), heads, heads * ((Sk + kTile - 1) / kTile * kTile),
+        const size_t few = 1024 + plan_few(heads * few_chunks(Sk, Hq / Hkv * Sq), heads * ((Sk + kTile - 1) / kTile * kTile),
                                            static_cast<int>(Hq / Hkv * Sq)).total;
         if (few > total) total = few;
     }
@@ -736,7 +736,11 @@ bool use_packed_tile(int Hq, int Hkv, int64_t Sq) { return Hq / Hkv > 1 && stati
 // sequence takes the same path by itself and in a packed batch.
 bool use_few(int Hq, int Hkv, int64_t Sq) { return static_cast<int64_t>(Hq / Hkv) * Sq <= kFewMaxRows; }
 
-int64_t few_chunks(int64_t Sk) { return ((Sk + kTile - 1) / kTile + kFewChunkTiles - 1) / kFewChunkTiles; }
+int64_t few_chunks(int64_t Sk, int64_t rows)
+{
+    const int n_tiles = static_cast<int>((Sk + kTile - 1) / kTile), per = few_chunk_tiles(n_tiles, static_cast<int>(rows));
+    return (n_tiles + per - 1) / per;
+}
 
 cudaError_t launch_forward(int producer, bool debug, bool fix8, int64_t items, cudaStream_t stream, const CUtensorMap& mq,
                            const CUtensorMap& mk, const CUtensorMap& mv, const FwdParams& P)
@@ -797,21 +801,23 @@ efq_status_t attention_impl(const void* q, const void* k, const void* v, float* 
         F.o = o;
         F.Hkv = Hkv; F.G = G; F.causal = causal ? 1 : 0;
         F.Sq = static_cast<int32_t>(Sq); F.Sk = static_cast<int32_t>(Sk); F.Sk_pad = static_cast<int32_t>(w.Sk_pad);
-        F.dense_chunks = static_cast<int32_t>(few_chunks(Sk));
+        F.dense_chunks = static_cast<int32_t>(few_chunks(Sk, G * Sq));
         F.q_row = 128; F.q_head = Sq * 128; F.q_seq = Hq * F.q_head;
         F.k_row = 128; F.k_head = Sk * 128; F.k_seq = Hkv * F.k_head;
         F.row_cap = static_cast<int32_t>(G * Sq);
-        F.n_counters = B * Hkv;
+        F.n_heads = B * Hkv;
         F.rescale_threshold = rescale_threshold;
         F.K = producer == 3 ? make_producer_consts_lut(softmax_scale) : make_producer_consts(softmax_scale, tau, h);
         const int64_t units = static_cast<int64_t>(B) * Hkv * F.dense_chunks;
-        const FewPlan fp = plan_few(units, F.n_counters, static_cast<int64_t>(B) * Hkv * w.Sk_pad, F.row_cap);
+        if (units > 0x7fffffffll) return EFQ_ERR_UNSUPPORTED;
+        F.n_units = static_cast<int32_t>(units);
+        const FewPlan fp = plan_few(units, static_cast<int64_t>(B) * Hkv * w.Sk_pad, F.row_cap);
         F.scores = reinterpret_cast<float*>(ws + 1024 + fp.scores); F.block_max = reinterpret_cast<float*>(ws + 1024 + fp.block_max);
-        F.partials = reinterpret_cast<float*>(ws + 1024 + fp.partials); F.counters = reinterpret_cast<uint32_t*>(ws + 1024 + fp.counters);
+        F.partials = reinterpret_cast<float*>(ws + 1024 + fp.partials);
         F.status = reinterpret_cast<uint32_t*>(ws);
         F.has_dbg = debug != nullptr ? 1 : 0;
         if (debug != nullptr) F.dbg = *debug;
-        return launch_few(producer, units, F, stream) == cudaSuccess ? EFQ_OK : EFQ_ERR_CUDA;
+        return launch_few(producer, F, stream) == cudaSuccess ? EFQ_OK : EFQ_ERR_CUDA;
     }
     const bool packed = use_packed_tile(Hq, Hkv, Sq);
     const int64_t q_rows = packed ? static_cast<int64_t>(B) * Hkv * kTile : static_cast<int64_t>(B) * Hq * w.Sq_pad;
@@ -893,7 +899,7 @@ bool plan_varlen(const int64_t* cu_q, const int64_t* cu_k, int n_seqs, int Hq, i
         if (use_few(Hq, Hkv, lq)) {
             ++p.n_few;
             p.few_rows = std::max(p.few_rows, static_cast<int>(Hq / Hkv * lq));
-            p.few_units += few_chunks(lk) * Hkv;
+            p.few_units += few_chunks(lk, Hq / Hkv * lq) * Hkv;
             p.few_keys += (lk + kTile - 1) / kTile * kTile;
             continue;
         }
@@ -924,7 +930,7 @@ bool plan_varlen(const int64_t* cu_q, const int64_t* cu_k, int n_seqs, int Hq, i
     p.few_table = off;
     if (p.n_few > kFewInlineSeqs) off = align_up(off + sizeof(FewSeq) * p.n_few, 1024);
     p.few = off;
-    if (p.n_few > 0) off += plan_few(p.few_units, static_cast<int64_t>(p.n_few) * Hkv, p.few_keys * Hkv, p.few_rows).total;
+    if (p.n_few > 0) off += plan_few(p.few_units, p.few_keys * Hkv, p.few_rows).total;
     p.total = off;
     return true;
 }
@@ -1214,7 +1220,7 @@ extern "C" efq_status_t efq_attention_fwd_varlen(const void* q, const void* k, c
             few_seqs[f++] = FewSeq{static_cast<int32_t>(lq), static_cast<int32_t>(lk), static_cast<int32_t>(q0), static_cast<int32_t>(k0),
                                    static_cast<int32_t>(few_key), static_cast<int32_t>(few_unit)};
             few_key += (lk + kTile - 1) / kTile * kTile;
-            few_unit += few_chunks(lk) * Hkv;
+            few_unit += few_chunks(lk, Hq / Hkv * lq) * Hkv;
             continue;
         }
         const bool packed = use_packed_tile(Hq, Hkv, lq);
@@ -1266,19 +1272,20 @@ extern "C" efq_status_t efq_attention_fwd_varlen(const void* q, const void* k, c
         F.q_head = 128; F.q_row = static_cast<int64_t>(Hq) * 128;
         F.k_head = 128; F.k_row = static_cast<int64_t>(Hkv) * 128;
         F.row_cap = p.few_rows;
-        F.n_counters = p.n_few * Hkv;
+        F.n_heads = p.n_few * Hkv;
+        F.n_units = static_cast<int32_t>(p.few_units);
         F.rescale_threshold = threshold;
         F.K = producer == 3 ? make_producer_consts_lut(softmax_scale) : make_producer_consts(softmax_scale, tau, h);
-        const FewPlan fp = plan_few(p.few_units, F.n_counters, p.few_keys * Hkv, p.few_rows);
+        const FewPlan fp = plan_few(p.few_units, p.few_keys * Hkv, p.few_rows);
         uint8_t* const fw = ws + p.few;
         F.scores = reinterpret_cast<float*>(fw + fp.scores); F.block_max = reinterpret_cast<float*>(fw + fp.block_max);
-        F.partials = reinterpret_cast<float*>(fw + fp.partials); F.counters = reinterpret_cast<uint32_t*>(fw + fp.counters);
+        F.partials = reinterpret_cast<float*>(fw + fp.partials);
         F.status = reinterpret_cast<uint32_t*>(ws);
         if (!few_long.empty()) {
             if (cudaMemcpyAsync(ws + p.few_table, few_long.data(), sizeof(FewSeq) * few_long.size(), cudaMemcpyHostToDevice, s) != cudaSuccess) return EFQ_ERR_CUDA;
             F.seqs = reinterpret_cast<const FewSeq*>(ws + p.few_table);
         }
-        if (launch_few(producer, p.few_units, F, s) != cudaSuccess) return EFQ_ERR_CUDA;
+        if (launch_few(producer, F, s) != cudaSuccess) return EFQ_ERR_CUDA;
         if (p.n_active == 0) return EFQ_OK;
     }
     if (p.n_active == 0)             // nothing to launch: the status word still has to read "no problem"

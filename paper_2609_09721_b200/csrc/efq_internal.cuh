@@ -66,9 +66,15 @@ struct ItemDesc {
 // ------------------------------------------------------------------------------------------------
 // 24 rows keep the scores in the workspace below the size of the MXFP4 copies that the general path would need there.
 constexpr int kFewMaxRows = 24;
-// Keys of a chunk: 4 tiles are 256 KB of K and V, enough to hide a CTA's start behind its neighbours, and small enough
-// that a single 8 K context spreads over the whole chip.
-constexpr int kFewChunkTiles = 4;
+// Tiles of a chunk of the KV range, by the sequence's own shape: short contexts are cut finely, so that one of them spreads
+// over the chip; with many rows a chunk's partial result (544 bytes a row) has to be small against its 64 KB of K and V a tile.
+constexpr int kFewMaxChunk = 4;
+__host__ __device__ inline int few_chunk_tiles(int n_tiles, int rows)
+{
+    return rows <= 8 ? (n_tiles < 16 ? 1 : n_tiles < 48 ? 2 : kFewMaxChunk) : n_tiles < 32 ? 2 : kFewMaxChunk;
+}
+// floats per query row of a chunk's partial result: 128 of O^T, the maximum they refer to, four parts of the denominator
+constexpr int kFewPartFloats = 136;
 constexpr int kFewInlineSeqs = 128;      // sequence tables up to this size travel as kernel parameters
 
 struct FewSeq {
@@ -86,20 +92,20 @@ struct FewParams {
     int32_t Sq, Sk, Sk_pad, dense_chunks;      // dense only
     int64_t q_seq, q_head, q_row, k_seq, k_head, k_row;    // strides in elements
     int32_t row_cap;                           // query rows the workspace holds per KV head (the most of any sequence)
-    int32_t n_counters;
+    int32_t n_units, n_heads;                  // chunks times KV heads, and KV heads, of all sequences
     float rescale_threshold;
     ProducerConsts K;
     float *scores, *block_max, *partials;      // workspace
-    uint32_t *counters, *status;
+    uint32_t* status;
     int32_t has_dbg;
     efq_debug_t dbg;
     const FewSeq* seqs;                        // device table; null: inline_seqs
     FewSeq inline_seqs[kFewInlineSeqs];
 };
 
-struct FewPlan { size_t scores, block_max, partials, counters, total; };   // offsets from a 1024-byte aligned base
-FewPlan plan_few(int64_t units, int64_t heads, int64_t keys_padded_all_heads, int rows);
-// units: chunks times KV heads of all sequences.  Clears the status words.
-cudaError_t launch_few(int producer, int64_t units, const FewParams& P, cudaStream_t stream);
+struct FewPlan { size_t scores, block_max, partials, total; };   // offsets from a 1024-byte aligned base
+FewPlan plan_few(int64_t units, int64_t keys_padded_all_heads, int rows);
+// Clears the status words.
+cudaError_t launch_few(int producer, const FewParams& P, cudaStream_t stream);
 
 }  // namespace efq
