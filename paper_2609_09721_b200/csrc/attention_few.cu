@@ -178,14 +178,22 @@ __global__ void __launch_bounds__(kFewThreads, N <= 8 ? 4 : 3) few_scores_kernel
     // bytes of every key - and so a quarter of each of the four blocks
     const int quad = tid & 3, key_in_tile = tid >> 2;
     uint4 kk[2][4];
+    const uint4* k_src = reinterpret_cast<const uint4*>(u.k + (u.j0 * kTile + key_in_tile) * P.k_row) + quad;
+    const int64_t k_half = 8 * P.k_row;                  // 64 keys on, in 16-byte pieces
     auto load_k = [&](int j) {
+        if ((j + 1) * kTile <= u.Sk) {
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int key = j * kTile + key_in_tile + 64 * h;
-            const uint4* src = reinterpret_cast<const uint4*>(u.k + key * P.k_row) + quad;
+            for (int i = 0; i < 4; ++i) kk[0][i] = __ldcs(k_src + 4 * i);
 #pragma unroll
-            for (int i = 0; i < 4; ++i) kk[h][i] = key < u.Sk ? __ldcs(src + 4 * i) : make_uint4(0, 0, 0, 0);
+            for (int i = 0; i < 4; ++i) kk[1][i] = __ldcs(k_src + k_half + 4 * i);
+        } else {
+            const bool in0 = j * kTile + key_in_tile < u.Sk, in1 = j * kTile + key_in_tile + 64 < u.Sk;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) kk[0][i] = in0 ? __ldcs(k_src + 4 * i) : make_uint4(0, 0, 0, 0);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) kk[1][i] = in1 ? __ldcs(k_src + k_half + 4 * i) : make_uint4(0, 0, 0, 0);
         }
+        k_src += 2 * k_half;
     };
     load_k(u.j0);
     // Q: one thread per (row, block)
@@ -210,8 +218,11 @@ __global__ void __launch_bounds__(kFewThreads, N <= 8 ? 4 : 3) few_scores_kernel
     const uint32_t tmem = sm->tmem_base;
     const int nblk = u.Sk_pad / 32;
     const int quarter = warp & 3, half = warp >> 2;      // 32 keys of the tile; rows 2 i + half
-    const int shift = P.causal ? u.Sk - u.Sq : u.Sk;     // key <= token + shift; without a mask every key of the sequence
+    // last visible key of row `lane`
+    const int limit = min(P.causal ? lane % u.Sq + u.Sk - u.Sq : u.Sk, u.Sk - 1);
 
+    float* dst = P.scores + u.s_off + half * u.Sk_pad + u.j0 * kTile + quarter * 32 + lane;
+    float* dst_max = P.block_max + u.s_off / 32 + half * nblk + u.j0 * 4 + quarter;
     // raw scores of a finished tile: thread = key, two rows of the half side by side
     auto put_scores = [&](int j) {
         const int buf = (j - u.j0) & 1;
@@ -222,23 +233,23 @@ __global__ void __launch_bounds__(kFewThreads, N <= 8 ? 4 : 3) few_scores_kernel
         ptx::tmem_wait_ld();
         ptx::tc_fence_before_sync();
         const int key = j * kTile + quarter * 32 + lane;
-        float* const dst = P.scores + u.s_off + key;
-        float* const dst_max = P.block_max + u.s_off / 32 + (key >> 5);
 #pragma unroll
         for (int i = 0; i < N; i += 4) {
             const int row = i + half;
             if (row < R) {
-                const float x0 = key < u.Sk && key <= row % u.Sq + shift ? (half ? s[i + 1] : s[i]) : -INFINITY;
-                const float x1 = key < u.Sk && key <= (row + 2) % u.Sq + shift ? (half ? s[i + 3] : s[i + 2]) : -INFINITY;
+                const float x0 = key <= __shfl_sync(0xffffffffu, limit, row) ? (half ? s[i + 1] : s[i]) : -INFINITY;
+                const float x1 = key <= __shfl_sync(0xffffffffu, limit, row + 2) ? (half ? s[i + 3] : s[i + 2]) : -INFINITY;
                 const float m0 = warp_max(x0), m1 = warp_max(x1);
-                dst[row * u.Sk_pad] = x0;
-                if (lane == 0) dst_max[row * nblk] = m0;
-                if (row + 2 < R) {
-                    dst[(row + 2) * u.Sk_pad] = x1;
-                    if (lane == 0) dst_max[(row + 2) * nblk] = m1;
+                dst[i * u.Sk_pad] = x0;
+                if (row + 2 < R) dst[(i + 2) * u.Sk_pad] = x1;
+                if (lane == 0) {
+                    dst_max[i * nblk] = m0;
+                    if (row + 2 < R) dst_max[(i + 2) * nblk] = m1;
                 }
             }
         }
+        dst += kTile;
+        dst_max += 4;
     };
 
     for (int j = u.j0; j < u.j1; ++j) {
@@ -374,17 +385,19 @@ __global__ void __launch_bounds__(kFewThreads, 3) few_values_kernel(const __grid
     // V: a lane takes eight channels of eight neighbouring keys, a warp 64 channels of a 32-key block: full 128-byte lines
     const int oct = lane & 7, kg = lane >> 3, v_half = warp & 1, v_blk = warp >> 1;
     uint4 vv[8];
+    const int64_t v_step = P.k_row / 8;                  // a key on, in 16-byte pieces
+    const uint4* v_src = reinterpret_cast<const uint4*>(u.v + (u.j0 * kTile + v_blk * 32 + kg * 8) * P.k_row + v_half * 64 + oct * 8);
     auto load_v = [&](int j) {
-        const int key0 = j * kTile + v_blk * 32 + kg * 8;
-        const uint4* src = reinterpret_cast<const uint4*>(u.v + key0 * P.k_row + v_half * 64 + oct * 8);
-        const int64_t step = P.k_row / 8;
         if ((j + 1) * kTile <= u.Sk) {
+            const uint4* src = v_src;
 #pragma unroll
-            for (int i = 0; i < 8; ++i) vv[i] = __ldcs(src + i * step);
+            for (int i = 0; i < 8; ++i, src += v_step) vv[i] = __ldcs(src);
         } else {
+            const int left = u.Sk - (j * kTile + v_blk * 32 + kg * 8);
 #pragma unroll
-            for (int i = 0; i < 8; ++i) vv[i] = key0 + i < u.Sk ? __ldcs(src + i * step) : make_uint4(0, 0, 0, 0);
+            for (int i = 0; i < 8; ++i) vv[i] = i < left ? __ldcs(v_src + i * v_step) : make_uint4(0, 0, 0, 0);
         }
+        v_src += kTile * v_step;
     };
     load_v(u.j0);       // an input: whatever produced it had finished before the scores kernel allowed this one to start
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -418,13 +431,14 @@ __global__ void __launch_bounds__(kFewThreads, 3) few_values_kernel(const __grid
     // Codes: thread = key of block `quarter`; the warps of a half take the rows 2 i + half.  O^T: thread = channel.
     constexpr int NH = N / 2;
     const int quarter = warp & 3, half = warp >> 2;
-    const float* const S = P.scores + u.s_off + half * u.Sk_pad + quarter * 32 + lane;
+    const float* s_src = P.scores + u.s_off + half * u.Sk_pad + u.j0 * kTile + quarter * 32 + lane;
     float x[NH];
-    auto load_scores = [&](int j) {
+    auto load_scores = [&]() {
 #pragma unroll
-        for (int i = 0; i < NH; ++i) x[i] = 2 * i + half < R ? __ldcg(S + j * kTile + 2 * i * u.Sk_pad) : -INFINITY;
+        for (int i = 0; i < NH; ++i) x[i] = 2 * i + half < R ? __ldcg(s_src + 2 * i * u.Sk_pad) : -INFINITY;
+        s_src += kTile;
     };
-    load_scores(u.j0);
+    load_scores();
     ptx::tc_fence_before_sync();
     __syncthreads();
     ptx::tc_fence_after_sync();
@@ -500,7 +514,7 @@ __global__ void __launch_bounds__(kFewThreads, 3) few_values_kernel(const __grid
             const float unit = byte != 0u ? __uint_as_float(byte << 23) : __uint_as_float(0x00400000u);
             l_run = l_run * sm->alpha[slot][my_row] + (PRODUCER == 6 ? psum : static_cast<float>(count) * 0.5f * unit);
         }
-        if (j + 1 < u.j1) load_scores(j + 1);
+        if (j + 1 < u.j1) load_scores();
         // ---- V^T operand of the tile: a channel pair per word, its block maximum over the four lanes of a channel group
         uint32_t w[8][4];
 #pragma unroll

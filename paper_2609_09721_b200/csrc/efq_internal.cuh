@@ -68,10 +68,10 @@ struct ItemDesc {
 constexpr int kFewMaxRows = 24;
 // Tiles of a chunk of the KV range, by the sequence's own shape: short contexts are cut finely, so that one of them spreads
 // over the chip; with many rows a chunk's partial result (544 bytes a row) has to be small against its 64 KB of K and V a tile.
-constexpr int kFewMaxChunk = 4;
+constexpr int kFewMaxChunk = 8;
 __host__ __device__ inline int few_chunk_tiles(int n_tiles, int rows)
 {
-    return rows <= 8 ? (n_tiles < 16 ? 1 : n_tiles < 48 ? 2 : kFewMaxChunk) : n_tiles < 32 ? 2 : kFewMaxChunk;
+    return rows <= 8 ? (n_tiles < 16 ? 1 : n_tiles < 32 ? 2 : n_tiles < 128 ? 4 : kFewMaxChunk) : n_tiles < 32 ? 2 : kFewMaxChunk;
 }
 // floats per query row of a chunk's partial result: 128 of O^T, the maximum they refer to, four parts of the denominator
 constexpr int kFewPartFloats = 136;
