@@ -1,6 +1,6 @@
-"""ctypes binding of libefq_b200.so: same names as the C ABI in include/efq.h.
+"""Python binding of libefq_b200.so: same names as the C ABI in include/efq.h.
 
-Argument marshalling only.  Tensors are torch CUDA tensors (torch is used for device
+Argument marshalling only: ctypes, and for the calls of a serving loop the CPython extension efq_fastcall.  Tensors are torch CUDA tensors (torch is used for device
 memory and streams); nothing here computes.  There is no CPU fallback: if the library
 has not been built, or a call returns a non-zero status, a RuntimeError is raised.
 """
@@ -48,6 +48,8 @@ class EfqError(RuntimeError):
 
 
 _lib = None
+_fast = None
+_raw_stream, _raw_device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice    # a tenth of torch.cuda.current_stream()
 
 
 def lib() -> C.CDLL:
@@ -113,6 +115,23 @@ def lib() -> C.CDLL:
     return _lib
 
 
+def _fastcall():
+    """The extension that calls the library's per-step entry points; raises if it has not been built."""
+    global _fast
+    if _fast is None:
+        L = lib()
+        try:
+            from . import efq_fastcall
+        except ImportError as e:
+            raise RuntimeError("efq_fastcall.so is missing: build it with `python -m paper_2609_09721_b200.build`") from e
+        address = lambda f: C.cast(f, C.c_void_p).value
+        efq_fastcall.set_functions(address(L.efq_attention_fwd), address(L.exp_then_quantize_attention_fwd),
+                                   address(L.efq_probgen), address(L.exp_then_quantize_probgen),
+                                   address(L.efq_attention_fwd_varlen), address(L.efq_attention_varlen_workspace_bytes))
+        _fast = efq_fastcall
+    return _fast
+
+
 def status_string(status: int) -> str:
     return lib().efq_status_string(int(status)).decode()
 
@@ -123,7 +142,7 @@ def version() -> str:
 
 def _stream(stream) -> int:
     if stream is None:
-        return torch.cuda.current_stream().cuda_stream
+        return _raw_stream(_raw_device())
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
@@ -137,6 +156,12 @@ def _params(params) -> Optional[EfqParams]:
     kv_tile = params[3] if len(params) > 3 else 0
     threshold = params[4] if len(params) > 4 else 0.0
     return EfqParams(float(tau), float(h), int(variant), int(kv_tile), float(threshold))
+
+
+def _params_address(params):
+    """(object to keep alive, its address or 0) for a params argument."""
+    p = _params(params)
+    return p, (0 if p is None else C.addressof(p))
 
 
 def _ptr(t) -> Optional[int]:
@@ -165,11 +190,12 @@ def efq_probgen(scores: torch.Tensor, row_max: torch.Tensor, score_scale: float 
     assert scores.is_cuda and scores.dtype == torch.float32 and scores.dim() == 2 and scores.stride(1) == 1
     assert row_max.is_cuda and row_max.dtype == torch.float32 and row_max.is_contiguous()
     codes, scales = _probgen_outputs(scores, codes, scales)
-    p = _params(params)
-    st = lib().efq_probgen(scores.data_ptr(), scores.stride(0), row_max.data_ptr(), scores.shape[0],
-                           scores.shape[1], float(score_scale), C.byref(p) if p is not None else None,
-                           codes.data_ptr(), scales.data_ptr(), _stream(stream))
-    _check(st, "efq_probgen")
+    keep, p = _params_address(params)
+    rows, cols = scores.shape
+    st = (_fast or _fastcall()).probgen(scores.data_ptr(), scores.stride(0), row_max.data_ptr(), rows, cols, score_scale, p,
+                                        codes.data_ptr(), scales.data_ptr(), _stream(stream))
+    if st:
+        _check(st, "efq_probgen")
     return codes, scales
 
 
@@ -180,10 +206,11 @@ def exp_then_quantize_probgen(scores: torch.Tensor, row_max: torch.Tensor, score
     assert scores.is_cuda and scores.dtype == torch.float32 and scores.dim() == 2 and scores.stride(1) == 1
     assert row_max.is_cuda and row_max.dtype == torch.float32 and row_max.is_contiguous()
     codes, scales = _probgen_outputs(scores, codes, scales)
-    st = lib().exp_then_quantize_probgen(scores.data_ptr(), scores.stride(0), row_max.data_ptr(), scores.shape[0],
-                                         scores.shape[1], float(score_scale), int(scale_mode), codes.data_ptr(),
-                                         scales.data_ptr(), _stream(stream))
-    _check(st, "exp_then_quantize_probgen")
+    rows, cols = scores.shape
+    st = (_fast or _fastcall()).etq_probgen(scores.data_ptr(), scores.stride(0), row_max.data_ptr(), rows, cols, score_scale,
+                                            int(scale_mode), codes.data_ptr(), scales.data_ptr(), _stream(stream))
+    if st:
+        _check(st, "exp_then_quantize_probgen")
     return codes, scales
 
 
@@ -207,11 +234,13 @@ class DebugDump:
 
 
 def _attn_args(q, k, v, o, workspace):
-    assert q.is_cuda and q.dtype == torch.bfloat16 and q.is_contiguous() and q.dim() == 4
-    assert k.is_cuda and k.dtype == torch.bfloat16 and k.is_contiguous() and k.shape == v.shape
-    assert v.is_cuda and v.dtype == torch.bfloat16 and v.is_contiguous()
+    bf16 = torch.bfloat16
+    ks = k.shape
+    assert q.is_cuda and q.dtype is bf16 and q.is_contiguous() and q.dim() == 4
+    assert k.is_cuda and k.dtype is bf16 and k.is_contiguous() and ks == v.shape
+    assert v.is_cuda and v.dtype is bf16 and v.is_contiguous()
     B, Hq, Sq, d = q.shape
-    _, Hkv, Sk, _ = k.shape
+    _, Hkv, Sk, _ = ks
     if o is None:
         o = torch.empty((B, Hq, Sq, d), dtype=torch.float32, device=q.device)
     if workspace is None:
@@ -225,12 +254,12 @@ def efq_attention_fwd(q, k, v, causal: bool = False, softmax_scale: float = 0.0,
     """Fused FP4 attention forward with EFQ probability generation.  q bf16 [B,Hq,Sq,d],
     k/v bf16 [B,Hkv,Sk,d]; returns o fp32 [B,Hq,Sq,d]."""
     B, Hq, Hkv, Sq, Sk, d, o, workspace = _attn_args(q, k, v, o, workspace)
-    p = _params(params)
-    st = lib().efq_attention_fwd(q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(), B, Hq, Hkv, Sq, Sk, d,
-                                 int(bool(causal)), float(softmax_scale), C.byref(p) if p is not None else None,
-                                 workspace.data_ptr(), workspace.numel(),
-                                 C.byref(debug.c) if debug is not None else None, _stream(stream))
-    _check(st, "efq_attention_fwd")
+    keep, p = _params_address(params)
+    st = (_fast or _fastcall()).attention(q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(), B, Hq, Hkv, Sq, Sk, d,
+                                          1 if causal else 0, softmax_scale, p, workspace.data_ptr(), workspace.numel(),
+                                          0 if debug is None else C.addressof(debug.c), _stream(stream))
+    if st:
+        _check(st, "efq_attention_fwd")
     return o
 
 
@@ -238,11 +267,11 @@ def exp_then_quantize_attention_fwd(q, k, v, causal: bool = False, softmax_scale
                                     o=None, workspace=None, debug: DebugDump = None, stream=None):
     """The MXFP4 comparison path: same pipeline, exp-then-quantize producer."""
     B, Hq, Hkv, Sq, Sk, d, o, workspace = _attn_args(q, k, v, o, workspace)
-    st = lib().exp_then_quantize_attention_fwd(q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(), B, Hq, Hkv,
-                                               Sq, Sk, d, int(bool(causal)), float(softmax_scale), int(scale_mode),
-                                               workspace.data_ptr(), workspace.numel(),
-                                               C.byref(debug.c) if debug is not None else None, _stream(stream))
-    _check(st, "exp_then_quantize_attention_fwd")
+    st = (_fast or _fastcall()).etq_attention(q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(), B, Hq, Hkv, Sq, Sk, d,
+                                              1 if causal else 0, softmax_scale, int(scale_mode), workspace.data_ptr(),
+                                              workspace.numel(), 0 if debug is None else C.addressof(debug.c), _stream(stream))
+    if st:
+        _check(st, "exp_then_quantize_attention_fwd")
     return o
 
 
@@ -275,21 +304,17 @@ def efq_attention_fwd_varlen(q, k, v, cu_seqlens_q, cu_seqlens_k, causal: bool =
     total_q, Hq, d = q.shape
     total_k, Hkv, _ = k.shape
     assert q.is_contiguous() and k.is_contiguous() and v.is_contiguous() and v.shape == k.shape
-    n = len(cu_seqlens_q) - 1
-    assert len(cu_seqlens_k) == n + 1 and int(cu_seqlens_q[-1]) == total_q and int(cu_seqlens_k[-1]) == total_k
-    cq = (C.c_int64 * (n + 1))(*[int(x) for x in cu_seqlens_q])
-    ck = (C.c_int64 * (n + 1))(*[int(x) for x in cu_seqlens_k])
+    fast = _fast or _fastcall()
     if workspace is None:
-        nbytes = lib().efq_attention_varlen_workspace_bytes(cq, ck, n, Hq, Hkv, d)
-        if nbytes == 0:
+        nbytes = fast.varlen(cu_seqlens_q, cu_seqlens_k, total_q, total_k, Hq, Hkv, d, None, 0, 0, 0, 0, 0.0, 0, 0, 0, 0, 0)
+        if nbytes <= 0:
             raise EfqError(1, "efq_attention_varlen_workspace_bytes")
         workspace = torch.empty(nbytes, dtype=torch.uint8, device=q.device)
     o = torch.empty((total_q, Hq, d), dtype=torch.float32, device=q.device)
-    p = _params(params)
-    st = lib().efq_attention_fwd_varlen(q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(), cq, ck, n, Hq, Hkv, d,
-                                        int(bool(causal)), float(softmax_scale), int(producer),
-                                        C.byref(p) if p is not None else None, workspace.data_ptr(), workspace.numel(),
-                                        _stream(stream))
+    keep, p = _params_address(params)
+    st = fast.varlen(cu_seqlens_q, cu_seqlens_k, total_q, total_k, Hq, Hkv, d, q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(),
+                     1 if causal else 0, softmax_scale, int(producer), p, workspace.data_ptr(), workspace.numel(), _stream(stream))
+    assert st != -1, "the prefix sums do not fit the tensors"
     _check(st, "efq_attention_fwd_varlen")
     return o
 

@@ -1,15 +1,19 @@
-"""Builds the C-ABI CUDA library in-tree: paper_2609_09721_b200/libefq_b200.so (sm_100a only)."""
+"""Builds the C-ABI CUDA library in-tree, paper_2609_09721_b200/libefq_b200.so (sm_100a only), and the CPython extension
+beside it that calls it, efq_fastcall.so."""
 from __future__ import annotations
 
 import glob
 import os
 import subprocess
 import sys
+import sysconfig
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(_HERE)
 CSRC = os.path.join(_HERE, "csrc")
 LIB = os.path.join(_HERE, "libefq_b200.so")
+FASTCALL_SRC = os.path.join(CSRC, "fastcall.c")
+FASTCALL = os.path.join(_HERE, "efq_fastcall.so")
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 
 FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-std=c++17", "-lineinfo",
@@ -22,10 +26,10 @@ def sources():
 
 
 def _stale() -> bool:
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(FASTCALL):
         return True
-    t = os.path.getmtime(LIB)
-    deps = sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(ROOT, "include", "*.h"))
+    t = min(os.path.getmtime(LIB), os.path.getmtime(FASTCALL))
+    deps = sources() + [FASTCALL_SRC] + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(ROOT, "include", "*.h"))
     return any(os.path.getmtime(d) > t for d in deps)
 
 
@@ -49,6 +53,10 @@ def build(force: bool = False, verbose: bool = False) -> str:
     tmp = LIB + f".tmp{os.getpid()}"
     subprocess.run([NVCC, "-shared", "-o", tmp, *objs, "-lcuda", "-cudart", "static"], check=True)
     os.replace(tmp, LIB)
+    tmp = FASTCALL + f".tmp{os.getpid()}"
+    subprocess.run([os.environ.get("CC", "gcc"), "-O2", "-Wall", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"],
+                    "-I", os.path.join(ROOT, "include"), FASTCALL_SRC, "-o", tmp], check=True)
+    os.replace(tmp, FASTCALL)
     return LIB
 
 

@@ -892,6 +892,7 @@ bool plan_varlen(const int64_t* cu_q, const int64_t* cu_k, int n_seqs, int Hq, i
     if (d != 128) { st = EFQ_ERR_UNSUPPORTED; return false; }
     if (n_seqs > 0 && (cu_q[0] != 0 || cu_k[0] != 0)) { st = EFQ_ERR_INVALID_ARG; return false; }
     p = VarlenPlan{};
+    size_t copies = 0;      // MXFP4 copies of the few-row sequences: not made, but the size a caller plans with still covers them
     for (int s = 0; s < n_seqs; ++s) {
         const int64_t lq = cu_q[s + 1] - cu_q[s], lk = cu_k[s + 1] - cu_k[s];
         if (lq < 0 || lk < 0) { st = EFQ_ERR_INVALID_ARG; return false; }
@@ -901,6 +902,7 @@ bool plan_varlen(const int64_t* cu_q, const int64_t* cu_k, int n_seqs, int Hq, i
             p.few_rows = std::max(p.few_rows, static_cast<int>(Hq / Hkv * lq));
             p.few_units += few_chunks(lk, Hq / Hkv * lq) * Hkv;
             p.few_keys += (lk + kTile - 1) / kTile * kTile;
+            copies += static_cast<size_t>(Hkv) * (kTile + 2 * ((lk + kTile - 1) / kTile * kTile)) * (64 + 4);
             continue;
         }
         const bool packed = use_packed_tile(Hq, Hkv, lq);
@@ -930,7 +932,7 @@ bool plan_varlen(const int64_t* cu_q, const int64_t* cu_k, int n_seqs, int Hq, i
     p.few_table = off;
     if (p.n_few > kFewInlineSeqs) off = align_up(off + sizeof(FewSeq) * p.n_few, 1024);
     p.few = off;
-    if (p.n_few > 0) off += plan_few(p.few_units, p.few_keys * Hkv, p.few_rows).total;
+    if (p.n_few > 0) off += std::max(plan_few(p.few_units, p.few_keys * Hkv, p.few_rows).total, align_up(copies, 1024));
     p.total = off;
     return true;
 }
