@@ -37,12 +37,6 @@ constexpr uint32_t kColD = 0;               // 2 x 32
 constexpr uint32_t kColSfA = 64;            // 2 x 4
 constexpr uint32_t kColSfB = 72;            // 2 x 4
 
-// The A operand (K or V^T codes of a tile) without swizzle: 8 rows x 16 bytes (a 32-element block) form a core matrix of
-// 128 bytes.  Strides that are no multiple of 128 keep the stores free of bank conflicts: lanes that write one row of
-// eight row groups (V^T) or eight rows of one block (K) meet 32 different banks.
-constexpr uint32_t kARowGroup = 144, kABlock = 16 * kARowGroup + 32;
-__device__ __forceinline__ uint32_t a_offset(uint32_t row, uint32_t blk) { return blk * kABlock + (row >> 3) * kARowGroup + (row & 7u) * 16u; }
-
 // One (sequence, KV head, chunk) of the grid.  Heads run fastest: the CTAs in flight read neighbouring heads of the same
 // tokens, which lie side by side in a token-major cache.
 struct Unit {
@@ -382,18 +376,17 @@ __global__ void __launch_bounds__(kFewThreads, 3) few_values_kernel(const __grid
     const Unit u = find_unit(P, static_cast<int>(blockIdx.x));
     const int R = P.G * u.Sq;
     few_setup(sm, warp);
-    // V: a lane takes eight channels of eight neighbouring keys, a warp 64 channels of a 32-key block: full 128-byte lines
-    const int oct = lane & 7, kg = lane >> 3, v_half = warp & 1, v_blk = warp >> 1;
+    const VTileLane L(warp, lane);
     uint4 vv[8];
     const int64_t v_step = P.k_row / 8;                  // a key on, in 16-byte pieces
-    const uint4* v_src = reinterpret_cast<const uint4*>(u.v + (u.j0 * kTile + v_blk * 32 + kg * 8) * P.k_row + v_half * 64 + oct * 8);
+    const uint4* v_src = reinterpret_cast<const uint4*>(u.v + (u.j0 * kTile + L.key) * P.k_row + L.ch);
     auto load_v = [&](int j) {
         if ((j + 1) * kTile <= u.Sk) {
             const uint4* src = v_src;
 #pragma unroll
             for (int i = 0; i < 8; ++i, src += v_step) vv[i] = __ldcs(src);
         } else {
-            const int left = u.Sk - (j * kTile + v_blk * 32 + kg * 8);
+            const int left = u.Sk - (j * kTile + L.key);
 #pragma unroll
             for (int i = 0; i < 8; ++i) vv[i] = i < left ? __ldcs(v_src + i * v_step) : make_uint4(0, 0, 0, 0);
         }
@@ -515,39 +508,9 @@ __global__ void __launch_bounds__(kFewThreads, 3) few_values_kernel(const __grid
             l_run = l_run * sm->alpha[slot][my_row] + (PRODUCER == 6 ? psum : static_cast<float>(count) * 0.5f * unit);
         }
         if (j + 1 < u.j1) load_scores();
-        // ---- V^T operand of the tile: a channel pair per word, its block maximum over the four lanes of a channel group
-        uint32_t w[8][4];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) { w[i][0] = vv[i].x; w[i][1] = vv[i].y; w[i][2] = vv[i].z; w[i][3] = vv[i].w; }
-        uint32_t fields[4];
-#pragma unroll
-        for (int p = 0; p < 4; ++p) {
-            fields[p] = bf16x2_absmax(bf16x2_absmax(bf16x2_absmax(w[0][p], w[1][p]), bf16x2_absmax(w[2][p], w[3][p])),
-                                      bf16x2_absmax(bf16x2_absmax(w[4][p], w[5][p]), bf16x2_absmax(w[6][p], w[7][p])));
-        }
-#pragma unroll
-        for (int p = 0; p < 4; ++p) fields[p] = bf16x2_absmax(fields[p], __shfl_xor_sync(0xffffffffu, fields[p], 8));
-#pragma unroll
-        for (int p = 0; p < 4; ++p) fields[p] = mxfp4_fields(bf16x2_absmax(fields[p], __shfl_xor_sync(0xffffffffu, fields[p], 16)));
-        uint8_t* const a_dst = sm->a[buf] + a_offset(v_half * 64 + oct * 8, v_blk) + kg * 4;
-#pragma unroll
-        for (int p = 0; p < 4; ++p) {
-            const uint32_t s2 = mxfp4_scales(fields[p]);
-            uint32_t e[8];
-#pragma unroll
-            for (int i = 0; i < 8; ++i) e[i] = bf16x2_mul(w[i][p], s2);
-            *reinterpret_cast<uint32_t*>(a_dst + 32 * p) = e2m1_word(bf16_lo(e[0]), bf16_lo(e[1]), bf16_lo(e[2]), bf16_lo(e[3]),
-                                                                     bf16_lo(e[4]), bf16_lo(e[5]), bf16_lo(e[6]), bf16_lo(e[7]));
-            *reinterpret_cast<uint32_t*>(a_dst + 32 * p + 16) = e2m1_word(bf16_hi(e[0]), bf16_hi(e[1]), bf16_hi(e[2]), bf16_hi(e[3]),
-                                                                          bf16_hi(e[4]), bf16_hi(e[5]), bf16_hi(e[6]), bf16_hi(e[7]));
-        }
+        // ---- V^T operand of the tile
+        mxfp4_v_tile(vv, L, sm->a[buf], sm->sf_a[buf]);
         if (j + 1 < u.j1) load_v(j + 1);
-        {   // scale bytes: lane group kg writes channel pair kg
-            const uint32_t f = kg < 2 ? (kg == 0 ? fields[0] : fields[1]) : (kg == 2 ? fields[2] : fields[3]);
-            uint8_t* const d = sm->sf_a[buf] + sf_tile_offset(v_half * 64 + oct * 8 + 2 * kg, v_blk);
-            d[0] = static_cast<uint8_t>(mxfp4_byte_lo(f));
-            d[16] = static_cast<uint8_t>(mxfp4_byte_hi(f));
-        }
         if (warp == ((t + 1) & 7) && j + 1 < u.j1 && lane < R)
             few_row_state<PRODUCER>(sm, P, t + 1, (t + 1) % kStateRing, sm->m_raw[slot][lane], lane);
         ptx::fence_proxy_async_smem();

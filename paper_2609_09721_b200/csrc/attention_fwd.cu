@@ -49,6 +49,8 @@ constexpr int kGroupWarps = 4;        // warps per probability group (one thread
 constexpr int kTileBytes = kTile * 64;          // 128 rows x 64 B of packed E2M1
 constexpr int kSfBytes = 512;
 constexpr int kVStageBytes = kTileBytes + 1024; // + 16 ones rows
+constexpr int kOutRowBytes = 528;       // staging row of the output: 512 bytes that start 4 banks apart, so that 128-bit stores
+                                        // of a warp (a row per lane) do not collide
 constexpr uint64_t kTimeoutCycles = 1500000000ull;
 
 // TMEM column map
@@ -62,7 +64,7 @@ constexpr uint32_t kTmemCols = 512;
 
 struct __align__(1024) Smem {
     uint8_t q[kTileBytes];
-    uint8_t k[kStages][kTileBytes];
+    uint8_t k[kStages][kTileBytes];     // k and v together: staging of the finished rows, once every load has been consumed
     uint8_t v[kStages][kVStageBytes];
     uint8_t p[2][kTileBytes];
     uint8_t sf_q[kSfBytes];
@@ -87,6 +89,8 @@ struct __align__(1024) Smem {
     uint32_t tmem_base;
     volatile uint32_t abort_flag;
 };
+
+static_assert(sizeof(Smem::k) + sizeof(Smem::v) >= kTile * kOutRowBytes, "finished rows fit where K and V were");
 
 struct FwdParams {
     int B, Hq, Hkv;
@@ -170,16 +174,16 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
     } else {
         Sq = P.Sq; Sk = P.Sk;
         packed = P.packed != 0;
-        const int64_t n_qtiles = packed ? 1 : P.Sq_pad / kTile;
-        const int64_t heads = packed ? P.Hkv : P.Hq;          // heads that own query tiles
-        const int64_t bh_count = static_cast<int64_t>(P.B) * heads;
-        const int64_t item = blockIdx.x;
-        const int64_t qt = n_qtiles - 1 - item / bh_count;
-        const int64_t bh = item % bh_count;
+        // 32-bit arithmetic: a 64-bit division costs hundreds of cycles that nothing hides here
+        const uint32_t n_qtiles = packed ? 1u : static_cast<uint32_t>(P.Sq_pad / kTile);
+        const uint32_t heads = packed ? P.Hkv : P.Hq;         // heads that own query tiles
+        const uint32_t bh_count = P.B * heads;
+        const uint32_t qt = n_qtiles - 1u - blockIdx.x / bh_count;
+        const uint32_t bh = blockIdx.x % bh_count;
         b = static_cast<int>(bh / heads);
         const int hh = static_cast<int>(bh % heads);
         if (packed) { hkv = hh; head0 = hkv * G; q0 = 0; q_row = static_cast<int>(bh * kTile); }
-        else { head0 = hh; hkv = hh / G; q0 = qt * kTile; q_row = static_cast<int>(bh * P.Sq_pad + q0); }
+        else { head0 = hh; hkv = hh / G; q0 = static_cast<int64_t>(qt) * kTile; q_row = static_cast<int>(bh * static_cast<uint32_t>(P.Sq_pad) + q0); }
         const int64_t kvh = static_cast<int64_t>(b) * P.Hkv + hkv;
         k_row0 = static_cast<int>(kvh * P.Sk_pad);
         v_x0 = 0;
@@ -196,42 +200,51 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         if (need < n_tiles) n_tiles = need;
     }
 
-    // ---- setup
-    if (threadIdx.x == 0) {
-        ptx::mbar_init(&sm->q_full, 1);
-        ptx::mbar_init(&sm->o_done, 1);
-        ptx::mbar_init(&sm->l_bar, 2 * kGroupWarps);
-        for (int s = 0; s < kStages; ++s) {
-            ptx::mbar_init(&sm->k_full[s], 1);
-            ptx::mbar_init(&sm->k_empty[s], 1);
-            ptx::mbar_init(&sm->v_full[s], 1);
-            ptx::mbar_init(&sm->v_empty[s], 1);
+    // ---- setup.  Warp 0 makes the barriers and goes on to load at once; the others wait for it in a named barrier that it
+    // only arrives at.
+    if (warp == 0) {
+        if (lane == 0) {
+            ptx::prefetch_tensormap(&map_q);
+            ptx::prefetch_tensormap(&map_k);
+            ptx::prefetch_tensormap(&map_v);
+            sm->abort_flag = 0u;
+            ptx::mbar_init(&sm->q_full, 1);
+            ptx::mbar_init(&sm->o_done, 1);
+            ptx::mbar_init(&sm->l_bar, 2 * kGroupWarps);
+            for (int s = 0; s < kStages; ++s) {
+                ptx::mbar_init(&sm->k_full[s], 1);
+                ptx::mbar_init(&sm->k_empty[s], 1);
+                ptx::mbar_init(&sm->v_full[s], 1);
+                ptx::mbar_init(&sm->v_empty[s], 1);
+            }
+            for (int i = 0; i < 2; ++i) {
+                ptx::mbar_init(&sm->s_full[i], 1);
+                ptx::mbar_init(&sm->s_empty[i], kGroupWarps);
+                ptx::mbar_init(&sm->p_full[i], kGroupWarps);
+                ptx::mbar_init(&sm->p_empty[i], 1);
+                ptx::mbar_init(&sm->o_ready[i], 4);
+                for (int qd = 0; qd < 4; ++qd) ptx::mbar_init(&sm->x_bar[i][qd], 1);
+            }
+            for (int i = 0; i < 4; ++i)
+                for (int qd = 0; qd < 4; ++qd) ptx::mbar_init(&sm->a_bar[i][qd], 1);
+            ptx::mbar_init_fence();
         }
-        for (int i = 0; i < 2; ++i) {
-            ptx::mbar_init(&sm->s_full[i], 1);
-            ptx::mbar_init(&sm->s_empty[i], kGroupWarps);
-            ptx::mbar_init(&sm->p_full[i], kGroupWarps);
-            ptx::mbar_init(&sm->p_empty[i], 1);
-            ptx::mbar_init(&sm->o_ready[i], 4);
-            for (int qd = 0; qd < 4; ++qd) ptx::mbar_init(&sm->x_bar[i][qd], 1);
-        }
-        for (int i = 0; i < 4; ++i)
-            for (int qd = 0; qd < 4; ++qd) ptx::mbar_init(&sm->a_bar[i][qd], 1);
-        sm->abort_flag = (*reinterpret_cast<volatile uint32_t*>(P.status) != 0u) ? 1u : 0u;
-        ptx::mbar_init_fence();
+        __syncwarp();
+        asm volatile("bar.arrive 1, 512;" ::: "memory");
+    } else {
+        if (warp == 1) ptx::tmem_alloc(&sm->tmem_base, kTmemCols);
+        // constant parts of the B operand of P~V: 16 rows of E2M1 1.0 (0x22) after each V^T stage, unit scales
+        for (int i = threadIdx.x - 32; i < kStages * 64; i += kThreads - 32)
+            reinterpret_cast<uint4*>(sm->v[i / 64] + kTileBytes)[i % 64] = make_uint4(0x22222222u, 0x22222222u, 0x22222222u, 0x22222222u);
+        for (int i = threadIdx.x - 32; i < kSfBytes / 4; i += kThreads - 32)
+            reinterpret_cast<uint32_t*>(sm->sf_ones)[i] = (i < 64 && (i & 3) == 0) ? 0x7f7f7f7fu : 0u;
+        ptx::fence_proxy_async_smem();
+        ptx::tc_fence_before_sync();
+        asm volatile("bar.sync 1, 512;" ::: "memory");
+        ptx::tc_fence_after_sync();
     }
-    // constant parts of the B operand of P~V: 16 rows of E2M1 1.0 (0x22) after each V^T stage, unit scales
-    for (int i = threadIdx.x; i < kStages * 256; i += kThreads)
-        reinterpret_cast<uint32_t*>(sm->v[i / 256] + kTileBytes)[i % 256] = 0x22222222u;
-    for (int i = threadIdx.x; i < kSfBytes / 4; i += kThreads)
-        reinterpret_cast<uint32_t*>(sm->sf_ones)[i] = (i < 64 && (i & 3) == 0) ? 0x7f7f7f7fu : 0u;
-    ptx::fence_proxy_async_smem();
-    if (warp == 1) ptx::tmem_alloc(&sm->tmem_base, kTmemCols);
-    ptx::tc_fence_before_sync();
-    __syncthreads();
-    ptx::tc_fence_after_sync();
-    const uint32_t tmem = sm->tmem_base;
-    const bool run = sm->abort_flag == 0 && n_tiles > 0;
+    const uint32_t tmem = warp == 0 ? 0u : sm->tmem_base;
+    const bool run = n_tiles > 0;
 
     // Register budget: the probability warpgroups take what the other two give up.  setmaxnreg moves registers
     // inside the CTA's own allocation only (512 threads x 128 at launch = 16 x 128 per lane), so the budgets must
@@ -259,6 +272,9 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
             ptx::bulk_load_1d(sm->sf_v[s], P.sf_v + (sfv_tile0 + j) * kSfBytes, kSfBytes, &sm->v_full[s]);
             if (++s == kStages) { s = 0; ph ^= 1u; }
         }
+    } else if (warp == 3 && lane == 0) {
+        // an earlier CTA of this launch gave up: the waits of this one end soon instead of after their limit
+        if (*reinterpret_cast<volatile uint32_t*>(P.status) != 0u) sm->abort_flag = 1u;
     } else if (run && warp == 1) {
         // =============================== S = Q K^T issuer ===============================
         // The whole warp runs the loop with warp-uniform state; one elected lane issues the tcgen05
@@ -539,30 +555,39 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
             ptx::tmem_ld32<32>(o_addr + 32, o);
             const uint32_t lcol = ptx::tmem_ld1(tmem + lane_base + kColO + 128);
             ptx::tmem_wait_ld();
-            if (row_valid) {
-                float l = __uint_as_float(lcol);
-                if (PRODUCER == 6) {
-                    // the accumulator refers to the maximum of the last tile, the larger of the two groups' references
-                    const float l0 = sm->lsum_x[0][row], l1 = sm->lsum_x[1][row];
-                    const float m0 = sm->mref_x[0][row], m1 = sm->mref_x[1][row];
-                    const float mf = fmaxf(m0, m1);
-                    l = (l0 != 0.0f ? l0 * ex2_approx(__fmul_rn(__fsub_rn(m0, mf), K.LOG2E)) : 0.0f) +
-                        (l1 != 0.0f ? l1 * ex2_approx(__fmul_rn(__fsub_rn(m1, mf), K.LOG2E)) : 0.0f);
-                }
-                const float inv = l > 0.0f ? 1.0f / l : 0.0f;
-                float4* dst = reinterpret_cast<float4*>(P.o + (o_base + hq * P.o_head + grow * P.o_row + 64 * group));
+            float l = __uint_as_float(lcol);
+            if (PRODUCER == 6) {
+                // the accumulator refers to the maximum of the last tile, the larger of the two groups' references
+                const float l0 = sm->lsum_x[0][row], l1 = sm->lsum_x[1][row];
+                const float m0 = sm->mref_x[0][row], m1 = sm->mref_x[1][row];
+                const float mf = fmaxf(m0, m1);
+                l = (l0 != 0.0f ? l0 * ex2_approx(__fmul_rn(__fsub_rn(m0, mf), K.LOG2E)) : 0.0f) +
+                    (l1 != 0.0f ? l1 * ex2_approx(__fmul_rn(__fsub_rn(m1, mf), K.LOG2E)) : 0.0f);
+            }
+            const float inv = l > 0.0f ? 1.0f / l : 0.0f;
+            // Through shared memory, inside the warp: a lane holds 256 bytes of a row, and storing them from registers would
+            // touch 32 rows per instruction (5000 cycles for the tile).  Read back, 16 lanes store 256 bytes of one row.
+            uint8_t* const stage = sm->k[0] + 256 * group + (row - lane) * kOutRowBytes;
 #pragma unroll
-                for (int i = 0; i < 16; ++i) {
-                    float4 v;
-                    v.x = __uint_as_float(o[4 * i + 0]) * inv;
-                    v.y = __uint_as_float(o[4 * i + 1]) * inv;
-                    v.z = __uint_as_float(o[4 * i + 2]) * inv;
-                    v.w = __uint_as_float(o[4 * i + 3]) * inv;
-                    dst[i] = v;
-                }
+            for (int i = 0; i < 16; ++i) {
+                float4 v;
+                v.x = __uint_as_float(o[4 * i + 0]) * inv;
+                v.y = __uint_as_float(o[4 * i + 1]) * inv;
+                v.z = __uint_as_float(o[4 * i + 2]) * inv;
+                v.w = __uint_as_float(o[4 * i + 3]) * inv;
+                *reinterpret_cast<float4*>(stage + lane * kOutRowBytes + 16 * i) = v;
+            }
+            __syncwarp();
+            const uint64_t my_dst = row_valid ? reinterpret_cast<uint64_t>(P.o + (o_base + hq * P.o_head + grow * P.o_row + 64 * group)) : 0ull;
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+                const int r = 2 * i + (lane >> 4);
+                const uint64_t dst = __shfl_sync(0xffffffffu, my_dst, r);
+                const float4 v = *reinterpret_cast<const float4*>(stage + r * kOutRowBytes + 16 * (lane & 15));
+                if (dst != 0ull) __stcs(reinterpret_cast<float4*>(dst) + (lane & 15), v);
             }
         }
-    } else if (sm->abort_flag == 0) {
+    } else {
         // no visible key for the whole tile: rows are zero
         if (row_valid) {
             float4* dst = reinterpret_cast<float4*>(P.o + (o_base + hq * P.o_head + grow * P.o_row + 64 * group));
@@ -872,7 +897,8 @@ efq_status_t attention_impl(const void* q, const void* k, const void* v, float* 
 // ------------------------------------------------------------------------------------------------
 // Packed variable-length batch: every sequence quantised by itself, all of them in two launches
 // ------------------------------------------------------------------------------------------------
-// Workspace: status words | tables (sequence table, item table, quantiser jobs, their CTA prefix sums) |
+// Workspace: status words | tables from the host (sequences, quantiser jobs, their CTA prefix sums, query tiles in the order
+// of their weight) | item table (written on the device: it has an entry per head) |
 // Q codes [rows of all sequences, 64 B] | Q scale tiles | K codes | K scale tiles |
 // V^T codes [Hkv * 128, sum of Sk_pad / 2 B] (the sequences side by side along the keys) | V scale tiles.
 struct VarlenPlan {
@@ -880,8 +906,8 @@ struct VarlenPlan {
     int n_few, few_rows;             // ... and the few-row path (attention_few.cu); the most query rows of one of them
     int64_t few_units, few_keys;     // their chunks times KV heads; their keys, padded to 128
     int64_t q_rows, k_rows, k_cols;  // rows of the Q and K code matrices, keys along V^T (all padded to 128)
-    int64_t items, quant_ctas;
-    size_t tables, seqs_off, items_off, jobs_off, prefix_off, qc, qsf, kc, ksf, vt, vsf, few_table, few, total;
+    int64_t items, groups, quant_ctas;
+    size_t tables, seqs_off, jobs_off, prefix_off, groups_off, items_off, qc, qsf, kc, ksf, vt, vsf, few_table, few, total;
 };
 
 // checks the two prefix arrays and lays the workspace out; false with st set on bad input
@@ -912,17 +938,19 @@ bool plan_varlen(const int64_t* cu_q, const int64_t* cu_k, int n_seqs, int Hq, i
         p.k_rows += Hkv * lk_pad;
         p.k_cols += lk_pad;
         p.items += packed ? Hkv : (lq_pad / kTile) * Hq;
-        p.quant_ctas += ((packed ? Hkv : Hq) * lq_pad * 4 + 255) / 256 + (Hkv * lk_pad * 4 + 255) / 256 + (Hkv * (lk_pad / 32) + 1) / 2;
+        p.groups += lq_pad / kTile;
+        p.quant_ctas += (packed ? Hkv : Hq) * (lq_pad / kTile) + 2 * Hkv * (lk_pad / kTile);
     }
     // 32-bit tile coordinates and grid sizes
     if (p.q_rows >= (1ll << 31) || p.k_rows >= (1ll << 31) || p.k_cols >= (1ll << 31) || p.items >= (1ll << 31) ||
         p.quant_ctas >= (1ll << 31) || p.few_units >= (1ll << 31) || p.few_keys >= (1ll << 31)) { st = EFQ_ERR_UNSUPPORTED; return false; }
     size_t off = 1024;
     p.seqs_off = off;   off = align_up(off + sizeof(SeqDesc) * p.n_active, 256);
-    p.items_off = off;  off = align_up(off + sizeof(ItemDesc) * static_cast<size_t>(p.items), 256);
     p.jobs_off = off;   off = align_up(off + sizeof(QuantJob) * 3 * p.n_active, 256);
-    p.prefix_off = off; off = align_up(off + sizeof(int32_t) * (3 * p.n_active + 1), 1024);
+    p.prefix_off = off; off = align_up(off + sizeof(int32_t) * (3 * p.n_active + 1), 256);
+    p.groups_off = off; off = align_up(off + sizeof(ItemGroup) * static_cast<size_t>(p.groups), 1024);
     p.tables = off - 1024;
+    p.items_off = off;  off = align_up(off + sizeof(ItemDesc) * static_cast<size_t>(p.items), 1024);
     p.qc = off;  off = align_up(off + static_cast<size_t>(p.q_rows) * 64, 1024);
     p.qsf = off; off = align_up(off + static_cast<size_t>(p.q_rows / kTile) * kSfBytes, 1024);
     p.kc = off;  off = align_up(off + static_cast<size_t>(p.k_rows) * 64, 1024);
@@ -1198,13 +1226,16 @@ extern "C" efq_status_t efq_attention_fwd_varlen(const void* q, const void* k, c
     // host copies of the tables, in the layout of the workspace's table region
     std::vector<uint8_t> tables(p.tables, 0);
     SeqDesc* seqs = reinterpret_cast<SeqDesc*>(tables.data() + (p.seqs_off - 1024));
-    ItemDesc* items = reinterpret_cast<ItemDesc*>(tables.data() + (p.items_off - 1024));
+    ItemGroup* groups = reinterpret_cast<ItemGroup*>(tables.data() + (p.groups_off - 1024));
     QuantJob* jobs = reinterpret_cast<QuantJob*>(tables.data() + (p.jobs_off - 1024));
     int32_t* prefix = reinterpret_cast<int32_t*>(tables.data() + (p.prefix_off - 1024));
     const __nv_bfloat16* qb = static_cast<const __nv_bfloat16*>(q);
     const __nv_bfloat16* kb = static_cast<const __nv_bfloat16*>(k);
     const __nv_bfloat16* vb = static_cast<const __nv_bfloat16*>(v);
-    int64_t q_row = 0, k_row = 0, k_col = 0, n_items = 0, ctas = 0, few_unit = 0, few_key = 0;
+    struct QueryTile { int32_t weight, seq, qt; };   // weight: KV tiles that it walks
+    std::vector<QueryTile> order;
+    order.reserve(static_cast<size_t>(p.groups));
+    int64_t q_row = 0, k_row = 0, k_col = 0, ctas = 0, few_unit = 0, few_key = 0;
     int a = 0, f = 0;
     FewParams F{};
     std::vector<FewSeq> few_long;            // more sequences than the kernel parameters hold
@@ -1232,12 +1263,10 @@ extern "C" efq_status_t efq_attention_fwd_varlen(const void* q, const void* k, c
         sd.q_row0 = static_cast<int32_t>(q_row); sd.Sq_pad = static_cast<int32_t>(lq_pad);
         sd.k_row0 = static_cast<int32_t>(k_row); sd.Sk_pad = static_cast<int32_t>(lk_pad);
         sd.k_col0 = static_cast<int32_t>(k_col); sd.packed = packed ? 1 : 0;
-        // work items: heaviest query tiles of a sequence first, the heads of a GQA group adjacent
-        if (packed) {
-            for (int hk = 0; hk < Hkv; ++hk) items[n_items++] = ItemDesc{a, 0, hk, 0};
-        } else {
-            for (int64_t qt = lq_pad / kTile - 1; qt >= 0; --qt)
-                for (int hh = 0; hh < Hq; ++hh) items[n_items++] = ItemDesc{a, static_cast<int32_t>(qt), hh, 0};
+        for (int64_t qt = 0; qt < lq_pad / kTile; ++qt) {
+            int64_t keys = lk;
+            if (causal) keys = std::min(lk, std::min((qt + 1) * kTile, lq) + lk - lq);
+            order.push_back(QueryTile{static_cast<int32_t>((std::max<int64_t>(keys, 0) + kTile - 1) / kTile), a, static_cast<int32_t>(qt)});
         }
         // quantiser jobs: the sequence's own Q, K, V (token-major source: a head is 128 elements, a token H * 128)
         QuantJob& jq = jobs[3 * a];
@@ -1293,11 +1322,19 @@ extern "C" efq_status_t efq_attention_fwd_varlen(const void* q, const void* k, c
     if (p.n_active == 0)             // nothing to launch: the status word still has to read "no problem"
         return cudaMemsetAsync(ws, 0, 4, s) == cudaSuccess ? EFQ_OK : EFQ_ERR_CUDA;
     prefix[3 * p.n_active] = static_cast<int32_t>(ctas);
+    // The heaviest query tiles of the whole batch first, so that the last CTAs to start are short ones.
+    std::stable_sort(order.begin(), order.end(), [](const QueryTile& x, const QueryTile& y) { return x.weight > y.weight; });
+    int64_t n_items = 0;
+    for (size_t i = 0; i < order.size(); ++i) {
+        groups[i] = ItemGroup{static_cast<int32_t>(n_items), order[i].seq, order[i].qt};
+        n_items += seqs[order[i].seq].packed ? Hkv : Hq;
+    }
 
     // Pageable host memory: the call returns once the bytes sit in the driver's staging area, so the vector may go.
     if (cudaMemcpyAsync(ws + 1024, tables.data(), p.tables, cudaMemcpyHostToDevice, s) != cudaSuccess) return EFQ_ERR_CUDA;
     if (launch_quantize_jobs(reinterpret_cast<const QuantJob*>(ws + p.jobs_off), reinterpret_cast<const int32_t*>(ws + p.prefix_off),
-                             3 * p.n_active, ctas, p.n_few > 0 ? nullptr : reinterpret_cast<uint32_t*>(ws), s) != cudaSuccess)
+                             3 * p.n_active, ctas, reinterpret_cast<const ItemGroup*>(ws + p.groups_off), static_cast<int>(order.size()), n_items,
+                             reinterpret_cast<ItemDesc*>(ws + p.items_off), p.n_few > 0 ? nullptr : reinterpret_cast<uint32_t*>(ws), s) != cudaSuccess)
         return EFQ_ERR_CUDA;
 
     CUtensorMap mq, mk, mv;

@@ -34,12 +34,19 @@ struct QuantJob {
     int32_t pad;
 };
 
+// The work items of one query tile of one sequence, one per head that owns it, in the order the fused forward takes them.
+// The host lists the tiles (heaviest first); the quantiser's launch spreads them into the item table.
+struct ItemGroup {
+    int32_t first_item, seq, qt;
+};
+struct ItemDesc;
+
 // Q, K and V of one [B, H, S, d] problem (or one sequence) in one launch; also clears the 256 status words.
 cudaError_t launch_quantize_qkv(const QuantSeg& q, const QuantSeg& k, const QuantSeg& v, uint32_t* status, cudaStream_t stream);
 // The jobs of a packed batch in one launch: jobs and first_cta (n_jobs + 1 prefix sums of CTAs) live in device memory.
 // status: the words to clear, null if an earlier launch of the call has cleared them.
-cudaError_t launch_quantize_jobs(const QuantJob* jobs, const int32_t* first_cta, int n_jobs, int64_t total_ctas, uint32_t* status,
-                                 cudaStream_t stream);
+cudaError_t launch_quantize_jobs(const QuantJob* jobs, const int32_t* first_cta, int n_jobs, int64_t total_ctas, const ItemGroup* groups,
+                                 int n_groups, int64_t n_items, ItemDesc* items, uint32_t* status, cudaStream_t stream);
 // CTAs a job needs (256 threads each)
 int64_t quantize_job_ctas(const QuantJob& job);
 

@@ -116,36 +116,9 @@ __device__ __forceinline__ void bulk_load_1d(void* smem_dst, const void* gmem_sr
         : "memory");
 }
 
-// 1-D bulk copy shared -> global, part of the thread's current bulk group; alignment and size as above.
-__device__ __forceinline__ void bulk_store_1d(void* gmem_dst, const void* smem_src, uint32_t bytes)
+__device__ __forceinline__ void prefetch_tensormap(const CUtensorMap* map)
 {
-    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;"
-                 ::"l"(gmem_dst), "r"(smem_u32(smem_src)), "r"(bytes) : "memory");
-}
-
-// ---------------------------------------------------------------- cluster launch control
-// Asks for a block of this grid that has not started yet; the 16-byte answer lands in shared memory and completes 16
-// bytes of the barrier's transaction.
-__device__ __forceinline__ void clc_try_cancel(void* smem_answer, uint64_t* bar)
-{
-    asm volatile("clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];"
-                 ::"r"(smem_u32(smem_answer)), "r"(smem_u32(bar)) : "memory");
-}
-// Block index of the block this CTA takes over, -1 if there was none left.
-__device__ __forceinline__ int clc_first_block(const void* smem_answer)
-{
-    uint32_t got, x;
-    asm volatile(
-        "{\n\t.reg .b128 h;\n\t.reg .pred p;\n\t"
-        "ld.shared.b128 h, [%2];\n\t"
-        "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, h;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t"
-        "mov.u32 %1, 0;\n\t"
-        "@p clusterlaunchcontrol.query_cancel.get_first_ctaid::x.b32.b128 %1, h;\n\t}\n"
-        : "=r"(got), "=r"(x)
-        : "r"(smem_u32(smem_answer))
-        : "memory");
-    return got ? static_cast<int>(x) : -1;
+    asm volatile("prefetch.tensormap [%0];" ::"l"(map) : "memory");
 }
 
 // ---------------------------------------------------------------- TMEM allocation (one full warp)
