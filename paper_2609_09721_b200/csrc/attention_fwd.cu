@@ -625,26 +625,27 @@ EncodeTiledFn get_encode()
     return fn;
 }
 
-// [rows, row_bytes] u8 matrix, box 64 B x 128 rows, 64-byte swizzle.  A descriptor depends on nothing but
-// (base, row_bytes, rows), so the last few are kept: a serving loop that calls with the same workspace and shape
-// (decode steps above all) does not pay for three driver calls per forward.
+// A descriptor depends on nothing but the base, the shape and the kind of map, so the last few are kept: a serving loop
+// that calls with the same buffers and shape (decode steps above all) does not pay for driver calls per forward.
+enum MapKind : uint32_t { kMapCodes, kMapBf16 };
 struct MapCacheEntry {
     const void* base;
     uint64_t row_bytes, rows;
+    MapKind kind;
     CUtensorMap map;
 };
-constexpr int kMapCacheSize = 24;
+constexpr int kMapCacheSize = 32;
 std::mutex g_map_mutex;
 MapCacheEntry g_map_cache[kMapCacheSize] = {};
 int g_map_next = 0;
 
-bool encode_map(CUtensorMap* map, const void* base, uint64_t row_bytes, uint64_t rows)
+bool encode_any(CUtensorMap* map, const void* base, uint64_t row_bytes, uint64_t rows, MapKind kind)
 {
     {
         std::lock_guard<std::mutex> lock(g_map_mutex);
         for (int i = 0; i < kMapCacheSize; ++i) {
             const MapCacheEntry& e = g_map_cache[i];
-            if (e.base == base && e.row_bytes == row_bytes && e.rows == rows) {
+            if (e.base == base && e.row_bytes == row_bytes && e.rows == rows && e.kind == kind) {
                 *map = e.map;
                 return true;
             }
@@ -652,19 +653,22 @@ bool encode_map(CUtensorMap* map, const void* base, uint64_t row_bytes, uint64_t
     }
     EncodeTiledFn enc = get_encode();
     if (!enc) return false;
-    cuuint64_t dims[2] = {row_bytes, rows};
+    const bool codes = kind == kMapCodes;
+    cuuint64_t dims[2] = {codes ? row_bytes : row_bytes / 2, rows};
     cuuint64_t strides[1] = {row_bytes};
     cuuint32_t box[2] = {64, 128};
     cuuint32_t estr[2] = {1, 1};
-    if (enc(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<void*>(base), dims, strides, box, estr,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+    if (enc(map, codes ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box,
+            estr, CU_TENSOR_MAP_INTERLEAVE_NONE, codes ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
+            CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return false;
     std::lock_guard<std::mutex> lock(g_map_mutex);
-    g_map_cache[g_map_next] = MapCacheEntry{base, row_bytes, rows, *map};
+    g_map_cache[g_map_next] = MapCacheEntry{base, row_bytes, rows, kind, *map};
     g_map_next = (g_map_next + 1) % kMapCacheSize;
     return true;
 }
+// [rows, row_bytes] matrix of packed codes, box 64 B x 128 rows, 64-byte swizzle
+bool encode_map(CUtensorMap* map, const void* base, uint64_t row_bytes, uint64_t rows) { return encode_any(map, base, row_bytes, rows, kMapCodes); }
 
 struct Workspace {
     size_t status, qc, qsf, kc, ksf, vt, vsf, total;
@@ -966,6 +970,9 @@ bool plan_varlen(const int64_t* cu_q, const int64_t* cu_k, int n_seqs, int Hq, i
 }
 
 }  // namespace
+
+bool encode_bf16_map(CUtensorMap* map, const void* base, uint64_t cols, uint64_t rows) { return encode_any(map, base, 2 * cols, rows, kMapBf16); }
+
 }  // namespace efq
 
 extern "C" size_t efq_attention_workspace_bytes(int B, int Hq, int Hkv, int64_t Sq, int64_t Sk, int d)

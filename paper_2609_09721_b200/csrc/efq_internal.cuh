@@ -2,6 +2,7 @@
 // the job descriptions of the quantiser and the tables a packed variable-length batch hands to the kernels.
 #pragma once
 
+#include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -49,6 +50,9 @@ cudaError_t launch_quantize_jobs(const QuantJob* jobs, const int32_t* first_cta,
                                  int n_groups, int64_t n_items, ItemDesc* items, uint32_t* status, cudaStream_t stream);
 // CTAs a job needs (256 threads each)
 int64_t quantize_job_ctas(const QuantJob& job);
+
+// Tensor map of a row-major bf16 matrix, box 64 columns (128 B) x 128 rows, 128-byte swizzle; the last few are kept.
+bool encode_bf16_map(CUtensorMap* map, const void* base, uint64_t cols, uint64_t rows);
 
 // One sequence of a packed batch as the fused forward sees it.
 struct SeqDesc {
