@@ -163,8 +163,8 @@ __global__ void __launch_bounds__(kFewThreads, N <= 8 ? 4 : 3) few_scores_kernel
     FewSmem* const sm = &smem;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     few_setup(sm, warp);
-    asm volatile("griddepcontrol.wait;" ::: "memory");                // the kernels before: inputs, and the workspace of an earlier call
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    ptx::grid_wait();                // the kernels before: inputs, and the workspace of an earlier call
+    ptx::grid_launch_next();
     const Unit u = find_unit(P, static_cast<int>(blockIdx.x));
     const int R = P.G * u.Sq;
     if (blockIdx.x == 0) P.status[tid] = 0u;
@@ -372,7 +372,7 @@ __global__ void __launch_bounds__(kFewThreads, 3) few_values_kernel(const __grid
     __shared__ FewSmem smem;
     FewSmem* const sm = &smem;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    ptx::grid_launch_next();
     const Unit u = find_unit(P, static_cast<int>(blockIdx.x));
     const int R = P.G * u.Sq;
     few_setup(sm, warp);
@@ -393,7 +393,7 @@ __global__ void __launch_bounds__(kFewThreads, 3) few_values_kernel(const __grid
         v_src += kTile * v_step;
     };
     load_v(u.j0);       // an input: whatever produced it had finished before the scores kernel allowed this one to start
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    ptx::grid_wait();
 
     // the chunk's block maxima and the running maximum of every row before the chunk
     const float* const bm = P.block_max + u.s_off / 32;
@@ -550,7 +550,7 @@ __global__ void __launch_bounds__(128) few_merge_kernel(const __grid_constant__ 
     const int head = static_cast<int>(blockIdx.x) % P.Hkv, seq = static_cast<int>(blockIdx.x) / P.Hkv;
     const int first_id = head + (P.n_seqs == 0 ? seq * P.dense_chunks * P.Hkv : (P.seqs != nullptr ? P.seqs : P.inline_seqs)[seq].first_unit);
     const Unit u = find_unit(P, first_id);
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    ptx::grid_wait();
     if (row >= P.G * u.Sq) return;
     const size_t part_floats = static_cast<size_t>(P.row_cap) * kFewPartFloats, step = part_floats * P.Hkv;
     const float* const first = P.partials + first_id * part_floats;
@@ -577,40 +577,24 @@ __global__ void __launch_bounds__(128) few_merge_kernel(const __grid_constant__ 
     u.o[g * P.q_head + (row - g * u.Sq) * P.q_row + threadIdx.x] = t * (d > 0.0f ? 1.0f / d : 0.0f);
 }
 
-// Each kernel may start while the one before it still runs; what it needs of that one it waits for itself.
-template <typename Kernel>
-cudaError_t launch_overlapped(Kernel kernel, dim3 grid, int threads, cudaStream_t stream, const FewParams& P)
-{
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = grid;
-    cfg.blockDim = dim3(threads);
-    cfg.stream = stream;
-    cudaLaunchAttribute at{};
-    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at.val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = &at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, P);
-}
-
 template <int N>
 cudaError_t launch_n(int producer, const FewParams& P, cudaStream_t stream)
 {
     const dim3 grid(static_cast<unsigned>(P.n_units));
-    cudaError_t e = launch_overlapped(few_scores_kernel<N>, grid, kFewThreads, stream, P);
+    cudaError_t e = launch_overlapped(few_scores_kernel<N>, grid, kFewThreads, 0, stream, P);
     if (e != cudaSuccess) return e;
     switch (producer) {
-        case 0: e = launch_overlapped(few_values_kernel<N, 0>, grid, kFewThreads, stream, P); break;
-        case 1: e = launch_overlapped(few_values_kernel<N, 1>, grid, kFewThreads, stream, P); break;
-        case 2: e = launch_overlapped(few_values_kernel<N, 2>, grid, kFewThreads, stream, P); break;
-        case 3: e = launch_overlapped(few_values_kernel<N, 3>, grid, kFewThreads, stream, P); break;
-        case 4: e = launch_overlapped(few_values_kernel<N, 4>, grid, kFewThreads, stream, P); break;
-        case 5: e = launch_overlapped(few_values_kernel<N, 5>, grid, kFewThreads, stream, P); break;
-        case 6: e = launch_overlapped(few_values_kernel<N, 6>, grid, kFewThreads, stream, P); break;
+        case 0: e = launch_overlapped(few_values_kernel<N, 0>, grid, kFewThreads, 0, stream, P); break;
+        case 1: e = launch_overlapped(few_values_kernel<N, 1>, grid, kFewThreads, 0, stream, P); break;
+        case 2: e = launch_overlapped(few_values_kernel<N, 2>, grid, kFewThreads, 0, stream, P); break;
+        case 3: e = launch_overlapped(few_values_kernel<N, 3>, grid, kFewThreads, 0, stream, P); break;
+        case 4: e = launch_overlapped(few_values_kernel<N, 4>, grid, kFewThreads, 0, stream, P); break;
+        case 5: e = launch_overlapped(few_values_kernel<N, 5>, grid, kFewThreads, 0, stream, P); break;
+        case 6: e = launch_overlapped(few_values_kernel<N, 6>, grid, kFewThreads, 0, stream, P); break;
         default: return cudaErrorInvalidValue;
     }
     if (e != cudaSuccess) return e;
-    return launch_overlapped(few_merge_kernel, dim3(static_cast<unsigned>(P.n_heads), static_cast<unsigned>(P.row_cap)), 128, stream, P);
+    return launch_overlapped(few_merge_kernel, dim3(static_cast<unsigned>(P.n_heads), static_cast<unsigned>(P.row_cap)), 128, 0, stream, P);
 }
 
 }  // namespace

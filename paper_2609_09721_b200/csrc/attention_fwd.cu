@@ -81,8 +81,7 @@ struct __align__(1024) Smem {
     uint64_t v_full[kStages], v_empty[kStages];
     uint64_t s_full[2], s_empty[2];
     uint64_t p_full[2], p_empty[2];
-    uint64_t x_bar[2][4];     // [group][lane quarter]: runmax of the group's latest tile is published
-    uint64_t a_bar[4][4];     // [tile mod 4][lane quarter]: alpha of that tile is published
+    uint64_t a_bar[4][4];     // [tile mod 4][lane quarter]: running maximum and alpha of that tile are published
     uint64_t o_ready[2];      // accumulator rows rescaled (or found unchanged) for the tile of this parity
     uint64_t o_done;          // the last P~V of the work item has completed
     uint64_t l_bar;           // FP32-denominator baseline only: all eight probability warps have written lsum_x / mref_x
@@ -161,6 +160,7 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
     int64_t sfv_tile0;
     bool packed;
     if (P.items != nullptr) {
+        ptx::grid_wait();                                     // the item table is written by the kernel before
         const ItemDesc it = P.items[blockIdx.x];
         const SeqDesc sd = P.seqs[it.seq];
         Sq = sd.Sq; Sk = sd.Sk; o_base = sd.o_off; b = it.seq;
@@ -223,7 +223,6 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                 ptx::mbar_init(&sm->p_full[i], kGroupWarps);
                 ptx::mbar_init(&sm->p_empty[i], 1);
                 ptx::mbar_init(&sm->o_ready[i], 4);
-                for (int qd = 0; qd < 4; ++qd) ptx::mbar_init(&sm->x_bar[i][qd], 1);
             }
             for (int i = 0; i < 4; ++i)
                 for (int qd = 0; qd < 4; ++qd) ptx::mbar_init(&sm->a_bar[i][qd], 1);
@@ -253,6 +252,8 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
     asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
     if (run && warp == 0 && lane == 0) {
         // =============================== TMA producer (one thread) ===============================
+        // The operands come from the kernel before.  Whatever else this kernel writes or reads follows from the loads.
+        ptx::grid_wait();
         ptx::mbar_arrive_expect_tx(&sm->q_full, kTileBytes + kSfBytes);
         ptx::tma_load_2d(sm->q, &map_q, 0, q_row, &sm->q_full);
         ptx::bulk_load_1d(sm->sf_q, P.sf_q + static_cast<int64_t>(q_row / kTile) * kSfBytes, kSfBytes, &sm->q_full);
@@ -273,6 +274,7 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
             if (++s == kStages) { s = 0; ph ^= 1u; }
         }
     } else if (warp == 3 && lane == 0) {
+        ptx::grid_wait();
         // an earlier CTA of this launch gave up: the waits of this one end soon instead of after their limit
         if (*reinterpret_cast<volatile uint32_t*>(P.status) != 0u) sm->abort_flag = 1u;
     } else if (run && warp == 1) {
@@ -444,7 +446,7 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
             bool have_prev;
             {
                 // polls whose answers are needed later travel while the scores do
-                have_prev = j == 0 || ptx::mbar_try_wait(&sm->x_bar[sb ^ 1][quarter], static_cast<uint32_t>(((j - 1) >> 1) & 1));
+                have_prev = j == 0 || ptx::mbar_try_wait(&sm->a_bar[(j - 1) & 3][quarter], static_cast<uint32_t>((j - 1) >> 2) & 1u);
                 ptx::tmem_wait_ld();
                 ptx::tc_fence_before_sync();          // the S buffer is handed back with the joint publication below
                 const int64_t key0 = j * kTile;
@@ -460,7 +462,7 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
             // ---- running row maximum (Eq. rowmax-update): handed over from the group that owns tile j-1
             float m_prev = -INFINITY;
             if (j > 0) {
-                if (!have_prev && !wait_all(&sm->x_bar[sb ^ 1][quarter], static_cast<uint32_t>(((j - 1) >> 1) & 1), sm, P.status)) { ok = false; break; }
+                if (!have_prev && !wait_all(&sm->a_bar[(j - 1) & 3][quarter], static_cast<uint32_t>((j - 1) >> 2) & 1u, sm, P.status)) { ok = false; break; }
                 m_prev = sm->runmax[sb ^ 1][row];
             }
             float m_new = fmaxf(fmaxf(m_prev, bmax[0]), max3(bmax[1], bmax[2], bmax[3]));
@@ -479,7 +481,6 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
             sm->alpha[j & 3][row] = alpha;
             __syncwarp();
             if (lane == 0) {
-                ptx::mbar_arrive(&sm->x_bar[sb][quarter]);
                 ptx::mbar_arrive(&sm->a_bar[j & 3][quarter]);
                 ptx::mbar_arrive(&sm->s_empty[sb]);           // every lane's scores are in registers (wait::ld above)
             }
@@ -589,6 +590,7 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         }
     } else {
         // no visible key for the whole tile: rows are zero
+        ptx::grid_wait();
         if (row_valid) {
             float4* dst = reinterpret_cast<float4*>(P.o + (o_base + hq * P.o_head + grow * P.o_row + 64 * group));
             for (int i = 0; i < 16; ++i) dst[i] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -735,8 +737,7 @@ cudaError_t launch_one(dim3 grid, size_t smem, cudaStream_t stream, const CUtens
             done[dev] = true;
         }
     }
-    attention_fwd_kernel<PRODUCER, DEBUG, FIX8><<<grid, kThreads, smem, stream>>>(mq, mk, mv, P);
-    return cudaGetLastError();
+    return launch_overlapped(attention_fwd_kernel<PRODUCER, DEBUG, FIX8>, grid, kThreads, smem, stream, mq, mk, mv, P);
 }
 
 template <int PRODUCER>

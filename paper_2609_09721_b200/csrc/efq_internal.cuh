@@ -11,6 +11,25 @@
 
 namespace efq {
 
+// Launches a kernel that may start while the one before it in the stream still runs (its blocks set up meanwhile); what it
+// needs of the work before it waits for itself with griddepcontrol.wait.  Takes about 2 microseconds off a call of two
+// kernels back to back.
+template <typename... Params, typename... Args>
+inline cudaError_t launch_overlapped(void (*kernel)(Params...), dim3 grid, int threads, size_t smem, cudaStream_t stream, const Args&... args)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(static_cast<unsigned>(threads));
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 // One operand of one sequence for the quantiser.  Rows of Q and K are quantised along d (blocks of 32), V along
 // the keys (blocks of 32 aligned to the sequence's own key index, per channel) and written transposed.
 struct QuantSeg {

@@ -23,6 +23,7 @@
 #include "efq_common.cuh"
 #include "efq_internal.cuh"
 #include "mxfp4.cuh"
+#include "sm100_ptx.cuh"
 
 namespace efq {
 
@@ -123,6 +124,8 @@ struct QuantArgs {
 __global__ void __launch_bounds__(256) quantize_qkv_kernel(const __grid_constant__ QuantArgs a)
 {
     __shared__ QuantSmem sm;
+    ptx::grid_wait();
+    ptx::grid_launch_next();
     const int cta = static_cast<int>(blockIdx.x);
     if (cta == 0) a.status[threadIdx.x] = 0u;
     if (cta < a.q_ctas) quantize_rows(a.q, cta);
@@ -137,6 +140,8 @@ __global__ void __launch_bounds__(256) quantize_jobs_kernel(const QuantJob* __re
                                                             int n_items, ItemDesc* __restrict__ items, uint32_t* status)
 {
     __shared__ QuantSmem sm;
+    ptx::grid_wait();
+    ptx::grid_launch_next();
     const int cta = blockIdx.x;
     if (cta == 0 && status != nullptr) status[threadIdx.x] = 0u;
     if (cta >= n_quant) {
@@ -173,8 +178,7 @@ cudaError_t launch_quantize_qkv(const QuantSeg& q, const QuantSeg& k, const Quan
     a.status = status;
     a.q_ctas = static_cast<int>(nq);
     a.k_ctas = static_cast<int>(nk);
-    quantize_qkv_kernel<<<static_cast<unsigned>(grid), 256, 0, stream>>>(a);
-    return cudaGetLastError();
+    return launch_overlapped(quantize_qkv_kernel, dim3(static_cast<unsigned>(grid)), 256, 0, stream, a);
 }
 
 cudaError_t launch_quantize_jobs(const QuantJob* jobs, const int32_t* first_cta, int n_jobs, int64_t total_ctas, const ItemGroup* groups,
@@ -182,9 +186,8 @@ cudaError_t launch_quantize_jobs(const QuantJob* jobs, const int32_t* first_cta,
 {
     const int64_t grid = total_ctas + (n_items + 255) / 256;
     if (n_jobs <= 0 || total_ctas <= 0 || grid > 0x7fffffffll) return cudaErrorInvalidValue;
-    quantize_jobs_kernel<<<static_cast<unsigned>(grid), 256, 0, stream>>>(jobs, first_cta, n_jobs, static_cast<int>(total_ctas), groups,
-                                                                          n_groups, static_cast<int>(n_items), items, status);
-    return cudaGetLastError();
+    return launch_overlapped(quantize_jobs_kernel, dim3(static_cast<unsigned>(grid)), 256, 0, stream, jobs, first_cta, n_jobs,
+                             static_cast<int>(total_ctas), groups, n_groups, static_cast<int>(n_items), items, status);
 }
 
 }  // namespace efq

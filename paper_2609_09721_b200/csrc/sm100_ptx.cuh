@@ -26,6 +26,12 @@ __device__ __forceinline__ bool elect_one()
     return pred != 0;
 }
 
+// ---------------------------------------------------------------- overlap with the neighbouring kernels of the stream
+// The work before this kernel has finished and is visible.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// The kernel after this one may start its blocks (it waits by grid_wait() for what it needs).
+__device__ __forceinline__ void grid_launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // ---------------------------------------------------------------- mbarrier
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count)
 {
