@@ -140,7 +140,7 @@ __device__ __forceinline__ bool wait_all(uint64_t* bar, uint32_t parity, Smem* s
     return __all_sync(__activemask(), ok);
 }
 
-template <int PRODUCER, bool DEBUG, bool FIX8>
+template <int PRODUCER, bool DEBUG>
 __global__ void __launch_bounds__(kThreads, 1)
 attention_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                      const __grid_constant__ CUtensorMap map_v, const FwdParams P)
@@ -497,7 +497,7 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
             for (int g = 0; g < 4; ++g) {
                 uint4 codes;
                 uint32_t byte;
-                produce32<PRODUCER, FIX8>(&r[g * 32], bmax[g], m_s, K, codes, byte, &lsum);
+                produce32<PRODUCER>(&r[g * 32], bmax[g], m_s, K, codes, byte, &lsum);
                 if (g == 0 && !have_p) {      // P~V of tile j-2 must have finished: it reads the group's P buffer
                     if (!wait_all(&sm->p_empty[sb], ph2 ^ 1u, sm, P.status)) { ok = false; break; }
                 }
@@ -719,7 +719,7 @@ bool shape_ok(int B, int Hq, int Hkv, int64_t Sq, int64_t Sk, int d)
            static_cast<int64_t>(B) * Hkv * ((Sk + kTile - 1) / kTile * kTile) < (1ll << 31);
 }
 
-template <int PRODUCER, bool DEBUG, bool FIX8>
+template <int PRODUCER, bool DEBUG>
 cudaError_t launch_one(dim3 grid, size_t smem, cudaStream_t stream, const CUtensorMap& mq, const CUtensorMap& mk,
                        const CUtensorMap& mv, const FwdParams& P)
 {
@@ -731,28 +731,20 @@ cudaError_t launch_one(dim3 grid, size_t smem, cudaStream_t stream, const CUtens
     {
         std::lock_guard<std::mutex> lock(mu);
         if (!done[dev]) {
-            cudaError_t e = cudaFuncSetAttribute(attention_fwd_kernel<PRODUCER, DEBUG, FIX8>,
+            cudaError_t e = cudaFuncSetAttribute(attention_fwd_kernel<PRODUCER, DEBUG>,
                                                  cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
             if (e != cudaSuccess) return e;
             done[dev] = true;
         }
     }
-    return launch_overlapped(attention_fwd_kernel<PRODUCER, DEBUG, FIX8>, grid, kThreads, smem, stream, mq, mk, mv, P);
+    return launch_overlapped(attention_fwd_kernel<PRODUCER, DEBUG>, grid, kThreads, smem, stream, mq, mk, mv, P);
 }
 
 template <int PRODUCER>
-cudaError_t launch_main(bool debug, bool fix8, dim3 grid, size_t smem, cudaStream_t stream, const CUtensorMap& mq,
-                        const CUtensorMap& mk, const CUtensorMap& mv, const FwdParams& P)
+cudaError_t launch_main(bool debug, dim3 grid, size_t smem, cudaStream_t stream, const CUtensorMap& mq, const CUtensorMap& mk,
+                        const CUtensorMap& mv, const FwdParams& P)
 {
-    if constexpr (PRODUCER != 0) {     // the 8 -> 7 fix belongs to the affine rule alone
-        return debug ? launch_one<PRODUCER, true, false>(grid, smem, stream, mq, mk, mv, P)
-                     : launch_one<PRODUCER, false, false>(grid, smem, stream, mq, mk, mv, P);
-    } else {
-        if (debug) return fix8 ? launch_one<PRODUCER, true, true>(grid, smem, stream, mq, mk, mv, P)
-                               : launch_one<PRODUCER, true, false>(grid, smem, stream, mq, mk, mv, P);
-        return fix8 ? launch_one<PRODUCER, false, true>(grid, smem, stream, mq, mk, mv, P)
-                    : launch_one<PRODUCER, false, false>(grid, smem, stream, mq, mk, mv, P);
-    }
+    return debug ? launch_one<PRODUCER, true>(grid, smem, stream, mq, mk, mv, P) : launch_one<PRODUCER, false>(grid, smem, stream, mq, mk, mv, P);
 }
 
 // The query heads of a KV group share one 128-row query tile when they fit: a decode step (one query token) of a
@@ -772,7 +764,7 @@ int64_t few_chunks(int64_t Sk, int64_t rows)
     return (n_tiles + per - 1) / per;
 }
 
-cudaError_t launch_forward(int producer, bool debug, bool fix8, int64_t items, cudaStream_t stream, const CUtensorMap& mq,
+cudaError_t launch_forward(int producer, bool debug, int64_t items, cudaStream_t stream, const CUtensorMap& mq,
                            const CUtensorMap& mk, const CUtensorMap& mv, const FwdParams& P)
 {
     if (items <= 0 || items > 0x7fffffffll) return cudaErrorInvalidValue;
@@ -780,19 +772,16 @@ cudaError_t launch_forward(int producer, bool debug, bool fix8, int64_t items, c
     // more than half of the SM's shared memory: one CTA per SM, since each CTA takes all 512 TMEM columns
     const size_t smem = sizeof(Smem) + 1024 > 120 * 1024 ? sizeof(Smem) + 1024 : 120 * 1024;
     switch (producer) {
-        case 0: return launch_main<0>(debug, fix8, grid, smem, stream, mq, mk, mv, P);
-        case 1: return launch_main<1>(debug, fix8, grid, smem, stream, mq, mk, mv, P);
-        case 2: return launch_main<2>(debug, fix8, grid, smem, stream, mq, mk, mv, P);
-        case 3: return launch_main<3>(debug, fix8, grid, smem, stream, mq, mk, mv, P);
-        case 4: return launch_main<4>(debug, fix8, grid, smem, stream, mq, mk, mv, P);
-        case 5: return launch_main<5>(debug, fix8, grid, smem, stream, mq, mk, mv, P);
-        case 6: return launch_main<6>(debug, fix8, grid, smem, stream, mq, mk, mv, P);
+        case 0: return launch_main<0>(debug, grid, smem, stream, mq, mk, mv, P);
+        case 1: return launch_main<1>(debug, grid, smem, stream, mq, mk, mv, P);
+        case 2: return launch_main<2>(debug, grid, smem, stream, mq, mk, mv, P);
+        case 3: return launch_main<3>(debug, grid, smem, stream, mq, mk, mv, P);
+        case 4: return launch_main<4>(debug, grid, smem, stream, mq, mk, mv, P);
+        case 5: return launch_main<5>(debug, grid, smem, stream, mq, mk, mv, P);
+        case 6: return launch_main<6>(debug, grid, smem, stream, mq, mk, mv, P);
         default: return cudaErrorInvalidValue;
     }
 }
-
-// fma(r, A, Bb) can reach 8 only if the residual of a block maximum, below ln 1.5, maps that high
-bool needs_fix8(float tau, float h) { return (log(1.5) - static_cast<double>(tau)) * static_cast<double>(h) + 1.0 > 7.999; }
 
 efq_status_t check_device()
 {
@@ -895,7 +884,7 @@ efq_status_t attention_impl(const void* q, const void* k, const void* v, float* 
     if (debug) P.dbg = *debug; else P.dbg = efq_debug_t{};
 
     const int64_t items = packed ? static_cast<int64_t>(B) * Hkv : (w.Sq_pad / kTile) * B * Hq;
-    return launch_forward(producer, debug != nullptr, needs_fix8(tau, h), items, stream, mq, mk, mv, P) == cudaSuccess ? EFQ_OK
+    return launch_forward(producer, debug != nullptr, items, stream, mq, mk, mv, P) == cudaSuccess ? EFQ_OK
                                                                                                                   : EFQ_ERR_CUDA;
 }
 
@@ -1367,7 +1356,7 @@ extern "C" efq_status_t efq_attention_fwd_varlen(const void* q, const void* k, c
     P.rescale_threshold = threshold;
     P.has_dbg = 0;
     P.dbg = efq_debug_t{};
-    return launch_forward(producer, false, needs_fix8(tau, h), n_items, s, mq, mk, mv, P) == cudaSuccess ? EFQ_OK : EFQ_ERR_CUDA;
+    return launch_forward(producer, false, n_items, s, mq, mk, mv, P) == cudaSuccess ? EFQ_OK : EFQ_ERR_CUDA;
 }
 
 extern "C" efq_status_t efq_poll_status(void* workspace, void* stream)

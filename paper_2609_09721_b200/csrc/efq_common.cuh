@@ -13,7 +13,7 @@ constexpr int kMxBlock = 32;  // keys per microscaling block
 
 // Revision of the fused forward kernel, part of efq_version().  Raise it whenever attention_fwd_kernel changes:
 // figures copied from a profiler capture (DRAM bytes per launch in the benchmark) are keyed to it.
-#define EFQ_FWD_KERNEL_REVISION "fwd.3"
+#define EFQ_FWD_KERNEL_REVISION "fwd.4"
 
 // Constants of the FP32 code rule, derived on the host in double and rounded once.
 // With x = sigma*r - m_s, k the block's scale exponent and z = x - k ln2 - ln6 (Eq. z-def):
@@ -167,6 +167,21 @@ __device__ __forceinline__ uint32_t cvt_e2m1x2(float lo, float hi)
         "  mov.b16 %0, {t, 0}; }\n"
         : "=h"(out)
         : "f"(lo), "f"(hi));
+    return out;
+}
+
+// Eight scaled elements -> eight codes, e0 in bits 0-3.  The conversions and the gathering of their bytes are one asm block
+// so that the bytes land in the word without shifts.
+__device__ __forceinline__ uint32_t e2m1_word(float e0, float e1, float e2, float e3, float e4, float e5, float e6, float e7)
+{
+    uint32_t out;
+    asm("{\n\t.reg .b8 b0, b1, b2, b3;\n\t"
+        "cvt.rn.satfinite.e2m1x2.f32 b0, %2, %1;\n\t"
+        "cvt.rn.satfinite.e2m1x2.f32 b1, %4, %3;\n\t"
+        "cvt.rn.satfinite.e2m1x2.f32 b2, %6, %5;\n\t"
+        "cvt.rn.satfinite.e2m1x2.f32 b3, %8, %7;\n\t"
+        "mov.b32 %0, {b0, b1, b2, b3};\n\t}\n"
+        : "=r"(out) : "f"(e0), "f"(e1), "f"(e2), "f"(e3), "f"(e4), "f"(e5), "f"(e6), "f"(e7));
     return out;
 }
 

@@ -42,15 +42,16 @@ __device__ __forceinline__ float block_max32(const float* r)
 // exponentials computed by a polynomial on the FMA pipe, 6 = producer 1 that also adds its 32 FP32 exponentials to
 // *psum (for the baseline whose denominator is the sum of the exponentials instead of the quantised operand).
 //
-// EFQ (Algorithm 1), three FMA-pipe instructions per element, bit-identical to
+// EFQ (Algorithm 1), two FMA-pipe instructions and half a pack per element, bit-identical to
 // c = floor(min(max(fma(r, A, Bb), 0), 7)):
-//   w  = fma.rn.sat(r, A/8, Bb/8)      = clamp(fma(r, A, Bb), 0, 8) / 8   (scaling by 2^-3 commutes with rounding)
-//   a' = fma.rm(w, 8, u)               = u + floor(8 w)                   (u an integer in [2^23, 2^24): ulp 1, round down)
-//   u' = fma.rn(a', 16, -15 * 2^23)    = 2^23 + 16 X                      (a' = 2^23 + X, exact)
-// so four elements accumulate Horner-style into X = c3 c2 c1 c0 (one nibble each) in the mantissa; the two
-// chain steps run as packed f32x2 FMAs on the low and high half of a 32-bit word at once.  floor(8 w) = 8 happens
-// only when fma(r, A, Bb) >= 8; FIX8 turns that nibble into 7 (needed when (ln 1.5 - tau) h + 1 can reach 8).
-template <int PRODUCER, bool FIX8>
+//   w = fma.rn.sat(r, A/8, Bb/8) = clamp(fma(r, A, Bb), 0, 8) / 8     (scaling by 2^-3 commutes with rounding)
+//   mul.rm(w, 2^-146)            = floor(8 w) 2^-149                  (a subnormal, whose bits are the integer itself)
+//   cvt.pack.sat.s4              two integers to two nibbles behind the ones packed before; 8 (only when the affine form
+//                                reaches 8) saturates to 7
+// Measured against four codes accumulated Horner-style in a mantissa by packed FMAs (0.75 more FMA-pipe instructions per
+// element, and a masked subtraction per word for the 8): 604 against 727 cycles per 128 x 128 tile with two warps per
+// scheduler, block maxima and operand stores included.
+template <int PRODUCER>
 __device__ __forceinline__ void produce32(const float* r, float rmax, float m_s, const ProducerConsts& K, uint4& codes,
                                           uint32_t& byte, float* psum = nullptr)
 {
@@ -59,22 +60,19 @@ __device__ __forceinline__ void produce32(const float* r, float rmax, float m_s,
         BlockScale s = efq_block_scale(rmax, m_s, K);
         byte = s.byte;
         const float A8 = K.A * 0.125f, B8 = s.Bb * 0.125f;
-        const uint64_t eight2 = pack2(8.0f, 8.0f), sixteen2 = pack2(16.0f, 16.0f);
-        const uint64_t magic2 = pack2(8388608.0f, 8388608.0f), back2 = pack2(-125829120.0f, -125829120.0f);
+        const float to_bits = __uint_as_float(8u);       // 2^-146
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-            uint64_t a2 = magic2;
+            uint32_t c[8];
 #pragma unroll
-            for (int i = 3; i >= 0; --i) {
-                const uint64_t w2 = pack2(fma_sat(r[q * 8 + i], A8, B8), fma_sat(r[q * 8 + 4 + i], A8, B8));
-                uint64_t u2 = magic2;
-                if (i != 3) asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(u2) : "l"(a2), "l"(sixteen2), "l"(back2));
-                asm("fma.rm.f32x2 %0, %1, %2, %3;" : "=l"(a2) : "l"(w2), "l"(eight2), "l"(u2));
+            for (int i = 0; i < 8; ++i) {
+                float t;
+                asm("mul.rm.f32 %0, %1, %2;" : "=f"(t) : "f"(fma_sat(r[q * 8 + i], A8, B8)), "f"(to_bits));
+                c[i] = __float_as_uint(t);
             }
-            uint32_t lo, hi;
-            asm("mov.b64 {%0, %1}, %2;" : "=r"(lo), "=r"(hi) : "l"(a2));
-            uint32_t word = __byte_perm(lo, hi, 0x5410);
-            if (FIX8) word -= (word >> 3) & 0x11111111u;
+            uint32_t word = 0u;
+#pragma unroll
+            for (int i = 3; i >= 0; --i) asm("cvt.pack.sat.s4.s32.b32 %0, %1, %2, %0;" : "+r"(word) : "r"(c[2 * i + 1]), "r"(c[2 * i]));
             w[q] = word;   // a block without a finite score has w = 0 everywhere (sat(-inf) and sat(NaN) are 0)
         }
     } else if (PRODUCER == 3) {
@@ -102,23 +100,21 @@ __device__ __forceinline__ void produce32(const float* r, float rmax, float m_s,
         };
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-            uint32_t word = 0;
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-                word |= (cvt_e2m1x2(ex2(q * 8 + 2 * i), ex2(q * 8 + 2 * i + 1)) & 0xffu) << (8 * i);
+            const uint32_t word = e2m1_word(ex2(q * 8), ex2(q * 8 + 1), ex2(q * 8 + 2), ex2(q * 8 + 3), ex2(q * 8 + 4), ex2(q * 8 + 5),
+                                            ex2(q * 8 + 6), ex2(q * 8 + 7));
             w[q] = f.live ? word : 0u;
         }
     } else {
         float p[32];
-        float amax = 0.0f, sum = 0.0f;
+        float sum = 0.0f;
 #pragma unroll
         for (int i = 0; i < 32; ++i) {
             float x = __fsub_rn(__fmul_rn(K.sigma, r[i]), m_s);
             p[i] = ex2_approx(__fmul_rn(x, K.LOG2E));
-            amax = fmaxf(amax, p[i]);
             if (PRODUCER == 6) sum += p[i];       // masked scores (-inf) give exactly 0
         }
         if (PRODUCER == 6) *psum += sum;
+        const float amax = fmaxf(block_max32(p), 0.0f);      // a row without a finite score has NaN everywhere: 0
         if (amax == 0.0f) {
             byte = 0;
             w[0] = w[1] = w[2] = w[3] = 0;
@@ -131,10 +127,8 @@ __device__ __forceinline__ void produce32(const float* r, float rmax, float m_s,
             byte = static_cast<uint32_t>(e + 127);
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                uint32_t word = 0;
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-                    word |= (cvt_e2m1x2(p[q * 8 + 2 * i] * s, p[q * 8 + 2 * i + 1] * s) & 0xffu) << (8 * i);
+                const float* x = p + q * 8;
+                const uint32_t word = e2m1_word(x[0] * s, x[1] * s, x[2] * s, x[3] * s, x[4] * s, x[5] * s, x[6] * s, x[7] * s);
                 w[q] = word;
             }
         }

@@ -69,7 +69,7 @@ __global__ void __launch_bounds__(128) fp4_peak_kernel(int iters, uint32_t* sink
     if (warp == 0) ptx::tmem_dealloc(tbase, 512);
 }
 
-template <int PRODUCER, bool FIX8>
+template <int PRODUCER>
 __global__ void __launch_bounds__(256) stage_kernel(ProducerConsts K, int iters, uint32_t* sink, long long* cycles)
 {
     float r[32];
@@ -87,7 +87,7 @@ __global__ void __launch_bounds__(256) stage_kernel(ProducerConsts K, int iters,
         uint4 codes;
         uint32_t byte;
         const float rmax = block_max32(r);
-        produce32<PRODUCER, FIX8>(r, rmax, m_s, K, codes, byte);
+        produce32<PRODUCER>(r, rmax, m_s, K, codes, byte);
         acc ^= codes.x ^ codes.y ^ codes.z ^ codes.w ^ byte;
         const float delta = __uint_as_float(0x3a000000u + (acc & 0xffu));   // keeps the loop from being hoisted
 #pragma unroll
@@ -126,18 +126,16 @@ extern "C" efq_status_t efq_stage_microbench(int producer, const efq_params_t* p
     if (params) { tau = params->tau; h = params->h; }
     if (!(h > 0.0f)) return EFQ_ERR_INVALID_ARG;
     const efq::ProducerConsts K = efq::make_producer_consts(0.08838834764831845f, tau, h);
-    const bool fix8 = (log(1.5) - static_cast<double>(tau)) * static_cast<double>(h) + 1.0 > 7.999;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     switch (producer) {
         case 0:
-            if (fix8) efq::stage_kernel<0, true><<<num_ctas, 256, 0, s>>>(K, iters, sink, cycles);
-            else efq::stage_kernel<0, false><<<num_ctas, 256, 0, s>>>(K, iters, sink, cycles);
+            efq::stage_kernel<0><<<num_ctas, 256, 0, s>>>(K, iters, sink, cycles);
             break;
-        case 1: efq::stage_kernel<1, false><<<num_ctas, 256, 0, s>>>(K, iters, sink, cycles); break;
-        case 2: efq::stage_kernel<2, false><<<num_ctas, 256, 0, s>>>(K, iters, sink, cycles); break;
-        case 5: efq::stage_kernel<5, false><<<num_ctas, 256, 0, s>>>(K, iters, sink, cycles); break;
-        case 4: efq::stage_kernel<4, false><<<num_ctas, 256, 0, s>>>(K, iters, sink, cycles); break;
-        case 3: efq::stage_kernel<3, false><<<num_ctas, 256, 0, s>>>(efq::make_producer_consts_lut(0.08838834764831845f), iters, sink, cycles); break;
+        case 1: efq::stage_kernel<1><<<num_ctas, 256, 0, s>>>(K, iters, sink, cycles); break;
+        case 2: efq::stage_kernel<2><<<num_ctas, 256, 0, s>>>(K, iters, sink, cycles); break;
+        case 5: efq::stage_kernel<5><<<num_ctas, 256, 0, s>>>(K, iters, sink, cycles); break;
+        case 4: efq::stage_kernel<4><<<num_ctas, 256, 0, s>>>(K, iters, sink, cycles); break;
+        case 3: efq::stage_kernel<3><<<num_ctas, 256, 0, s>>>(efq::make_producer_consts_lut(0.08838834764831845f), iters, sink, cycles); break;
         default: return EFQ_ERR_INVALID_ARG;
     }
     return cudaGetLastError() == cudaSuccess ? EFQ_OK : EFQ_ERR_CUDA;

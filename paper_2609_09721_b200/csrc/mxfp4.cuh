@@ -25,21 +25,6 @@ __device__ __forceinline__ uint32_t bf16x2_mul(uint32_t a, uint32_t b)
 __device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }
 __device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
 
-// Eight scaled elements -> eight codes, e0 in bits 0-3.  The conversions and the gathering of their bytes are one asm block
-// so that the bytes land in the word without shifts.
-__device__ __forceinline__ uint32_t e2m1_word(float e0, float e1, float e2, float e3, float e4, float e5, float e6, float e7)
-{
-    uint32_t out;
-    asm("{\n\t.reg .b8 b0, b1, b2, b3;\n\t"
-        "cvt.rn.satfinite.e2m1x2.f32 b0, %2, %1;\n\t"
-        "cvt.rn.satfinite.e2m1x2.f32 b1, %4, %3;\n\t"
-        "cvt.rn.satfinite.e2m1x2.f32 b2, %6, %5;\n\t"
-        "cvt.rn.satfinite.e2m1x2.f32 b3, %8, %7;\n\t"
-        "mov.b32 %0, {b0, b1, b2, b3};\n\t}\n"
-        : "=r"(out) : "f"(e0), "f"(e1), "f"(e2), "f"(e3), "f"(e4), "f"(e5), "f"(e6), "f"(e7));
-    return out;
-}
-
 // Shared exponents of two blocks at once, from the packed magnitudes of their largest elements: field is the exponent field
 // (in place, at least 2), the scale byte of a block is its field - 2 (e = field - 129 >= -127), and the elements are taken
 // times 2^-e, returned as packed bf16.
