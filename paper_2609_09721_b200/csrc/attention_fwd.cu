@@ -82,7 +82,7 @@ struct __align__(1024) Smem {
     uint64_t s_full[2], s_empty[2];
     uint64_t p_full[2], p_empty[2];
     uint64_t a_bar[4][4];     // [tile mod 4][lane quarter]: running maximum and alpha of that tile are published
-    uint64_t o_ready[2];      // accumulator rows rescaled (or found unchanged) for the tile of this parity
+    uint64_t o_ready[4];      // [tile mod 4]: accumulator rows rescaled (or found unchanged) for that tile
     uint64_t o_done;          // the last P~V of the work item has completed
     uint64_t l_bar;           // FP32-denominator baseline only: all eight probability warps have written lsum_x / mref_x
     uint32_t tmem_base;
@@ -140,6 +140,18 @@ __device__ __forceinline__ bool wait_all(uint64_t* bar, uint32_t parity, Smem* s
     return __all_sync(__activemask(), ok);
 }
 
+// o[0 .. 31] *= a, two at a time
+__device__ __forceinline__ void scale32(uint32_t* o, uint64_t a)
+{
+#pragma unroll
+    for (int i = 0; i < 32; i += 2) {
+        uint64_t v;
+        asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "r"(o[i]), "r"(o[i + 1]));
+        asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(v) : "l"(v), "l"(a));
+        asm("mov.b64 {%0, %1}, %2;" : "=r"(o[i]), "=r"(o[i + 1]) : "l"(v));
+    }
+}
+
 template <int PRODUCER, bool DEBUG>
 __global__ void __launch_bounds__(kThreads, 1)
 attention_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
@@ -192,11 +204,11 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         o_base = static_cast<int64_t>(b) * P.Hq * P.o_head;
     }
     const int64_t shift = Sk - Sq;                         // causal: query i sees keys <= i + shift
-    int64_t n_tiles = (Sk + kTile - 1) / kTile;
+    int n_tiles = static_cast<int>((Sk + kTile - 1) / kTile);          // shapes stay below 2^31 rows: 32-bit tile counters
     if (P.causal) {
         int64_t last_row = packed ? Sq - 1 : (q0 + kTile - 1 < Sq ? q0 + kTile - 1 : Sq - 1);
         int64_t last_key = last_row + shift;               // may be negative: nothing visible
-        int64_t need = last_key < 0 ? 0 : last_key / kTile + 1;
+        const int need = last_key < 0 ? 0 : static_cast<int>(last_key / kTile) + 1;
         if (need < n_tiles) n_tiles = need;
     }
 
@@ -222,8 +234,8 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                 ptx::mbar_init(&sm->s_empty[i], kGroupWarps);
                 ptx::mbar_init(&sm->p_full[i], kGroupWarps);
                 ptx::mbar_init(&sm->p_empty[i], 1);
-                ptx::mbar_init(&sm->o_ready[i], 4);
             }
+            for (int i = 0; i < 4; ++i) ptx::mbar_init(&sm->o_ready[i], 4);
             for (int i = 0; i < 4; ++i)
                 for (int qd = 0; qd < 4; ++qd) ptx::mbar_init(&sm->a_bar[i][qd], 1);
             ptx::mbar_init_fence();
@@ -247,7 +259,7 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
 
     // Register budget: the probability warpgroups take what the other two give up.  setmaxnreg moves registers
     // inside the CTA's own allocation only (512 threads x 128 at launch = 16 x 128 per lane), so the budgets must
-    // add up to no more than that: 4 x 56 + 8 x 200 + 4 x 56 = 2048.  A role that asks for more waits for good.
+    // add up to no more than that: 4 x 56 + 8 x 184 + 4 x 88 = 2048.  A role that asks for more waits for good.
     if (warp < 4) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
     if (run && warp == 0 && lane == 0) {
@@ -260,7 +272,7 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         const int64_t sfk_tile0 = k_row0 / kTile;
         int s = 0;
         uint32_t ph = 0;
-        for (int64_t j = 0; j < (P.inject_skip_loads ? 0 : n_tiles); ++j) {
+        for (int j = 0; j < (P.inject_skip_loads ? 0 : n_tiles); ++j) {
             // Stage barriers of their own: a waiter on a barrier that other roles may complete twice before it
             // looks (S runs ahead) could not tell which completion it sees by parity.
             if (!wait1(&sm->k_empty[s], ph ^ 1u, sm, P.status)) break;
@@ -290,7 +302,7 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         if (ok && ptx::elect_one()) ptx::tmem_cp_sf(sfq, d_sf + (ptx::smem_u32(sm->sf_q) >> 4));
         int ks = 0;
         uint32_t kph = 0;
-        for (int64_t t = 0; ok && t < n_tiles; ++t) {
+        for (int t = 0; ok && t < n_tiles; ++t) {
             const int sb = static_cast<int>(t & 1);
             if (!wait_all(&sm->k_full[ks], kph, sm, P.status)) break;
             if (!wait_all(&sm->s_empty[sb], static_cast<uint32_t>((t >> 1) & 1) ^ 1u, sm, P.status)) break;
@@ -320,11 +332,11 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         __syncwarp();
         int vs = 0;
         uint32_t vph = 0;
-        for (int64_t j = 0; j < n_tiles; ++j) {
+        for (int j = 0; j < n_tiles; ++j) {
             const int pb = static_cast<int>(j & 1);
             if (!wait_all(&sm->v_full[vs], vph, sm, P.status)) break;
             if (!wait_all(&sm->p_full[pb], static_cast<uint32_t>((j >> 1) & 1), sm, P.status)) break;
-            if (!wait_all(&sm->o_ready[pb], static_cast<uint32_t>((j >> 1) & 1), sm, P.status)) break;
+            if (!wait_all(&sm->o_ready[j & 3], static_cast<uint32_t>((j >> 2) & 1), sm, P.status)) break;
             ptx::tc_fence_after_sync();
             if (ptx::elect_one()) {
                 const uint32_t sfp = tmem + kColSfP + 4 * pb;
@@ -347,51 +359,56 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
     // =============================== historical rescaling (Eq. alpha) ===============================
     // One warp per TMEM lane quarter.  When a row's maximum grew in tile j, its accumulator row and its
     // denominator are multiplied by alpha_j after P~V_{j-1} has landed and before P~V_j is released; this runs
-    // beside the code generation of tile j instead of inside it.
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
+    // beside the code generation of tile j instead of inside it.  A quarter without growth releases P~V_j at once, so it
+    // may run behind P~V_{j-1} without a gap.  Bound: P~V waits for this step, and what takes its time is the latency of
+    // the TMEM accesses and the issue slots that the probability warps leave.  So the load of the next 32 columns is on
+    // its way while 32 are multiplied and stored.  S = 16384 (causal, 32 heads): 1589 us with one buffer and 56 registers
+    // (which spilled), 1509 with 88 registers, 1497 with two buffers; 64 columns at a time spills again (1885).
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 88;");
     const int quarter = warp & 3;
     const uint32_t row = quarter * 32 + lane;
     const uint32_t o_addr = tmem + (static_cast<uint32_t>(quarter * 32) << 16) + kColO;
     if (run) {
-        for (int64_t j = 0; j < n_tiles; ++j) {
-            const int sb = static_cast<int>(j & 1);
-            // every tile, so that each phase of this barrier is seen in order
+        for (int j = 0; j < n_tiles; ++j) {
             if (!wait_all(&sm->a_bar[j & 3][quarter], static_cast<uint32_t>((j >> 2) & 1), sm, P.status)) break;
-            if (j > 0) {
-                const float alpha = sm->alpha[j & 3][row];
-                const bool any = __any_sync(0xffffffffu, alpha != 1.0f);
-                // every tile, so that each phase of this barrier is seen in order
-                if (!wait_all(&sm->p_empty[sb ^ 1], static_cast<uint32_t>(((j - 1) >> 1) & 1), sm, P.status)) break;
-                if (any) {
-                    ptx::tc_fence_after_sync();
-                    uint32_t o[32];
-                    const uint64_t alpha2 = pack2(alpha, alpha);
-                    uint32_t lcol = 0;
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        ptx::tmem_ld32<0>(o_addr + 32 * c, o);
-                        if (c == 0) lcol = ptx::tmem_ld1(o_addr + 128);     // the denominator travels with the first chunk
-                        ptx::tmem_wait_ld();
-#pragma unroll
-                        for (int i = 0; i < 32; i += 2) {
-                            uint64_t v2;
-                            asm("mov.b64 %0, {%1, %2};" : "=l"(v2) : "r"(o[i]), "r"(o[i + 1]));
-                            asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(v2) : "l"(v2), "l"(alpha2));
-                            asm("mov.b64 {%0, %1}, %2;" : "=r"(o[i]), "=r"(o[i + 1]) : "l"(v2));
-                        }
-                        ptx::tmem_st32<0>(o_addr + 32 * c, o);
-                        if (c == 0) ptx::tmem_st1(o_addr + 128, __float_as_uint(__uint_as_float(lcol) * alpha));
-                        ptx::tmem_wait_st();   // the store reads o[] asynchronously: not before this may o[] be reused
-                    }
-                    ptx::tc_fence_before_sync();
-                }
+            const float alpha = sm->alpha[j & 3][row];
+            if (j > 0 && __any_sync(0xffffffffu, alpha != 1.0f)) {
+                // The end of P~V_{j-1} frees its V stage.  Of the four tiles that share this barrier's parity only j - 5 can be
+                // confused with j - 1, and it is over: the scores' warps waited for it before they published tile j - 1.
+                if (!wait_all(&sm->v_empty[(j - 1) & 3], static_cast<uint32_t>((j - 1) >> 2) & 1u, sm, P.status)) break;
+                ptx::tc_fence_after_sync();
+                const uint64_t alpha2 = pack2(alpha, alpha);
+                uint32_t oa[32], ob[32];
+                // a store reads its registers asynchronously: not before wait::st may a load overwrite them
+                ptx::tmem_ld32<0>(o_addr, oa);
+                const uint32_t lcol = ptx::tmem_ld1(o_addr + 128);            // the denominator travels with the first columns
+                ptx::tmem_wait_ld();
+                ptx::tmem_ld32<0>(o_addr + 32, ob);
+                scale32(oa, alpha2);
+                ptx::tmem_st32<0>(o_addr, oa);
+                ptx::tmem_st1(o_addr + 128, __float_as_uint(__uint_as_float(lcol) * alpha));
+                ptx::tmem_wait_ld();
+                scale32(ob, alpha2);
+                ptx::tmem_wait_st();
+                ptx::tmem_ld32<0>(o_addr + 64, oa);
+                ptx::tmem_st32<0>(o_addr + 32, ob);
+                ptx::tmem_wait_ld();
+                scale32(oa, alpha2);
+                ptx::tmem_wait_st();
+                ptx::tmem_ld32<0>(o_addr + 96, ob);
+                ptx::tmem_st32<0>(o_addr + 64, oa);
+                ptx::tmem_wait_ld();
+                scale32(ob, alpha2);
+                ptx::tmem_st32<0>(o_addr + 96, ob);
+                ptx::tmem_wait_st();
+                ptx::tc_fence_before_sync();
             }
             __syncwarp();
-            if (lane == 0) ptx::mbar_arrive(&sm->o_ready[sb]);
+            if (lane == 0) ptx::mbar_arrive(&sm->o_ready[j & 3]);
         }
     }
     } else {
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 200;");
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 184;");
     const int quarter = warp & 3;                       // TMEM lane quarter this warp may touch
     const int group = (warp - 4) >> 2;                  // group 0 takes the even KV tiles, group 1 the odd ones
     const uint32_t row = quarter * 32 + lane;           // row inside the query tile: one thread owns one row
@@ -450,7 +467,7 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                 ptx::tmem_wait_ld();
                 ptx::tc_fence_before_sync();          // the S buffer is handed back with the joint publication below
                 const int64_t key0 = j * kTile;
-                if (key0 + 127 > limit) {     // diagonal or ragged tile: keys past the row's limit are masked in place
+                if (__any_sync(0xffffffffu, key0 + 127 > limit)) {     // diagonal or ragged tile: keys past the row's limit are masked in place
 #pragma unroll
                     for (int i = 0; i < 128; ++i)
                         if (key0 + i > limit) r[i] = -INFINITY;
