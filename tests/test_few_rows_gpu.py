@@ -1,0 +1,79 @@
+"""The path for few query rows (query heads of a KV group times query tokens: at most 24) at its edges, against the CPU
+oracle: 1 row to 24 and the first size past it, key counts around the 128-key tile and around the sizes where the chunk of
+a CTA grows, each producer, and a packed batch too large for the sequence table that travels with the launch."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2609_09721_b200 import binding, inputs
+from test_attention_gpu import MEAN, TOL_O, _all_rows, _case_tensors, _check_dump
+
+pytestmark = pytest.mark.gpu
+
+# producer: (oracle path, tolerance)
+PRODUCERS = {"efq": ("efq", TOL_O), "lut": ("efq_lut", TOL_O), "etq0": ("etq", 5e-3), "etq1": ("etq6", 5e-3), "etq2": ("etq", 5e-3)}
+
+
+def _forward(dq, dk, dv, causal, producer, threshold=0.0, debug=None):
+    if producer.startswith("etq"):
+        return binding.exp_then_quantize_attention_fwd(dq, dk, dv, causal, 0.0, int(producer[3:]), debug=debug)
+    return binding.efq_attention_fwd(dq, dk, dv, causal, 0.0, (MEAN[0], MEAN[1], int(producer == "lut"), 0, threshold), debug=debug)
+
+
+@pytest.mark.parametrize("Hq,Hkv,Sq,Sk,causal,producer,threshold", [
+    (1, 1, 1, 1, True, "efq", 0.0), (4, 4, 1, 127, False, "efq", 0.0), (8, 1, 1, 129, True, "efq", 0.0),        # 1, 1, 8 rows
+    (2, 2, 9, 2047, True, "efq", 0.0), (4, 1, 4, 2049, True, "efq", 0.0), (2, 1, 8, 128, False, "efq", 0.0),    # 9, 16, 16 rows
+    (1, 1, 17, 4095, True, "efq", 0.0), (8, 1, 3, 4097, False, "efq", 0.0), (1, 1, 24, 16, True, "efq", 0.0),   # 17, 24, 24 rows
+    (5, 1, 5, 1500, True, "efq", 0.0),                                                                        # 25 rows: the general path
+    (8, 2, 1, 16385, True, "efq", 0.0), (6, 2, 2, 1793, True, "efq", 2.0),
+    (8, 2, 1, 1025, True, "lut", 0.0), (3, 1, 7, 600, True, "etq0", 0.0), (8, 2, 1, 2100, False, "etq1", 0.0), (4, 1, 6, 333, True, "etq2", 0.0),
+])
+def test_few_rows_against_the_oracle(oracle, Hq, Hkv, Sq, Sk, causal, producer, threshold):
+    case = inputs.AttentionCase("few", 1, Hq, Hkv, Sq, Sk, 128, causal, 500 + Sk, "k_outliers")
+    (q, k, v), (dq, dk, dv) = _case_tensors(case)
+    head = Hq - 1
+    dump = binding.DebugDump(0, head, 0, Sq, Sk)
+    o = _forward(dq, dk, dv, causal, producer, threshold, debug=dump)
+    production = _forward(dq, dk, dv, causal, producer, threshold)
+    torch.cuda.synchronize()
+    assert torch.equal(o, production)
+    path, tol = PRODUCERS[producer]
+    rows = np.array([(0, h, i) for h in range(Hq) for i in range(Sq)], np.int64)
+    want = oracle.attention_rows(q, k, v, rows, causal, case.softmax_scale, path, rescale_threshold=threshold)
+    got = o.cpu().numpy().reshape(-1, 128)
+    assert np.abs(got - want).max() <= tol
+    if causal and Sq > Sk:                      # queries before the first key see nothing
+        assert np.all(got.reshape(Hq, Sq, 128)[:, : Sq - Sk] == 0.0)
+    else:
+        _check_dump(oracle, case, dump, _all_rows(case, head, 0, Sq), MEAN, producer=path, threshold=threshold)
+
+
+@pytest.mark.parametrize("n_seqs", [128, 129])
+def test_packed_batch_of_few_row_sequences(n_seqs):
+    """128 sequences are described in the launch itself, more in device memory: each equals its forward alone bit for bit."""
+    Hq, Hkv = 4, 2
+    g = torch.Generator(device="cuda").manual_seed(7)
+    lens = [(1 + n % 12, 1 + (37 * n) % 700) for n in range(n_seqs)]
+    cu_q = np.concatenate([[0], np.cumsum([a for a, _ in lens])])
+    cu_k = np.concatenate([[0], np.cumsum([b for _, b in lens])])
+    q = torch.randn(int(cu_q[-1]), Hq, 128, generator=g, device="cuda").bfloat16()
+    k, v = (torch.randn(int(cu_k[-1]), Hkv, 128, generator=g, device="cuda").bfloat16() for _ in range(2))
+    o = binding.efq_attention_fwd_varlen(q, k, v, cu_q, cu_k, True)
+    for n in range(n_seqs):
+        a, b, c, d = cu_q[n], cu_q[n + 1], cu_k[n], cu_k[n + 1]
+        alone = binding.efq_attention_fwd(*(t.permute(1, 0, 2)[None].contiguous() for t in (q[a:b], k[c:d], v[c:d])), True)
+        assert torch.equal(o[a:b].permute(1, 0, 2), alone[0]), f"sequence {n}"
+
+
+@pytest.mark.parametrize("S,Hq,Hkv", [(127, 2, 1), (129, 1, 1), (257, 3, 3)])
+def test_inputs_at_a_16_byte_boundary(S, Hq, Hkv):
+    """Operand preparation loads 32 bytes at a time where the input allows it: inputs that start 16 bytes off give the same."""
+    g = torch.Generator(device="cuda").manual_seed(11)
+
+    def pair(heads):
+        t = torch.randn(1, heads, S, 128, generator=g, device="cuda").bfloat16()
+        shifted = torch.empty(t.numel() + 16, dtype=torch.bfloat16, device="cuda")[8:8 + t.numel()].view(t.shape)
+        return t, shifted.copy_(t)
+
+    (q, q2), (k, k2), (v, v2) = pair(Hq), pair(Hkv), pair(Hkv)
+    assert torch.equal(binding.efq_attention_fwd(q, k, v, True), binding.efq_attention_fwd(q2, k2, v2, True))
