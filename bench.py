@@ -445,7 +445,7 @@ def run_cuda(args):
         del sets
 
     # accuracy beside the speed: relative Frobenius error of each producer's output against FP32 attention on
-    # the unquantised inputs, on the whole benchmarked problem (reference kernel: plain CUDA cores, run once)
+    # the unquantised inputs, on the whole benchmarked problem (reference kernel, run once)
     accuracy = None
     if rank == 0 and not args.skip_error and case.flops <= 2.0e13:
         t0 = time.time()

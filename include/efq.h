@@ -180,8 +180,9 @@ efq_status_t efq_attention_fwd_quantized(float* o, int B, int Hq, int Hkv, int64
  * quantised by themselves, so the result of a sequence equals efq_attention_fwd on that sequence alone, bit for
  * bit.  A sequence without queries is skipped; one without keys gets zero rows.  `producer` as for
  * efq_attention_fwd_quantized.
- * The whole batch takes two kernel launches on `stream` whatever the number of sequences: one operand preparation
- * over all sequences (each quantised on its own: V blocks of 32 keys are aligned to the sequence's own key index)
+ * The whole batch takes at most five kernel launches on `stream` whatever the number of sequences.  The sequences with at
+ * most 24 query rows a KV head (Hq / Hkv * len_q: decode steps) take three that read K and V as they are; the others take two:
+ * one operand preparation over all of them (each quantised on its own: V blocks of 32 keys are aligned to the sequence's own key index)
  * and one fused forward whose work items come from a table in the workspace.  A sequence with so few query tokens
  * that the query heads of a KV group fit into one 128-row tile (Hq / Hkv * len_q <= 128: decode steps, short
  * chunks) is run with those heads sharing a tile, so its K/V tiles are read once per KV head.  The same packing is
@@ -261,8 +262,8 @@ efq_status_t efq_attention_fwd_static(const void* q, const void* k, const void* 
 
 /* Softmax attention in FP32 on the unquantised bf16 inputs (the problem statement of Sec. 3.1 with no low-bit
  * operand anywhere): O = softmax(scale Q K^T + mask) V, online over the keys, exponentials by expf.  This is the
- * reference output O_ref of the calibration objective and the "exact" side of the error figures; a plain
- * CUDA-core kernel, not a fast path.  Arguments as for efq_attention_fwd (no workspace); B * Hq <= 65535. */
+ * reference output O_ref of the calibration objective and the "exact" side of the error figures; on the
+ * tensor cores, with bf16 products that are exact in FP32 and probabilities split into three bf16 terms.  Arguments as for efq_attention_fwd (no workspace); B * Hq <= 65535. */
 efq_status_t efq_exact_attention_fwd(const void* q, const void* k, const void* v, float* o, int B, int Hq, int Hkv,
                                      int64_t Sq, int64_t Sk, int d, int causal, float softmax_scale, void* stream);
 

@@ -903,12 +903,12 @@ efq_status_t attention_impl(const void* q, const void* k, const void* v, float* 
     if (debug) P.dbg = *debug; else P.dbg = efq_debug_t{};
 
     const int64_t items = packed ? static_cast<int64_t>(B) * Hkv : (w.Sq_pad / kTile) * B * Hq;
-    return launch_forward(producer, debug != nullptr, items, stream, mq, mk, mv, P) == cudaSuccess ? EFQ_OK
-                                                                                                                  : EFQ_ERR_CUDA;
+    return launch_forward(producer, debug != nullptr, items, stream, mq, mk, mv, P) == cudaSuccess ? EFQ_OK : EFQ_ERR_CUDA;
 }
 
 // ------------------------------------------------------------------------------------------------
-// Packed variable-length batch: every sequence quantised by itself, all of them in two launches
+// Packed variable-length batch: every sequence quantised by itself.  Two launches for all sequences of the general path,
+// three for all that have few query rows (attention_few.cu).
 // ------------------------------------------------------------------------------------------------
 // Workspace: status words | tables from the host (sequences, quantiser jobs, their CTA prefix sums, query tiles in the order
 // of their weight) | item table (written on the device: it has an entry per head) |
