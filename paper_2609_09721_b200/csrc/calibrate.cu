@@ -59,13 +59,13 @@ __device__ __forceinline__ uint32_t bf16_pair(float lo, float hi)
 // load while the tensor core and the exponentials do not need their buffer.
 __global__ void __launch_bounds__(256, 1)
 exact_attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
-                       float* __restrict__ o, int Hq, int Hkv, int Sq, int Sk, int causal, float sigma)
+                       float* __restrict__ o, int heads, int Hq, int Hkv, int Sq, int Sk, int causal, float sigma)
 {
     extern __shared__ uint8_t smem_raw[];
     ExactSmem* const sm = reinterpret_cast<ExactSmem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int bh = blockIdx.x, hkv_row = (bh / Hq) * Hkv + (bh % Hq) / (Hq / Hkv);
-    const int q0 = (static_cast<int>(gridDim.y) - 1 - static_cast<int>(blockIdx.y)) * kTile;      // long rows first
+    const int bh = static_cast<int>(blockIdx.x % static_cast<unsigned>(heads)), hkv_row = (bh / Hq) * Hkv + (bh % Hq) / (Hq / Hkv);
+    const int q0 = static_cast<int>((gridDim.x - 1u - blockIdx.x) / static_cast<unsigned>(heads)) * kTile;      // long rows first
     int n_steps = (Sk + kTile - 1) / kTile;
     if (causal) {
         const int last_key = min(q0 + kTile, Sq) - 1 + Sk - Sq;
@@ -284,7 +284,7 @@ extern "C" efq_status_t efq_exact_attention_fwd(const void* q, const void* k, co
     if (!efq::is_sm100()) return EFQ_ERR_ARCH;
     const float sigma = softmax_scale > 0.0f ? softmax_scale : 0.08838834764831845f;
     const int64_t rows_q = static_cast<int64_t>(B) * Hq * Sq, rows_k = static_cast<int64_t>(B) * Hkv * Sk, q_tiles = (Sq + efq::kTile - 1) / efq::kTile;
-    if (rows_q >= (1ll << 31) - 128 || rows_k >= (1ll << 31) - 128 || q_tiles > 65535) return EFQ_ERR_UNSUPPORTED;      // 32-bit tile coordinates
+    if (rows_q >= (1ll << 31) - 128 || rows_k >= (1ll << 31) - 128 || q_tiles * B * Hq >= (1ll << 31)) return EFQ_ERR_UNSUPPORTED;      // 32-bit tile coordinates
     constexpr int smem = static_cast<int>(sizeof(efq::ExactSmem)) + 1024;
     static std::atomic<uint64_t> done{0};        // the shared-memory attribute belongs to the device: set once for each
     int dev = 0;
@@ -297,8 +297,8 @@ extern "C" efq_status_t efq_exact_attention_fwd(const void* q, const void* k, co
     if (!efq::encode_bf16_map(&mq, q, 128, static_cast<uint64_t>(rows_q)) || !efq::encode_bf16_map(&mk, k, 128, static_cast<uint64_t>(rows_k)) ||
         !efq::encode_bf16_map(&mv, v, 128, static_cast<uint64_t>(rows_k)))
         return EFQ_ERR_CUDA;
-    const dim3 grid(static_cast<unsigned>(B * Hq), static_cast<unsigned>(q_tiles));
-    efq::exact_attention_kernel<<<grid, 256, smem, static_cast<cudaStream_t>(stream)>>>(mq, mk, mv, o, Hq, Hkv, static_cast<int>(Sq),
+    const dim3 grid(static_cast<unsigned>(q_tiles * B * Hq));
+    efq::exact_attention_kernel<<<grid, 256, smem, static_cast<cudaStream_t>(stream)>>>(mq, mk, mv, o, B * Hq, Hq, Hkv, static_cast<int>(Sq),
                                                                                         static_cast<int>(Sk), causal ? 1 : 0, sigma);
     return cudaGetLastError() == cudaSuccess ? EFQ_OK : EFQ_ERR_CUDA;
 }
