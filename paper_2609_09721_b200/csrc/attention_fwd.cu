@@ -29,6 +29,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <mutex>
 #include <vector>
 
@@ -622,6 +623,8 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
     if (warp == 1) ptx::tmem_dealloc(tmem, kTmemCols);
 }
 
+#include "attention_short.cuh"
+
 // ------------------------------------------------------------------------------------------------
 // host side
 // ------------------------------------------------------------------------------------------------
@@ -759,6 +762,38 @@ cudaError_t launch_one(dim3 grid, size_t smem, cudaStream_t stream, const CUtens
     return launch_overlapped(attention_fwd_kernel<PRODUCER, DEBUG>, grid, kThreads, smem, stream, mq, mk, mv, P);
 }
 
+// Short KV walks and more query tiles than SMs: persistent CTAs (the measurements are in attention_short.cuh).  The line lies
+// where the gain is still 2 to 4 %, causal or not: 24 KV tiles.
+constexpr int kShortTiles = 24;
+bool use_short(int producer, bool debug, int64_t items, int sms, const FwdParams& P)
+{
+    return !debug && producer != 6 && P.items == nullptr && !P.packed && !P.inject_skip_loads && items > sms &&
+           P.Sk <= static_cast<int64_t>(kShortTiles) * kTile;
+}
+
+template <int PRODUCER>
+cudaError_t launch_short(unsigned sms, int dev, cudaStream_t stream, const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv,
+                         const FwdParams& P)
+{
+    constexpr int smem = static_cast<int>(sizeof(ShortSmem)) + 1024;
+    static std::atomic<uint64_t> done{0};        // the shared-memory attribute belongs to (function, device): set once for each
+    if ((done.load(std::memory_order_relaxed) >> dev & 1u) == 0u) {
+        const cudaError_t e = cudaFuncSetAttribute(attention_short_kernel<PRODUCER>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return e;
+        done.fetch_or(1ull << dev, std::memory_order_relaxed);
+    }
+    return launch_overlapped(attention_short_kernel<PRODUCER>, dim3(sms), kThreads, smem, stream, mq, mk, mv, P);
+}
+
+// SMs of a device, asked for once
+int sm_count(int dev)
+{
+    static std::atomic<int> known[kMaxDevices] = {};
+    int n = known[dev].load(std::memory_order_relaxed);
+    if (n == 0 && cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess) known[dev].store(n, std::memory_order_relaxed);
+    return n;
+}
+
 template <int PRODUCER>
 cudaError_t launch_main(bool debug, dim3 grid, size_t smem, cudaStream_t stream, const CUtensorMap& mq, const CUtensorMap& mk,
                         const CUtensorMap& mv, const FwdParams& P)
@@ -787,6 +822,20 @@ cudaError_t launch_forward(int producer, bool debug, int64_t items, cudaStream_t
                            const CUtensorMap& mk, const CUtensorMap& mv, const FwdParams& P)
 {
     if (items <= 0 || items > 0x7fffffffll) return cudaErrorInvalidValue;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+    const int sms = sm_count(dev);
+    if (sms > 0 && use_short(producer, debug, items, sms, P)) {
+        switch (producer) {
+            case 0: return launch_short<0>(sms, dev, stream, mq, mk, mv, P);
+            case 1: return launch_short<1>(sms, dev, stream, mq, mk, mv, P);
+            case 2: return launch_short<2>(sms, dev, stream, mq, mk, mv, P);
+            case 3: return launch_short<3>(sms, dev, stream, mq, mk, mv, P);
+            case 4: return launch_short<4>(sms, dev, stream, mq, mk, mv, P);
+            case 5: return launch_short<5>(sms, dev, stream, mq, mk, mv, P);
+            default: return cudaErrorInvalidValue;
+        }
+    }
     dim3 grid(static_cast<unsigned>(items));
     // more than half of the SM's shared memory: one CTA per SM, since each CTA takes all 512 TMEM columns
     const size_t smem = sizeof(Smem) + 1024 > 120 * 1024 ? sizeof(Smem) + 1024 : 120 * 1024;

@@ -1,0 +1,433 @@
+// Fused forward for short KV walks: the kernel of attention_fwd.cu (which includes this file) with persistent CTAs.
+//
+// A CTA of attention_fwd_kernel spends about 10000 cycles outside its tiles: start, barriers, TMEM, the latency of the first
+// loads and scores, the last P~V, the rows on their way out.  Against 512 keys, 4 tiles of about 1500 cycles, that is more than
+// the work.  Here one CTA per SM walks a list of query tiles and nothing of that stands between two of them: Q is
+// double-buffered and loads run ahead into the next item, S of its first tiles is computed while the last codes of this one
+// are generated, and the rescaling warps write the finished rows while the probability warps are in the next item.  The
+// tile counter t runs over all items of the CTA: it picks buffers and phases, the tile j inside the item picks the keys.
+// Everything else, the arithmetic above all, is that of attention_fwd_kernel, and so is the result, bit for bit.
+//
+// Why not for all shapes: in the steady state the looped form is 3 to 4 % slower.  Measured against the other kernel (whole
+// call, 24 heads, 16000 queries, not causal): 128 keys 153 -> 90 us, 256 keys 164 -> 111, 512 keys 195 -> 142, 1024 keys
+// 255 -> 211, 2048 keys 373 -> 342, 3072 keys 488 -> 468, 4096 keys 604 -> 594, 8192 keys 1064 -> 1098.  Causal, 32 heads: 32 x 128
+// tokens 60 -> 39 us, 4 x 1024 tokens 74 -> 67, 2048 tokens 51 -> 48, 3000 tokens 89 -> 87, 4096 tokens 134 -> 136.
+#pragma once
+
+struct __align__(1024) ShortSmem : Smem {
+    uint8_t q1[kTileBytes];                // query tile of every other item (the first one's is Smem::q)
+    uint8_t stage[kTile * kOutRowBytes];   // finished rows on their way out
+    uint8_t sf_q1[kSfBytes];
+    uint64_t q_ready[2], q_empty[2];
+};
+constexpr uint32_t kColSfQ1 = 440;         // scales of q1: 4 columns behind those of V
+
+// The k-th item of this CTA: the CTAs take items in turn, every other round in reverse, so that the heavier items of a round
+// go to those that had the lighter ones before.
+__device__ __forceinline__ uint32_t short_item(uint32_t k) { return k * gridDim.x + ((k & 1u) ? gridDim.x - 1u - blockIdx.x : blockIdx.x); }
+
+// A query tile of a [B, H, S, d] batch: heaviest query tiles first, the heads of a GQA group adjacent.
+struct ShortItem {
+    uint32_t bh, hkv_b;    // head of Q and of K, V, counted over the batch
+    int q0, n_tiles;
+};
+__device__ __forceinline__ ShortItem short_decode(const FwdParams& P, uint32_t index)
+{
+    ShortItem w;
+    const uint32_t heads = static_cast<uint32_t>(P.B) * P.Hq;
+    const uint32_t qt = static_cast<uint32_t>(P.Sq_pad / kTile) - 1u - index / heads;
+    w.bh = index % heads;
+    w.hkv_b = w.bh / static_cast<uint32_t>(P.Hq / P.Hkv);      // B * Hkv heads, G of Q for each
+    w.q0 = static_cast<int>(qt) * kTile;
+    w.n_tiles = static_cast<int>((P.Sk + kTile - 1) / kTile);
+    if (P.causal) {
+        const int64_t last_row = w.q0 + kTile - 1 < P.Sq ? w.q0 + kTile - 1 : P.Sq - 1;
+        const int64_t last_key = last_row + P.Sk - P.Sq;       // may be negative: nothing visible
+        const int need = last_key < 0 ? 0 : static_cast<int>(last_key / kTile) + 1;
+        if (need < w.n_tiles) w.n_tiles = need;
+    }
+    return w;
+}
+
+template <int PRODUCER>
+__global__ void __launch_bounds__(kThreads, 1)
+attention_short_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
+                       const __grid_constant__ CUtensorMap map_v, const FwdParams P)
+{
+    static_assert(PRODUCER != 6, "the denominator of FP32 exponentials is summed by attention_fwd_kernel only");
+    extern __shared__ uint8_t smem_raw[];
+    ShortSmem* sm = reinterpret_cast<ShortSmem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
+    const int warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31;
+    const uint32_t n_items = static_cast<uint32_t>(P.Sq_pad / kTile) * static_cast<uint32_t>(P.B) * P.Hq;
+
+    if (warp == 0) {
+        if (lane == 0) {
+            ptx::prefetch_tensormap(&map_q);
+            ptx::prefetch_tensormap(&map_k);
+            ptx::prefetch_tensormap(&map_v);
+            sm->abort_flag = 0u;
+            for (int s = 0; s < kStages; ++s) {
+                ptx::mbar_init(&sm->k_full[s], 1);
+                ptx::mbar_init(&sm->k_empty[s], 1);
+                ptx::mbar_init(&sm->v_full[s], 1);
+                ptx::mbar_init(&sm->v_empty[s], 1);
+            }
+            for (int i = 0; i < 2; ++i) {
+                ptx::mbar_init(&sm->q_ready[i], 1);
+                ptx::mbar_init(&sm->q_empty[i], 1);
+                ptx::mbar_init(&sm->s_full[i], 1);
+                ptx::mbar_init(&sm->s_empty[i], kGroupWarps);
+                ptx::mbar_init(&sm->p_full[i], kGroupWarps);
+                ptx::mbar_init(&sm->p_empty[i], 1);
+            }
+            for (int i = 0; i < 4; ++i) ptx::mbar_init(&sm->o_ready[i], 4);
+            for (int i = 0; i < 4; ++i)
+                for (int qd = 0; qd < 4; ++qd) ptx::mbar_init(&sm->a_bar[i][qd], 1);
+            ptx::mbar_init_fence();
+        }
+        __syncwarp();
+        asm volatile("bar.arrive 1, 512;" ::: "memory");
+    } else {
+        if (warp == 1) ptx::tmem_alloc(&sm->tmem_base, kTmemCols);
+        // constant parts of the B operand of P~V: 16 rows of E2M1 1.0 (0x22) after each V^T stage, unit scales
+        for (int i = threadIdx.x - 32; i < kStages * 64; i += kThreads - 32)
+            reinterpret_cast<uint4*>(sm->v[i / 64] + kTileBytes)[i % 64] = make_uint4(0x22222222u, 0x22222222u, 0x22222222u, 0x22222222u);
+        for (int i = threadIdx.x - 32; i < kSfBytes / 4; i += kThreads - 32)
+            reinterpret_cast<uint32_t*>(sm->sf_ones)[i] = (i < 64 && (i & 3) == 0) ? 0x7f7f7f7fu : 0u;
+        ptx::fence_proxy_async_smem();
+        ptx::tc_fence_before_sync();
+        asm volatile("bar.sync 1, 512;" ::: "memory");
+        ptx::tc_fence_after_sync();
+    }
+    const uint32_t tmem = warp == 0 ? 0u : sm->tmem_base;
+
+    // 4 x 56 + 8 x 184 + 4 x 88 = 2048 registers per lane, what the launch holds
+    if (warp < 4) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
+    if (warp == 0 && lane == 0) {
+        // =============================== TMA producer (one thread) ===============================
+        // The operands come from the kernel before.  Whatever else this kernel writes or reads follows from the loads.
+        ptx::grid_wait();
+        int s = 0, n = 0;
+        uint32_t ph = 0, idx;
+        bool ok = true;
+        for (uint32_t k = 0; ok && (idx = short_item(k)) < n_items; ++k) {
+            const ShortItem w = short_decode(P, idx);
+            if (w.n_tiles <= 0) continue;
+            const int qb = n & 1;
+            if (!wait1(&sm->q_empty[qb], (static_cast<uint32_t>(n >> 1) & 1u) ^ 1u, sm, P.status)) break;
+            ptx::mbar_arrive_expect_tx(&sm->q_ready[qb], kTileBytes + kSfBytes);
+            const int q_row = static_cast<int>(w.bh * static_cast<uint32_t>(P.Sq_pad)) + w.q0;
+            ptx::tma_load_2d(qb ? sm->q1 : sm->q, &map_q, 0, q_row, &sm->q_ready[qb]);
+            ptx::bulk_load_1d(qb ? sm->sf_q1 : sm->sf_q, P.sf_q + static_cast<int64_t>(q_row / kTile) * kSfBytes, kSfBytes, &sm->q_ready[qb]);
+            ++n;
+            const int k_row0 = static_cast<int>(w.hkv_b * static_cast<uint32_t>(P.Sk_pad)), v_row0 = static_cast<int>(w.hkv_b) * kTile;
+            const int64_t tile0 = k_row0 / kTile;          // of the scale tiles of K and of V
+            for (int j = 0; j < w.n_tiles; ++j) {
+                // Stage barriers of their own: a waiter on a barrier that other roles may complete twice before it
+                // looks (S runs ahead) could not tell which completion it sees by parity.
+                if (!wait1(&sm->k_empty[s], ph ^ 1u, sm, P.status)) { ok = false; break; }
+                ptx::mbar_arrive_expect_tx(&sm->k_full[s], kTileBytes + kSfBytes);
+                ptx::tma_load_2d(sm->k[s], &map_k, 0, k_row0 + j * kTile, &sm->k_full[s]);
+                ptx::bulk_load_1d(sm->sf_k[s], P.sf_k + (tile0 + j) * kSfBytes, kSfBytes, &sm->k_full[s]);
+                if (!wait1(&sm->v_empty[s], ph ^ 1u, sm, P.status)) { ok = false; break; }
+                ptx::mbar_arrive_expect_tx(&sm->v_full[s], kTileBytes + kSfBytes);
+                ptx::tma_load_2d(sm->v[s], &map_v, j * 64, v_row0, &sm->v_full[s]);
+                ptx::bulk_load_1d(sm->sf_v[s], P.sf_v + (tile0 + j) * kSfBytes, kSfBytes, &sm->v_full[s]);
+                if (++s == kStages) { s = 0; ph ^= 1u; }
+            }
+        }
+    } else if (warp == 3 && lane == 0) {
+        ptx::grid_wait();
+        // an earlier CTA of this launch gave up: the waits of this one end soon instead of after their limit
+        if (*reinterpret_cast<volatile uint32_t*>(P.status) != 0u) sm->abort_flag = 1u;
+    } else if (warp == 1) {
+        // =============================== S = Q K^T issuer ===============================
+        // The whole warp runs the loop with warp-uniform state; one elected lane issues the tcgen05
+        // instructions.  Descriptors differ from tile to tile only in the start-address field (address >> 4).
+        const uint64_t d_sw64 = ptx::smem_desc(0, 16, 512, ptx::kLayoutSw64);
+        const uint64_t d_sf = ptx::smem_desc(0, 16, 128, ptx::kLayoutNone);
+        int ks = 0, n = 0;
+        uint32_t t = 0;                                       // t: tiles of this CTA so far, over all of its items
+        uint32_t kph = 0, idx;
+        bool ok = true;
+        for (uint32_t k = 0; ok && (idx = short_item(k)) < n_items; ++k) {
+            const int n_tiles = short_decode(P, idx).n_tiles;
+            if (n_tiles <= 0) continue;
+            const int qb = n & 1;
+            const uint64_t dq0 = d_sw64 + (ptx::smem_u32(qb ? sm->q1 : sm->q) >> 4);
+            const uint32_t sfq = tmem + (qb ? kColSfQ1 : kColSfQ);
+            if (!wait_all(&sm->q_ready[qb], static_cast<uint32_t>(n >> 1) & 1u, sm, P.status)) break;
+            ++n;
+            ptx::tc_fence_after_sync();
+            if (ptx::elect_one()) ptx::tmem_cp_sf(sfq, d_sf + (ptx::smem_u32(qb ? sm->sf_q1 : sm->sf_q) >> 4));
+            __syncwarp();
+            for (int j = 0; j < n_tiles; ++j, ++t) {
+                const int sb = static_cast<int>(t & 1u);
+                if (!wait_all(&sm->k_full[ks], kph, sm, P.status)) { ok = false; break; }
+                if (!wait_all(&sm->s_empty[sb], ((t >> 1) & 1u) ^ 1u, sm, P.status)) { ok = false; break; }
+                ptx::tc_fence_after_sync();
+                if (ptx::elect_one()) {
+                    const uint32_t sfk = tmem + kColSfK + 4 * sb;
+                    ptx::tmem_cp_sf(sfk, d_sf + (ptx::smem_u32(sm->sf_k[ks]) >> 4));
+                    const uint64_t dk0 = d_sw64 + (ptx::smem_u32(sm->k[ks]) >> 4);
+                    const uint32_t d_s = tmem + kColS + 128 * sb;
+                    ptx::mma_mxf4(d_s, dq0, dk0, ptx::mxf4_idesc(128, 0), sfq, sfk, 0u);
+                    ptx::mma_mxf4(d_s, dq0 + 2, dk0 + 2, ptx::mxf4_idesc(128, 2), sfq | (2u << 30), sfk | (2u << 30), 1u);
+                    ptx::mma_commit(&sm->s_full[sb]);
+                    ptx::mma_commit(&sm->k_empty[ks]);
+                    if (j + 1 == n_tiles) ptx::mma_commit(&sm->q_empty[qb]);
+                }
+                __syncwarp();
+                if (++ks == kStages) { ks = 0; kph ^= 1u; }
+            }
+        }
+    } else if (warp == 2) {
+        // =============================== [dA | dl] = P~ [V | 1] issuer ===============================
+        const uint64_t d_sw64 = ptx::smem_desc(0, 16, 512, ptx::kLayoutSw64);
+        const uint64_t d_sf = ptx::smem_desc(0, 16, 128, ptx::kLayoutNone);
+        if (ptx::elect_one()) {
+            const uint64_t d1 = d_sf + (ptx::smem_u32(sm->sf_ones) >> 4);
+            ptx::tmem_cp_sf(tmem + kColSfV + 4, d1);
+            ptx::tmem_cp_sf(tmem + kColSfV + 12, d1);
+        }
+        __syncwarp();
+        uint32_t t = 0, idx;
+        bool ok = true;
+        for (uint32_t k = 0; ok && (idx = short_item(k)) < n_items; ++k) {
+            const int n_tiles = short_decode(P, idx).n_tiles;
+            for (int j = 0; j < n_tiles; ++j, ++t) {
+                const int pb = static_cast<int>(t & 1u), vs = static_cast<int>(t % kStages);
+                if (!wait_all(&sm->v_full[vs], (t / kStages) & 1u, sm, P.status)) { ok = false; break; }
+                if (!wait_all(&sm->p_full[pb], (t >> 1) & 1u, sm, P.status)) { ok = false; break; }
+                if (!wait_all(&sm->o_ready[t & 3u], (t >> 2) & 1u, sm, P.status)) { ok = false; break; }
+                ptx::tc_fence_after_sync();
+                if (ptx::elect_one()) {
+                    const uint32_t sfp = tmem + kColSfP + 4 * pb;
+                    const uint32_t sfv = tmem + kColSfV + 8 * pb;
+                    ptx::tmem_cp_sf(sfp, d_sf + (ptx::smem_u32(sm->sf_p[pb]) >> 4));
+                    ptx::tmem_cp_sf(sfv, d_sf + (ptx::smem_u32(sm->sf_v[vs]) >> 4));
+                    const uint64_t dp0 = d_sw64 + (ptx::smem_u32(sm->p[pb]) >> 4);
+                    const uint64_t dv0 = d_sw64 + (ptx::smem_u32(sm->v[vs]) >> 4);
+                    ptx::mma_mxf4(tmem + kColO, dp0, dv0, ptx::mxf4_idesc(144, 0), sfp, sfv, j > 0 ? 1u : 0u);
+                    ptx::mma_mxf4(tmem + kColO, dp0 + 2, dv0 + 2, ptx::mxf4_idesc(144, 2), sfp | (2u << 30), sfv | (2u << 30), 1u);
+                    ptx::mma_commit(&sm->p_empty[pb]);
+                    ptx::mma_commit(&sm->v_empty[vs]);
+                }
+                __syncwarp();
+            }
+        }
+    }
+    } else if (warp >= 12) {
+    // =============================== historical rescaling (Eq. alpha), rows out ===============================
+    // One warp per TMEM lane quarter: the accumulator rows that grew, as in attention_fwd_kernel, and the finished rows of an
+    // item, whose way out takes no time from the probability warps here.
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 88;");
+    const int quarter = warp & 3;
+    const uint32_t row = quarter * 32 + lane;
+    const uint32_t o_addr = tmem + (static_cast<uint32_t>(quarter * 32) << 16) + kColO;
+    ptx::grid_wait();
+    uint32_t t = 0, idx;
+    bool ok = true;
+    if (lane == 0) ptx::mbar_arrive(&sm->o_ready[0]);         // the first tile overwrites the accumulator
+    __syncwarp();
+    for (uint32_t k = 0; ok && (idx = short_item(k)) < n_items; ++k) {
+        const ShortItem w = short_decode(P, idx);
+        uint64_t my_dst = 0ull;                               // this lane's row of the output, if it exists
+        if (w.q0 + static_cast<int64_t>(row) < P.Sq) my_dst = reinterpret_cast<uint64_t>(P.o + (static_cast<int64_t>(w.bh) * P.o_head + (w.q0 + static_cast<int64_t>(row)) * P.o_row));
+        __syncwarp();
+        uint8_t* const stage = sm->stage + (row - lane) * kOutRowBytes;
+        if (w.n_tiles > 0) {
+            for (int j = 0; j < w.n_tiles; ++j, ++t) {
+                if (j == 0) continue;                         // released when the accumulator was free, below
+                if (!wait_all(&sm->a_bar[t & 3u][quarter], (t >> 2) & 1u, sm, P.status)) { ok = false; break; }
+                const float alpha = sm->alpha[t & 3u][row];
+                if (__any_sync(0xffffffffu, alpha != 1.0f)) {
+                    // The end of P~V of the tile before frees its V stage.  The parity says so only if the stage's use before has
+                    // ended, and it has: the probability warps waited for it before they stored the codes of the tile two before.
+                    if (!wait_all(&sm->v_empty[(t - 1u) & 3u], ((t - 1u) >> 2) & 1u, sm, P.status)) { ok = false; break; }
+                    ptx::tc_fence_after_sync();
+                    const uint64_t alpha2 = pack2(alpha, alpha);
+                    uint32_t oa[32], ob[32];
+                    // a store reads its registers asynchronously: not before wait::st may a load overwrite them
+                    ptx::tmem_ld32<0>(o_addr, oa);
+                    const uint32_t lcol = ptx::tmem_ld1(o_addr + 128);            // the denominator travels with the first columns
+                    ptx::tmem_wait_ld();
+                    ptx::tmem_ld32<0>(o_addr + 32, ob);
+                    scale32(oa, alpha2);
+                    ptx::tmem_st32<0>(o_addr, oa);
+                    ptx::tmem_st1(o_addr + 128, __float_as_uint(__uint_as_float(lcol) * alpha));
+                    ptx::tmem_wait_ld();
+                    scale32(ob, alpha2);
+                    ptx::tmem_wait_st();
+                    ptx::tmem_ld32<0>(o_addr + 64, oa);
+                    ptx::tmem_st32<0>(o_addr + 32, ob);
+                    ptx::tmem_wait_ld();
+                    scale32(oa, alpha2);
+                    ptx::tmem_wait_st();
+                    ptx::tmem_ld32<0>(o_addr + 96, ob);
+                    ptx::tmem_st32<0>(o_addr + 64, oa);
+                    ptx::tmem_wait_ld();
+                    scale32(ob, alpha2);
+                    ptx::tmem_st32<0>(o_addr + 96, ob);
+                    ptx::tmem_wait_st();
+                    ptx::tc_fence_before_sync();
+                }
+                __syncwarp();
+                if (lane == 0) ptx::mbar_arrive(&sm->o_ready[t & 3u]);
+                __syncwarp();
+            }
+            // ---- final normalisation O = A / l: out of TMEM first, so that P~V of the next item may start, then to memory
+            if (!ok || !wait_all(&sm->v_empty[(t - 1u) & 3u], ((t - 1u) >> 2) & 1u, sm, P.status)) break;
+            ptx::tc_fence_after_sync();
+            const uint32_t lcol = ptx::tmem_ld1(o_addr + 128);
+            ptx::tmem_wait_ld();
+            const float l = __uint_as_float(lcol);
+            const float inv = l > 0.0f ? 1.0f / l : 0.0f;
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                uint32_t o[32];
+                ptx::tmem_ld32<0>(o_addr + 32 * c, o);
+                ptx::tmem_wait_ld();
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+                    *reinterpret_cast<float4*>(stage + lane * kOutRowBytes + 128 * c + 16 * i) =
+                        make_float4(__uint_as_float(o[4 * i]) * inv, __uint_as_float(o[4 * i + 1]) * inv, __uint_as_float(o[4 * i + 2]) * inv, __uint_as_float(o[4 * i + 3]) * inv);
+            }
+            ptx::tc_fence_before_sync();
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive(&sm->o_ready[t & 3u]);        // first tile of the next item, if there is one
+        } else {
+            // no visible key for the whole tile: rows are zero
+            for (int i = 0; i < 32; ++i) *reinterpret_cast<float4*>(stage + i * kOutRowBytes + 16 * lane) = make_float4(0.f, 0.f, 0.f, 0.f);
+            __syncwarp();
+        }
+        // through shared memory, inside the warp: a lane holds a row, and storing it from registers would touch 32 rows per instruction
+#pragma unroll 8
+        for (int r = 0; r < 32; ++r) {
+            const uint64_t dst = __shfl_sync(0xffffffffu, my_dst, r);
+            const float4 v = *reinterpret_cast<const float4*>(stage + r * kOutRowBytes + 16 * lane);
+            if (dst != 0ull) __stcs(reinterpret_cast<float4*>(dst) + lane, v);
+        }
+        __syncwarp();
+    }
+    } else {
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 184;");
+    const int quarter = warp & 3;                       // TMEM lane quarter this warp may touch
+    const int group = (warp - 4) >> 2;                  // group 0 takes the even KV tiles, group 1 the odd ones
+    const uint32_t row = quarter * 32 + lane;           // row inside the query tile: one thread owns one row
+    const uint32_t lane_base = static_cast<uint32_t>(quarter * 32) << 16;
+    const ProducerConsts K = P.K;
+    uint32_t base = 0, idx;                             // tiles of this CTA before the item: buffers and phases count over all items
+    bool ok = true;
+    float r[128];
+    const uint32_t s_addr = tmem + lane_base + kColS + 128 * group;
+    for (uint32_t k = 0; ok && (idx = short_item(k)) < n_items; ++k) {
+        const ShortItem w = short_decode(P, idx);
+        const int n_tiles = w.n_tiles;
+        if (n_tiles <= 0) continue;
+        int64_t limit = P.causal ? w.q0 + static_cast<int64_t>(row) + P.Sk - P.Sq : P.Sk - 1;   // last visible key of this row
+        if (limit > P.Sk - 1) limit = P.Sk - 1;
+        bool in_flight = false;           // the scores of this tile were asked for at the end of the group's previous tile
+        __syncwarp();
+
+        for (int64_t j = (base & 1u) ^ static_cast<uint32_t>(group); j < n_tiles; j += 2) {
+            const uint32_t t = base + static_cast<uint32_t>(j);
+            const int sb = group;                                         // S, P and exchange buffers belong to the group
+            const uint32_t ph2 = (t >> 1) & 1u;
+
+            // ---- scores of tile j: TMEM -> registers (Algorithm 2, step 1 happened on the tensor core)
+            if (!in_flight) {
+                if (!wait_all(&sm->s_full[sb], ph2, sm, P.status)) { ok = false; break; }
+                ptx::tc_fence_after_sync();
+                ptx::tmem_ld32f<0>(s_addr, r);
+                ptx::tmem_ld32f<32>(s_addr + 32, r);
+                ptx::tmem_ld32f<64>(s_addr + 64, r);
+                ptx::tmem_ld32f<96>(s_addr + 96, r);
+            }
+            float bmax[4];
+            bool have_prev;
+            float m_prev = -INFINITY;
+            {
+                // the other group's publication and the maximum it carries are asked for while the scores travel
+                // (S = 131072: 78.2 ms, 79.3 with the maximum read after the scores)
+                have_prev = t == 0 || ptx::mbar_try_wait(&sm->a_bar[(t - 1u) & 3u][quarter], ((t - 1u) >> 2) & 1u);
+                if (j > 0 && have_prev) m_prev = sm->runmax[sb ^ 1][row];
+                ptx::tmem_wait_ld();
+                ptx::tc_fence_before_sync();          // the S buffer is handed back with the joint publication below
+                const int64_t key0 = j * kTile;
+                if (__any_sync(0xffffffffu, key0 + 127 > limit)) {     // diagonal or ragged tile: keys past the row's limit are masked in place
+#pragma unroll
+                    for (int i = 0; i < 128; ++i)
+                        if (key0 + i > limit) r[i] = -INFINITY;
+                }
+            }
+#pragma unroll
+            for (int g = 0; g < 4; ++g) bmax[g] = block_max32(&r[32 * g]);
+
+            // ---- running row maximum (Eq. rowmax-update): handed over from the group that owns tile j-1
+            if (!have_prev) {
+                if (!wait_all(&sm->a_bar[(t - 1u) & 3u][quarter], ((t - 1u) >> 2) & 1u, sm, P.status)) { ok = false; break; }
+                if (j > 0) m_prev = sm->runmax[sb ^ 1][row];
+            }
+            float m_new = fmaxf(fmaxf(m_prev, bmax[0]), max3(bmax[1], bmax[2], bmax[3]));
+            if (P.rescale_threshold > 0.0f && m_prev != -INFINITY) {      // optional policy: keep the old maximum
+                const float ahead = __fsub_rn(__fmul_rn(K.sigma, m_new), __fmul_rn(K.sigma, m_prev));
+                if (!(ahead > P.rescale_threshold)) m_new = m_prev;
+            }
+            const float m_s_prev = __fmul_rn(K.sigma, m_prev);
+            const float m_s = __fmul_rn(K.sigma, m_new);
+            const bool grew = m_new > m_prev && m_prev != -INFINITY;      // history exists and must be rescaled
+            const float alpha = grew ? ex2_approx(__fmul_rn(__fsub_rn(m_s_prev, m_s), K.LOG2E)) : 1.0f;
+            // One publication for both readers: the running maximum for the other group, alpha for the rescaling
+            // warps.  alpha sits in a ring of four tiles: slot j mod 4 was last read for tile j-4, before P~V_{j-4}
+            // was released, and this group waited for the end of P~V_{j-4} before it stored the codes of tile j-2.
+            sm->runmax[sb][row] = m_new;
+            sm->alpha[t & 3u][row] = alpha;
+            __syncwarp();
+            if (lane == 0) {
+                ptx::mbar_arrive(&sm->a_bar[t & 3u][quarter]);
+                ptx::mbar_arrive(&sm->s_empty[sb]);           // every lane's scores are in registers (wait::ld above)
+            }
+            // P~V of tile j-2 reads the group's P buffer: asked here, answered while block 0 is computed
+            const bool have_p = ptx::mbar_try_wait(&sm->p_empty[sb], ph2 ^ 1u);
+
+            // ---- probability operand (Algorithm 1 per block): codes and scales straight into the MMA operand
+            uint32_t sfword = 0;
+#pragma unroll
+            for (int g = 0; g < 4; ++g) {
+                uint4 codes;
+                uint32_t byte;
+                produce32<PRODUCER>(&r[g * 32], bmax[g], m_s, K, codes, byte);
+                if (g == 0 && !have_p) {      // P~V of tile j-2 must have finished: it reads the group's P buffer
+                    if (!wait_all(&sm->p_empty[sb], ph2 ^ 1u, sm, P.status)) { ok = false; break; }
+                }
+                *reinterpret_cast<uint4*>(sm->p[sb] + code_tile_offset(row, g)) = codes;
+                sfword |= byte << (8 * g);
+            }
+            if (!ok) break;               // the bounded wait inside the block loop gave up
+            *reinterpret_cast<uint32_t*>(sm->sf_p[sb] + (row & 31u) * 16u + (row >> 5) * 4u) = sfword;
+            // The registers are free: if S of the group's next tile is there already (it is as a rule, S runs ahead),
+            // its scores set out now and travel while the operand is handed over and the loop turns.
+            in_flight = j + 2 < n_tiles && ptx::mbar_try_wait(&sm->s_full[sb], ph2 ^ 1u);
+            if (in_flight) {
+                ptx::tc_fence_after_sync();
+                ptx::tmem_ld32f<0>(s_addr, r);
+                ptx::tmem_ld32f<32>(s_addr + 32, r);
+                ptx::tmem_ld32f<64>(s_addr + 64, r);
+                ptx::tmem_ld32f<96>(s_addr + 96, r);
+            }
+            ptx::fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive(&sm->p_full[sb]);
+        }
+        base += static_cast<uint32_t>(n_tiles);
+        ptx::tmem_wait_ld();              // nothing may be in flight when a bounded wait gave up inside the loop
+    }
+    }
+
+    ptx::tc_fence_before_sync();
+    __syncthreads();
+    if (warp == 1) ptx::tmem_dealloc(tmem, kTmemCols);
+}

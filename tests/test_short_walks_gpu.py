@@ -1,0 +1,43 @@
+"""Persistent CTAs for short KV walks (more query tiles than SMs): every row equals, bit for bit, what the kernel with one
+CTA per query tile returns (it is the one that runs when the operand is dumped), and sampled rows match the CPU oracle.  Key
+counts at the edges of a tile and of the dispatch rule, ragged query tiles, GQA, batches, items without a visible key."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2609_09721_b200 import binding, inputs
+from test_attention_gpu import MEAN, TOL_O, _case_tensors
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("B,Hq,Hkv,Sq,Sk,causal,producer,threshold", [
+    (1, 24, 24, 1000, 1, False, "efq", 0.0), (1, 8, 2, 2500, 128, False, "efq", 0.0), (2, 8, 8, 1281, 129, False, "efq", 0.0),
+    (1, 24, 24, 2100, 512, False, "efq", 0.0), (1, 12, 4, 3000, 1000, False, "efq", 0.0), (1, 8, 4, 2560, 3072, False, "efq", 0.0),
+    (1, 8, 4, 2560, 3073, False, "efq", 0.0),                                # one key past the rule: one CTA per query tile
+    (100, 4, 2, 127, 127, True, "efq", 0.0), (40, 4, 1, 130, 256, True, "efq", 0.0), (3, 16, 4, 600, 1024, True, "efq", 0.0),
+    (5, 8, 2, 900, 200, True, "efq", 0.0),                                   # the first 700 queries see nothing
+    (2, 16, 4, 700, 400, False, "efq", 1.0), (2, 16, 4, 700, 400, False, "lut", 0.0),
+    (2, 16, 4, 700, 400, False, "etq0", 0.0), (2, 16, 4, 700, 400, False, "etq1", 0.0),
+    (2, 16, 4, 700, 400, True, "etq2", 0.0), (2, 16, 4, 700, 400, False, "etq3", 0.0), (2, 16, 4, 700, 400, False, "etq4", 0.0),
+])
+def test_short_walks_equal_one_cta_per_tile(oracle, B, Hq, Hkv, Sq, Sk, causal, producer, threshold):
+    case = inputs.AttentionCase("short", B, Hq, Hkv, Sq, Sk, 128, causal, 600 + Sk, "k_outliers")
+    (q, k, v), (dq, dk, dv) = _case_tensors(case)
+
+    def forward(debug=None):
+        if producer.startswith("etq"):
+            return binding.exp_then_quantize_attention_fwd(dq, dk, dv, causal, 0.0, int(producer[3:]), debug=debug)
+        return binding.efq_attention_fwd(dq, dk, dv, causal, 0.0, (MEAN[0], MEAN[1], int(producer == "lut"), 0, threshold), debug=debug)
+
+    o = forward()
+    assert torch.equal(o, forward(binding.DebugDump(B - 1, Hq - 1, 0, 1, Sk)))
+    if producer in ("efq", "lut"):
+        rng = np.random.default_rng(Sk)
+        rows = np.stack([rng.integers(0, n, 64) for n in (B, Hq, Sq)], 1)
+        rows[0], rows[1] = (0, 0, 0), (B - 1, Hq - 1, Sq - 1)
+        want = oracle.attention_rows(q, k, v, rows, causal, case.softmax_scale, {"efq": "efq", "lut": "efq_lut"}[producer], rescale_threshold=threshold)
+        got = o[rows[:, 0], rows[:, 1], rows[:, 2]].cpu().numpy()
+        assert np.abs(got - want).max() <= TOL_O
+    if causal and Sq > Sk:
+        assert torch.all(o[:, :, : Sq - Sk] == 0)
