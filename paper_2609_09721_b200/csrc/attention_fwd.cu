@@ -763,26 +763,36 @@ cudaError_t launch_one(dim3 grid, size_t smem, cudaStream_t stream, const CUtens
 }
 
 // Short KV walks and more query tiles than SMs: persistent CTAs (the measurements are in attention_short.cuh).  The line lies
-// where the gain is still 2 to 4 %, causal or not: 24 KV tiles.
-constexpr int kShortTiles = 24;
+// where the gain is still 2 to 4 %, causal or not: 24 KV tiles.  The plain exponential producers (1, 2) in a packed batch, whose
+// code generation is long enough to hide the other kernel's start, gain only on short sequences (4 of 200 to 400 tokens 33 -> 29
+// us) and lose on long ones (6 of up to 3000 tokens 167 -> 179 us): 4 tiles.
+constexpr int kShortTiles = 24, kShortTilesPlainTable = 4;
+// P.Sk: the keys of the problem or of the longest sequence.
 bool use_short(int producer, bool debug, int64_t items, int sms, const FwdParams& P)
 {
-    return !debug && producer != 6 && P.items == nullptr && !P.packed && !P.inject_skip_loads && items > sms &&
-           P.Sk <= static_cast<int64_t>(kShortTiles) * kTile;
+    return !debug && producer != 6 && !P.packed && !P.inject_skip_loads && items > sms &&
+           P.Sk <= (P.items && (producer == 1 || producer == 2) ? kShortTilesPlainTable : kShortTiles) * static_cast<int64_t>(kTile);
 }
 
-template <int PRODUCER>
-cudaError_t launch_short(unsigned sms, int dev, cudaStream_t stream, const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv,
+template <int PRODUCER, bool TABLE>
+cudaError_t launch_short_one(unsigned items, unsigned sms, int dev, cudaStream_t stream, const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv,
                          const FwdParams& P)
 {
     constexpr int smem = static_cast<int>(sizeof(ShortSmem)) + 1024;
     static std::atomic<uint64_t> done{0};        // the shared-memory attribute belongs to (function, device): set once for each
     if ((done.load(std::memory_order_relaxed) >> dev & 1u) == 0u) {
-        const cudaError_t e = cudaFuncSetAttribute(attention_short_kernel<PRODUCER>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        const cudaError_t e = cudaFuncSetAttribute(attention_short_kernel<PRODUCER, TABLE>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess) return e;
         done.fetch_or(1ull << dev, std::memory_order_relaxed);
     }
-    return launch_overlapped(attention_short_kernel<PRODUCER>, dim3(sms), kThreads, smem, stream, mq, mk, mv, P);
+    return launch_overlapped(attention_short_kernel<PRODUCER, TABLE>, dim3(sms), kThreads, smem, stream, mq, mk, mv, P, items);
+}
+
+template <int PRODUCER>
+cudaError_t launch_short(unsigned items, unsigned sms, int dev, cudaStream_t stream, const CUtensorMap& mq, const CUtensorMap& mk,
+                         const CUtensorMap& mv, const FwdParams& P)
+{
+    return P.items ? launch_short_one<PRODUCER, true>(items, sms, dev, stream, mq, mk, mv, P) : launch_short_one<PRODUCER, false>(items, sms, dev, stream, mq, mk, mv, P);
 }
 
 // SMs of a device, asked for once
@@ -827,12 +837,12 @@ cudaError_t launch_forward(int producer, bool debug, int64_t items, cudaStream_t
     const int sms = sm_count(dev);
     if (sms > 0 && use_short(producer, debug, items, sms, P)) {
         switch (producer) {
-            case 0: return launch_short<0>(sms, dev, stream, mq, mk, mv, P);
-            case 1: return launch_short<1>(sms, dev, stream, mq, mk, mv, P);
-            case 2: return launch_short<2>(sms, dev, stream, mq, mk, mv, P);
-            case 3: return launch_short<3>(sms, dev, stream, mq, mk, mv, P);
-            case 4: return launch_short<4>(sms, dev, stream, mq, mk, mv, P);
-            case 5: return launch_short<5>(sms, dev, stream, mq, mk, mv, P);
+            case 0: return launch_short<0>(static_cast<unsigned>(items), static_cast<unsigned>(sms), dev, stream, mq, mk, mv, P);
+            case 1: return launch_short<1>(static_cast<unsigned>(items), static_cast<unsigned>(sms), dev, stream, mq, mk, mv, P);
+            case 2: return launch_short<2>(static_cast<unsigned>(items), static_cast<unsigned>(sms), dev, stream, mq, mk, mv, P);
+            case 3: return launch_short<3>(static_cast<unsigned>(items), static_cast<unsigned>(sms), dev, stream, mq, mk, mv, P);
+            case 4: return launch_short<4>(static_cast<unsigned>(items), static_cast<unsigned>(sms), dev, stream, mq, mk, mv, P);
+            case 5: return launch_short<5>(static_cast<unsigned>(items), static_cast<unsigned>(sms), dev, stream, mq, mk, mv, P);
             default: return cudaErrorInvalidValue;
         }
     }
@@ -969,6 +979,7 @@ struct VarlenPlan {
     int64_t few_units, few_keys;     // their chunks times KV heads; their keys, padded to 128
     int64_t q_rows, k_rows, k_cols;  // rows of the Q and K code matrices, keys along V^T (all padded to 128)
     int64_t items, groups, quant_ctas;
+    int64_t longest;                 // keys of the longest sequence of the general path
     size_t tables, seqs_off, jobs_off, prefix_off, groups_off, items_off, qc, qsf, kc, ksf, vt, vsf, few_table, few, total;
 };
 
@@ -999,6 +1010,7 @@ bool plan_varlen(const int64_t* cu_q, const int64_t* cu_k, int n_seqs, int Hq, i
         p.q_rows += (packed ? Hkv : Hq) * lq_pad;
         p.k_rows += Hkv * lk_pad;
         p.k_cols += lk_pad;
+        p.longest = std::max(p.longest, lk);
         p.items += packed ? Hkv : (lq_pad / kTile) * Hq;
         p.groups += lq_pad / kTile;
         p.quant_ctas += (packed ? Hkv : Hq) * (lq_pad / kTile) + 2 * Hkv * (lk_pad / kTile);
@@ -1408,7 +1420,7 @@ extern "C" efq_status_t efq_attention_fwd_varlen(const void* q, const void* k, c
     if (!encode_map(&mv, ws + p.vt, static_cast<uint64_t>(p.k_cols / 2), static_cast<uint64_t>(Hkv) * 128)) return EFQ_ERR_CUDA;
 
     FwdParams P{};
-    P.B = p.n_active; P.Hq = Hq; P.Hkv = Hkv; P.Sq = 0; P.Sk = 0; P.Sq_pad = 0; P.Sk_pad = 0;
+    P.B = p.n_active; P.Hq = Hq; P.Hkv = Hkv; P.Sq = 0; P.Sk = p.longest; P.Sq_pad = 0; P.Sk_pad = 0;
     P.causal = causal ? 1 : 0;
     P.K = producer == 3 ? make_producer_consts_lut(softmax_scale) : make_producer_consts(softmax_scale, tau, h);
     P.sf_q = ws + p.qsf; P.sf_k = ws + p.ksf; P.sf_v = ws + p.vsf;

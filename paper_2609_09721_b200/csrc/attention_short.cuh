@@ -12,6 +12,7 @@
 // call, 24 heads, 16000 queries, not causal): 128 keys 153 -> 90 us, 256 keys 164 -> 111, 512 keys 195 -> 142, 1024 keys
 // 255 -> 211, 2048 keys 373 -> 342, 3072 keys 488 -> 468, 4096 keys 604 -> 594, 8192 keys 1064 -> 1098.  Causal, 32 heads: 32 x 128
 // tokens 60 -> 39 us, 4 x 1024 tokens 74 -> 67, 2048 tokens 51 -> 48, 3000 tokens 89 -> 87, 4096 tokens 134 -> 136.
+// Packed batches: 16 sequences of 100 to 3000 tokens 565 -> 513 us, 40 of 100 to 500 235 -> 188, 64 of 64 to 128 132 -> 94.
 #pragma once
 
 struct __align__(1024) ShortSmem : Smem {
@@ -26,40 +27,68 @@ constexpr uint32_t kColSfQ1 = 440;         // scales of q1: 4 columns behind tho
 // go to those that had the lighter ones before.
 __device__ __forceinline__ uint32_t short_item(uint32_t k) { return k * gridDim.x + ((k & 1u) ? gridDim.x - 1u - blockIdx.x : blockIdx.x); }
 
-// A query tile of a [B, H, S, d] batch: heaviest query tiles first, the heads of a GQA group adjacent.
+// One work item: rows q0 .. q0 + 127 of a query head or - "packed", in a variable-length batch - row r = token r % Sq of query
+// head r / Sq of a KV group.  Each role uses the fields that it needs; the others are never computed.
 struct ShortItem {
-    uint32_t bh, hkv_b;    // head of Q and of K, V, counted over the batch
-    int q0, n_tiles;
+    int n_tiles, q0;
+    int q_row, k_row0, v_x0, v_row0;      // where its operands start in the code matrices
+    int64_t sfv_tile0, Sq, Sk, o;         // o: element offset of row 0 of its (first) query head in the output
+    bool packed;
 };
+// TABLE = false: [B, H, S, d] batch, heaviest query tiles first, the heads of a GQA group adjacent (a template parameter because
+// the table's fields cost registers in every role).  TABLE = true: variable-length batch, items sorted by weight in memory.
+template <bool TABLE>
 __device__ __forceinline__ ShortItem short_decode(const FwdParams& P, uint32_t index)
 {
     ShortItem w;
-    const uint32_t heads = static_cast<uint32_t>(P.B) * P.Hq;
-    const uint32_t qt = static_cast<uint32_t>(P.Sq_pad / kTile) - 1u - index / heads;
-    w.bh = index % heads;
-    w.hkv_b = w.bh / static_cast<uint32_t>(P.Hq / P.Hkv);      // B * Hkv heads, G of Q for each
-    w.q0 = static_cast<int>(qt) * kTile;
-    w.n_tiles = static_cast<int>((P.Sk + kTile - 1) / kTile);
+    if (TABLE) {
+        const ItemDesc it = P.items[index];
+        const SeqDesc sd = P.seqs[it.seq];
+        const int G = P.Hq / P.Hkv;
+        w.packed = sd.packed != 0;
+        const int hkv = w.packed ? it.head : it.head / G, head0 = w.packed ? it.head * G : it.head;
+        w.q0 = w.packed ? 0 : it.qt * kTile;
+        w.q_row = sd.q_row0 + (w.packed ? hkv * kTile : head0 * sd.Sq_pad + w.q0);
+        w.k_row0 = sd.k_row0 + hkv * sd.Sk_pad;
+        w.v_x0 = sd.k_col0 / 2;
+        w.v_row0 = hkv * kTile;
+        w.sfv_tile0 = static_cast<int64_t>(hkv) * P.v_tiles_per_head + sd.k_col0 / kTile;
+        w.Sq = sd.Sq; w.Sk = sd.Sk;
+        w.o = sd.o_off + head0 * P.o_head;
+    } else {
+        const uint32_t heads = static_cast<uint32_t>(P.B) * P.Hq;
+        const uint32_t qt = static_cast<uint32_t>(P.Sq_pad / kTile) - 1u - index / heads;
+        const uint32_t bh = index % heads, kvh = bh / static_cast<uint32_t>(P.Hq / P.Hkv);      // B * Hkv heads, G of Q for each
+        w.packed = false;
+        w.q0 = static_cast<int>(qt) * kTile;
+        w.q_row = static_cast<int>(bh * static_cast<uint32_t>(P.Sq_pad)) + w.q0;
+        w.k_row0 = static_cast<int>(kvh * static_cast<uint32_t>(P.Sk_pad));
+        w.v_x0 = 0;
+        w.v_row0 = static_cast<int>(kvh) * kTile;
+        w.sfv_tile0 = w.k_row0 / kTile;
+        w.Sq = P.Sq; w.Sk = P.Sk;
+        w.o = static_cast<int64_t>(bh) * P.o_head;
+    }
+    w.n_tiles = static_cast<int>((w.Sk + kTile - 1) / kTile);
     if (P.causal) {
-        const int64_t last_row = w.q0 + kTile - 1 < P.Sq ? w.q0 + kTile - 1 : P.Sq - 1;
-        const int64_t last_key = last_row + P.Sk - P.Sq;       // may be negative: nothing visible
+        const int64_t last_row = !(TABLE && w.packed) && w.q0 + kTile - 1 < w.Sq ? w.q0 + kTile - 1 : w.Sq - 1;
+        const int64_t last_key = last_row + w.Sk - w.Sq;       // may be negative: nothing visible
         const int need = last_key < 0 ? 0 : static_cast<int>(last_key / kTile) + 1;
         if (need < w.n_tiles) w.n_tiles = need;
     }
     return w;
 }
 
-template <int PRODUCER>
+template <int PRODUCER, bool TABLE>
 __global__ void __launch_bounds__(kThreads, 1)
 attention_short_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
-                       const __grid_constant__ CUtensorMap map_v, const FwdParams P)
+                       const __grid_constant__ CUtensorMap map_v, const FwdParams P, const uint32_t n_items)
 {
     static_assert(PRODUCER != 6, "the denominator of FP32 exponentials is summed by attention_fwd_kernel only");
     extern __shared__ uint8_t smem_raw[];
     ShortSmem* sm = reinterpret_cast<ShortSmem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
-    const uint32_t n_items = static_cast<uint32_t>(P.Sq_pad / kTile) * static_cast<uint32_t>(P.B) * P.Hq;
 
     if (warp == 0) {
         if (lane == 0) {
@@ -113,28 +142,26 @@ attention_short_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
         uint32_t ph = 0, idx;
         bool ok = true;
         for (uint32_t k = 0; ok && (idx = short_item(k)) < n_items; ++k) {
-            const ShortItem w = short_decode(P, idx);
+            const ShortItem w = short_decode<TABLE>(P, idx);
             if (w.n_tiles <= 0) continue;
             const int qb = n & 1;
             if (!wait1(&sm->q_empty[qb], (static_cast<uint32_t>(n >> 1) & 1u) ^ 1u, sm, P.status)) break;
             ptx::mbar_arrive_expect_tx(&sm->q_ready[qb], kTileBytes + kSfBytes);
-            const int q_row = static_cast<int>(w.bh * static_cast<uint32_t>(P.Sq_pad)) + w.q0;
-            ptx::tma_load_2d(qb ? sm->q1 : sm->q, &map_q, 0, q_row, &sm->q_ready[qb]);
-            ptx::bulk_load_1d(qb ? sm->sf_q1 : sm->sf_q, P.sf_q + static_cast<int64_t>(q_row / kTile) * kSfBytes, kSfBytes, &sm->q_ready[qb]);
+            ptx::tma_load_2d(qb ? sm->q1 : sm->q, &map_q, 0, w.q_row, &sm->q_ready[qb]);
+            ptx::bulk_load_1d(qb ? sm->sf_q1 : sm->sf_q, P.sf_q + static_cast<int64_t>(w.q_row / kTile) * kSfBytes, kSfBytes, &sm->q_ready[qb]);
             ++n;
-            const int k_row0 = static_cast<int>(w.hkv_b * static_cast<uint32_t>(P.Sk_pad)), v_row0 = static_cast<int>(w.hkv_b) * kTile;
-            const int64_t tile0 = k_row0 / kTile;          // of the scale tiles of K and of V
+            const int64_t sfk_tile0 = w.k_row0 / kTile;
             for (int j = 0; j < w.n_tiles; ++j) {
                 // Stage barriers of their own: a waiter on a barrier that other roles may complete twice before it
                 // looks (S runs ahead) could not tell which completion it sees by parity.
                 if (!wait1(&sm->k_empty[s], ph ^ 1u, sm, P.status)) { ok = false; break; }
                 ptx::mbar_arrive_expect_tx(&sm->k_full[s], kTileBytes + kSfBytes);
-                ptx::tma_load_2d(sm->k[s], &map_k, 0, k_row0 + j * kTile, &sm->k_full[s]);
-                ptx::bulk_load_1d(sm->sf_k[s], P.sf_k + (tile0 + j) * kSfBytes, kSfBytes, &sm->k_full[s]);
+                ptx::tma_load_2d(sm->k[s], &map_k, 0, w.k_row0 + j * kTile, &sm->k_full[s]);
+                ptx::bulk_load_1d(sm->sf_k[s], P.sf_k + (sfk_tile0 + j) * kSfBytes, kSfBytes, &sm->k_full[s]);
                 if (!wait1(&sm->v_empty[s], ph ^ 1u, sm, P.status)) { ok = false; break; }
                 ptx::mbar_arrive_expect_tx(&sm->v_full[s], kTileBytes + kSfBytes);
-                ptx::tma_load_2d(sm->v[s], &map_v, j * 64, v_row0, &sm->v_full[s]);
-                ptx::bulk_load_1d(sm->sf_v[s], P.sf_v + (tile0 + j) * kSfBytes, kSfBytes, &sm->v_full[s]);
+                ptx::tma_load_2d(sm->v[s], &map_v, w.v_x0 + j * 64, w.v_row0, &sm->v_full[s]);
+                ptx::bulk_load_1d(sm->sf_v[s], P.sf_v + (w.sfv_tile0 + j) * kSfBytes, kSfBytes, &sm->v_full[s]);
                 if (++s == kStages) { s = 0; ph ^= 1u; }
             }
         }
@@ -148,12 +175,13 @@ attention_short_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
         // instructions.  Descriptors differ from tile to tile only in the start-address field (address >> 4).
         const uint64_t d_sw64 = ptx::smem_desc(0, 16, 512, ptx::kLayoutSw64);
         const uint64_t d_sf = ptx::smem_desc(0, 16, 128, ptx::kLayoutNone);
+        if (TABLE) ptx::grid_wait();                           // the item table is written by the kernel before
         int ks = 0, n = 0;
         uint32_t t = 0;                                       // t: tiles of this CTA so far, over all of its items
         uint32_t kph = 0, idx;
         bool ok = true;
         for (uint32_t k = 0; ok && (idx = short_item(k)) < n_items; ++k) {
-            const int n_tiles = short_decode(P, idx).n_tiles;
+            const int n_tiles = short_decode<TABLE>(P, idx).n_tiles;
             if (n_tiles <= 0) continue;
             const int qb = n & 1;
             const uint64_t dq0 = d_sw64 + (ptx::smem_u32(qb ? sm->q1 : sm->q) >> 4);
@@ -193,10 +221,11 @@ attention_short_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
             ptx::tmem_cp_sf(tmem + kColSfV + 12, d1);
         }
         __syncwarp();
+        if (TABLE) ptx::grid_wait();
         uint32_t t = 0, idx;
         bool ok = true;
         for (uint32_t k = 0; ok && (idx = short_item(k)) < n_items; ++k) {
-            const int n_tiles = short_decode(P, idx).n_tiles;
+            const int n_tiles = short_decode<TABLE>(P, idx).n_tiles;
             for (int j = 0; j < n_tiles; ++j, ++t) {
                 const int pb = static_cast<int>(t & 1u), vs = static_cast<int>(t % kStages);
                 if (!wait_all(&sm->v_full[vs], (t / kStages) & 1u, sm, P.status)) { ok = false; break; }
@@ -233,9 +262,14 @@ attention_short_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
     if (lane == 0) ptx::mbar_arrive(&sm->o_ready[0]);         // the first tile overwrites the accumulator
     __syncwarp();
     for (uint32_t k = 0; ok && (idx = short_item(k)) < n_items; ++k) {
-        const ShortItem w = short_decode(P, idx);
+        const ShortItem w = short_decode<TABLE>(P, idx);
         uint64_t my_dst = 0ull;                               // this lane's row of the output, if it exists
-        if (w.q0 + static_cast<int64_t>(row) < P.Sq) my_dst = reinterpret_cast<uint64_t>(P.o + (static_cast<int64_t>(w.bh) * P.o_head + (w.q0 + static_cast<int64_t>(row)) * P.o_row));
+        if (TABLE && w.packed) {
+            const int gq = static_cast<int>(row) / static_cast<int>(w.Sq), token = static_cast<int>(row) - gq * static_cast<int>(w.Sq);
+            if (gq < P.Hq / P.Hkv) my_dst = reinterpret_cast<uint64_t>(P.o + (w.o + gq * P.o_head + token * P.o_row));
+        } else if (w.q0 + static_cast<int64_t>(row) < w.Sq) {
+            my_dst = reinterpret_cast<uint64_t>(P.o + (w.o + (w.q0 + static_cast<int64_t>(row)) * P.o_row));
+        }
         __syncwarp();
         uint8_t* const stage = sm->stage + (row - lane) * kOutRowBytes;
         if (w.n_tiles > 0) {
@@ -319,16 +353,18 @@ attention_short_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
     const uint32_t row = quarter * 32 + lane;           // row inside the query tile: one thread owns one row
     const uint32_t lane_base = static_cast<uint32_t>(quarter * 32) << 16;
     const ProducerConsts K = P.K;
+    if (TABLE) ptx::grid_wait();
     uint32_t base = 0, idx;                             // tiles of this CTA before the item: buffers and phases count over all items
     bool ok = true;
     float r[128];
     const uint32_t s_addr = tmem + lane_base + kColS + 128 * group;
     for (uint32_t k = 0; ok && (idx = short_item(k)) < n_items; ++k) {
-        const ShortItem w = short_decode(P, idx);
+        const ShortItem w = short_decode<TABLE>(P, idx);
         const int n_tiles = w.n_tiles;
         if (n_tiles <= 0) continue;
-        int64_t limit = P.causal ? w.q0 + static_cast<int64_t>(row) + P.Sk - P.Sq : P.Sk - 1;   // last visible key of this row
-        if (limit > P.Sk - 1) limit = P.Sk - 1;
+        const int64_t token = TABLE && w.packed ? static_cast<int>(row) % static_cast<int>(w.Sq) : w.q0 + static_cast<int64_t>(row);
+        int64_t limit = P.causal ? token + w.Sk - w.Sq : w.Sk - 1;   // last visible key of this row
+        if (limit > w.Sk - 1) limit = w.Sk - 1;
         bool in_flight = false;           // the scores of this tile were asked for at the end of the group's previous tile
         __syncwarp();
 

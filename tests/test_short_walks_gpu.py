@@ -41,3 +41,24 @@ def test_short_walks_equal_one_cta_per_tile(oracle, B, Hq, Hkv, Sq, Sk, causal, 
         assert np.abs(got - want).max() <= TOL_O
     if causal and Sq > Sk:
         assert torch.all(o[:, :, : Sq - Sk] == 0)
+
+
+@pytest.mark.parametrize("Hq,Hkv,causal,longest,producer", [(8, 2, True, 1000, 0), (6, 6, False, 3072, 0), (8, 4, True, 3073, 0), (8, 2, True, 700, 1), (8, 2, False, 640, 1)])
+def test_short_walks_of_a_packed_batch(Hq, Hkv, causal, longest, producer):
+    """Sequences of mixed lengths, up to the longest that the rule takes and one past it: shared query tiles (few tokens), the
+    few-row path beside them, queries that see nothing, none at all.  Each equals its forward alone bit for bit."""
+    g = torch.Generator(device="cuda").manual_seed(13)
+    lens = [(500, longest), (40, 300), (1, 200), (300, 100), (129, 129), (0, 50), (30, 257), (128, 128), (70, 0), (1300, 640), (257, 384), (1000, 512)]
+    cu_q = np.concatenate([[0], np.cumsum([a for a, _ in lens])])
+    cu_k = np.concatenate([[0], np.cumsum([b for _, b in lens])])
+    q = torch.randn(int(cu_q[-1]), Hq, 128, generator=g, device="cuda").bfloat16()
+    k, v = (torch.randn(int(cu_k[-1]), Hkv, 128, generator=g, device="cuda").bfloat16() for _ in range(2))
+    o = binding.efq_attention_fwd_varlen(q, k, v, cu_q, cu_k, causal, 0.0, producer)
+    for n, (lq, lk) in enumerate(lens):
+        got = o[cu_q[n]:cu_q[n + 1]].permute(1, 0, 2)
+        if lq == 0 or lk == 0:
+            assert torch.all(got == 0)
+            continue
+        one = [t.permute(1, 0, 2)[None].contiguous() for t in (q[cu_q[n]:cu_q[n + 1]], k[cu_k[n]:cu_k[n + 1]], v[cu_k[n]:cu_k[n + 1]])]
+        alone = binding.exp_then_quantize_attention_fwd(*one, causal, 0.0, 0) if producer else binding.efq_attention_fwd(*one, causal)
+        assert torch.equal(got, alone[0]), f"sequence {n}"
