@@ -31,6 +31,7 @@
 #include <algorithm>
 #include <atomic>
 #include <mutex>
+#include <type_traits>
 #include <vector>
 
 #include "efq_common.cuh"
@@ -763,15 +764,16 @@ cudaError_t launch_one(dim3 grid, size_t smem, cudaStream_t stream, const CUtens
 }
 
 // Short KV walks and more query tiles than SMs: persistent CTAs (the measurements are in attention_short.cuh).  The line lies
-// where the gain is still 2 to 4 %, causal or not: 24 KV tiles.  The plain exponential producers (1, 2) in a packed batch, whose
-// code generation is long enough to hide the other kernel's start, gain only on short sequences (4 of 200 to 400 tokens 33 -> 29
-// us) and lose on long ones (6 of up to 3000 tokens 167 -> 179 us): 4 tiles.
-constexpr int kShortTiles = 24, kShortTilesPlainTable = 4;
+// where the gain is still 2 to 4 %, causal or not: 24 KV tiles for the affine rule and its table form.  The exponential producers
+// gain on long walks too; 128 tiles is as far as the plain forms (1, 2) do (no difference at 16384 keys, not causal).
+constexpr int kShortTiles = 24, kShortTilesPlain = 128, kShortTilesFolded = 1 << 24;
 // P.Sk: the keys of the problem or of the longest sequence.
 bool use_short(int producer, bool debug, int64_t items, int sms, const FwdParams& P)
 {
     return !debug && producer != 6 && !P.packed && !P.inject_skip_loads && items > sms &&
-           P.Sk <= (P.items && (producer == 1 || producer == 2) ? kShortTilesPlainTable : kShortTiles) * static_cast<int64_t>(kTile);
+           P.Sk <= (producer == 1 || producer == 2   ? kShortTilesPlain
+                    : producer == 4 || producer == 5 ? kShortTilesFolded
+                                                     : kShortTiles) * static_cast<int64_t>(kTile);
 }
 
 template <int PRODUCER, bool TABLE>

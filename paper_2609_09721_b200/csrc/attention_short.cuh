@@ -12,6 +12,8 @@
 // call, 24 heads, 16000 queries, not causal): 128 keys 153 -> 90 us, 256 keys 164 -> 111, 512 keys 195 -> 142, 1024 keys
 // 255 -> 211, 2048 keys 373 -> 342, 3072 keys 488 -> 468, 4096 keys 604 -> 594, 8192 keys 1064 -> 1098.  Causal, 32 heads: 32 x 128
 // tokens 60 -> 39 us, 4 x 1024 tokens 74 -> 67, 2048 tokens 51 -> 48, 3000 tokens 89 -> 87, 4096 tokens 134 -> 136.
+// The exponential producers gain at every length, their code generation hides what the loop costs: S = 2048 65 -> 58 us, 4096
+// 191 -> 182, 16384 2348 -> 2305; folded scale 56 -> 46, 157 -> 143, 1859 -> 1765.
 // Packed batches: 16 sequences of 100 to 3000 tokens 565 -> 513 us, 40 of 100 to 500 235 -> 188, 64 of 64 to 128 132 -> 94.
 #pragma once
 
@@ -85,6 +87,9 @@ attention_short_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
                        const __grid_constant__ CUtensorMap map_v, const FwdParams P, const uint32_t n_items)
 {
     static_assert(PRODUCER != 6, "the denominator of FP32 exponentials is summed by attention_fwd_kernel only");
+    // Keys and tiles of the probability warps fit 32 bits (shapes stay below 2^31 rows).  The affine rule is faster with 64 all the
+    // same (512 keys 277 -> 286 us with 32), the others with 32 (exponential, S = 4096: 198 -> 184): what the compiler makes of it.
+    using Index = typename std::conditional<PRODUCER == 0, int64_t, int>::type;
     extern __shared__ uint8_t smem_raw[];
     ShortSmem* sm = reinterpret_cast<ShortSmem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
     const int warp = threadIdx.x >> 5;
@@ -363,12 +368,12 @@ attention_short_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
         const int n_tiles = w.n_tiles;
         if (n_tiles <= 0) continue;
         const int64_t token = TABLE && w.packed ? static_cast<int>(row) % static_cast<int>(w.Sq) : w.q0 + static_cast<int64_t>(row);
-        int64_t limit = P.causal ? token + w.Sk - w.Sq : w.Sk - 1;   // last visible key of this row
-        if (limit > w.Sk - 1) limit = w.Sk - 1;
+        const int64_t sees = P.causal ? token + w.Sk - w.Sq : w.Sk - 1;
+        const Index limit = static_cast<Index>(sees > w.Sk - 1 ? w.Sk - 1 : sees < -1 ? -1 : sees);   // last visible key of this row
         bool in_flight = false;           // the scores of this tile were asked for at the end of the group's previous tile
         __syncwarp();
 
-        for (int64_t j = (base & 1u) ^ static_cast<uint32_t>(group); j < n_tiles; j += 2) {
+        for (Index j = static_cast<Index>((base & 1u) ^ static_cast<uint32_t>(group)); j < n_tiles; j += 2) {
             const uint32_t t = base + static_cast<uint32_t>(j);
             const int sb = group;                                         // S, P and exchange buffers belong to the group
             const uint32_t ph2 = (t >> 1) & 1u;
@@ -392,11 +397,11 @@ attention_short_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
                 if (j > 0 && have_prev) m_prev = sm->runmax[sb ^ 1][row];
                 ptx::tmem_wait_ld();
                 ptx::tc_fence_before_sync();          // the S buffer is handed back with the joint publication below
-                const int64_t key0 = j * kTile;
-                if (__any_sync(0xffffffffu, key0 + 127 > limit)) {     // diagonal or ragged tile: keys past the row's limit are masked in place
+                const Index last = limit - j * kTile;     // last visible key of the row inside the tile
+                if (__any_sync(0xffffffffu, last < 127)) {     // diagonal or ragged tile: keys past the row's limit are masked in place
 #pragma unroll
                     for (int i = 0; i < 128; ++i)
-                        if (key0 + i > limit) r[i] = -INFINITY;
+                        if (i > last) r[i] = -INFINITY;
                 }
             }
 #pragma unroll
