@@ -763,17 +763,16 @@ cudaError_t launch_one(dim3 grid, size_t smem, cudaStream_t stream, const CUtens
     return launch_overlapped(attention_fwd_kernel<PRODUCER, DEBUG>, grid, kThreads, smem, stream, mq, mk, mv, P);
 }
 
-// Short KV walks and more query tiles than SMs: persistent CTAs (the measurements are in attention_short.cuh).  The line lies
-// where the gain is still 2 to 4 %, causal or not: 24 KV tiles for the affine rule and its table form.  The exponential producers
-// gain on long walks too; 128 tiles is as far as the plain forms (1, 2) do (no difference at 16384 keys, not causal).
-constexpr int kShortTiles = 24, kShortTilesPlain = 128, kShortTilesFolded = 1 << 24;
-// P.Sk: the keys of the problem or of the longest sequence.
+// Short KV walks and more query tiles than SMs: persistent CTAs (the measurements are in attention_short.cuh).  The line is drawn
+// by the mean walk of a query tile, half of a causal square, where the gain is down to 1 or 2 %: 40 KV tiles for the affine rule,
+// 24 for its table form.  The exponential producers gain on long walks too; 128 tiles is as far as the plain forms (1, 2) do.
+// P.Sk: the keys of the problem or, with P.Sq = 0, of the longest sequence.
 bool use_short(int producer, bool debug, int64_t items, int sms, const FwdParams& P)
 {
-    return !debug && producer != 6 && !P.packed && !P.inject_skip_loads && items > sms &&
-           P.Sk <= (producer == 1 || producer == 2   ? kShortTilesPlain
-                    : producer == 4 || producer == 5 ? kShortTilesFolded
-                                                     : kShortTiles) * static_cast<int64_t>(kTile);
+    if (debug || producer == 6 || P.packed || P.inject_skip_loads || items <= sms) return false;
+    const int64_t tiles = producer == 0 ? 40 : producer == 3 ? 24 : producer <= 2 ? 128 : 1 << 24;
+    const int64_t mean = P.causal ? P.Sk - std::min(P.Sq, P.Sk) / 2 : P.Sk;
+    return mean <= tiles * kTile;
 }
 
 template <int PRODUCER, bool TABLE>

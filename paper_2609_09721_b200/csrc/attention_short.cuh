@@ -8,10 +8,11 @@
 // tile counter t runs over all items of the CTA: it picks buffers and phases, the tile j inside the item picks the keys.
 // Everything else, the arithmetic above all, is that of attention_fwd_kernel, and so is the result, bit for bit.
 //
-// Why not for all shapes: in the steady state the looped form is 3 to 4 % slower.  Measured against the other kernel (whole
-// call, 24 heads, 16000 queries, not causal): 128 keys 153 -> 90 us, 256 keys 164 -> 111, 512 keys 195 -> 142, 1024 keys
-// 255 -> 211, 2048 keys 373 -> 342, 3072 keys 488 -> 468, 4096 keys 604 -> 594, 8192 keys 1064 -> 1098.  Causal, 32 heads: 32 x 128
-// tokens 60 -> 39 us, 4 x 1024 tokens 74 -> 67, 2048 tokens 51 -> 48, 3000 tokens 89 -> 87, 4096 tokens 134 -> 136.
+// Why not for all shapes: in the steady state the looped form is 3 % slower.  Measured against the other kernel (whole
+// call, 24 heads, 16000 queries, not causal): 128 keys 153 -> 89 us, 256 keys 164 -> 111, 512 keys 195 -> 140, 1024 keys
+// 255 -> 211, 2048 keys 373 -> 342, 3072 keys 487 -> 459, 4096 keys 604 -> 583, 6144 keys 834 -> 827, 8192 keys 1064 -> 1070,
+// 16384 keys 1988 -> 2052.  Causal, 32 heads: 32 x 128 tokens 60 -> 39 us, 4 x 1024 tokens 74 -> 61, 2048 tokens 51 -> 46, 4096
+// tokens 133 -> 129, 8192 tokens 428 -> 421, 16384 tokens 1466 -> 1472.
 // The exponential producers gain at every length, their code generation hides what the loop costs: S = 2048 65 -> 58 us, 4096
 // 191 -> 182, 16384 2348 -> 2305; folded scale 56 -> 46, 157 -> 143, 1859 -> 1765.
 // Packed batches: 16 sequences of 100 to 3000 tokens 565 -> 513 us, 40 of 100 to 500 235 -> 188, 64 of 64 to 128 132 -> 94.
