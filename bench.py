@@ -37,10 +37,10 @@ NOMINAL_FP4_OVER_BF16 = 4.0          # dense FP4 : dense bf16 tensor throughput 
 FALLBACK_BF16_TFLOPS = 1590.0
 FALLBACK_HBM_GBS = 6650.0
 # dram__bytes_read.sum + dram__bytes_write.sum of one launch of the fused kernel: NOT measured by this run, copied
-# from the single-pass ncu capture summarised in the named profile, and valid only for the kernel revision that
+# from the ncu capture summarised in the named profile, and valid only for the kernel revision that
 # capture saw (the library's version tag); for any other revision the line carries null.
 NCU_DRAM_BYTES_PER_LAUNCH = {
-    "qwen3_8b_16k": {"bytes": 57717248 + 217710080, "kernel_revision": "fwd.3", "profile": "profiles/attention_fwd_qwen3_8b_16k.md"},
+    "qwen3_8b_16k": {"bytes": 53586944 + 211130112, "kernel_revision": "fwd.5", "profile": "profiles/attention_fwd_current.md"},
 }
 BURST_REGION_S = 1.0   # a timed region shorter than this runs at burst clocks: its roofline uses the burst peak
 
