@@ -103,6 +103,10 @@ __host__ __device__ inline int few_chunk_tiles(int n_tiles, int rows)
 {
     return rows <= 8 ? (n_tiles < 16 ? 1 : n_tiles < 32 ? 2 : n_tiles < 128 ? 4 : kFewMaxChunk) : n_tiles < 32 ? 2 : kFewMaxChunk;
 }
+// Start of row `row` of the scores of a KV head (row_len keys) or of its block maxima: 64-bit, since 24 rows pass 2^31 scores
+// from 97.6 million keys on.
+__host__ __device__ constexpr int64_t few_row_offset(int row, int row_len) { return static_cast<int64_t>(row_len) * row; }
+static_assert(few_row_offset(kFewMaxRows - 2, 100000000) == 2200000000ll, "rows of a long context are addressed in 64 bits");
 // floats per query row of a chunk's partial result: 128 of O^T, the maximum they refer to, four parts of the denominator
 constexpr int kFewPartFloats = 136;
 constexpr int kFewInlineSeqs = 128;      // sequence tables up to this size travel as kernel parameters

@@ -77,3 +77,20 @@ def test_inputs_at_a_16_byte_boundary(S, Hq, Hkv):
 
     (q, q2), (k, k2), (v, v2) = pair(Hq), pair(Hkv), pair(Hkv)
     assert torch.equal(binding.efq_attention_fwd(q, k, v, True), binding.efq_attention_fwd(q2, k2, v2, True))
+
+
+def test_rows_past_two_to_the_31_scores():
+    """24 rows on 98 million keys: the scores of rows 22 and 23 start past 2^31.  Every row asks the same, so every row answers
+    what one row by itself does, bit for bit (both lengths of context are cut into the same chunks)."""
+    Sk = 98_000_001
+    assert 22 * Sk > 2 ** 31
+    g = torch.Generator(device="cuda").manual_seed(17)
+    kv = torch.empty(1, 1, Sk, 128, dtype=torch.bfloat16, device="cuda").normal_(generator=g)
+    q = torch.randn(1, 1, 1, 128, generator=g, device="cuda").bfloat16()
+    one = binding.efq_attention_fwd(q, kv, kv)
+    rows = binding.efq_attention_fwd(q.expand(1, 1, 24, 128).contiguous(), kv, kv)
+    assert torch.isfinite(one).all() and one.abs().max() > 0
+    for r in range(24):
+        assert torch.equal(rows[0, 0, r], one[0, 0, 0]), f"row {r}"
+    del kv, one, rows
+    torch.cuda.empty_cache()
