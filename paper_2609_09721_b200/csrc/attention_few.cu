@@ -7,7 +7,7 @@
 //                       maxima of the 32-key blocks go to the workspace (4 bytes per row and key against 256 of K)
 //   few_values_kernel   the running maximum of every row before the chunk from the block maxima; Algorithm 1 with
 //                       thread = key (a microscaling block is a warp); V tile -> MXFP4 operand, transposed;
-//                       O^T[channel, row] += V^^T P~; partial sums of a chunk to the workspace
+//                       O^T[channel, row] += V^^T P~; the partial sums of a chunk take the place of its first tile's scores
 //   few_merge_kernel    the chunks of a row added up
 //
 // The KV range is cut into chunks by a rule on the sequence's own shape, so the result of a sequence does not depend on
@@ -525,14 +525,16 @@ __global__ void __launch_bounds__(kFewThreads, 3) few_values_kernel(const __grid
     }
     add_tile(u.j1 - u.j0 - 1);
 
-    // ---- partial result of the chunk: [row][128] O^T | maximum [row] | denominator [key block][row]
-    float* const part = P.partials + blockIdx.x * (static_cast<size_t>(P.row_cap) * kFewPartFloats);
+    // ---- partial result of the chunk.  Its scores may go: the block's threads used the last of them before the barrier of the last
+    // tile, and no other block reads them.
+    float* const part = P.scores + u.s_off + few_row_offset(half, u.Sk_pad) + u.j0 * kTile + quarter * 32 + lane;
 #pragma unroll
     for (int i = 0; i < NH; ++i)
-        if (2 * i + half < R) part[(2 * i + half) * 128 + quarter * 32 + lane] = acc[i];
+        if (2 * i + half < R) part[few_row_offset(2 * i, u.Sk_pad)] = acc[i];
     if (has_row) {
-        if (quarter == 0) part[P.row_cap * 128 + my_row] = sm->m_s[(u.j1 - u.j0 - 1) % kStateRing][my_row];
-        part[P.row_cap * (129 + quarter) + my_row] = l_run;
+        float* const stat = P.stats + (static_cast<size_t>(blockIdx.x) * P.row_cap + my_row) * kFewStatFloats;
+        stat[quarter] = l_run;
+        if (quarter == 0) stat[4] = sm->m_s[(u.j1 - u.j0 - 1) % kStateRing][my_row];
     }
     ptx::tc_fence_before_sync();
     __syncthreads();
@@ -552,18 +554,20 @@ __global__ void __launch_bounds__(128) few_merge_kernel(const __grid_constant__ 
     const Unit u = find_unit(P, first_id);
     ptx::grid_wait();
     if (row >= P.G * u.Sq) return;
-    const size_t part_floats = static_cast<size_t>(P.row_cap) * kFewPartFloats, step = part_floats * P.Hkv;
-    const float* const first = P.partials + first_id * part_floats;
-    const float m_last = __ldcg(first + (u.n_chunks - 1) * step + P.row_cap * 128 + row);
+    // the row's partial results: u is the first chunk, whose length is that of all but the last
+    const float4* const part = reinterpret_cast<const float4*>(P.scores + u.s_off + few_row_offset(row, u.Sk_pad)) + lane;
+    const int part_step = u.j1 * (kTile / 4);
+    const float* const stat = P.stats + (static_cast<size_t>(first_id) * P.row_cap + row) * kFewStatFloats;
+    const size_t stat_step = static_cast<size_t>(P.Hkv) * P.row_cap * kFewStatFloats;
+    const float m_last = __ldcg(stat + (u.n_chunks - 1) * stat_step + 4);
     float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
     float l = 0.0f;
 #pragma unroll 4
     for (int c = warp; c < u.n_chunks; c += 4) {
-        const float* p = first + c * step;
-        const float m = __ldcg(p + P.row_cap * 128 + row);
-        const float4 x = __ldcg(reinterpret_cast<const float4*>(p + row * 128) + lane);
-        const float lc = (__ldcg(p + P.row_cap * 129 + row) + __ldcg(p + P.row_cap * 130 + row)) +
-                         (__ldcg(p + P.row_cap * 131 + row) + __ldcg(p + P.row_cap * 132 + row));
+        const float m = __ldcg(stat + c * stat_step + 4);
+        const float4 x = __ldcg(part + static_cast<int64_t>(c) * part_step);
+        const float4 lp = __ldcg(reinterpret_cast<const float4*>(stat + c * stat_step));
+        const float lc = (lp.x + lp.y) + (lp.z + lp.w);
         const float w = m == -INFINITY ? 0.0f : ex2_approx(__fmul_rn(__fsub_rn(m, m_last), P.K.LOG2E));
         l = fmaf(lc, w, l);
         a.x = fmaf(x.x, w, a.x); a.y = fmaf(x.y, w, a.y); a.z = fmaf(x.z, w, a.z); a.w = fmaf(x.w, w, a.w);
@@ -614,7 +618,7 @@ FewPlan plan_few(int64_t units, int64_t keys_padded_all_heads, int rows)
     auto take = [&](size_t bytes) { const size_t at = off; off = (off + bytes + 1023) / 1024 * 1024; return at; };
     w.scores = take(static_cast<size_t>(keys_padded_all_heads) * rows * sizeof(float));
     w.block_max = take(static_cast<size_t>(keys_padded_all_heads / 32) * rows * sizeof(float));
-    w.partials = take(static_cast<size_t>(units) * rows * kFewPartFloats * sizeof(float));
+    w.stats = take(static_cast<size_t>(units) * rows * kFewStatFloats * sizeof(float));
     w.total = off;
     return w;
 }

@@ -911,7 +911,7 @@ efq_status_t attention_impl(const void* q, const void* k, const void* v, float* 
         F.n_units = static_cast<int32_t>(units);
         const FewPlan fp = plan_few(units, static_cast<int64_t>(B) * Hkv * w.Sk_pad, F.row_cap);
         F.scores = reinterpret_cast<float*>(ws + 1024 + fp.scores); F.block_max = reinterpret_cast<float*>(ws + 1024 + fp.block_max);
-        F.partials = reinterpret_cast<float*>(ws + 1024 + fp.partials);
+        F.stats = reinterpret_cast<float*>(ws + 1024 + fp.stats);
         F.status = reinterpret_cast<uint32_t*>(ws);
         F.has_dbg = debug != nullptr ? 1 : 0;
         if (debug != nullptr) F.dbg = *debug;
@@ -1388,7 +1388,7 @@ extern "C" efq_status_t efq_attention_fwd_varlen(const void* q, const void* k, c
         const FewPlan fp = plan_few(p.few_units, p.few_keys * Hkv, p.few_rows);
         uint8_t* const fw = ws + p.few;
         F.scores = reinterpret_cast<float*>(fw + fp.scores); F.block_max = reinterpret_cast<float*>(fw + fp.block_max);
-        F.partials = reinterpret_cast<float*>(fw + fp.partials);
+        F.stats = reinterpret_cast<float*>(fw + fp.stats);
         F.status = reinterpret_cast<uint32_t*>(ws);
         if (!few_long.empty()) {
             if (cudaMemcpyAsync(ws + p.few_table, few_long.data(), sizeof(FewSeq) * few_long.size(), cudaMemcpyHostToDevice, s) != cudaSuccess) return EFQ_ERR_CUDA;

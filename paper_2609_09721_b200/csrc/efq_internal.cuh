@@ -94,7 +94,6 @@ struct ItemDesc {
 // ------------------------------------------------------------------------------------------------
 // Few query rows (attention_few.cu): the query rows of a KV group, Hq / Hkv * Sq of them, are at most kFewMaxRows
 // ------------------------------------------------------------------------------------------------
-// 24 rows keep the scores in the workspace below the size of the MXFP4 copies that the general path would need there.
 constexpr int kFewMaxRows = 24;
 // Tiles of a chunk of the KV range, by the sequence's own shape: short contexts are cut finely, so that one of them spreads
 // over the chip; with many rows a chunk's partial result (544 bytes a row) has to be small against its 64 KB of K and V a tile.
@@ -107,8 +106,12 @@ __host__ __device__ inline int few_chunk_tiles(int n_tiles, int rows)
 // from 97.6 million keys on.
 __host__ __device__ constexpr int64_t few_row_offset(int row, int row_len) { return static_cast<int64_t>(row_len) * row; }
 static_assert(few_row_offset(kFewMaxRows - 2, 100000000) == 2200000000ll, "rows of a long context are addressed in 64 bits");
-// floats per query row of a chunk's partial result: 128 of O^T, the maximum they refer to, four parts of the denominator
-constexpr int kFewPartFloats = 136;
+// A chunk's partial result: the 128 values of a row's O^T take the place of the row's scores of the chunk's first tile, which
+// nobody reads any more by then; beside them, per row, four parts of the denominator, the maximum they refer to, three unused.
+// So a KV head needs rows * (528 tiles + 32 chunks) bytes, at 24 rows and a tile a chunk 13440 a tile: less than the 17408 of the
+// MXFP4 copies of K and V, and what fits a workspace on the general path fits it here.  (With O^T in a place of its own, 544
+// bytes a row and chunk, 22 to 24 rows below 32 tiles did not; longer chunks would fit, and take 29 us instead of 20 there.)
+constexpr int kFewStatFloats = 8;
 constexpr int kFewInlineSeqs = 128;      // sequence tables up to this size travel as kernel parameters
 
 struct FewSeq {
@@ -129,7 +132,7 @@ struct FewParams {
     int32_t n_units, n_heads;                  // chunks times KV heads, and KV heads, of all sequences
     float rescale_threshold;
     ProducerConsts K;
-    float *scores, *block_max, *partials;      // workspace
+    float *scores, *block_max, *stats;         // workspace
     uint32_t* status;
     int32_t has_dbg;
     efq_debug_t dbg;
@@ -137,7 +140,7 @@ struct FewParams {
     FewSeq inline_seqs[kFewInlineSeqs];
 };
 
-struct FewPlan { size_t scores, block_max, partials, total; };   // offsets from a 1024-byte aligned base
+struct FewPlan { size_t scores, block_max, stats, total; };   // offsets from a 1024-byte aligned base
 FewPlan plan_few(int64_t units, int64_t keys_padded_all_heads, int rows);
 // Clears the status words.
 cudaError_t launch_few(int producer, const FewParams& P, cudaStream_t stream);

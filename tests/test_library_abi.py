@@ -75,3 +75,29 @@ def test_workspace_planning_is_host_logic():
     assert _varlen_bytes([0, 5, 3], [0, 5, 9], 8, 2) == 0                              # and never decrease
     assert _varlen_bytes([0, 5], [0, 5], 8, 3) == 0
     assert _varlen_bytes([0], [0], 8, 2) > 0                                           # an empty batch is valid
+
+
+def _round_up(x, a):
+    return (x + a - 1) // a * a
+
+
+def _mxfp4_bytes(B, Hq, Hkv, Sq, Sk):
+    """Status words and the MXFP4 copies of Q, K and V, each part on a 1 KiB boundary: what the general path lays out."""
+    q, k = B * Hq * _round_up(Sq, 128), B * Hkv * _round_up(Sk, 128)
+    return 1024 + sum(_round_up(rows * 64, 1024) + _round_up(rows * 4, 1024) for rows in (q, k, k))
+
+
+def test_few_row_shapes_need_no_more_workspace_than_the_general_path():
+    """The path for few query rows lays the workspace out differently but never needs more of it, so what fits a workspace (the
+    4 MiB of efq_attention_fwd_static among them) does not depend on the path, and a workspace that is large enough for some
+    query length is so for every shorter one."""
+    size = binding.efq_attention_workspace_bytes
+    for G in (1, 2, 3, 8, 24):
+        for Sq in range(1, 26 // G + 1):
+            for Hkv in (1, 2, 8, 31, 65):
+                for Sk in list(range(64, 6000, 128)) + [129, 8192, 16383, 60001]:
+                    assert size(1, G * Hkv, Hkv, Sq, Sk, 128) == _mxfp4_bytes(1, G * Hkv, Hkv, Sq, Sk), (G, Sq, Hkv, Sk)
+    assert size(3, 8, 8, 24, 777, 128) == _mxfp4_bytes(3, 8, 8, 24, 777)
+    # at the edge of the built-in scratch, where 22 to 24 rows a KV head did not fit
+    for Hq, Hkv, Sq, Sk in ((32, 8, 6, 3400), (24, 24, 24, 1100), (65, 65, 24, 300)):
+        assert size(1, Hq, Hkv, Sq, Sk, 128) <= binding.STATIC_SCRATCH_BYTES

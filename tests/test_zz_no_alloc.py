@@ -54,3 +54,12 @@ def test_static_entry_applies_the_argument_rules_of_the_regular_forward():
     with pytest.raises(binding.EfqError) as e:       # Hq % Hkv != 0 is an invalid argument here too
         binding.efq_attention_fwd_static(q, k, k, False, o=torch.empty((1, 3, 128, 128), dtype=torch.float32, device="cuda"))
     assert e.value.status == binding.STATUS_NAMES.index("EFQ_ERR_INVALID_ARG")
+
+
+@pytest.mark.parametrize("Hq,Hkv,Sq,Sk", [(32, 8, 6, 3400), (24, 24, 24, 1100)])
+def test_static_scratch_takes_few_row_shapes_at_its_edge(Hq, Hkv, Sq, Sk):
+    """24 query rows a KV head on the path for few rows: the largest part of the scratch per key."""
+    g = torch.Generator(device="cuda").manual_seed(5)
+    q = torch.randn(1, Hq, Sq, 128, generator=g, device="cuda").bfloat16()
+    k, v = (torch.randn(1, Hkv, Sk, 128, generator=g, device="cuda").bfloat16() for _ in range(2))
+    assert torch.equal(binding.efq_attention_fwd_static(q, k, v, True), binding.efq_attention_fwd(q, k, v, True))
