@@ -1,7 +1,9 @@
 /* Call path from Python into the C ABI for the entry points that a serving loop calls per step: a CPython extension that
  * takes plain integers (addresses, sizes, a stream) and passes them on.  Marshalling only, like the ctypes binding beside
  * it, which costs 2.3 microseconds for the 17 arguments of a forward (and tens for the prefix sums of a packed batch)
- * where this takes a few tenths.  The library is not linked: the binding hands over the addresses of its functions. */
+ * where this takes a few tenths.  The library is not linked: the binding hands over the addresses of its functions.
+ * As in ctypes, the interpreter lock is released around every call: a launch waits while the stream's queue is full, and the
+ * table copy of a packed batch may wait for the stream, and neither may stop the other threads of a server. */
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 #include <stdint.h>
@@ -28,6 +30,9 @@ static struct {
     varlen_fn varlen;
     varlen_bytes_fn varlen_bytes;
 } fn;
+
+/* The call without the interpreter lock; its arguments are plain C values by then. */
+#define UNLOCKED(type, call) type st; Py_BEGIN_ALLOW_THREADS st = call; Py_END_ALLOW_THREADS
 
 /* Arguments are converted first and errors looked at once: a conversion that fails leaves the exception set. */
 static void* ptr(PyObject* o) { return o == Py_None ? NULL : (void*)(uintptr_t)PyLong_AsUnsignedLongLong(o); }
@@ -67,7 +72,8 @@ static PyObject* attention(PyObject* self, PyObject* const* a, Py_ssize_t n)
     const float scale = f32(a[11]);
     void *params = ptr(a[12]), *ws = ptr(a[13]), *debug = ptr(a[15]), *stream = ptr(a[16]);
     if (PyErr_Occurred()) return NULL;
-    return PyLong_FromLong(fn.attention(q, k, v, o, B, Hq, Hkv, Sq, Sk, d, causal, scale, params, ws, (size_t)bytes, debug, stream));
+    UNLOCKED(efq_status_t, fn.attention(q, k, v, o, B, Hq, Hkv, Sq, Sk, d, causal, scale, params, ws, (size_t)bytes, debug, stream))
+    return PyLong_FromLong(st);
 }
 
 static PyObject* etq_attention(PyObject* self, PyObject* const* a, Py_ssize_t n)
@@ -80,7 +86,8 @@ static PyObject* etq_attention(PyObject* self, PyObject* const* a, Py_ssize_t n)
     const float scale = f32(a[11]);
     void *ws = ptr(a[13]), *debug = ptr(a[15]), *stream = ptr(a[16]);
     if (PyErr_Occurred()) return NULL;
-    return PyLong_FromLong(fn.etq_attention(q, k, v, o, B, Hq, Hkv, Sq, Sk, d, causal, scale, mode, ws, (size_t)bytes, debug, stream));
+    UNLOCKED(efq_status_t, fn.etq_attention(q, k, v, o, B, Hq, Hkv, Sq, Sk, d, causal, scale, mode, ws, (size_t)bytes, debug, stream))
+    return PyLong_FromLong(st);
 }
 
 /* scores, ld, row_max, rows, cols, scale, params or scale mode, codes, scales, stream */
@@ -92,7 +99,8 @@ static PyObject* probgen(PyObject* self, PyObject* const* a, Py_ssize_t n)
     const int64_t ld = i64(a[1]), rows = i64(a[3]), cols = i64(a[4]);
     const float scale = f32(a[5]);
     if (PyErr_Occurred()) return NULL;
-    return PyLong_FromLong(fn.probgen(scores, ld, row_max, rows, cols, scale, params, codes, scales, stream));
+    UNLOCKED(efq_status_t, fn.probgen(scores, ld, row_max, rows, cols, scale, params, codes, scales, stream))
+    return PyLong_FromLong(st);
 }
 
 static PyObject* etq_probgen(PyObject* self, PyObject* const* a, Py_ssize_t n)
@@ -104,7 +112,8 @@ static PyObject* etq_probgen(PyObject* self, PyObject* const* a, Py_ssize_t n)
     const float scale = f32(a[5]);
     const int mode = i32(a[6]);
     if (PyErr_Occurred()) return NULL;
-    return PyLong_FromLong(fn.etq_probgen(scores, ld, row_max, rows, cols, scale, mode, codes, scales, stream));
+    UNLOCKED(efq_status_t, fn.etq_probgen(scores, ld, row_max, rows, cols, scale, mode, codes, scales, stream))
+    return PyLong_FromLong(st);
 }
 
 /* A sequence of integers as a C array; NULL with an exception set on failure. */
@@ -147,12 +156,15 @@ static PyObject* varlen(PyObject* self, PyObject* const* a, Py_ssize_t n)
     const float scale = f32(a[12]);
     PyObject* result = NULL;
     if (!PyErr_Occurred()) {
-        if (nq < 1 || nk != nq || cq[nq - 1] != total_q || ck[nk - 1] != total_k)
+        if (nq < 1 || nk != nq || cq[nq - 1] != total_q || ck[nk - 1] != total_k) {
             result = PyLong_FromLong(-1);
-        else if (a[7] == Py_None)
-            result = PyLong_FromSize_t(fn.varlen_bytes(cq, ck, (int)(nq - 1), Hq, Hkv, d));
-        else
-            result = PyLong_FromLong(fn.varlen(q, k, v, o, cq, ck, (int)(nq - 1), Hq, Hkv, d, causal, scale, producer, params, ws, (size_t)bytes, stream));
+        } else if (a[7] == Py_None) {
+            UNLOCKED(size_t, fn.varlen_bytes(cq, ck, (int)(nq - 1), Hq, Hkv, d))
+            result = PyLong_FromSize_t(st);
+        } else {
+            UNLOCKED(efq_status_t, fn.varlen(q, k, v, o, cq, ck, (int)(nq - 1), Hq, Hkv, d, causal, scale, producer, params, ws, (size_t)bytes, stream))
+            result = PyLong_FromLong(st);
+        }
     }
     free(cq);
     free(ck);

@@ -2,6 +2,9 @@
 import ctypes
 import os
 import re
+import subprocess
+import threading
+import time
 
 import pytest
 
@@ -114,3 +117,37 @@ def test_few_row_sequences_of_a_packed_batch_take_no_more_than_their_copies(lens
     cu_k = [sum(b for _, b in lens[:i]) for i in range(len(lens) + 1)]
     copies = sum(Hkv * (128 + 2 * _round_up(lk, 128)) * 68 for _, lk in lens)
     assert _varlen_bytes(cu_q, cu_k, Hkv, Hkv) <= copies + 32 * len(lens) + 16384
+
+
+def test_calls_do_not_hold_the_interpreter_lock(tmp_path):
+    """While a call of the extension waits (here in functions that sleep in the place of the library's), other Python threads
+    run: the counting thread gets on during each of the six calls."""
+    (tmp_path / "slow.c").write_text("#include <unistd.h>\nlong slow(void) { usleep(200000); return 0; }\n")
+    subprocess.run(["gcc", "-shared", "-fPIC", str(tmp_path / "slow.c"), "-o", str(tmp_path / "slow.so")], check=True)
+    slow = ctypes.cast(ctypes.CDLL(str(tmp_path / "slow.so")).slow, ctypes.c_void_p).value
+    fast = binding._fastcall()
+    count, stop = [0], threading.Event()
+
+    def run():
+        while not stop.is_set():
+            count[0] += 1
+            time.sleep(0.002)
+
+    thread = threading.Thread(target=run)
+    fast.set_functions(*[slow] * 6)
+    try:
+        thread.start()
+        for name, call in {"attention": lambda: fast.attention(*[0] * 11, 0.0, *[0] * 5),
+                           "etq_attention": lambda: fast.etq_attention(*[0] * 11, 0.0, *[0] * 5),
+                           "probgen": lambda: fast.probgen(*[0] * 5, 1.0, *[0] * 4),
+                           "etq_probgen": lambda: fast.etq_probgen(*[0] * 5, 1.0, *[0] * 4),
+                           "varlen_bytes": lambda: fast.varlen([0], [0], *[0] * 5, None, *[0] * 4, 0.0, *[0] * 5),
+                           "varlen": lambda: fast.varlen([0], [0], *[0] * 10, 0.0, *[0] * 5)}.items():
+            before = count[0]
+            assert call() == 0
+            assert count[0] - before >= 5, f"{name}: the other thread stood still"
+    finally:
+        stop.set()
+        thread.join()
+        binding._fast = None
+        binding._fastcall()             # the library's own functions again
