@@ -442,7 +442,7 @@ def efq_stage_microbench(producer: int, num_ctas: int, iters: int, params=None, 
 
 
 def efq_attention_fwd_inject_timeout(q, k, v, o, workspace, stream=None) -> None:
-    """Test hook: the forward with K/V loads left out, so a bounded device-side wait expires (see efq.h)."""
+    """Test hook: the forward with K/V loads (few query rows: MMAs) left out, so a bounded device-side wait expires (see efq.h)."""
     B, Hq, Sq, d = q.shape
     _, Hkv, Sk, _ = k.shape
     st = lib().efq_attention_fwd_inject_timeout(q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(), B, Hq, Hkv, Sq,

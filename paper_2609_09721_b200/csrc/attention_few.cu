@@ -88,15 +88,6 @@ __device__ __forceinline__ Unit find_unit(const FewParams& P, int id)
     return u;
 }
 
-// Bounded wait for a completion of this CTA's own MMAs.  On expiry the status word takes the error; the CTA carries on
-// with whatever the accumulator holds, so that every thread still meets the block's barriers.
-__device__ __forceinline__ void wait_done(uint64_t* bar, uint32_t parity, uint32_t* status)
-{
-    for (int i = 0; i < 20000; ++i)
-        if (ptx::mbar_try_wait_suspend(bar, parity, 50000u)) return;
-    atomicExch(status, static_cast<uint32_t>(EFQ_ERR_DEVICE_TIMEOUT));
-}
-
 __device__ __forceinline__ float warp_max(float x)
 {
     float m;
@@ -128,7 +119,23 @@ struct __align__(1024) FewSmem {
     float4 bmax[kFewMaxChunk][32];  // [tile of the chunk][row]: its block maxima
     uint64_t mma_done[2];
     uint32_t tmem_base;
+    volatile uint32_t gave_up;      // a bounded wait of this CTA ran out
 };
+
+// Bounded wait for a completion of this CTA's own MMAs.  On expiry (about a second) the status word takes the error; the CTA
+// carries on with whatever the accumulator holds, so that every thread still meets the block's barriers, and no further wait of
+// it lasts.  A wait that has gone on for some milliseconds also looks whether another CTA has given up already: block 0 cleared the
+// word long before.
+__device__ __forceinline__ void wait_done(FewSmem* sm, int buf, uint32_t parity, uint32_t* status)
+{
+    for (int i = 1; i <= 20000; ++i) {
+        if (ptx::mbar_try_wait_suspend(&sm->mma_done[buf], parity, 50000u)) return;
+        if (sm->gave_up != 0u) return;
+        if ((i & 127) == 0 && *reinterpret_cast<volatile uint32_t*>(status) != 0u) break;
+    }
+    sm->gave_up = 1u;
+    atomicExch(status, static_cast<uint32_t>(EFQ_ERR_DEVICE_TIMEOUT));
+}
 
 // Operand rows past the last query row are never written: they only reach accumulator columns that nobody reads.
 __device__ __forceinline__ void few_setup(FewSmem* sm, int warp)
@@ -137,13 +144,15 @@ __device__ __forceinline__ void few_setup(FewSmem* sm, int warp)
     if (threadIdx.x == 32) {
         ptx::mbar_init(&sm->mma_done[0], 1);
         ptx::mbar_init(&sm->mma_done[1], 1);
+        sm->gave_up = 0u;
         ptx::mbar_init_fence();
     }
 }
 
 // D[128, N] = A B^T of one tile: two K = 64 steps, a fresh accumulator
-__device__ __forceinline__ void few_mma(FewSmem* sm, uint32_t tmem, int buf, int b_buf, uint32_t n)
+__device__ __forceinline__ void few_mma(const FewParams& P, FewSmem* sm, uint32_t tmem, int buf, int b_buf, uint32_t n)
 {
+    if (P.inject_skip_mma) return;
     const uint64_t d_sw64 = ptx::smem_desc(0, 16, 512, ptx::kLayoutSw64);
     const uint64_t d_sf = ptx::smem_desc(0, 16, 128, ptx::kLayoutNone);
     const uint32_t sfa = tmem + kColSfA + 4 * buf, sfb = tmem + kColSfB + 4 * b_buf, d = tmem + kColD + 32 * buf;
@@ -220,7 +229,7 @@ __global__ void __launch_bounds__(kFewThreads, N <= 8 ? 4 : 3) few_scores_kernel
     // raw scores of a finished tile: thread = key, two rows of the half side by side
     auto put_scores = [&](int j) {
         const int buf = (j - u.j0) & 1;
-        wait_done(&sm->mma_done[buf], static_cast<uint32_t>(j - u.j0) >> 1 & 1u, P.status);
+        wait_done(sm, buf, static_cast<uint32_t>(j - u.j0) >> 1 & 1u, P.status);
         ptx::tc_fence_after_sync();
         float s[N];
         tmem_ld_cols<N>(tmem + (static_cast<uint32_t>(quarter * 32) << 16) + kColD + 32 * buf, s);
@@ -280,7 +289,7 @@ __global__ void __launch_bounds__(kFewThreads, N <= 8 ? 4 : 3) few_scores_kernel
         __syncthreads();
         if (warp == 0) {
             ptx::tc_fence_after_sync();
-            if (ptx::elect_one()) few_mma(sm, tmem, buf, 0, N);
+            if (ptx::elect_one()) few_mma(P, sm, tmem, buf, 0, N);
             __syncwarp();
         }
         if (j > u.j0) put_scores(j - 1);
@@ -447,7 +456,7 @@ __global__ void __launch_bounds__(kFewThreads, 3) few_values_kernel(const __grid
     for (int i = 0; i < NH; ++i) acc[i] = 0.0f;
     auto add_tile = [&](int t) {
         const int buf = t & 1;
-        wait_done(&sm->mma_done[buf], static_cast<uint32_t>(t >> 1) & 1u, P.status);
+        wait_done(sm, buf, static_cast<uint32_t>(t >> 1) & 1u, P.status);
         ptx::tc_fence_after_sync();
         float d[N];
         tmem_ld_cols<N>(tmem + (static_cast<uint32_t>(quarter * 32) << 16) + kColD + 32 * buf, d);
@@ -518,7 +527,7 @@ __global__ void __launch_bounds__(kFewThreads, 3) few_values_kernel(const __grid
         __syncthreads();
         if (warp == 0) {
             ptx::tc_fence_after_sync();
-            if (ptx::elect_one()) few_mma(sm, tmem, buf, buf, N);
+            if (ptx::elect_one()) few_mma(P, sm, tmem, buf, buf, N);
             __syncwarp();
         }
         if (t > 0) add_tile(t - 1);

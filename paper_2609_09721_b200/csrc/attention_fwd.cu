@@ -873,7 +873,7 @@ efq_status_t check_device()
 efq_status_t attention_impl(const void* q, const void* k, const void* v, float* o, int B, int Hq, int Hkv, int64_t Sq,
                             int64_t Sk, int d, int causal, float softmax_scale, int producer, float tau, float h,
                             void* workspace, size_t workspace_bytes, const efq_debug_t* debug, cudaStream_t stream,
-                            bool do_quantize, bool do_forward, bool inject_skip_loads = false, float rescale_threshold = 0.0f)
+                            bool do_quantize, bool do_forward, bool inject = false, float rescale_threshold = 0.0f)
 {
     // q [B, Hq, Sq, d], k, v [B, Hkv, Sk, d], o [B, Hq, Sq, d]
     if (!q || !k || !v || !o) return EFQ_ERR_INVALID_ARG;
@@ -893,7 +893,7 @@ efq_status_t attention_impl(const void* q, const void* k, const void* v, float* 
 
     uint8_t* ws = static_cast<uint8_t*>(workspace);
     const int G = Hq / Hkv;
-    if (do_quantize && do_forward && !inject_skip_loads && use_few(Hq, Hkv, Sq)) {
+    if (do_quantize && do_forward && use_few(Hq, Hkv, Sq)) {
         FewParams F{};
         F.q = static_cast<const __nv_bfloat16*>(q); F.k = static_cast<const __nv_bfloat16*>(k); F.v = static_cast<const __nv_bfloat16*>(v);
         F.o = o;
@@ -913,6 +913,7 @@ efq_status_t attention_impl(const void* q, const void* k, const void* v, float* 
         F.scores = reinterpret_cast<float*>(ws + 1024 + fp.scores); F.block_max = reinterpret_cast<float*>(ws + 1024 + fp.block_max);
         F.stats = reinterpret_cast<float*>(ws + 1024 + fp.stats);
         F.status = reinterpret_cast<uint32_t*>(ws);
+        F.inject_skip_mma = inject ? 1 : 0;
         F.has_dbg = debug != nullptr ? 1 : 0;
         if (debug != nullptr) F.dbg = *debug;
         return launch_few(producer, F, stream) == cudaSuccess ? EFQ_OK : EFQ_ERR_CUDA;
@@ -957,7 +958,7 @@ efq_status_t attention_impl(const void* q, const void* k, const void* v, float* 
     P.status = reinterpret_cast<uint32_t*>(ws + w.status);
     P.packed = packed ? 1 : 0;
     P.seqs = nullptr; P.items = nullptr; P.v_tiles_per_head = 0;
-    P.inject_skip_loads = inject_skip_loads ? 1 : 0;
+    P.inject_skip_loads = inject ? 1 : 0;
     P.rescale_threshold = rescale_threshold;
     P.has_dbg = debug ? 1 : 0;
     if (debug) P.dbg = *debug; else P.dbg = efq_debug_t{};

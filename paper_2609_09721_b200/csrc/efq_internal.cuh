@@ -134,6 +134,7 @@ struct FewParams {
     ProducerConsts K;
     float *scores, *block_max, *stats;         // workspace
     uint32_t* status;
+    int32_t inject_skip_mma;                   // test hook: no MMA is issued, so the first wait for one runs out
     int32_t has_dbg;
     efq_debug_t dbg;
     const FewSeq* seqs;                        // device table; null: inline_seqs

@@ -5,6 +5,8 @@ own FP32 raw scores and running maxima; the raw scores themselves equal the orac
 products of the dequantised operands; (L2) max |O_gpu - O_oracle| <= 2e-3 end to end from the same
 bf16 inputs.  The error against exact (unquantised, FP32-softmax) attention is reported, not bounded
 tightly: the paper prints no figure for it."""
+import time
+
 import numpy as np
 import pytest
 import torch
@@ -447,6 +449,33 @@ def test_bounded_wait_expires_and_context_stays_usable(oracle):
     rows = _all_rows(case, 0, 0, 256)
     want = oracle.attention_rows(q, k, v, rows, False, case.softmax_scale, "efq")
     assert np.abs(o.cpu().numpy()[0, 0] - want).max() <= TOL_O
+
+
+def _kernels(call):
+    """Names of the kernels that the call launched."""
+    with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as prof:
+        call()
+        torch.cuda.synchronize()
+    return " ".join(e.key for e in prof.key_averages())
+
+
+@pytest.mark.parametrize("B,Hq,Hkv,Sq,Sk", [(1, 8, 2, 1, 1000), (64, 32, 8, 1, 2000)])      # one wave of CTAs, seven
+def test_bounded_wait_expires_in_the_few_row_kernels(B, Hq, Hkv, Sq, Sk):
+    """No MMA is issued: both kernels report the expired wait, the CTAs after the first ones do not wait their full second again,
+    and the next forward on the same workspace is what it was before."""
+    g = torch.Generator(device="cuda").manual_seed(3)
+    q = torch.randn(B, Hq, Sq, 128, generator=g, device="cuda").bfloat16()
+    k, v = (torch.randn(B, Hkv, Sk, 128, generator=g, device="cuda").bfloat16() for _ in range(2))
+    ws = torch.empty(binding.efq_attention_workspace_bytes(B, Hq, Hkv, Sq, Sk, 128), dtype=torch.uint8, device="cuda")
+    want = binding.efq_attention_fwd(q, k, v, workspace=ws)
+    assert binding.efq_poll_status(ws) == 0
+    t0 = time.perf_counter()
+    names = _kernels(lambda: binding.efq_attention_fwd_inject_timeout(q, k, v, torch.empty_like(want), ws))
+    assert "few_scores_kernel" in names and "few_values_kernel" in names
+    assert binding.efq_poll_status(ws) == binding.STATUS_NAMES.index("EFQ_ERR_DEVICE_TIMEOUT")
+    assert time.perf_counter() - t0 < 4.0
+    assert torch.equal(binding.efq_attention_fwd(q, k, v, workspace=ws), want)
+    assert binding.efq_poll_status(ws) == 0
 
 
 def test_batch_two_and_quantized_workspace_reuse(oracle):
