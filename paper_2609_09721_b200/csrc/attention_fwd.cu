@@ -769,7 +769,7 @@ cudaError_t launch_one(dim3 grid, size_t smem, cudaStream_t stream, const CUtens
 // P.Sk: the keys of the problem or, with P.Sq = 0, of the longest sequence.
 bool use_short(int producer, bool debug, int64_t items, int sms, const FwdParams& P)
 {
-    if (debug || producer == 6 || P.packed || P.inject_skip_loads || items <= sms) return false;
+    if (debug || producer == 6 || P.packed || items <= sms) return false;
     const int64_t tiles = producer == 0 ? 40 : producer == 3 ? 24 : producer <= 2 ? 128 : 1 << 24;
     const int64_t mean = P.causal ? P.Sk - std::min(P.Sq, P.Sk) / 2 : P.Sk;
     return mean <= tiles * kTile;

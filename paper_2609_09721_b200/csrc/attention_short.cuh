@@ -157,7 +157,7 @@ attention_short_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
             ptx::bulk_load_1d(qb ? sm->sf_q1 : sm->sf_q, P.sf_q + static_cast<int64_t>(w.q_row / kTile) * kSfBytes, kSfBytes, &sm->q_ready[qb]);
             ++n;
             const int64_t sfk_tile0 = w.k_row0 / kTile;
-            for (int j = 0; j < w.n_tiles; ++j) {
+            for (int j = 0; j < (P.inject_skip_loads ? 0 : w.n_tiles); ++j) {
                 // Stage barriers of their own: a waiter on a barrier that other roles may complete twice before it
                 // looks (S runs ahead) could not tell which completion it sees by parity.
                 if (!wait1(&sm->k_empty[s], ph ^ 1u, sm, P.status)) { ok = false; break; }

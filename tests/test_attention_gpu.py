@@ -478,6 +478,23 @@ def test_bounded_wait_expires_in_the_few_row_kernels(B, Hq, Hkv, Sq, Sk):
     assert binding.efq_poll_status(ws) == 0
 
 
+@pytest.mark.parametrize("B,Hq,Hkv,Sq,Sk", [(1, 16, 4, 1300, 400), (3, 24, 8, 2000, 700)])      # about one item a CTA, eight
+def test_bounded_wait_expires_with_persistent_ctas(B, Hq, Hkv, Sq, Sk):
+    """The same in the kernel for short KV walks: each role leaves its loop over the items."""
+    g = torch.Generator(device="cuda").manual_seed(4)
+    q = torch.randn(B, Hq, Sq, 128, generator=g, device="cuda").bfloat16()
+    k, v = (torch.randn(B, Hkv, Sk, 128, generator=g, device="cuda").bfloat16() for _ in range(2))
+    ws = torch.empty(binding.efq_attention_workspace_bytes(B, Hq, Hkv, Sq, Sk, 128), dtype=torch.uint8, device="cuda")
+    want = binding.efq_attention_fwd(q, k, v, workspace=ws)
+    t0 = time.perf_counter()
+    names = _kernels(lambda: binding.efq_attention_fwd_inject_timeout(q, k, v, torch.empty_like(want), ws))
+    assert "attention_short_kernel" in names
+    assert binding.efq_poll_status(ws) == binding.STATUS_NAMES.index("EFQ_ERR_DEVICE_TIMEOUT")
+    assert time.perf_counter() - t0 < 4.0
+    assert torch.equal(binding.efq_attention_fwd(q, k, v, workspace=ws), want)
+    assert binding.efq_poll_status(ws) == 0
+
+
 def test_batch_two_and_quantized_workspace_reuse(oracle):
     """B = 2 with GQA; the two-call form (quantise once, forward twice with different producers and parameters)
     gives the same results as the one-call forms."""
