@@ -263,7 +263,8 @@ efq_status_t efq_attention_fwd_static(const void* q, const void* k, const void* 
 /* Softmax attention in FP32 on the unquantised bf16 inputs (the problem statement of Sec. 3.1 with no low-bit
  * operand anywhere): O = softmax(scale Q K^T + mask) V, online over the keys, exponentials by expf.  This is the
  * reference output O_ref of the calibration objective and the "exact" side of the error figures; on the
- * tensor cores, with bf16 products that are exact in FP32 and probabilities split into three bf16 terms.  Arguments as for efq_attention_fwd (no workspace); B * Hq <= 65535. */
+ * tensor cores, with bf16 products that are exact in FP32 and probabilities split into three bf16 terms.  Arguments as for
+ * efq_attention_fwd (no workspace); B * Hq <= 65535.  Rows of a block in which a bounded device-side wait expired are NaN. */
 efq_status_t efq_exact_attention_fwd(const void* q, const void* k, const void* v, float* o, int B, int Hq, int Hkv,
                                      int64_t Sq, int64_t Sk, int d, int causal, float softmax_scale, void* stream);
 
@@ -313,13 +314,18 @@ efq_status_t efq_stage_microbench(int producer, const efq_params_t* params, int 
 
 /* Test hook for the bounded-wait path (no GPU fault is involved): efq_attention_fwd, on the kernels that the shape takes there,
  * with the K/V loads left out - for at most 24 query rows a KV head, whose kernels load by themselves, the MMAs - so that the
- * first device-side wait on them runs out after its limit (about a second).  Every role then
+ * first device-side wait on them runs out after its limit (under a second).  Every role then
  * drains, tensor memory is released, the kernel returns normally and the status word reads
  * EFQ_ERR_DEVICE_TIMEOUT through efq_poll_status(); `o` is undefined.  The context stays usable and the next
  * efq_attention_fwd on the same workspace clears the status. */
 efq_status_t efq_attention_fwd_inject_timeout(const void* q, const void* k, const void* v, float* o, int B, int Hq,
                                               int Hkv, int64_t Sq, int64_t Sk, int d, void* workspace,
                                               size_t workspace_bytes, void* stream);
+
+/* The same for efq_exact_attention_fwd (not causal): K and V are not loaded.  There is no status word; a block whose wait ran out
+ * writes NaN to its rows of `o`. */
+efq_status_t efq_exact_attention_fwd_inject_timeout(const void* q, const void* k, const void* v, float* o, int B, int Hq, int Hkv,
+                                                    int64_t Sq, int64_t Sk, int d, void* stream);
 
 const char* efq_status_string(efq_status_t status);
 

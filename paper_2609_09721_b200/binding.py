@@ -26,8 +26,8 @@ EXPORTS = ["efq_probgen", "exp_then_quantize_probgen", "efq_attention_workspace_
            "efq_attention_fwd_host", "efq_attention_fwd_host_pipelined", "efq_attention_fwd_static", "efq_poll_status",
            "efq_attention_varlen_workspace_bytes", "efq_attention_fwd_varlen",
            "efq_exact_attention_fwd", "efq_relative_error", "efq_calibrate",
-           "efq_fp4_mma_peak_probe", "efq_stage_microbench", "efq_attention_fwd_inject_timeout", "efq_status_string",
-           "efq_version"]
+           "efq_fp4_mma_peak_probe", "efq_stage_microbench", "efq_attention_fwd_inject_timeout",
+           "efq_exact_attention_fwd_inject_timeout", "efq_status_string", "efq_version"]
 
 
 class EfqParams(C.Structure):
@@ -94,6 +94,8 @@ def lib() -> C.CDLL:
                                                C.POINTER(EfqParams), vp]
         L.efq_attention_fwd_inject_timeout.restype = i32
         L.efq_attention_fwd_inject_timeout.argtypes = [vp, vp, vp, vp, i32, i32, i32, i64, i64, i32, vp, C.c_size_t, vp]
+        L.efq_exact_attention_fwd_inject_timeout.restype = i32
+        L.efq_exact_attention_fwd_inject_timeout.argtypes = [vp, vp, vp, vp, i32, i32, i32, i64, i64, i32, vp]
         L.efq_exact_attention_fwd.restype = i32
         L.efq_exact_attention_fwd.argtypes = [vp, vp, vp, vp, i32, i32, i32, i64, i64, i32, i32, f32, vp]
         L.efq_relative_error.restype = i32
@@ -448,3 +450,12 @@ def efq_attention_fwd_inject_timeout(q, k, v, o, workspace, stream=None) -> None
     st = lib().efq_attention_fwd_inject_timeout(q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(), B, Hq, Hkv, Sq,
                                                 Sk, d, workspace.data_ptr(), workspace.numel(), _stream(stream))
     _check(st, "efq_attention_fwd_inject_timeout")
+
+
+def efq_exact_attention_fwd_inject_timeout(q, k, v, o, stream=None) -> None:
+    """Test hook: the reference attention with K/V loads left out; the rows of `o` become NaN (see efq.h)."""
+    B, Hq, Sq, d = q.shape
+    _, Hkv, Sk, _ = k.shape
+    st = lib().efq_exact_attention_fwd_inject_timeout(q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(), B, Hq, Hkv, Sq,
+                                                      Sk, d, _stream(stream))
+    _check(st, "efq_exact_attention_fwd_inject_timeout")

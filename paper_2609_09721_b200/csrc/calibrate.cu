@@ -35,16 +35,20 @@ struct __align__(1024) ExactSmem {
     float l_half[2][kTile];
     uint64_t q_full, k_full, v_full, s_done, o_done;
     uint32_t tmem_base;
-    uint32_t failed;
+    volatile uint32_t failed;
 };
 
-// Bounded; on expiry the block is marked as failed and everyone carries on to the end with what is there.
-__device__ __forceinline__ void wait_for(uint64_t* bar, uint32_t parity, ExactSmem* sm)
+// Bounded (20000 polls, 0.07 s when nothing comes); on expiry the block is marked as failed, which ends its other waits too.  What depends on the wait -
+// a load into the buffer, an MMA - is left out after a false: a barrier whose phase has not ended must not get another arrival.
+__device__ __forceinline__ bool wait_for(uint64_t* bar, uint32_t parity, ExactSmem* sm)
 {
-    if (ptx::mbar_try_wait(bar, parity)) return;
-    for (int i = 0; i < 20000; ++i)
-        if (ptx::mbar_try_wait_suspend(bar, parity, 50000u)) return;
+    if (ptx::mbar_try_wait(bar, parity)) return true;
+    for (int i = 0; i < 20000; ++i) {
+        if (ptx::mbar_try_wait_suspend(bar, parity, 50000u)) return true;
+        if (sm->failed != 0u) return false;
+    }
     sm->failed = 1u;
+    return false;
 }
 
 __device__ __forceinline__ uint32_t bf16_pair(float lo, float hi)
@@ -59,7 +63,7 @@ __device__ __forceinline__ uint32_t bf16_pair(float lo, float hi)
 // load while the tensor core and the exponentials do not need their buffer.
 __global__ void __launch_bounds__(256, 1)
 exact_attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
-                       float* __restrict__ o, int heads, int Hq, int Hkv, int Sq, int Sk, int causal, float sigma)
+                       float* __restrict__ o, int heads, int Hq, int Hkv, int Sq, int Sk, int causal, float sigma, int inject_skip_loads)
 {
     extern __shared__ uint8_t smem_raw[];
     ExactSmem* const sm = reinterpret_cast<ExactSmem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
@@ -94,8 +98,10 @@ exact_attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
         ptx::mbar_init(&sm->o_done, 1);
         ptx::mbar_init_fence();
         load_pair(sm->q, &map_q, bh * Sq + q0, &sm->q_full);
-        load_pair(sm->k, &map_k, hkv_row * Sk, &sm->k_full);
-        load_pair(sm->v, &map_v, hkv_row * Sk, &sm->v_full);
+        if (!inject_skip_loads) {
+            load_pair(sm->k, &map_k, hkv_row * Sk, &sm->k_full);
+            load_pair(sm->v, &map_v, hkv_row * Sk, &sm->v_full);
+        }
     }
     ptx::tc_fence_before_sync();
     __syncthreads();
@@ -128,17 +134,20 @@ exact_attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
 #pragma unroll
     for (int i = 0; i < 64; ++i) acc[i] = 0.0f;
     if (warp == 0) {
-        wait_for(&sm->q_full, 0, sm);
-        wait_for(&sm->k_full, 0, sm);
+        const bool ok = __all_sync(0xffffffffu, wait_for(&sm->q_full, 0, sm) && wait_for(&sm->k_full, 0, sm));
         ptx::tc_fence_after_sync();
-        if (ptx::elect_one()) issue_s();
+        if (ok && ptx::elect_one()) issue_s();
         __syncwarp();
     }
+    int k_loads = inject_skip_loads ? 0 : 1, v_loads = k_loads;       // what thread 32 has asked for
     for (int j = 0; j < n_steps; ++j) {
         const uint32_t ph = j & 1;
-        wait_for(&sm->s_done, ph, sm);
+        const bool s_ready = wait_for(&sm->s_done, ph, sm);
         ptx::tc_fence_after_sync();
-        if (tid == 32 && j + 1 < n_steps) load_pair(sm->k, &map_k, hkv_row * Sk + (j + 1) * kTile, &sm->k_full);
+        if (tid == 32 && s_ready && j + 1 < n_steps) {
+            load_pair(sm->k, &map_k, hkv_row * Sk + (j + 1) * kTile, &sm->k_full);
+            ++k_loads;
+        }
         const int key0 = j * kTile + 64 * half;
         float s[64];
         ptx::tmem_ld32f<0>(tmem + lane_base + kColS + 64 * half, s);
@@ -160,6 +169,7 @@ exact_attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
             ptx::fence_proxy_async_smem();
         }
         __syncthreads();
+        if (sm->failed != 0u) break;         // the same for all: nobody waits, and so nobody fails, between the two barriers
         const float m_new = fmaxf(m, fmaxf(sm->tile_max[ph][0][row], sm->tile_max[ph][1][row]));
         const float alpha = m == -INFINITY ? 0.0f : expf(m - m_new);
         const float base = m_new == -INFINITY ? 0.0f : m_new;        // nothing visible yet: every exponential is exp(-inf) = 0
@@ -184,18 +194,20 @@ exact_attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
         ptx::tc_fence_before_sync();
         __syncthreads();
         if (warp == 0) {
-            wait_for(&sm->v_full, ph, sm);
-            if (j + 1 < n_steps) wait_for(&sm->k_full, ph ^ 1u, sm);
+            const bool ok = __all_sync(0xffffffffu, wait_for(&sm->v_full, ph, sm) && (j + 1 == n_steps || wait_for(&sm->k_full, ph ^ 1u, sm)));
             ptx::tc_fence_after_sync();
-            if (ptx::elect_one()) {
+            if (ok && ptx::elect_one()) {
                 issue_pv();
                 if (j + 1 < n_steps) issue_s();
             }
             __syncwarp();
         }
-        wait_for(&sm->o_done, ph, sm);
+        const bool o_ready = wait_for(&sm->o_done, ph, sm);
         ptx::tc_fence_after_sync();
-        if (tid == 32 && j + 1 < n_steps) load_pair(sm->v, &map_v, hkv_row * Sk + (j + 1) * kTile, &sm->v_full);
+        if (tid == 32 && o_ready && j + 1 < n_steps) {
+            load_pair(sm->v, &map_v, hkv_row * Sk + (j + 1) * kTile, &sm->v_full);
+            ++v_loads;
+        }
         float d[64];
         ptx::tmem_ld32f<0>(tmem + lane_base + kColO + 64 * half, d);
         ptx::tmem_ld32f<32>(tmem + lane_base + kColO + 64 * half + 32, d);
@@ -203,6 +215,14 @@ exact_attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
         ptx::tc_fence_before_sync();
 #pragma unroll
         for (int i = 0; i < 64; ++i) acc[i] = fmaf(acc[i], alpha, d[i]);
+    }
+    if (tid == 32 && sm->failed != 0u) {     // its own copies in flight end before the block does
+        auto landed = [](uint64_t* bar, int loads) {
+            for (int i = 0; loads > 0 && i < 1000 && !ptx::mbar_try_wait_suspend(bar, (loads - 1) & 1, 50000u); ++i) {}
+        };
+        landed(&sm->q_full, 1);
+        landed(&sm->k_full, k_loads);
+        landed(&sm->v_full, v_loads);
     }
     sm->l_half[half][row] = l;
     __syncthreads();
@@ -270,9 +290,8 @@ bool is_sm100()
 }  // namespace
 }  // namespace efq
 
-extern "C" efq_status_t efq_exact_attention_fwd(const void* q, const void* k, const void* v, float* o, int B, int Hq,
-                                                int Hkv, int64_t Sq, int64_t Sk, int d, int causal,
-                                                float softmax_scale, void* stream)
+static efq_status_t exact_attention(const void* q, const void* k, const void* v, float* o, int B, int Hq, int Hkv, int64_t Sq, int64_t Sk, int d,
+                                    int causal, float softmax_scale, void* stream, bool inject_skip_loads)
 {
     if (!q || !k || !v || !o) return EFQ_ERR_INVALID_ARG;
     if (B <= 0 || Hq <= 0 || Hkv <= 0 || Sq <= 0 || Sk <= 0 || Hq % Hkv != 0) return EFQ_ERR_INVALID_ARG;
@@ -299,8 +318,22 @@ extern "C" efq_status_t efq_exact_attention_fwd(const void* q, const void* k, co
         return EFQ_ERR_CUDA;
     const dim3 grid(static_cast<unsigned>(q_tiles * B * Hq));
     efq::exact_attention_kernel<<<grid, 256, smem, static_cast<cudaStream_t>(stream)>>>(mq, mk, mv, o, B * Hq, Hq, Hkv, static_cast<int>(Sq),
-                                                                                        static_cast<int>(Sk), causal ? 1 : 0, sigma);
+                                                                                        static_cast<int>(Sk), causal ? 1 : 0, sigma,
+                                                                                        inject_skip_loads ? 1 : 0);
     return cudaGetLastError() == cudaSuccess ? EFQ_OK : EFQ_ERR_CUDA;
+}
+
+extern "C" efq_status_t efq_exact_attention_fwd(const void* q, const void* k, const void* v, float* o, int B, int Hq,
+                                                int Hkv, int64_t Sq, int64_t Sk, int d, int causal,
+                                                float softmax_scale, void* stream)
+{
+    return exact_attention(q, k, v, o, B, Hq, Hkv, Sq, Sk, d, causal, softmax_scale, stream, false);
+}
+
+extern "C" efq_status_t efq_exact_attention_fwd_inject_timeout(const void* q, const void* k, const void* v, float* o, int B, int Hq, int Hkv,
+                                                               int64_t Sq, int64_t Sk, int d, void* stream)
+{
+    return exact_attention(q, k, v, o, B, Hq, Hkv, Sq, Sk, d, 0, 0.0f, stream, true);
 }
 
 static cudaError_t launch_error_sums(const float* a, const float* ref, int64_t n, double* sums, cudaStream_t s)

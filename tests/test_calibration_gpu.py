@@ -1,5 +1,7 @@
 """GPU parity of the calibration helpers (Algorithm 3): the FP32 reference attention, the relative
 Frobenius error and the (tau, h) grid search, each against the CPU oracle, through the C ABI."""
+import time
+
 import numpy as np
 import pytest
 import torch
@@ -47,6 +49,22 @@ def test_exact_attention_batch_and_explicit_scale(oracle):
     got = o.cpu().numpy()
     for n, (b, h, i) in enumerate(rows):
         assert np.abs(got[b, h, i] - want[n]).max() <= 2e-5
+
+
+@pytest.mark.parametrize("Sk", [100, 300, 1024])           # a ragged tile alone, one behind others, none
+def test_bounded_wait_expires_in_the_reference_attention(Sk):
+    """K and V are never loaded: every block gives up once (its later waits do not last), the rows are NaN instead of a wrong
+    number, and the next call is what it was before."""
+    g = torch.Generator(device="cuda").manual_seed(9)
+    q, k, v = (torch.randn(1, 2, n, 128, generator=g, device="cuda").bfloat16() for n in (200, Sk, Sk))
+    want = binding.efq_exact_attention_fwd(q, k, v)
+    torch.cuda.synchronize()
+    o, t0 = torch.zeros_like(want), time.perf_counter()
+    binding.efq_exact_attention_fwd_inject_timeout(q, k, v, o)
+    torch.cuda.synchronize()
+    assert time.perf_counter() - t0 < 3.0
+    assert torch.isnan(o).all()
+    assert torch.equal(binding.efq_exact_attention_fwd(q, k, v), want)
 
 
 def test_relative_error_is_the_frobenius_ratio():
