@@ -764,14 +764,16 @@ cudaError_t launch_one(dim3 grid, size_t smem, cudaStream_t stream, const CUtens
     return launch_overlapped(attention_fwd_kernel<PRODUCER, DEBUG>, grid, kThreads, smem, stream, mq, mk, mv, P);
 }
 
-// Short KV walks and more query tiles than SMs: persistent CTAs (the measurements are in attention_short.cuh).  The line is drawn
-// by the mean walk of a query tile, half of a causal square, where the gain is down to 1 or 2 %: 40 KV tiles for the affine rule,
-// 24 for its table form.  The exponential producers gain on long walks too; 128 tiles is as far as the plain forms (1, 2) do.
+// Short KV walks and more query tiles than SMs: persistent CTAs (the measurements are in attention_short.cuh).  The line lies where
+// both forms take the same time: 40 KV tiles for the affine rule, 16 for its table form, 64 for the plain exponentials (1, 2); the
+// folded ones gain at every length.  A [B, H, S, d] problem is judged by the mean walk of a query tile, half of a causal square, a
+// packed batch by its longest sequence: nothing up to the line is slower for it, though a batch of short sequences with one long
+// one would gain past it (63 of 64 to 500 tokens and one of 6000, causal: 530 -> 451 us for the affine rule).
 // P.Sk: the keys of the problem or, with P.Sq = 0, of the longest sequence.
 bool use_short(int producer, bool debug, int64_t items, int sms, const FwdParams& P)
 {
     if (debug || producer == 6 || P.packed || items <= sms) return false;
-    const int64_t tiles = producer == 0 ? 40 : producer == 3 ? 24 : producer <= 2 ? 128 : 1 << 24;
+    const int64_t tiles = producer == 0 ? 40 : producer == 3 ? 16 : producer <= 2 ? 64 : 1 << 24;
     const int64_t mean = P.causal ? P.Sk - std::min(P.Sq, P.Sk) / 2 : P.Sk;
     return mean <= tiles * kTile;
 }

@@ -8,14 +8,21 @@
 // tile counter t runs over all items of the CTA: it picks buffers and phases, the tile j inside the item picks the keys.
 // Everything else, the arithmetic above all, is that of attention_fwd_kernel, and so is the result, bit for bit.
 //
-// Why not for all shapes: in the steady state the looped form is 3 % slower.  Measured against the other kernel (whole
+// Why not for all shapes: in the steady state the looped form is 3 % slower.  Measured for the affine rule against the other kernel (whole
 // call, 24 heads, 16000 queries, not causal): 128 keys 153 -> 89 us, 256 keys 164 -> 111, 512 keys 195 -> 140, 1024 keys
 // 255 -> 211, 2048 keys 373 -> 342, 3072 keys 487 -> 459, 4096 keys 604 -> 583, 6144 keys 834 -> 827, 8192 keys 1064 -> 1070,
 // 16384 keys 1988 -> 2052.  Causal, 32 heads: 32 x 128 tokens 60 -> 39 us, 4 x 1024 tokens 74 -> 61, 2048 tokens 51 -> 46, 4096
 // tokens 133 -> 129, 8192 tokens 428 -> 421, 16384 tokens 1466 -> 1472.
-// The exponential producers gain at every length, their code generation hides what the loop costs: S = 2048 65 -> 58 us, 4096
-// 191 -> 182, 16384 2348 -> 2305; folded scale 56 -> 46, 157 -> 143, 1859 -> 1765.
-// Packed batches: 16 sequences of 100 to 3000 tokens 565 -> 513 us, 40 of 100 to 500 235 -> 188, 64 of 64 to 128 132 -> 94.
+// Packed batches, 32 / 8 heads: 64 sequences of 64 to 128 tokens 132 -> 94 us; 16 of 100 to 3000 343 -> 300 causal, 448 -> 420 not;
+// 16 of 500 to 5120 961 -> 884 and 1395 -> 1324; 8 x 5120 1590 -> 1504 and 2517 -> 2426.
+// The table form of the rule loses more in the loop.  24 heads, 8000 queries, not causal: 1024 keys 181 -> 164 us, 1536 238 -> 228, 2048
+// 296 -> 291, 3072 410 -> 416, 4096 524 -> 540; causal: 4096 tokens 205 -> 204, 8192 698 -> 708.  Packed: 8 x 2000 tokens 534 -> 521
+// causal, 797 -> 772 not; 16 of 100 to 2000 286 -> 265, 373 -> 369; 16 of 100 to 3000 448 -> 423 but 626 -> 637.
+// The plain exponentials (scale4; scale6 is the same within 1 %): causal S = 4096 195 -> 187 us, 8192 657 -> 637, 16384 2364 -> 2343,
+// 32768 8871 -> 8985; not causal, 24 heads, 8000 queries: 4096 keys 506 -> 481, 8192 932 -> 922, 12288 1354 -> 1358, 16384 1771 -> 1802.
+// Packed: 6 of 500 to 3000 tokens 340 -> 322 causal, 501 -> 479 not; 4 x 8192 2630 -> 2619, 4693 -> 4659; 4 x 16384 9435 -> 9581.
+// The folded ones gain at every length, their code generation hides what the loop costs: causal S = 4096 157 -> 143, 16384 1859 -> 1765,
+// 131072 103.3 -> 101.9 ms; 4 x 16384 tokens packed 7515 -> 7111 us; with the polynomial 131072 108.1 -> 105.7 ms.
 #pragma once
 
 struct __align__(1024) ShortSmem : Smem {
@@ -392,8 +399,8 @@ attention_short_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
             bool have_prev;
             float m_prev = -INFINITY;
             {
-                // the other group's publication and the maximum it carries are asked for while the scores travel
-                // (S = 131072: 78.2 ms, 79.3 with the maximum read after the scores)
+                // the other group's publication and the maximum it carries are asked for while the scores travel, as in
+                // attention_fwd_kernel
                 have_prev = t == 0 || ptx::mbar_try_wait(&sm->a_bar[(t - 1u) & 3u][quarter], ((t - 1u) >> 2) & 1u);
                 if (j > 0 && have_prev) m_prev = sm->runmax[sb ^ 1][row];
                 ptx::tmem_wait_ld();

@@ -21,6 +21,8 @@ pytestmark = pytest.mark.gpu
     (2, 16, 4, 700, 400, False, "etq0", 0.0), (2, 16, 4, 700, 400, False, "etq1", 0.0),
     (2, 16, 4, 700, 400, True, "etq2", 0.0), (2, 16, 4, 700, 400, False, "etq3", 0.0), (2, 16, 4, 700, 400, False, "etq4", 0.0),
     (1, 16, 4, 1300, 4000, True, "etq0", 0.0), (1, 16, 4, 1300, 4000, True, "etq2", 0.0), (2, 16, 4, 700, 400, True, "lut", 0.0), (1, 8, 2, 2600, 6400, True, "efq", 0.0),
+    (1, 8, 4, 2560, 2048, False, "lut", 0.0), (1, 8, 4, 2560, 2049, False, "lut", 0.0),          # at the lines of the other producers
+    (1, 8, 4, 2560, 8192, False, "etq0", 0.0), (1, 8, 4, 2560, 8193, False, "etq1", 0.0), (1, 8, 4, 2560, 9000, False, "etq2", 0.0),
 ])
 def test_short_walks_equal_one_cta_per_tile(oracle, B, Hq, Hkv, Sq, Sk, causal, producer, threshold):
     case = inputs.AttentionCase("short", B, Hq, Hkv, Sq, Sk, 128, causal, 600 + Sk, "k_outliers")
