@@ -478,6 +478,8 @@ attention_short_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
 
     ptx::tc_fence_before_sync();
     __syncthreads();
-    if (sm->abort_flag) __nanosleep(1000000u);      // loads may be in flight: a millisecond, before shared memory is another CTA's
-    if (warp == 1) ptx::tmem_dealloc(tmem, kTmemCols);
+    if (warp == 1) {
+        if (sm->abort_flag) __nanosleep(1000000u);  // loads may be in flight: a millisecond, before shared memory is another CTA's
+        ptx::tmem_dealloc(tmem, kTmemCols);
+    }
 }
