@@ -112,7 +112,7 @@ efq_status_t efq_probgen(const float* scores, int64_t ld, const float* row_max, 
  * with scale_mode 0 except at rounding knife-edges.
  * scale_mode 3 is scale_mode 2 with 2 of every 8 exponentials computed on the FMA pipe (floor, cubic polynomial
  * of the fraction with relative error 8.6e-5, exponent insertion) to take load off the exponential unit.  Measured
- * on B200 it gains 3 % in the register-resident stage and loses 6 % in the fused forward, where issue slots and
+ * on B200 it loses 6 % in the register-resident stage and 4 % in the fused forward, where issue slots and
  * not the exponential unit are short; it is kept as the record of that comparison.  Codes differ from
  * scale_mode 0 on a few elements in ten thousand (the polynomial's error against the E2M1 rounding step). */
 efq_status_t exp_then_quantize_probgen(const float* scores, int64_t ld, const float* row_max, int64_t rows,
