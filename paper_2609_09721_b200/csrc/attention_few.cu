@@ -577,7 +577,8 @@ __global__ void __launch_bounds__(128) few_merge_kernel(const __grid_constant__ 
         const float4 x = __ldcg(part + static_cast<int64_t>(c) * part_step);
         const float4 lp = __ldcg(reinterpret_cast<const float4*>(stat + c * stat_step));
         const float lc = (lp.x + lp.y) + (lp.z + lp.w);
-        const float w = m == -INFINITY ? 0.0f : ex2_approx(__fmul_rn(__fsub_rn(m, m_last), P.K.LOG2E));
+        // equal maxima by comparison: both are infinite where the inputs or a score overflowed
+        const float w = m == -INFINITY ? 0.0f : m == m_last ? 1.0f : ex2_approx(__fmul_rn(__fsub_rn(m, m_last), P.K.LOG2E));
         l = fmaf(lc, w, l);
         a.x = fmaf(x.x, w, a.x); a.y = fmaf(x.y, w, a.y); a.z = fmaf(x.z, w, a.z); a.w = fmaf(x.w, w, a.w);
     }

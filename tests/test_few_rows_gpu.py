@@ -79,6 +79,34 @@ def test_inputs_at_a_16_byte_boundary(S, Hq, Hkv):
     assert torch.equal(binding.efq_attention_fwd(q, k, v, True), binding.efq_attention_fwd(q2, k2, v2, True))
 
 
+@pytest.mark.parametrize("B,Hq,Hkv,Sq,Sk", [(1, 4, 4, 1, 700), (1, 8, 2, 3, 1300), (2, 2, 2, 24, 500)])
+@pytest.mark.parametrize("value", [float("inf"), float("-inf"), float("nan"), 3.38e38])
+@pytest.mark.parametrize("where", ["q", "k", "v"])
+def test_non_finite_inputs_as_on_the_general_path(B, Hq, Hkv, Sq, Sk, value, where):
+    """Infinities, NaN and the largest values (whose scores overflow): the row maximum is infinite from some tile on, and the
+    chunks add up as on the general path, which the two-call form always takes.  Both add FP32 numbers in different orders:
+    2^-23 per addition of a tile, below 1e-5 of the row's largest value."""
+    g = torch.Generator(device="cuda").manual_seed(Sk)
+    t = {"q": torch.randn(B, Hq, Sq, 128, generator=g, device="cuda").bfloat16(),
+         "k": torch.randn(B, Hkv, Sk, 128, generator=g, device="cuda").bfloat16(),
+         "v": torch.randn(B, Hkv, Sk, 128, generator=g, device="cuda").bfloat16()}
+    x = t[where].view(-1)
+    if where == "v":
+        value = min(max(value, -1e30), 1e30) if value == value else 1e30     # larger ones overflow in one order of the sum and not in another
+    x[torch.randint(0, x.numel(), (max(1, x.numel() // 2000),), generator=g, device="cuda")] = value
+    q, k, v = t["q"], t["k"], t["v"]
+    shape = (B, Hq, Hkv, Sq, Sk, 128)
+    ws = torch.empty(binding.efq_attention_workspace_bytes(*shape), dtype=torch.uint8, device="cuda")
+    for causal in (False, True):
+        for producer in (0, 1, 4):
+            got = binding.exp_then_quantize_attention_fwd(q, k, v, causal, 0.0, {1: 0, 4: 2}[producer]) if producer else binding.efq_attention_fwd(q, k, v, causal)
+            binding.efq_quantize_qkv(q, k, v, ws)
+            want = binding.efq_attention_fwd_quantized(torch.empty_like(got), shape, ws, causal, 0.0, producer)
+            assert torch.isfinite(want).all()
+            scale = want.abs().amax(dim=-1, keepdim=True)
+            assert ((got - want).abs() <= 1e-5 * scale).all(), (causal, producer)
+
+
 def test_rows_past_two_to_the_31_scores():
     """24 rows on 98 million keys: the scores of rows 22 and 23 start past 2^31.  Every row asks the same, so every row answers
     what one row by itself does, bit for bit (both lengths of context are cut into the same chunks)."""
