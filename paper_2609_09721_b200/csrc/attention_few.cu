@@ -317,7 +317,7 @@ __device__ __forceinline__ uint32_t key_code(float r, float par, const ProducerC
         return cvt_e2m1x2(e, 0.0f) & 15u;
     } else {
         p = ex2_approx(__fmul_rn(__fsub_rn(__fmul_rn(K.sigma, r), par), K.LOG2E));
-        const float amax = warp_max(p);
+        const float amax = fmaxf(warp_max(p), 0.0f);      // a row without a finite score has NaN everywhere: 0
         if (amax == 0.0f) { byte = 0u; return 0u; }
         const uint32_t bits = __float_as_uint(amax);
         const int E = static_cast<int>((bits >> 23) & 0xffu) - 127;

@@ -11,7 +11,8 @@ from test_attention_gpu import MEAN, TOL_O, _all_rows, _case_tensors, _check_dum
 pytestmark = pytest.mark.gpu
 
 # producer: (oracle path, tolerance)
-PRODUCERS = {"efq": ("efq", TOL_O), "lut": ("efq_lut", TOL_O), "etq0": ("etq", 5e-3), "etq1": ("etq6", 5e-3), "etq2": ("etq", 5e-3)}
+PRODUCERS = {"efq": ("efq", TOL_O), "lut": ("efq_lut", TOL_O), "etq0": ("etq", 5e-3), "etq1": ("etq6", 5e-3), "etq2": ("etq", 5e-3),
+             "etq3": ("etq", 5e-3), "etq4": ("etq_fp32den", 5e-3)}
 
 
 def _forward(dq, dk, dv, causal, producer, threshold=0.0, debug=None):
@@ -26,6 +27,8 @@ def _forward(dq, dk, dv, causal, producer, threshold=0.0, debug=None):
     (1, 1, 17, 4095, True, "efq", 0.0), (8, 1, 3, 4097, False, "efq", 0.0), (1, 1, 24, 16, True, "efq", 0.0),   # 17, 24, 24 rows
     (5, 1, 5, 1500, True, "efq", 0.0),                                                                        # 25 rows: the general path
     (8, 2, 1, 16385, True, "efq", 0.0), (6, 2, 2, 1793, True, "efq", 2.0),
+    (4, 1, 5, 2, True, "lut", 0.0), (4, 1, 5, 2, True, "etq0", 0.0), (4, 1, 5, 2, True, "etq1", 0.0),           # three queries see nothing
+    (4, 1, 5, 2, True, "etq2", 0.0), (4, 1, 5, 2, True, "etq3", 0.0), (4, 1, 5, 2, True, "etq4", 0.0), (1, 1, 24, 20, True, "etq0", 0.0),
     (8, 2, 1, 1025, True, "lut", 0.0), (3, 1, 7, 600, True, "etq0", 0.0), (8, 2, 1, 2100, False, "etq1", 0.0), (4, 1, 6, 333, True, "etq2", 0.0),
 ])
 def test_few_rows_against_the_oracle(oracle, Hq, Hkv, Sq, Sk, causal, producer, threshold):
