@@ -264,7 +264,8 @@ efq_status_t efq_attention_fwd_static(const void* q, const void* k, const void* 
  * operand anywhere): O = softmax(scale Q K^T + mask) V, online over the keys, exponentials by expf.  This is the
  * reference output O_ref of the calibration objective and the "exact" side of the error figures; on the
  * tensor cores, with bf16 products that are exact in FP32 and probabilities split into three bf16 terms.  Arguments as for
- * efq_attention_fwd (no workspace); B * Hq <= 65535.  Rows of a block in which a bounded device-side wait expired are NaN. */
+ * efq_attention_fwd (no workspace); B * Hq <= 65535.  Rows of a block in which a bounded device-side wait expired are NaN.
+ * V has to be finite: an infinity or NaN in it makes NaN of its channel in every row whose 128-key tile holds it. */
 efq_status_t efq_exact_attention_fwd(const void* q, const void* k, const void* v, float* o, int B, int Hq, int Hkv,
                                      int64_t Sq, int64_t Sk, int d, int causal, float softmax_scale, void* stream);
 

@@ -1,8 +1,8 @@
 """Python binding of libefq_b200.so: same names as the C ABI in include/efq.h.
 
-Argument marshalling only: ctypes, and for the calls of a serving loop the CPython extension efq_fastcall.  Tensors are torch CUDA tensors (torch is used for device
-memory and streams); nothing here computes.  There is no CPU fallback: if the library
-has not been built, or a call returns a non-zero status, a RuntimeError is raised.
+Argument marshalling only: ctypes, and for the calls of a serving loop the CPython extension efq_fastcall.  Tensors are
+torch CUDA tensors (torch is used for device memory and streams); nothing here computes.  There is no CPU fallback: if the
+library has not been built, or a call returns a non-zero status, a RuntimeError is raised.
 """
 from __future__ import annotations
 
@@ -309,7 +309,8 @@ def efq_attention_fwd_varlen(q, k, v, cu_seqlens_q, cu_seqlens_k, causal: bool =
     fast = _fast or _fastcall()
     if workspace is None:
         nbytes = fast.varlen(cu_seqlens_q, cu_seqlens_k, total_q, total_k, Hq, Hkv, d, None, 0, 0, 0, 0, 0.0, 0, 0, 0, 0, 0)
-        if nbytes <= 0:
+        assert nbytes != -1, "the prefix sums do not fit the tensors"
+        if nbytes == 0:
             raise EfqError(1, "efq_attention_varlen_workspace_bytes")
         workspace = torch.empty(nbytes, dtype=torch.uint8, device=q.device)
     o = torch.empty((total_q, Hq, d), dtype=torch.float32, device=q.device)

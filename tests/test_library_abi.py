@@ -7,6 +7,7 @@ import threading
 import time
 
 import pytest
+import torch
 
 from paper_2609_09721_b200 import binding, build
 
@@ -151,3 +152,12 @@ def test_calls_do_not_hold_the_interpreter_lock(tmp_path):
         thread.join()
         binding._fast = None
         binding._fastcall()             # the library's own functions again
+
+
+@pytest.mark.parametrize("cu_q,cu_k", [([0, 4], [0, 9]), ([0, 5], [0, 8]), ([0, 2, 5], [0, 9]), ([0, 5], [0, 4, 9])])
+@pytest.mark.parametrize("workspace", [None, torch.empty(64, dtype=torch.uint8)])
+def test_prefix_sums_that_do_not_fit_the_tensors_are_an_assertion(cu_q, cu_k, workspace):
+    """Found by the binding before the library is called, with a workspace of the caller's or without."""
+    q, k = torch.empty(5, 2, 128, dtype=torch.bfloat16), torch.empty(9, 2, 128, dtype=torch.bfloat16)
+    with pytest.raises(AssertionError, match="prefix sums"):
+        binding.efq_attention_fwd_varlen(q, k, k, cu_q, cu_k, workspace=workspace, stream=0)
