@@ -180,8 +180,9 @@ efq_status_t efq_attention_fwd_quantized(float* o, int B, int Hq, int Hkv, int64
  * quantised by themselves, so the result of a sequence equals efq_attention_fwd on that sequence alone, bit for
  * bit.  A sequence without queries is skipped; one without keys gets zero rows.  `producer` as for
  * efq_attention_fwd_quantized.
- * The whole batch takes at most five kernel launches on `stream` whatever the number of sequences.  The sequences with at
- * most 24 query rows a KV head (Hq / Hkv * len_q: decode steps) take three that read K and V as they are; the others take two:
+ * The whole batch takes at most five kernel launches on `stream` whatever the number of sequences.  The sequences with few
+ * query rows a KV head (Hq / Hkv * len_q: at most 16, 24 from 8065 keys on: decode steps) take three that read K
+ * and V as they are; the others take two:
  * one operand preparation over all of them (each quantised on its own: V blocks of 32 keys are aligned to the sequence's own key index)
  * and one fused forward whose work items come from a table in the workspace.  A sequence with so few query tokens
  * that the query heads of a KV group fit into one 128-row tile (Hq / Hkv * len_q <= 128: decode steps, short
@@ -314,7 +315,7 @@ efq_status_t efq_stage_microbench(int producer, const efq_params_t* params, int 
                                   long long* cycles, void* stream);
 
 /* Test hook for the bounded-wait path (no GPU fault is involved): efq_attention_fwd, on the kernels that the shape takes there,
- * with the K/V loads left out - for at most 24 query rows a KV head, whose kernels load by themselves, the MMAs - so that the
+ * with the K/V loads left out - on the path for few query rows, whose kernels load by themselves, the MMAs - so that the
  * first device-side wait on them runs out after its limit (under a second).  Every role then
  * drains, tensor memory is released, the kernel returns normally and the status word reads
  * EFQ_ERR_DEVICE_TIMEOUT through efq_poll_status(); `o` is undefined.  The context stays usable and the next

@@ -705,7 +705,7 @@ struct Workspace {
 
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
-bool use_few(int Hq, int Hkv, int64_t Sq);
+bool use_few(int Hq, int Hkv, int64_t Sq, int64_t Sk);
 int64_t few_chunks(int64_t Sk, int64_t rows);
 
 Workspace plan_workspace(int B, int Hq, int Hkv, int64_t Sq, int64_t Sk)
@@ -729,7 +729,7 @@ Workspace plan_workspace(int B, int Hq, int Hkv, int64_t Sq, int64_t Sk)
 size_t workspace_bytes_for(int B, int Hq, int Hkv, int64_t Sq, int64_t Sk)
 {
     size_t total = plan_workspace(B, Hq, Hkv, Sq, Sk).total;
-    if (use_few(Hq, Hkv, Sq)) {
+    if (use_few(Hq, Hkv, Sq, Sk)) {
         const int64_t heads = static_cast<int64_t>(B) * Hkv;
         const size_t few = 1024 + plan_few(heads * few_chunks(Sk, Hq / Hkv * Sq), heads * ((Sk + kTile - 1) / kTile * kTile),
                                            static_cast<int>(Hq / Hkv * Sq)).total;
@@ -823,10 +823,10 @@ cudaError_t launch_main(bool debug, dim3 grid, size_t smem, cudaStream_t stream,
 // the unpacked one bit for bit.
 bool use_packed_tile(int Hq, int Hkv, int64_t Sq) { return Hq / Hkv > 1 && static_cast<int64_t>(Hq / Hkv) * Sq <= kTile; }
 
-// At most kFewMaxRows query rows per KV group: K and V are read once whatever the kernel does, so the path that quantises
-// them on the way to the tensor core takes over (attention_few.cu).  Depends on the sequence's own shape alone, so that a
-// sequence takes the same path by itself and in a packed batch.
-bool use_few(int Hq, int Hkv, int64_t Sq) { return static_cast<int64_t>(Hq / Hkv) * Sq <= kFewMaxRows; }
+// Few query rows per KV group: K and V are read once whatever the kernel does, so the path that quantises them on the way to
+// the tensor core takes over (attention_few.cu; the line and its measurements: few_takes).  Depends on the sequence's own shape
+// alone, so that a sequence takes the same path by itself and in a packed batch.
+bool use_few(int Hq, int Hkv, int64_t Sq, int64_t Sk) { return few_takes(static_cast<int64_t>(Hq / Hkv) * Sq, (Sk + kTile - 1) / kTile); }
 
 int64_t few_chunks(int64_t Sk, int64_t rows)
 {
@@ -898,7 +898,7 @@ efq_status_t attention_impl(const void* q, const void* k, const void* v, float* 
 
     uint8_t* ws = static_cast<uint8_t*>(workspace);
     const int G = Hq / Hkv;
-    if (do_quantize && do_forward && use_few(Hq, Hkv, Sq)) {
+    if (do_quantize && do_forward && use_few(Hq, Hkv, Sq, Sk)) {
         FewParams F{};
         F.q = static_cast<const __nv_bfloat16*>(q); F.k = static_cast<const __nv_bfloat16*>(k); F.v = static_cast<const __nv_bfloat16*>(v);
         F.o = o;
@@ -1003,7 +1003,7 @@ bool plan_varlen(const int64_t* cu_q, const int64_t* cu_k, int n_seqs, int Hq, i
         const int64_t lq = cu_q[s + 1] - cu_q[s], lk = cu_k[s + 1] - cu_k[s];
         if (lq < 0 || lk < 0) { st = EFQ_ERR_INVALID_ARG; return false; }
         if (lq == 0 || lk == 0) continue;
-        if (use_few(Hq, Hkv, lq)) {
+        if (use_few(Hq, Hkv, lq, lk)) {
             ++p.n_few;
             p.few_rows = std::max(p.few_rows, static_cast<int>(Hq / Hkv * lq));
             p.few_units += few_chunks(lk, Hq / Hkv * lq) * Hkv;
@@ -1333,7 +1333,7 @@ extern "C" efq_status_t efq_attention_fwd_varlen(const void* q, const void* k, c
             if (cudaMemsetAsync(o + q0 * Hq * 128, 0, static_cast<size_t>(lq) * Hq * 128 * sizeof(float), s) != cudaSuccess) return EFQ_ERR_CUDA;
             continue;
         }
-        if (use_few(Hq, Hkv, lq)) {
+        if (use_few(Hq, Hkv, lq, lk)) {
             few_seqs[f++] = FewSeq{static_cast<int32_t>(lq), static_cast<int32_t>(lk), static_cast<int32_t>(q0), static_cast<int32_t>(k0),
                                    static_cast<int32_t>(few_key), static_cast<int32_t>(few_unit)};
             few_key += (lk + kTile - 1) / kTile * kTile;

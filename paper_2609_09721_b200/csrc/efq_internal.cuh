@@ -92,9 +92,22 @@ struct ItemDesc {
 };
 
 // ------------------------------------------------------------------------------------------------
-// Few query rows (attention_few.cu): the query rows of a KV group, Hq / Hkv * Sq of them, are at most kFewMaxRows
+// Few query rows (attention_few.cu): the query rows of a KV group are Hq / Hkv * Sq
 // ------------------------------------------------------------------------------------------------
 constexpr int kFewMaxRows = 24;
+// The contexts that take it, by the sequence's own shape: up to 16 rows all, 17 to 24 rows from 64 KV tiles on.  Its time grows with
+// the rows (each has its codes made and its scores written for itself), that of the general path does not up to 128; but the
+// general path walks a whole context in one CTA a KV head.  Measured, this path against the general one, us, with 1 / 64 / 256 KV heads:
+//    8 rows: 1000 keys 11.7 / 20.4 / - against 13.5 / 18.7 / -, 4000 keys 19.7 / 43.5 / - against 29.9 / 52.9 / -
+//   16 rows: 1000 keys 15.5 / 23.3 / 58 against 13.3 / 18.8 / 48; 2000 keys 15.7 / 35 / 101 against 19.1 / 29 / 84; 4000 keys 38 / 62 / 159
+//            against 30 / 53 / 155; 8000 keys 39 / 93 / 292 against 51 / 99 / 289; 16000 keys 40 / 154 / 561 against 92 / 189 / 563
+//   24 rows: 1000 keys 19.2 / 29.5 / 75 against 13.5 / 18.9 / 49; 2000 keys 19.8 / 45 / 130 against 19.3 / 29 / 84; 3000 keys 20.2 / 56 / 192
+//            against 24.9 / 41 / 119; 4000 keys 51 / 80 / 218 against 31 / 54 / 155; 8000 keys 52 / 124 / 385 against 52 / 100 / 289;
+//            16000 keys 53 / 214 / 746 against 92 / 189 / 561
+// The number of heads and sequences must not matter to the line (a sequence gives the same bits alone and in a batch).  Up to 16
+// rows the gains of a few long contexts outweigh a loss of a fifth in wide batches of short ones; above, the line lies where a few
+// heads begin to gain.
+__host__ __device__ inline bool few_takes(int64_t rows, int64_t n_tiles) { return rows <= 16 || (rows <= kFewMaxRows && n_tiles >= 64); }
 // Tiles of a chunk of the KV range, by the sequence's own shape: short contexts are cut finely, so that one of them spreads
 // over the chip; with many rows a chunk's partial result (544 bytes a row) has to be small against its 64 KB of K and V a tile.
 constexpr int kFewMaxChunk = 8;
@@ -109,8 +122,7 @@ static_assert(few_row_offset(kFewMaxRows - 2, 100000000) == 2200000000ll, "rows 
 // A chunk's partial result: the 128 values of a row's O^T take the place of the row's scores of the chunk's first tile, which
 // nobody reads any more by then; beside them, per row, four parts of the denominator, the maximum they refer to, three unused.
 // So a KV head needs rows * (528 tiles + 32 chunks) bytes, at 24 rows and a tile a chunk 13440 a tile: less than the 17408 of the
-// MXFP4 copies of K and V, and what fits a workspace on the general path fits it here.  (With O^T in a place of its own, 544
-// bytes a row and chunk, 22 to 24 rows below 32 tiles did not; longer chunks would fit, and take 29 us instead of 20 there.)
+// MXFP4 copies of K and V, and what fits a workspace on the general path fits it here.
 constexpr int kFewStatFloats = 8;
 constexpr int kFewInlineSeqs = 128;      // sequence tables up to this size travel as kernel parameters
 

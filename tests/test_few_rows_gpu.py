@@ -27,8 +27,11 @@ def _forward(dq, dk, dv, causal, producer, threshold=0.0, debug=None):
     (1, 1, 17, 4095, True, "efq", 0.0), (8, 1, 3, 4097, False, "efq", 0.0), (1, 1, 24, 16, True, "efq", 0.0),   # 17, 24, 24 rows
     (5, 1, 5, 1500, True, "efq", 0.0),                                                                        # 25 rows: the general path
     (8, 2, 1, 16385, True, "efq", 0.0), (6, 2, 2, 1793, True, "efq", 2.0),
-    (4, 1, 5, 2, True, "lut", 0.0), (4, 1, 5, 2, True, "etq0", 0.0), (4, 1, 5, 2, True, "etq1", 0.0),           # three queries see nothing
-    (4, 1, 5, 2, True, "etq2", 0.0), (4, 1, 5, 2, True, "etq3", 0.0), (4, 1, 5, 2, True, "etq4", 0.0), (1, 1, 24, 20, True, "etq0", 0.0),
+    (2, 1, 4, 1, True, "lut", 0.0), (2, 1, 4, 1, True, "etq0", 0.0), (2, 1, 4, 1, True, "etq1", 0.0),           # three queries see nothing
+    (2, 1, 4, 1, True, "etq2", 0.0), (2, 1, 4, 1, True, "etq3", 0.0), (2, 1, 4, 1, True, "etq4", 0.0), (1, 1, 8, 3, True, "etq0", 0.0),
+    (2, 1, 8, 3968, True, "efq", 0.0), (2, 1, 8, 3969, True, "etq2", 0.0), (1, 1, 9, 600, True, "lut", 0.0),      # 16 rows: chunks of 2 and 8 tiles
+    (8, 1, 3, 8064, False, "efq", 0.0), (1, 1, 17, 8065, True, "efq", 0.0), (8, 1, 3, 8193, False, "lut", 0.0),   # the line for 17 to 24 rows
+    (3, 1, 7, 8300, True, "etq0", 0.0), (4, 1, 6, 9000, True, "etq1", 0.0), (1, 1, 24, 8192, True, "etq4", 0.0),
     (8, 2, 1, 1025, True, "lut", 0.0), (3, 1, 7, 600, True, "etq0", 0.0), (8, 2, 1, 2100, False, "etq1", 0.0), (4, 1, 6, 333, True, "etq2", 0.0),
 ])
 def test_few_rows_against_the_oracle(oracle, Hq, Hkv, Sq, Sk, causal, producer, threshold):
@@ -48,15 +51,16 @@ def test_few_rows_against_the_oracle(oracle, Hq, Hkv, Sq, Sk, causal, producer, 
     if causal and Sq > Sk:                      # queries before the first key see nothing
         assert np.all(got.reshape(Hq, Sq, 128)[:, : Sq - Sk] == 0.0)
     else:
-        _check_dump(oracle, case, dump, _all_rows(case, head, 0, Sq), MEAN, producer=path, threshold=threshold)
+        _check_dump(oracle, case, dump, _all_rows(case, head, 0, Sq), MEAN, producer=path.replace("_fp32den", ""), threshold=threshold)
 
 
-@pytest.mark.parametrize("n_seqs", [128, 129])
-def test_packed_batch_of_few_row_sequences(n_seqs):
-    """128 sequences are described in the launch itself, more in device memory: each equals its forward alone bit for bit."""
+@pytest.mark.parametrize("n_seqs,tokens", [(128, 12), (129, 12), (128, 4), (129, 4)])
+def test_packed_batch_of_few_row_sequences(n_seqs, tokens):
+    """128 sequences of few rows (4 tokens: up to 8) are described in the launch itself, more in device memory; of those with up to
+    12 tokens some go the general way beside them.  Each equals its forward alone bit for bit."""
     Hq, Hkv = 4, 2
     g = torch.Generator(device="cuda").manual_seed(7)
-    lens = [(1 + n % 12, 1 + (37 * n) % 700) for n in range(n_seqs)]
+    lens = [(1 + n % tokens, 1 + (37 * n) % 700) for n in range(n_seqs)]
     cu_q = np.concatenate([[0], np.cumsum([a for a, _ in lens])])
     cu_k = np.concatenate([[0], np.cumsum([b for _, b in lens])])
     q = torch.randn(int(cu_q[-1]), Hq, 128, generator=g, device="cuda").bfloat16()
@@ -82,7 +86,7 @@ def test_inputs_at_a_16_byte_boundary(S, Hq, Hkv):
     assert torch.equal(binding.efq_attention_fwd(q, k, v, True), binding.efq_attention_fwd(q2, k2, v2, True))
 
 
-@pytest.mark.parametrize("B,Hq,Hkv,Sq,Sk", [(1, 4, 4, 1, 700), (1, 8, 2, 3, 1300), (2, 2, 2, 24, 500)])
+@pytest.mark.parametrize("B,Hq,Hkv,Sq,Sk", [(1, 4, 4, 1, 700), (1, 8, 2, 3, 1500), (2, 2, 2, 24, 8100)])
 @pytest.mark.parametrize("value", [float("inf"), float("-inf"), float("nan"), 3.38e38])
 @pytest.mark.parametrize("where", ["q", "k", "v"])
 def test_non_finite_inputs_as_on_the_general_path(B, Hq, Hkv, Sq, Sk, value, where):

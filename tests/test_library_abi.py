@@ -104,12 +104,12 @@ def test_few_row_shapes_need_no_more_workspace_than_the_general_path():
                 for Sk in list(range(64, 6000, 128)) + [129, 8192, 16383, 60001]:
                     assert size(1, G * Hkv, Hkv, Sq, Sk, 128) == _mxfp4_bytes(1, G * Hkv, Hkv, Sq, Sk), (G, Sq, Hkv, Sk)
     assert size(3, 8, 8, 24, 777, 128) == _mxfp4_bytes(3, 8, 8, 24, 777)
-    # at the edge of the built-in scratch, where 22 to 24 rows a KV head did not fit
+    # at the edge of the built-in scratch
     for Hq, Hkv, Sq, Sk in ((32, 8, 6, 3400), (24, 24, 24, 1100), (65, 65, 24, 300)):
         assert size(1, Hq, Hkv, Sq, Sk, 128) <= binding.STATIC_SCRATCH_BYTES
 
 
-@pytest.mark.parametrize("lens", [[(24, 1900)] + [(1, 1900)] * 63, [(24, 100)] + [(1, 128)] * 200, [(1 + n % 24, 1 + 37 * n) for n in range(150)]])
+@pytest.mark.parametrize("lens", [[(24, 8100)] + [(1, 1900)] * 63, [(16, 1500)] + [(1, 128)] * 200, [(1 + n % 24, 1 + 137 * n) for n in range(150)]])
 def test_few_row_sequences_of_a_packed_batch_take_no_more_than_their_copies(lens):
     """The size of a packed batch is that of its sequences (MXFP4 copies, which the path for few rows stays below), also where a
     sequence of 24 rows among sequences of one row makes room for 24 rows in each."""
@@ -117,7 +117,7 @@ def test_few_row_sequences_of_a_packed_batch_take_no_more_than_their_copies(lens
     cu_q = [sum(a for a, _ in lens[:i]) for i in range(len(lens) + 1)]
     cu_k = [sum(b for _, b in lens[:i]) for i in range(len(lens) + 1)]
     copies = sum(Hkv * (128 + 2 * _round_up(lk, 128)) * 68 for _, lk in lens)
-    assert _varlen_bytes(cu_q, cu_k, Hkv, Hkv) <= copies + 32 * len(lens) + 16384
+    assert _varlen_bytes(cu_q, cu_k, Hkv, Hkv) <= copies + 1024 * len(lens) + 16384        # a table entry each on the general path
 
 
 def test_calls_do_not_hold_the_interpreter_lock(tmp_path):

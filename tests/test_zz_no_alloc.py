@@ -56,9 +56,9 @@ def test_static_entry_applies_the_argument_rules_of_the_regular_forward():
     assert e.value.status == binding.STATUS_NAMES.index("EFQ_ERR_INVALID_ARG")
 
 
-@pytest.mark.parametrize("Hq,Hkv,Sq,Sk", [(32, 8, 6, 3400), (24, 24, 24, 1100)])
+@pytest.mark.parametrize("Hq,Hkv,Sq,Sk", [(32, 8, 6, 3400), (24, 24, 24, 1100), (3, 3, 24, 8100), (16, 8, 8, 3500)])
 def test_static_scratch_takes_few_row_shapes_at_its_edge(Hq, Hkv, Sq, Sk):
-    """24 query rows a KV head on the path for few rows: the largest part of the scratch per key."""
+    """The largest shapes of few query rows that fit: 24 rows a KV head on the general path and on the one for few rows, 16 rows there."""
     g = torch.Generator(device="cuda").manual_seed(5)
     q = torch.randn(1, Hq, Sq, 128, generator=g, device="cuda").bfloat16()
     k, v = (torch.randn(1, Hkv, Sk, 128, generator=g, device="cuda").bfloat16() for _ in range(2))
