@@ -219,13 +219,13 @@ __global__ void __launch_bounds__(kFewThreads, N <= 8 ? 4 : 3) few_scores_kernel
     __syncthreads();
     ptx::tc_fence_after_sync();
     const uint32_t tmem = sm->tmem_base;
-    const int nblk = u.Sk_pad / 32;
+    const int n_tiles = u.Sk_pad / kTile, nblk = 4 * n_tiles;
     const int quarter = warp & 3, half = warp >> 2;      // 32 keys of the tile; rows 2 i + half
     // last visible key of row `lane`
     const int limit = min(P.causal ? lane % u.Sq + u.Sk - u.Sq : u.Sk, u.Sk - 1);
 
-    float* dst = P.scores + u.s_off + few_row_offset(half, u.Sk_pad) + u.j0 * kTile + quarter * 32 + lane;
-    float* dst_max = P.block_max + u.s_off / 32 + few_row_offset(half, nblk) + u.j0 * 4 + quarter;
+    float* dst = P.scores + u.s_off + few_row_offset(half, n_tiles) + u.j0 * kTile + quarter * 32 + lane;
+    float* dst_max = P.block_max + u.s_off / 32 + half * nblk + u.j0 * 4 + quarter;
     // raw scores of a finished tile: thread = key, two rows of the half side by side
     auto put_scores = [&](int j) {
         const int buf = (j - u.j0) & 1;
@@ -243,11 +243,11 @@ __global__ void __launch_bounds__(kFewThreads, N <= 8 ? 4 : 3) few_scores_kernel
                 const float x0 = key <= __shfl_sync(0xffffffffu, limit, row) ? (half ? s[i + 1] : s[i]) : -INFINITY;
                 const float x1 = key <= __shfl_sync(0xffffffffu, limit, row + 2) ? (half ? s[i + 3] : s[i + 2]) : -INFINITY;
                 const float m0 = warp_max(x0), m1 = warp_max(x1);
-                dst[few_row_offset(i, u.Sk_pad)] = x0;
-                if (row + 2 < R) dst[few_row_offset(i + 2, u.Sk_pad)] = x1;
+                dst[few_row_offset(i, n_tiles)] = x0;
+                if (row + 2 < R) dst[few_row_offset(i + 2, n_tiles)] = x1;
                 if (lane == 0) {
-                    dst_max[few_row_offset(i, nblk)] = m0;
-                    if (row + 2 < R) dst_max[few_row_offset(i + 2, nblk)] = m1;
+                    dst_max[i * nblk] = m0;
+                    if (row + 2 < R) dst_max[(i + 2) * nblk] = m1;
                 }
             }
         }
@@ -406,16 +406,16 @@ __global__ void __launch_bounds__(kFewThreads, 3) few_values_kernel(const __grid
 
     // the chunk's block maxima and the running maximum of every row before the chunk
     const float* const bm = P.block_max + u.s_off / 32;
-    const int nblk = u.Sk_pad / 32;
+    const int n_tiles = u.Sk_pad / kTile, nblk = 4 * n_tiles;
     for (int i = tid; i < R * (u.j1 - u.j0); i += kFewThreads) {
         const int t = i / R, row = i - t * R;
-        sm->bmax[t][row] = __ldcg(reinterpret_cast<const float4*>(bm + few_row_offset(row, nblk)) + u.j0 + t);
+        sm->bmax[t][row] = __ldcg(reinterpret_cast<const float4*>(bm + row * nblk) + u.j0 + t);
     }
     if (!(P.rescale_threshold > 0.0f)) {
         for (int row = warp; row < R; row += 8) {
             float m = -INFINITY;
             for (int b = lane; b < u.j0; b += 32) {
-                const float4 x = __ldcg(reinterpret_cast<const float4*>(bm + few_row_offset(row, nblk)) + b);
+                const float4 x = __ldcg(reinterpret_cast<const float4*>(bm + row * nblk) + b);
                 m = fmaxf(fmaxf(m, fmaxf(x.x, x.y)), fmaxf(x.z, x.w));
             }
             m = warp_max(m);
@@ -424,7 +424,7 @@ __global__ void __launch_bounds__(kFewThreads, 3) few_values_kernel(const __grid
     } else if (tid < R) {                    // optional policy: the kept maximum depends on the order of the tiles
         float m = -INFINITY;
         for (int j = 0; j < u.j0; ++j) {
-            const float4 b = __ldcg(reinterpret_cast<const float4*>(bm + few_row_offset(tid, nblk)) + j);
+            const float4 b = __ldcg(reinterpret_cast<const float4*>(bm + tid * nblk) + j);
             const float c = fmaxf(m, fmaxf(fmaxf(b.x, b.y), fmaxf(b.z, b.w)));
             if (m == -INFINITY || __fsub_rn(__fmul_rn(P.K.sigma, c), __fmul_rn(P.K.sigma, m)) > P.rescale_threshold) m = c;
         }
@@ -433,11 +433,11 @@ __global__ void __launch_bounds__(kFewThreads, 3) few_values_kernel(const __grid
     // Codes: thread = key of block `quarter`; the warps of a half take the rows 2 i + half.  O^T: thread = channel.
     constexpr int NH = N / 2;
     const int quarter = warp & 3, half = warp >> 2;
-    const float* s_src = P.scores + u.s_off + few_row_offset(half, u.Sk_pad) + u.j0 * kTile + quarter * 32 + lane;
+    float* s_src = P.scores + u.s_off + few_row_offset(half, n_tiles) + u.j0 * kTile + quarter * 32 + lane;
     float x[NH];
     auto load_scores = [&]() {
 #pragma unroll
-        for (int i = 0; i < NH; ++i) x[i] = 2 * i + half < R ? __ldcg(s_src + few_row_offset(2 * i, u.Sk_pad)) : -INFINITY;
+        for (int i = 0; i < NH; ++i) x[i] = 2 * i + half < R ? __ldcg(s_src + few_row_offset(2 * i, n_tiles)) : -INFINITY;
         s_src += kTile;
     };
     load_scores();
@@ -536,10 +536,10 @@ __global__ void __launch_bounds__(kFewThreads, 3) few_values_kernel(const __grid
 
     // ---- partial result of the chunk.  Its scores may go: the block's threads used the last of them before the barrier of the last
     // tile, and no other block reads them.
-    float* const part = P.scores + u.s_off + few_row_offset(half, u.Sk_pad) + u.j0 * kTile + quarter * 32 + lane;
+    float* const part = s_src - (u.j1 - u.j0) * kTile;          // it has gone past the chunk's tiles
 #pragma unroll
     for (int i = 0; i < NH; ++i)
-        if (2 * i + half < R) part[few_row_offset(2 * i, u.Sk_pad)] = acc[i];
+        if (2 * i + half < R) part[few_row_offset(2 * i, n_tiles)] = acc[i];
     if (has_row) {
         float* const stat = P.stats + (static_cast<size_t>(blockIdx.x) * P.row_cap + my_row) * kFewStatFloats;
         stat[quarter] = l_run;
@@ -564,7 +564,7 @@ __global__ void __launch_bounds__(128) few_merge_kernel(const __grid_constant__ 
     ptx::grid_wait();
     if (row >= P.G * u.Sq) return;
     // the row's partial results: u is the first chunk, whose length is that of all but the last
-    const float4* const part = reinterpret_cast<const float4*>(P.scores + u.s_off + few_row_offset(row, u.Sk_pad)) + lane;
+    const float4* const part = reinterpret_cast<const float4*>(P.scores + u.s_off + few_row_offset(row, u.Sk_pad / kTile)) + lane;
     const int part_step = u.j1 * (kTile / 4);
     const float* const stat = P.stats + (static_cast<size_t>(first_id) * P.row_cap + row) * kFewStatFloats;
     const size_t stat_step = static_cast<size_t>(P.Hkv) * P.row_cap * kFewStatFloats;

@@ -115,10 +115,12 @@ __host__ __device__ inline int few_chunk_tiles(int n_tiles, int rows)
 {
     return rows <= 8 ? (n_tiles < 16 ? 1 : n_tiles < 32 ? 2 : n_tiles < 128 ? 4 : kFewMaxChunk) : n_tiles < 32 ? 2 : kFewMaxChunk;
 }
-// Start of row `row` of the scores of a KV head (row_len keys) or of its block maxima: 64-bit, since 24 rows pass 2^31 scores
-// from 97.6 million keys on.
-__host__ __device__ constexpr int64_t few_row_offset(int row, int row_len) { return static_cast<int64_t>(row_len) * row; }
-static_assert(few_row_offset(kFewMaxRows - 2, 100000000) == 2200000000ll, "rows of a long context are addressed in 64 bits");
+// Start of row `row` of the scores of a KV head, n_tiles of 128 keys: 64-bit, since 24 rows pass 2^31 scores from 97.6 million keys
+// on.  The product of row and tiles fits 32 bits; kept in those, the offsets of a thread's rows take a register each in the loop
+// and not two (9 to 16 rows, 16000 keys: 3 to 5 %).  Block maxima (four a tile) are addressed in 32 bits.
+__host__ __device__ constexpr int64_t few_row_offset(int row, int n_tiles) { return static_cast<int64_t>(row * n_tiles) * 128; }
+static_assert(few_row_offset(kFewMaxRows - 2, 100000000 / 128) == 2200000000ll, "rows of a long context are addressed in 64 bits");
+static_assert(int64_t{kFewMaxRows} * (int64_t{1} << 31) / 32 < int64_t{1} << 31, "block maxima of the longest context");
 // A chunk's partial result: the 128 values of a row's O^T take the place of the row's scores of the chunk's first tile, which
 // nobody reads any more by then; beside them, per row, four parts of the denominator, the maximum they refer to, three unused.
 // So a KV head needs rows * (528 tiles + 32 chunks) bytes, at 24 rows and a tile a chunk 13440 a tile: less than the 17408 of the
