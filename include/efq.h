@@ -191,7 +191,7 @@ efq_status_t efq_attention_fwd_quantized(float* o, int B, int Hq, int Hkv, int64
  * not depend on it.
  * The workspace holds the MXFP4 copies of all sequences side by side plus the tables:
  * efq_attention_varlen_workspace_bytes() gives the size for the given prefix sums (0 for invalid arguments).  The
- * two prefix arrays are read during the call only.
+ * two prefix arrays are read during the call only; a graph that the call is recorded into keeps the tables made from them.
  * Asynchronous; efq_poll_status(workspace, stream) reports a device-side problem of any sequence.
  * Errors: INVALID_ARG (null pointer, n_seqs < 0, prefix sums not starting at 0 or decreasing, bad params),
  * UNSUPPORTED (d != 128, a batch too long for the 32-bit tile coordinates), ALIGNMENT, WORKSPACE, ARCH, CUDA. */

@@ -1046,6 +1046,25 @@ bool plan_varlen(const int64_t* cu_q, const int64_t* cu_k, int n_seqs, int Hq, i
     return true;
 }
 
+// Host table to the workspace.  Pageable memory: the call returns once the bytes sit in the driver's staging area, so the vector
+// may go - but a copy recorded into a graph reads them at every replay, so there the graph takes the vector over and frees it when it
+// and all that was instantiated from it are destroyed.
+template <typename T>
+cudaError_t copy_table(void* dst, std::vector<T>& host, cudaStream_t stream)
+{
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    cudaGraph_t graph = nullptr;
+    cudaError_t e = cudaStreamGetCaptureInfo(stream, &capture, nullptr, &graph, nullptr, nullptr);
+    if (e != cudaSuccess) return e;
+    e = cudaMemcpyAsync(dst, host.data(), sizeof(T) * host.size(), cudaMemcpyHostToDevice, stream);
+    if (e != cudaSuccess || capture != cudaStreamCaptureStatusActive) return e;
+    auto* const kept = new std::vector<T>(std::move(host));          // the bytes stay where they are
+    cudaUserObject_t owner;
+    e = cudaUserObjectCreate(&owner, kept, [](void* p) { delete static_cast<std::vector<T>*>(p); }, 1, cudaUserObjectNoDestructorSync);
+    if (e != cudaSuccess) { host = std::move(*kept); delete kept; return e; }
+    return cudaGraphRetainUserObject(graph, owner, 1, cudaGraphUserObjectMove);
+}
+
 }  // namespace
 
 bool encode_bf16_map(CUtensorMap* map, const void* base, uint64_t cols, uint64_t rows) { return encode_any(map, base, 2 * cols, rows, kMapBf16); }
@@ -1397,7 +1416,7 @@ extern "C" efq_status_t efq_attention_fwd_varlen(const void* q, const void* k, c
         F.stats = reinterpret_cast<float*>(fw + fp.stats);
         F.status = reinterpret_cast<uint32_t*>(ws);
         if (!few_long.empty()) {
-            if (cudaMemcpyAsync(ws + p.few_table, few_long.data(), sizeof(FewSeq) * few_long.size(), cudaMemcpyHostToDevice, s) != cudaSuccess) return EFQ_ERR_CUDA;
+            if (copy_table(ws + p.few_table, few_long, s) != cudaSuccess) return EFQ_ERR_CUDA;
             F.seqs = reinterpret_cast<const FewSeq*>(ws + p.few_table);
         }
         if (launch_few(producer, F, s) != cudaSuccess) return EFQ_ERR_CUDA;
@@ -1414,8 +1433,7 @@ extern "C" efq_status_t efq_attention_fwd_varlen(const void* q, const void* k, c
         n_items += seqs[order[i].seq].packed ? Hkv : Hq;
     }
 
-    // Pageable host memory: the call returns once the bytes sit in the driver's staging area, so the vector may go.
-    if (cudaMemcpyAsync(ws + 1024, tables.data(), p.tables, cudaMemcpyHostToDevice, s) != cudaSuccess) return EFQ_ERR_CUDA;
+    if (copy_table(ws + 1024, tables, s) != cudaSuccess) return EFQ_ERR_CUDA;
     if (launch_quantize_jobs(reinterpret_cast<const QuantJob*>(ws + p.jobs_off), reinterpret_cast<const int32_t*>(ws + p.prefix_off),
                              3 * p.n_active, ctas, reinterpret_cast<const ItemGroup*>(ws + p.groups_off), static_cast<int>(order.size()), n_items,
                              reinterpret_cast<ItemDesc*>(ws + p.items_off), p.n_few > 0 ? nullptr : reinterpret_cast<uint32_t*>(ws), s) != cudaSuccess)

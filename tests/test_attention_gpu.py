@@ -575,3 +575,33 @@ def test_pipelined_host_entry_point_matches_device_entry_point(B, Hq, Hkv, S, ch
     with pytest.raises(binding.EfqError) as e:
         binding.efq_attention_fwd_host_pipelined(hq, hk, hv, ho, dq, dk, dv, do, streams, True, 0.0, 0, None, ws, 0)
     assert e.value.status == 1
+
+
+@pytest.mark.parametrize("lens", [[(300, 500), (1, 700), (20, 300), (130, 130)], [(1 + n % 3, 40 + n) for n in range(140)]])
+def test_packed_batch_recorded_into_a_graph(lens):
+    """The tables of a packed batch come from host memory of the call; a graph reads them at every replay and so keeps them.
+    (140 few-row sequences: more than travel with the launch.)  Replays on new inputs equal the call."""
+    Hq, Hkv = 8, 2
+    g = torch.Generator(device="cuda").manual_seed(23)
+    cu_q = np.concatenate([[0], np.cumsum([a for a, _ in lens])])
+    cu_k = np.concatenate([[0], np.cumsum([b for _, b in lens])])
+    q = torch.randn(int(cu_q[-1]), Hq, 128, generator=g, device="cuda").bfloat16()
+    k, v = (torch.randn(int(cu_k[-1]), Hkv, 128, generator=g, device="cuda").bfloat16() for _ in range(2))
+    ws = torch.empty(64 << 20, dtype=torch.uint8, device="cuda")
+    side = torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(side):
+        binding.efq_attention_fwd_varlen(q, k, v, cu_q, cu_k, True, workspace=ws)
+    torch.cuda.current_stream().wait_stream(side)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        o = binding.efq_attention_fwd_varlen(q, k, v, cu_q, cu_k, True, workspace=ws)
+    for _ in range(3):
+        q.normal_(generator=g)
+        k.normal_(generator=g)
+        want = binding.efq_attention_fwd_varlen(q, k, v, cu_q, cu_k, True)
+        host = [np.full(4096, 0xFF, np.uint8) for _ in range(200)]       # takes what the call freed on the host, if it did
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(o, want)
+        del host
