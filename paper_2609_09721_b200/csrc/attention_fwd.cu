@@ -53,7 +53,7 @@ constexpr int kSfBytes = 512;
 constexpr int kVStageBytes = kTileBytes + 1024; // + 16 ones rows
 constexpr int kOutRowBytes = 528;       // staging row of the output: 512 bytes that start 4 banks apart, so that 128-bit stores
                                         // of a warp (a row per lane) do not collide
-constexpr uint64_t kTimeoutCycles = 1500000000ull;
+constexpr uint32_t kTimeoutCycles = 1500000000u;
 
 // TMEM column map
 constexpr uint32_t kColS = 0;         // 2 x 128
@@ -89,6 +89,7 @@ struct __align__(1024) Smem {
     uint64_t l_bar;           // FP32-denominator baseline only: all eight probability warps have written lsum_x / mref_x
     uint32_t tmem_base;
     volatile uint32_t abort_flag;
+    volatile uint32_t progress; // tiles whose P~V has been issued
 };
 
 static_assert(sizeof(Smem::k) + sizeof(Smem::v) >= kTile * kOutRowBytes, "finished rows fit where K and V were");
@@ -102,6 +103,7 @@ struct FwdParams {
     const uint8_t* sf_k;      // [B*Hkv*Sk_pad/128][512]
     const uint8_t* sf_v;
     float* o;
+    int64_t o_tokens;         // packed batch: query tokens in all
     int64_t o_head, o_row;    // strides of o in elements: row i of (batch b, head h) starts at o[(b * Hq + h) * o_head + i * o_row]
     uint32_t* status;
     efq_debug_t dbg;
@@ -109,37 +111,45 @@ struct FwdParams {
     int packed;               // dense batch with few query tokens: the query heads of a KV group share one query tile
     const SeqDesc* seqs;      // packed variable-length batch: sequence table and one item per CTA (device memory);
     const ItemDesc* items;    //   NULL for a [B, H, S, d] batch, whose items follow from the block index
+    uint32_t heads_magic;     // [B, H, S, d]: ceil(2^32 / (B * Hq)), 0 for one head (persistent kernel)
     int64_t v_tiles_per_head; // packed batch: 128-key tiles per KV head in the V^T code matrix (all sequences)
     int inject_skip_loads;    // test hook: the TMA thread loads Q only, so the first wait on K/V runs out
     float rescale_threshold;  // 0: Algorithm 2; > 0: the shifting maximum is kept while the true one is at most this far above
 };
 
-// Bounded wait of one thread.  Returns false on timeout (recorded in the status word) or CTA-wide abort.
-// The polling loop is kept to the barrier test itself; the abort flag and the clock are looked at every 64th
-// round only, because every instruction a waiting warp issues is taken from the warps that compute.
-__device__ __forceinline__ bool wait1(uint64_t* bar, uint32_t parity, Smem* sm, uint32_t* status)
+// Waits end with the completion or, false, when the CTA gave up.  That is one warp's business (stalled below): the kernels inline
+// some twenty-five waits, and a clock in each of them made a sixth of the code, which outgrows the instruction cache as it is.
+__device__ __forceinline__ bool wait1(uint64_t* bar, uint32_t parity, Smem* sm)
 {
-    if (ptx::mbar_try_wait(bar, parity)) return true;
-    const long long t0 = clock64();
-    for (uint32_t spins = 1;; ++spins) {
-        if (ptx::mbar_try_wait_suspend(bar, parity, 20000u)) return true;
-        if ((spins & 63u) == 0u) {
-            if (sm->abort_flag) return false;
-            if (static_cast<uint64_t>(clock64() - t0) > kTimeoutCycles) {
-                sm->abort_flag = 1;
-                atomicExch(status, static_cast<uint32_t>(EFQ_ERR_DEVICE_TIMEOUT));
-                return false;
-            }
-        }
-    }
+#pragma unroll 1
+    while (!ptx::mbar_try_wait(bar, parity))
+        if (sm->abort_flag) return false;
+    return true;
 }
 // The same wait executed by all lanes of a warp.  All lanes poll the same barrier; only the rare timeout path
 // can split a warp, so the verdict is made warp-uniform there and nowhere else.
-__device__ __forceinline__ bool wait_all(uint64_t* bar, uint32_t parity, Smem* sm, uint32_t* status)
+__device__ __forceinline__ bool wait_all(uint64_t* bar, uint32_t parity, Smem* sm)
 {
     if (ptx::mbar_try_wait(bar, parity)) return true;
-    const bool ok = wait1(bar, parity, sm, status);
-    return __all_sync(__activemask(), ok);
+    return __all_sync(__activemask(), wait1(bar, parity, sm));
+}
+// The watch over all waits of the CTA, by the one thread that waits for its result: between two of its own polls it looks whether
+// P~V goes on.  Without another tile within the limit the CTA gives up, and the status word says so.
+__device__ __forceinline__ bool wait_watching(uint64_t* bar, uint32_t parity, Smem* sm, uint32_t* status)
+{
+    uint32_t t0 = ptx::clock32(), seen = sm->progress;
+#pragma unroll 1
+    while (!ptx::mbar_try_wait(bar, parity)) {
+        if (sm->abort_flag) return false;
+        const uint32_t now = sm->progress;
+        if (now != seen) { seen = now; t0 = ptx::clock32(); }
+        if (ptx::clock32() - t0 > kTimeoutCycles) {
+            sm->abort_flag = 1u;
+            atomicExch(status, static_cast<uint32_t>(EFQ_ERR_DEVICE_TIMEOUT));
+            return false;
+        }
+    }
+    return true;
 }
 
 // o[0 .. 31] *= a, two at a time
@@ -160,7 +170,7 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                      const __grid_constant__ CUtensorMap map_v, const FwdParams P)
 {
     extern __shared__ uint8_t smem_raw[];
-    Smem* sm = reinterpret_cast<Smem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
+    Smem* sm = reinterpret_cast<Smem*>(smem_raw + ptx::smem_round_up(smem_raw, 1024u));
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
 
@@ -222,6 +232,7 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
             ptx::prefetch_tensormap(&map_k);
             ptx::prefetch_tensormap(&map_v);
             sm->abort_flag = 0u;
+            sm->progress = 0u;
             ptx::mbar_init(&sm->q_full, 1);
             ptx::mbar_init(&sm->o_done, 1);
             ptx::mbar_init(&sm->l_bar, 2 * kGroupWarps);
@@ -277,11 +288,11 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         for (int j = 0; j < (P.inject_skip_loads ? 0 : n_tiles); ++j) {
             // Stage barriers of their own: a waiter on a barrier that other roles may complete twice before it
             // looks (S runs ahead) could not tell which completion it sees by parity.
-            if (!wait1(&sm->k_empty[s], ph ^ 1u, sm, P.status)) break;
+            if (!wait1(&sm->k_empty[s], ph ^ 1u, sm)) break;
             ptx::mbar_arrive_expect_tx(&sm->k_full[s], kTileBytes + kSfBytes);
             ptx::tma_load_2d(sm->k[s], &map_k, 0, k_row0 + static_cast<int>(j * kTile), &sm->k_full[s]);
             ptx::bulk_load_1d(sm->sf_k[s], P.sf_k + (sfk_tile0 + j) * kSfBytes, kSfBytes, &sm->k_full[s]);
-            if (!wait1(&sm->v_empty[s], ph ^ 1u, sm, P.status)) break;
+            if (!wait1(&sm->v_empty[s], ph ^ 1u, sm)) break;
             ptx::mbar_arrive_expect_tx(&sm->v_full[s], kTileBytes + kSfBytes);
             ptx::tma_load_2d(sm->v[s], &map_v, v_x0 + static_cast<int>(j * 64), v_y0, &sm->v_full[s]);
             ptx::bulk_load_1d(sm->sf_v[s], P.sf_v + (sfv_tile0 + j) * kSfBytes, kSfBytes, &sm->v_full[s]);
@@ -291,6 +302,7 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         ptx::grid_wait();
         // an earlier CTA of this launch gave up: the waits of this one end soon instead of after their limit
         if (*reinterpret_cast<volatile uint32_t*>(P.status) != 0u) sm->abort_flag = 1u;
+        if (run) wait_watching(&sm->o_done, 0, sm, P.status);
     } else if (run && warp == 1) {
         // =============================== S = Q K^T issuer ===============================
         // The whole warp runs the loop with warp-uniform state; one elected lane issues the tcgen05
@@ -299,15 +311,15 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         const uint64_t d_sf = ptx::smem_desc(0, 16, 128, ptx::kLayoutNone);
         const uint64_t dq0 = d_sw64 + (ptx::smem_u32(sm->q) >> 4);
         const uint32_t sfq = tmem + kColSfQ;
-        bool ok = wait_all(&sm->q_full, 0, sm, P.status);
+        bool ok = wait_all(&sm->q_full, 0, sm);
         ptx::tc_fence_after_sync();
         if (ok && ptx::elect_one()) ptx::tmem_cp_sf(sfq, d_sf + (ptx::smem_u32(sm->sf_q) >> 4));
         int ks = 0;
         uint32_t kph = 0;
         for (int t = 0; ok && t < n_tiles; ++t) {
             const int sb = static_cast<int>(t & 1);
-            if (!wait_all(&sm->k_full[ks], kph, sm, P.status)) break;
-            if (!wait_all(&sm->s_empty[sb], static_cast<uint32_t>((t >> 1) & 1) ^ 1u, sm, P.status)) break;
+            if (!wait_all(&sm->k_full[ks], kph, sm)) break;
+            if (!wait_all(&sm->s_empty[sb], static_cast<uint32_t>((t >> 1) & 1) ^ 1u, sm)) break;
             ptx::tc_fence_after_sync();
             if (ptx::elect_one()) {
                 const uint32_t sfk = tmem + kColSfK + 4 * sb;
@@ -336,9 +348,9 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         uint32_t vph = 0;
         for (int j = 0; j < n_tiles; ++j) {
             const int pb = static_cast<int>(j & 1);
-            if (!wait_all(&sm->v_full[vs], vph, sm, P.status)) break;
-            if (!wait_all(&sm->p_full[pb], static_cast<uint32_t>((j >> 1) & 1), sm, P.status)) break;
-            if (!wait_all(&sm->o_ready[j & 3], static_cast<uint32_t>((j >> 2) & 1), sm, P.status)) break;
+            if (!wait_all(&sm->v_full[vs], vph, sm)) break;
+            if (!wait_all(&sm->p_full[pb], static_cast<uint32_t>((j >> 1) & 1), sm)) break;
+            if (!wait_all(&sm->o_ready[j & 3], static_cast<uint32_t>((j >> 2) & 1), sm)) break;
             ptx::tc_fence_after_sync();
             if (ptx::elect_one()) {
                 const uint32_t sfp = tmem + kColSfP + 4 * pb;
@@ -352,6 +364,7 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                 ptx::mma_commit(&sm->p_empty[pb]);
                 ptx::mma_commit(&sm->v_empty[vs]);
                 if (j + 1 == n_tiles) ptx::mma_commit(&sm->o_done);
+                sm->progress = static_cast<uint32_t>(j) + 1u;
             }
             __syncwarp();
             if (++vs == kStages) { vs = 0; vph ^= 1u; }
@@ -372,12 +385,12 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
     const uint32_t o_addr = tmem + (static_cast<uint32_t>(quarter * 32) << 16) + kColO;
     if (run) {
         for (int j = 0; j < n_tiles; ++j) {
-            if (!wait_all(&sm->a_bar[j & 3][quarter], static_cast<uint32_t>((j >> 2) & 1), sm, P.status)) break;
+            if (!wait_all(&sm->a_bar[j & 3][quarter], static_cast<uint32_t>((j >> 2) & 1), sm)) break;
             const float alpha = sm->alpha[j & 3][row];
             if (j > 0 && __any_sync(0xffffffffu, alpha != 1.0f)) {
                 // The end of P~V_{j-1} frees its V stage.  The parity says so only if P~V_{j-5}, the stage's use before, has ended,
                 // and it has: the probability warps waited for it before they stored the codes of tile j-3.
-                if (!wait_all(&sm->v_empty[(j - 1) & 3], static_cast<uint32_t>((j - 1) >> 2) & 1u, sm, P.status)) break;
+                if (!wait_all(&sm->v_empty[(j - 1) & 3], static_cast<uint32_t>((j - 1) >> 2) & 1u, sm)) break;
                 ptx::tc_fence_after_sync();
                 const uint64_t alpha2 = pack2(alpha, alpha);
                 uint32_t oa[32], ob[32];
@@ -454,7 +467,7 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
 
             // ---- scores of tile j: TMEM -> registers (Algorithm 2, step 1 happened on the tensor core)
             if (!in_flight) {
-                if (!wait_all(&sm->s_full[sb], ph2, sm, P.status)) { ok = false; break; }
+                if (!wait_all(&sm->s_full[sb], ph2, sm)) { ok = false; break; }
                 ptx::tc_fence_after_sync();
                 ptx::tmem_ld32f<0>(s_addr, r);
                 ptx::tmem_ld32f<32>(s_addr + 32, r);
@@ -471,11 +484,17 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                 if (j > 0 && have_prev) m_prev = sm->runmax[sb ^ 1][row];
                 ptx::tmem_wait_ld();
                 ptx::tc_fence_before_sync();          // the S buffer is handed back with the joint publication below
-                const int64_t key0 = j * kTile;
-                if (__any_sync(0xffffffffu, key0 + 127 > limit)) {     // diagonal or ragged tile: keys past the row's limit are masked in place
+                const int64_t last64 = limit - j * kTile;              // last visible key of the row inside the tile
+                if (__any_sync(0xffffffffu, last64 < 127)) {           // diagonal or ragged tile: keys past the row's limit are masked in place
+                    const int last = static_cast<int>(last64 < -1 ? -1 : last64 > 127 ? 127 : last64);
 #pragma unroll
-                    for (int i = 0; i < 128; ++i)
-                        if (key0 + i > limit) r[i] = -INFINITY;
+                    for (int g = 0; g < 4; ++g) {          // a bit per key: predicates come out of a word seven at a time
+                        const int n = last - 32 * g + 1;   // keys of the block that the row sees
+                        const uint32_t bits = n >= 32 ? 0xffffffffu : n <= 0 ? 0u : (1u << n) - 1u;
+#pragma unroll
+                        for (int i = 0; i < 32; ++i)
+                            if ((bits & (1u << i)) == 0u) r[32 * g + i] = -INFINITY;
+                    }
                 }
             }
 #pragma unroll
@@ -483,7 +502,7 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
 
             // ---- running row maximum (Eq. rowmax-update): handed over from the group that owns tile j-1
             if (!have_prev) {
-                if (!wait_all(&sm->a_bar[(j - 1) & 3][quarter], static_cast<uint32_t>((j - 1) >> 2) & 1u, sm, P.status)) { ok = false; break; }
+                if (!wait_all(&sm->a_bar[(j - 1) & 3][quarter], static_cast<uint32_t>((j - 1) >> 2) & 1u, sm)) { ok = false; break; }
                 m_prev = sm->runmax[sb ^ 1][row];
             }
             float m_new = fmaxf(fmaxf(m_prev, bmax[0]), max3(bmax[1], bmax[2], bmax[3]));
@@ -520,7 +539,7 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                 uint32_t byte;
                 produce32<PRODUCER>(&r[g * 32], bmax[g], m_s, K, codes, byte, &lsum);
                 if (g == 0 && !have_p) {      // P~V of tile j-2 must have finished: it reads the group's P buffer
-                    if (!wait_all(&sm->p_empty[sb], ph2 ^ 1u, sm, P.status)) { ok = false; break; }
+                    if (!wait_all(&sm->p_empty[sb], ph2 ^ 1u, sm)) { ok = false; break; }
                 }
                 *reinterpret_cast<uint4*>(sm->p[sb] + code_tile_offset(row, g)) = codes;
                 sfword |= byte << (8 * g);
@@ -567,8 +586,8 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         // ---- final normalisation O = A / l: each group writes 64 of the 128 channels
         // (a barrier of its own: a group that skipped a phase of the other group's p_empty could not tell
         // an old completion from the last one by parity)
-        if (ok) ok = wait_all(&sm->o_done, 0, sm, P.status);
-        if (ok && PRODUCER == 6) ok = wait_all(&sm->l_bar, 0, sm, P.status);
+        if (ok) ok = wait_all(&sm->o_done, 0, sm);
+        if (ok && PRODUCER == 6) ok = wait_all(&sm->l_bar, 0, sm);
         if (ok) {
             ptx::tc_fence_after_sync();
             uint32_t o[64];
@@ -655,10 +674,11 @@ EncodeTiledFn get_encode()
 
 // A descriptor depends on nothing but the base, the shape and the kind of map, so the last few are kept: a serving loop
 // that calls with the same buffers and shape (decode steps above all) does not pay for driver calls per forward.
-enum MapKind : uint32_t { kMapCodes, kMapBf16 };
+// kMapRowsOut: FP32 rows of 128 channels, [heads, tokens] or, kMapRowsOutPacked, [tokens, heads]; coordinates (channel, token, head).
+enum MapKind : uint32_t { kMapCodes, kMapBf16, kMapRowsOut, kMapRowsOutPacked };
 struct MapCacheEntry {
     const void* base;
-    uint64_t row_bytes, rows;
+    uint64_t row_bytes, rows;      // of the outputs: heads, tokens
     MapKind kind;
     CUtensorMap map;
 };
@@ -681,15 +701,24 @@ bool encode_any(CUtensorMap* map, const void* base, uint64_t row_bytes, uint64_t
     }
     EncodeTiledFn enc = get_encode();
     if (!enc) return false;
-    const bool codes = kind == kMapCodes;
-    cuuint64_t dims[2] = {codes ? row_bytes : row_bytes / 2, rows};
-    cuuint64_t strides[1] = {row_bytes};
-    cuuint32_t box[2] = {64, 128};
-    cuuint32_t estr[2] = {1, 1};
-    if (enc(map, codes ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box,
-            estr, CU_TENSOR_MAP_INTERLEAVE_NONE, codes ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
-            CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-        return false;
+    const cuuint32_t estr[3] = {1, 1, 1};
+    CUresult r;
+    if (kind == kMapCodes || kind == kMapBf16) {
+        const bool codes = kind == kMapCodes;
+        const cuuint64_t dims[2] = {codes ? row_bytes : row_bytes / 2, rows}, strides[1] = {row_bytes};
+        const cuuint32_t box[2] = {64, 128};
+        r = enc(map, codes ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box,
+                estr, CU_TENSOR_MAP_INTERLEAVE_NONE, codes ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
+                CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    } else {
+        const uint64_t heads = row_bytes;
+        const cuuint64_t dims[3] = {128, rows, heads};
+        const cuuint64_t strides[2] = {kind == kMapRowsOut ? 512 : 512 * heads, kind == kMapRowsOut ? 512 * rows : 512};
+        const cuuint32_t box[3] = {32, 32, 1};
+        r = enc(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    }
+    if (r != CUDA_SUCCESS) return false;
     std::lock_guard<std::mutex> lock(g_map_mutex);
     g_map_cache[g_map_next] = MapCacheEntry{base, row_bytes, rows, kind, *map};
     g_map_next = (g_map_next + 1) % kMapCacheSize;
@@ -782,7 +811,7 @@ bool use_short(int producer, bool debug, int64_t items, int sms, const FwdParams
 
 template <int PRODUCER, bool TABLE>
 cudaError_t launch_short_one(unsigned items, unsigned sms, int dev, cudaStream_t stream, const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv,
-                         const FwdParams& P)
+                         const CUtensorMap& mo, const FwdParams& P)
 {
     constexpr int smem = static_cast<int>(sizeof(ShortSmem)) + 1024;
     static std::atomic<uint64_t> done{0};        // the shared-memory attribute belongs to (function, device): set once for each
@@ -791,14 +820,14 @@ cudaError_t launch_short_one(unsigned items, unsigned sms, int dev, cudaStream_t
         if (e != cudaSuccess) return e;
         done.fetch_or(1ull << dev, std::memory_order_relaxed);
     }
-    return launch_overlapped(attention_short_kernel<PRODUCER, TABLE>, dim3(sms), kThreads, smem, stream, mq, mk, mv, P, items);
+    return launch_overlapped(attention_short_kernel<PRODUCER, TABLE>, dim3(sms), kThreads, smem, stream, mq, mk, mv, mo, P, items);
 }
 
 template <int PRODUCER>
 cudaError_t launch_short(unsigned items, unsigned sms, int dev, cudaStream_t stream, const CUtensorMap& mq, const CUtensorMap& mk,
-                         const CUtensorMap& mv, const FwdParams& P)
+                         const CUtensorMap& mv, const CUtensorMap& mo, const FwdParams& P)
 {
-    return P.items ? launch_short_one<PRODUCER, true>(items, sms, dev, stream, mq, mk, mv, P) : launch_short_one<PRODUCER, false>(items, sms, dev, stream, mq, mk, mv, P);
+    return P.items ? launch_short_one<PRODUCER, true>(items, sms, dev, stream, mq, mk, mv, mo, P) : launch_short_one<PRODUCER, false>(items, sms, dev, stream, mq, mk, mv, mo, P);
 }
 
 // SMs of a device, asked for once
@@ -842,13 +871,18 @@ cudaError_t launch_forward(int producer, bool debug, int64_t items, cudaStream_t
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
     const int sms = sm_count(dev);
     if (sms > 0 && use_short(producer, debug, items, sms, P)) {
+        CUtensorMap mo;
+        const bool packed_batch = P.items != nullptr;
+        if (!encode_any(&mo, P.o, packed_batch ? P.Hq : static_cast<uint64_t>(P.B) * P.Hq, packed_batch ? P.o_tokens : P.Sq,
+                        packed_batch ? kMapRowsOutPacked : kMapRowsOut))
+            return cudaErrorInvalidValue;
         switch (producer) {
-            case 0: return launch_short<0>(static_cast<unsigned>(items), static_cast<unsigned>(sms), dev, stream, mq, mk, mv, P);
-            case 1: return launch_short<1>(static_cast<unsigned>(items), static_cast<unsigned>(sms), dev, stream, mq, mk, mv, P);
-            case 2: return launch_short<2>(static_cast<unsigned>(items), static_cast<unsigned>(sms), dev, stream, mq, mk, mv, P);
-            case 3: return launch_short<3>(static_cast<unsigned>(items), static_cast<unsigned>(sms), dev, stream, mq, mk, mv, P);
-            case 4: return launch_short<4>(static_cast<unsigned>(items), static_cast<unsigned>(sms), dev, stream, mq, mk, mv, P);
-            case 5: return launch_short<5>(static_cast<unsigned>(items), static_cast<unsigned>(sms), dev, stream, mq, mk, mv, P);
+            case 0: return launch_short<0>(static_cast<unsigned>(items), static_cast<unsigned>(sms), dev, stream, mq, mk, mv, mo, P);
+            case 1: return launch_short<1>(static_cast<unsigned>(items), static_cast<unsigned>(sms), dev, stream, mq, mk, mv, mo, P);
+            case 2: return launch_short<2>(static_cast<unsigned>(items), static_cast<unsigned>(sms), dev, stream, mq, mk, mv, mo, P);
+            case 3: return launch_short<3>(static_cast<unsigned>(items), static_cast<unsigned>(sms), dev, stream, mq, mk, mv, mo, P);
+            case 4: return launch_short<4>(static_cast<unsigned>(items), static_cast<unsigned>(sms), dev, stream, mq, mk, mv, mo, P);
+            case 5: return launch_short<5>(static_cast<unsigned>(items), static_cast<unsigned>(sms), dev, stream, mq, mk, mv, mo, P);
             default: return cudaErrorInvalidValue;
         }
     }
@@ -968,6 +1002,8 @@ efq_status_t attention_impl(const void* q, const void* k, const void* v, float* 
     P.has_dbg = debug ? 1 : 0;
     if (debug) P.dbg = *debug; else P.dbg = efq_debug_t{};
 
+    const uint64_t heads = static_cast<uint64_t>(B) * Hq;
+    P.heads_magic = heads > 1 ? static_cast<uint32_t>(((1ull << 32) + heads - 1) / heads) : 0u;
     const int64_t items = packed ? static_cast<int64_t>(B) * Hkv : (w.Sq_pad / kTile) * B * Hq;
     return launch_forward(producer, debug != nullptr, items, stream, mq, mk, mv, P) == cudaSuccess ? EFQ_OK : EFQ_ERR_CUDA;
 }
@@ -1362,7 +1398,7 @@ extern "C" efq_status_t efq_attention_fwd_varlen(const void* q, const void* k, c
         const bool packed = use_packed_tile(Hq, Hkv, lq);
         const int64_t lq_pad = packed ? kTile : (lq + kTile - 1) / kTile * kTile, lk_pad = (lk + kTile - 1) / kTile * kTile;
         SeqDesc& sd = seqs[a];
-        sd.Sq = lq; sd.Sk = lk; sd.o_off = q0 * Hq * 128;
+        sd.Sq = lq; sd.Sk = lk; sd.o_off = q0 * Hq * 128; sd.token0 = static_cast<int32_t>(q0);
         sd.q_row0 = static_cast<int32_t>(q_row); sd.Sq_pad = static_cast<int32_t>(lq_pad);
         sd.k_row0 = static_cast<int32_t>(k_row); sd.Sk_pad = static_cast<int32_t>(lk_pad);
         sd.k_col0 = static_cast<int32_t>(k_col); sd.packed = packed ? 1 : 0;
@@ -1429,8 +1465,10 @@ extern "C" efq_status_t efq_attention_fwd_varlen(const void* q, const void* k, c
     std::stable_sort(order.begin(), order.end(), [](const QueryTile& x, const QueryTile& y) { return x.weight > y.weight; });
     int64_t n_items = 0;
     for (size_t i = 0; i < order.size(); ++i) {
-        groups[i] = ItemGroup{static_cast<int32_t>(n_items), order[i].seq, order[i].qt};
-        n_items += seqs[order[i].seq].packed ? Hkv : Hq;
+        const SeqDesc& sd = seqs[order[i].seq];
+        groups[i] = ItemGroup{static_cast<int32_t>(n_items), order[i].seq, order[i].qt, order[i].weight, static_cast<int32_t>(sd.Sq),
+                              static_cast<int32_t>(sd.Sk), sd.packed};
+        n_items += sd.packed ? Hkv : Hq;
     }
 
     if (copy_table(ws + 1024, tables, s) != cudaSuccess) return EFQ_ERR_CUDA;
@@ -1452,6 +1490,7 @@ extern "C" efq_status_t efq_attention_fwd_varlen(const void* q, const void* k, c
     P.o = o;
     P.o_head = 128;                                   // token-major: a head is 128 elements, a token Hq * 128
     P.o_row = static_cast<int64_t>(Hq) * 128;
+    P.o_tokens = cu_seqlens_q[n_seqs];
     P.status = reinterpret_cast<uint32_t*>(ws);
     P.packed = 0;
     P.seqs = reinterpret_cast<const SeqDesc*>(ws + p.seqs_off);

@@ -27,64 +27,110 @@
 
 struct __align__(1024) ShortSmem : Smem {
     uint8_t q1[kTileBytes];                // query tile of every other item (the first one's is Smem::q)
-    uint8_t stage[kTile * kOutRowBytes];   // finished rows on their way out
+    uint8_t stage[4][kTile * 128];         // finished rows on their way out: 32 channels of each, 128-byte swizzle
     uint8_t sf_q1[kSfBytes];
     uint64_t q_ready[2], q_empty[2];
+    uint64_t finished;                     // the rescaling warps have left their loop
 };
 constexpr uint32_t kColSfQ1 = 440;         // scales of q1: 4 columns behind those of V
 
-// The k-th item of this CTA: the CTAs take items in turn, every other round in reverse, so that the heavier items of a round
-// go to those that had the lighter ones before.
-__device__ __forceinline__ uint32_t short_item(uint32_t k) { return k * gridDim.x + ((k & 1u) ? gridDim.x - 1u - blockIdx.x : blockIdx.x); }
-
-// One work item: rows q0 .. q0 + 127 of a query head or - "packed", in a variable-length batch - row r = token r % Sq of query
-// head r / Sq of a KV group.  Each role uses the fields that it needs; the others are never computed.
-struct ShortItem {
-    int n_tiles, q0;
-    int q_row, k_row0, v_x0, v_row0;      // where its operands start in the code matrices
-    int64_t sfv_tile0, Sq, Sk, o;         // o: element offset of row 0 of its (first) query head in the output
-    bool packed;
-};
-// TABLE = false: [B, H, S, d] batch, heaviest query tiles first, the heads of a GQA group adjacent (a template parameter because
-// the table's fields cost registers in every role).  TABLE = true: variable-length batch, items sorted by weight in memory.
+// The items of this CTA, one after the other: the CTAs take items in turn, every other round in reverse, so that the heavier items
+// of a round go to those that had the lighter ones before.  Every role walks them for itself, so a step has to be short: it
+// stands between the last tile of an item and the first of the next.  [B, H, S, d] batch (heaviest query tiles first, the heads of a
+// GQA group adjacent): query tile and head by additions.  Packed batch (TABLE; items sorted by weight in memory): the
+// entry of the next item is on its way while this one is worked on.
 template <bool TABLE>
-__device__ __forceinline__ ShortItem short_decode(const FwdParams& P, uint32_t index)
+struct ShortWalk {
+    uint32_t k;                    // items before this one
+    uint32_t quo, rem;             // dense: index of the item divided by the heads
+    uint32_t step[2];              // dense: the way to the next item after an even, an odd k: quotient << 16 | remainder
+    ItemDesc it, next;             // packed batch; n_tiles < 0 past the last item
+
+    __device__ __forceinline__ ItemDesc fetch(const FwdParams& P, uint32_t n_items, uint32_t i) const
+    {
+        const uint32_t index = i * gridDim.x + ((i & 1u) ? gridDim.x - 1u - blockIdx.x : blockIdx.x);
+        ItemDesc d;
+        d.n_tiles = -1;
+        if (index < n_items) d = P.items[index];
+        return d;
+    }
+    __device__ __forceinline__ ShortWalk(const FwdParams& P, uint32_t n_items) : k(0)
+    {
+        if (TABLE) {
+            it = fetch(P, n_items, 0);
+            next = fetch(P, n_items, 1);
+        } else {
+            const uint32_t heads = static_cast<uint32_t>(P.B) * P.Hq, even = 2u * (gridDim.x - blockIdx.x) - 1u, odd = 2u * blockIdx.x + 1u;
+            // numbers up to twice the SMs: exact for every count of heads, and a remainder fits 16 bits
+            auto div = [&](uint32_t x) { return P.heads_magic != 0u ? __umulhi(x, P.heads_magic) : x; };
+            quo = div(blockIdx.x); rem = blockIdx.x - quo * heads;
+            step[0] = div(even); step[0] = step[0] << 16 | (even - step[0] * heads);
+            step[1] = div(odd); step[1] = step[1] << 16 | (odd - step[1] * heads);
+        }
+    }
+    __device__ __forceinline__ void advance(const FwdParams& P, uint32_t n_items)
+    {
+        ++k;
+        if (TABLE) {
+            it = next;
+            next = fetch(P, n_items, k + 1);
+        } else {
+            const uint32_t heads = static_cast<uint32_t>(P.B) * P.Hq, s = (k & 1u) ? step[0] : step[1];
+            quo += s >> 16;
+            rem += s & 0xffffu;
+            if (rem >= heads) { rem -= heads; ++quo; }
+        }
+    }
+    __device__ __forceinline__ bool valid(const FwdParams& P) const { return TABLE ? it.n_tiles >= 0 : quo < static_cast<uint32_t>(P.Sq_pad) / kTile; }
+    __device__ __forceinline__ bool packed() const { return TABLE && it.packed != 0; }
+    __device__ __forceinline__ int Sq(const FwdParams& P) const { return TABLE ? it.Sq : static_cast<int>(P.Sq); }
+    __device__ __forceinline__ int Sk(const FwdParams& P) const { return TABLE ? it.Sk : static_cast<int>(P.Sk); }
+    __device__ __forceinline__ int q0(const FwdParams& P) const     // first row (packed: 0)
+    {
+        return TABLE ? it.qt * kTile : static_cast<int>(static_cast<uint32_t>(P.Sq_pad) / kTile - 1u - quo) * kTile;
+    }
+    __device__ __forceinline__ int n_tiles(const FwdParams& P) const
+    {
+        if (TABLE) return it.n_tiles;
+        const int all = (Sk(P) + kTile - 1) / kTile;
+        if (!P.causal) return all;
+        const int last_key = min(q0(P) + kTile, Sq(P)) - 1 + Sk(P) - Sq(P);       // may be negative: nothing visible
+        return last_key < 0 ? 0 : min(all, last_key / kTile + 1);
+    }
+};
+
+// Where an item's operands and rows lie: rows q0 .. q0 + 127 of a query head or - "packed", in a variable-length batch - row r =
+// token r % Sq of query head r / Sq of a KV group.  Each role uses the fields that it needs; the others are never computed.
+struct ShortItem {
+    int q_row, k_row0, v_x0, v_row0;      // in the code matrices
+    int64_t sfv_tile0, o;                 // o: element offset of row 0 of its (first) query head in the output
+    int o_y, o_z;                         // the item's first row in the tensor map of the output: token, head
+};
+template <bool TABLE>
+__device__ __forceinline__ ShortItem short_decode(const FwdParams& P, const ShortWalk<TABLE>& walk)
 {
     ShortItem w;
+    const int q0 = walk.q0(P);
     if (TABLE) {
-        const ItemDesc it = P.items[index];
-        const SeqDesc sd = P.seqs[it.seq];
-        const int G = P.Hq / P.Hkv;
-        w.packed = sd.packed != 0;
-        const int hkv = w.packed ? it.head : it.head / G, head0 = w.packed ? it.head * G : it.head;
-        w.q0 = w.packed ? 0 : it.qt * kTile;
-        w.q_row = sd.q_row0 + (w.packed ? hkv * kTile : head0 * sd.Sq_pad + w.q0);
+        const SeqDesc sd = P.seqs[walk.it.seq];
+        const int G = P.Hq / P.Hkv, head = walk.it.head;
+        const int hkv = walk.packed() ? head : head / G, head0 = walk.packed() ? head * G : head;
+        w.q_row = sd.q_row0 + (walk.packed() ? hkv * kTile : head0 * sd.Sq_pad + q0);
         w.k_row0 = sd.k_row0 + hkv * sd.Sk_pad;
         w.v_x0 = sd.k_col0 / 2;
         w.v_row0 = hkv * kTile;
         w.sfv_tile0 = static_cast<int64_t>(hkv) * P.v_tiles_per_head + sd.k_col0 / kTile;
-        w.Sq = sd.Sq; w.Sk = sd.Sk;
         w.o = sd.o_off + head0 * P.o_head;
+        w.o_y = sd.token0 + q0; w.o_z = head0;
     } else {
-        const uint32_t heads = static_cast<uint32_t>(P.B) * P.Hq;
-        const uint32_t qt = static_cast<uint32_t>(P.Sq_pad / kTile) - 1u - index / heads;
-        const uint32_t bh = index % heads, kvh = bh / static_cast<uint32_t>(P.Hq / P.Hkv);      // B * Hkv heads, G of Q for each
-        w.packed = false;
-        w.q0 = static_cast<int>(qt) * kTile;
-        w.q_row = static_cast<int>(bh * static_cast<uint32_t>(P.Sq_pad)) + w.q0;
+        const uint32_t bh = walk.rem, kvh = bh / static_cast<uint32_t>(P.Hq / P.Hkv);      // B * Hkv heads, G of Q for each
+        w.q_row = static_cast<int>(bh * static_cast<uint32_t>(P.Sq_pad)) + q0;
         w.k_row0 = static_cast<int>(kvh * static_cast<uint32_t>(P.Sk_pad));
         w.v_x0 = 0;
         w.v_row0 = static_cast<int>(kvh) * kTile;
         w.sfv_tile0 = w.k_row0 / kTile;
-        w.Sq = P.Sq; w.Sk = P.Sk;
         w.o = static_cast<int64_t>(bh) * P.o_head;
-    }
-    w.n_tiles = static_cast<int>((w.Sk + kTile - 1) / kTile);
-    if (P.causal) {
-        const int64_t last_row = !(TABLE && w.packed) && w.q0 + kTile - 1 < w.Sq ? w.q0 + kTile - 1 : w.Sq - 1;
-        const int64_t last_key = last_row + w.Sk - w.Sq;       // may be negative: nothing visible
-        const int need = last_key < 0 ? 0 : static_cast<int>(last_key / kTile) + 1;
-        if (need < w.n_tiles) w.n_tiles = need;
+        w.o_y = q0; w.o_z = static_cast<int>(bh);
     }
     return w;
 }
@@ -92,14 +138,11 @@ __device__ __forceinline__ ShortItem short_decode(const FwdParams& P, uint32_t i
 template <int PRODUCER, bool TABLE>
 __global__ void __launch_bounds__(kThreads, 1)
 attention_short_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
-                       const __grid_constant__ CUtensorMap map_v, const FwdParams P, const uint32_t n_items)
+                       const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_o, const FwdParams P, const uint32_t n_items)
 {
     static_assert(PRODUCER != 6, "the denominator of FP32 exponentials is summed by attention_fwd_kernel only");
-    // Keys and tiles of the probability warps fit 32 bits (shapes stay below 2^31 rows).  The affine rule is faster with 64 all the
-    // same (512 keys 277 -> 286 us with 32), the others with 32 (exponential, S = 4096: 198 -> 184): what the compiler makes of it.
-    using Index = typename std::conditional<PRODUCER == 0, int64_t, int>::type;
     extern __shared__ uint8_t smem_raw[];
-    ShortSmem* sm = reinterpret_cast<ShortSmem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
+    ShortSmem* sm = reinterpret_cast<ShortSmem*>(smem_raw + ptx::smem_round_up(smem_raw, 1024u));
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
 
@@ -108,7 +151,9 @@ attention_short_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
             ptx::prefetch_tensormap(&map_q);
             ptx::prefetch_tensormap(&map_k);
             ptx::prefetch_tensormap(&map_v);
+            ptx::prefetch_tensormap(&map_o);
             sm->abort_flag = 0u;
+            sm->progress = 0u;
             for (int s = 0; s < kStages; ++s) {
                 ptx::mbar_init(&sm->k_full[s], 1);
                 ptx::mbar_init(&sm->k_empty[s], 1);
@@ -123,6 +168,7 @@ attention_short_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
                 ptx::mbar_init(&sm->p_full[i], kGroupWarps);
                 ptx::mbar_init(&sm->p_empty[i], 1);
             }
+            ptx::mbar_init(&sm->finished, 4);
             for (int i = 0; i < 4; ++i) ptx::mbar_init(&sm->o_ready[i], 4);
             for (int i = 0; i < 4; ++i)
                 for (int qd = 0; qd < 4; ++qd) ptx::mbar_init(&sm->a_bar[i][qd], 1);
@@ -152,26 +198,27 @@ attention_short_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
         // The operands come from the kernel before.  Whatever else this kernel writes or reads follows from the loads.
         ptx::grid_wait();
         int s = 0, n = 0;
-        uint32_t ph = 0, idx;
+        uint32_t ph = 0;
         bool ok = true;
-        for (uint32_t k = 0; ok && (idx = short_item(k)) < n_items; ++k) {
-            const ShortItem w = short_decode<TABLE>(P, idx);
-            if (w.n_tiles <= 0) continue;
+        for (ShortWalk<TABLE> walk(P, n_items); ok && walk.valid(P); walk.advance(P, n_items)) {
+            const int n_tiles = walk.n_tiles(P);
+            if (n_tiles <= 0) continue;
+            const ShortItem w = short_decode<TABLE>(P, walk);
             const int qb = n & 1;
-            if (!wait1(&sm->q_empty[qb], (static_cast<uint32_t>(n >> 1) & 1u) ^ 1u, sm, P.status)) break;
+            if (!wait1(&sm->q_empty[qb], (static_cast<uint32_t>(n >> 1) & 1u) ^ 1u, sm)) break;
             ptx::mbar_arrive_expect_tx(&sm->q_ready[qb], kTileBytes + kSfBytes);
             ptx::tma_load_2d(qb ? sm->q1 : sm->q, &map_q, 0, w.q_row, &sm->q_ready[qb]);
             ptx::bulk_load_1d(qb ? sm->sf_q1 : sm->sf_q, P.sf_q + static_cast<int64_t>(w.q_row / kTile) * kSfBytes, kSfBytes, &sm->q_ready[qb]);
             ++n;
             const int64_t sfk_tile0 = w.k_row0 / kTile;
-            for (int j = 0; j < (P.inject_skip_loads ? 0 : w.n_tiles); ++j) {
+            for (int j = 0; j < (P.inject_skip_loads ? 0 : n_tiles); ++j) {
                 // Stage barriers of their own: a waiter on a barrier that other roles may complete twice before it
                 // looks (S runs ahead) could not tell which completion it sees by parity.
-                if (!wait1(&sm->k_empty[s], ph ^ 1u, sm, P.status)) { ok = false; break; }
+                if (!wait1(&sm->k_empty[s], ph ^ 1u, sm)) { ok = false; break; }
                 ptx::mbar_arrive_expect_tx(&sm->k_full[s], kTileBytes + kSfBytes);
                 ptx::tma_load_2d(sm->k[s], &map_k, 0, w.k_row0 + j * kTile, &sm->k_full[s]);
                 ptx::bulk_load_1d(sm->sf_k[s], P.sf_k + (sfk_tile0 + j) * kSfBytes, kSfBytes, &sm->k_full[s]);
-                if (!wait1(&sm->v_empty[s], ph ^ 1u, sm, P.status)) { ok = false; break; }
+                if (!wait1(&sm->v_empty[s], ph ^ 1u, sm)) { ok = false; break; }
                 ptx::mbar_arrive_expect_tx(&sm->v_full[s], kTileBytes + kSfBytes);
                 ptx::tma_load_2d(sm->v[s], &map_v, w.v_x0 + j * 64, w.v_row0, &sm->v_full[s]);
                 ptx::bulk_load_1d(sm->sf_v[s], P.sf_v + (w.sfv_tile0 + j) * kSfBytes, kSfBytes, &sm->v_full[s]);
@@ -182,6 +229,7 @@ attention_short_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
         ptx::grid_wait();
         // an earlier CTA of this launch gave up: the waits of this one end soon instead of after their limit
         if (*reinterpret_cast<volatile uint32_t*>(P.status) != 0u) sm->abort_flag = 1u;
+        wait_watching(&sm->finished, 0, sm, P.status);
     } else if (warp == 1) {
         // =============================== S = Q K^T issuer ===============================
         // The whole warp runs the loop with warp-uniform state; one elected lane issues the tcgen05
@@ -191,23 +239,23 @@ attention_short_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
         if (TABLE) ptx::grid_wait();                           // the item table is written by the kernel before
         int ks = 0, n = 0;
         uint32_t t = 0;                                       // t: tiles of this CTA so far, over all of its items
-        uint32_t kph = 0, idx;
+        uint32_t kph = 0;
         bool ok = true;
-        for (uint32_t k = 0; ok && (idx = short_item(k)) < n_items; ++k) {
-            const int n_tiles = short_decode<TABLE>(P, idx).n_tiles;
+        for (ShortWalk<TABLE> walk(P, n_items); ok && walk.valid(P); walk.advance(P, n_items)) {
+            const int n_tiles = walk.n_tiles(P);
             if (n_tiles <= 0) continue;
             const int qb = n & 1;
             const uint64_t dq0 = d_sw64 + (ptx::smem_u32(qb ? sm->q1 : sm->q) >> 4);
             const uint32_t sfq = tmem + (qb ? kColSfQ1 : kColSfQ);
-            if (!wait_all(&sm->q_ready[qb], static_cast<uint32_t>(n >> 1) & 1u, sm, P.status)) break;
+            if (!wait_all(&sm->q_ready[qb], static_cast<uint32_t>(n >> 1) & 1u, sm)) break;
             ++n;
             ptx::tc_fence_after_sync();
             if (ptx::elect_one()) ptx::tmem_cp_sf(sfq, d_sf + (ptx::smem_u32(qb ? sm->sf_q1 : sm->sf_q) >> 4));
             __syncwarp();
             for (int j = 0; j < n_tiles; ++j, ++t) {
                 const int sb = static_cast<int>(t & 1u);
-                if (!wait_all(&sm->k_full[ks], kph, sm, P.status)) { ok = false; break; }
-                if (!wait_all(&sm->s_empty[sb], ((t >> 1) & 1u) ^ 1u, sm, P.status)) { ok = false; break; }
+                if (!wait_all(&sm->k_full[ks], kph, sm)) { ok = false; break; }
+                if (!wait_all(&sm->s_empty[sb], ((t >> 1) & 1u) ^ 1u, sm)) { ok = false; break; }
                 ptx::tc_fence_after_sync();
                 if (ptx::elect_one()) {
                     const uint32_t sfk = tmem + kColSfK + 4 * sb;
@@ -235,15 +283,15 @@ attention_short_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
         }
         __syncwarp();
         if (TABLE) ptx::grid_wait();
-        uint32_t t = 0, idx;
+        uint32_t t = 0;
         bool ok = true;
-        for (uint32_t k = 0; ok && (idx = short_item(k)) < n_items; ++k) {
-            const int n_tiles = short_decode<TABLE>(P, idx).n_tiles;
+        for (ShortWalk<TABLE> walk(P, n_items); ok && walk.valid(P); walk.advance(P, n_items)) {
+            const int n_tiles = walk.n_tiles(P);
             for (int j = 0; j < n_tiles; ++j, ++t) {
                 const int pb = static_cast<int>(t & 1u), vs = static_cast<int>(t % kStages);
-                if (!wait_all(&sm->v_full[vs], (t / kStages) & 1u, sm, P.status)) { ok = false; break; }
-                if (!wait_all(&sm->p_full[pb], (t >> 1) & 1u, sm, P.status)) { ok = false; break; }
-                if (!wait_all(&sm->o_ready[t & 3u], (t >> 2) & 1u, sm, P.status)) { ok = false; break; }
+                if (!wait_all(&sm->v_full[vs], (t / kStages) & 1u, sm)) { ok = false; break; }
+                if (!wait_all(&sm->p_full[pb], (t >> 1) & 1u, sm)) { ok = false; break; }
+                if (!wait_all(&sm->o_ready[t & 3u], (t >> 2) & 1u, sm)) { ok = false; break; }
                 ptx::tc_fence_after_sync();
                 if (ptx::elect_one()) {
                     const uint32_t sfp = tmem + kColSfP + 4 * pb;
@@ -256,6 +304,7 @@ attention_short_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
                     ptx::mma_mxf4(tmem + kColO, dp0 + 2, dv0 + 2, ptx::mxf4_idesc(144, 2), sfp | (2u << 30), sfv | (2u << 30), 1u);
                     ptx::mma_commit(&sm->p_empty[pb]);
                     ptx::mma_commit(&sm->v_empty[vs]);
+                    sm->progress = t + 1u;
                 }
                 __syncwarp();
             }
@@ -269,31 +318,25 @@ attention_short_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
     const int quarter = warp & 3;
     const uint32_t row = quarter * 32 + lane;
     const uint32_t o_addr = tmem + (static_cast<uint32_t>(quarter * 32) << 16) + kColO;
+    // this lane's row of the staging: 16-byte pieces, their order turned by the row
+    uint8_t* const my_stage = sm->stage[0] + row * 128;
+    const uint32_t turn = (row & 7u) * 16u;
     ptx::grid_wait();
-    uint32_t t = 0, idx;
+    uint32_t t = 0;
     bool ok = true;
     if (lane == 0) ptx::mbar_arrive(&sm->o_ready[0]);         // the first tile overwrites the accumulator
     __syncwarp();
-    for (uint32_t k = 0; ok && (idx = short_item(k)) < n_items; ++k) {
-        const ShortItem w = short_decode<TABLE>(P, idx);
-        uint64_t my_dst = 0ull;                               // this lane's row of the output, if it exists
-        if (TABLE && w.packed) {
-            const int gq = static_cast<int>(row) / static_cast<int>(w.Sq), token = static_cast<int>(row) - gq * static_cast<int>(w.Sq);
-            if (gq < P.Hq / P.Hkv) my_dst = reinterpret_cast<uint64_t>(P.o + (w.o + gq * P.o_head + token * P.o_row));
-        } else if (w.q0 + static_cast<int64_t>(row) < w.Sq) {
-            my_dst = reinterpret_cast<uint64_t>(P.o + (w.o + (w.q0 + static_cast<int64_t>(row)) * P.o_row));
-        }
-        __syncwarp();
-        uint8_t* const stage = sm->stage + (row - lane) * kOutRowBytes;
-        if (w.n_tiles > 0) {
-            for (int j = 0; j < w.n_tiles; ++j, ++t) {
+    for (ShortWalk<TABLE> walk(P, n_items); ok && walk.valid(P); walk.advance(P, n_items)) {
+        const int n_tiles = walk.n_tiles(P);
+        if (n_tiles > 0) {
+            for (int j = 0; j < n_tiles; ++j, ++t) {
                 if (j == 0) continue;                         // released when the accumulator was free, below
-                if (!wait_all(&sm->a_bar[t & 3u][quarter], (t >> 2) & 1u, sm, P.status)) { ok = false; break; }
+                if (!wait_all(&sm->a_bar[t & 3u][quarter], (t >> 2) & 1u, sm)) { ok = false; break; }
                 const float alpha = sm->alpha[t & 3u][row];
                 if (__any_sync(0xffffffffu, alpha != 1.0f)) {
                     // The end of P~V of the tile before frees its V stage.  The parity says so only if the stage's use before has
                     // ended, and it has: the probability warps waited for it before they stored the codes of the tile two before.
-                    if (!wait_all(&sm->v_empty[(t - 1u) & 3u], ((t - 1u) >> 2) & 1u, sm, P.status)) { ok = false; break; }
+                    if (!wait_all(&sm->v_empty[(t - 1u) & 3u], ((t - 1u) >> 2) & 1u, sm)) { ok = false; break; }
                     ptx::tc_fence_after_sync();
                     const uint64_t alpha2 = pack2(alpha, alpha);
                     uint32_t oa[32], ob[32];
@@ -325,21 +368,23 @@ attention_short_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
                 if (lane == 0) ptx::mbar_arrive(&sm->o_ready[t & 3u]);
                 __syncwarp();
             }
-            // ---- final normalisation O = A / l: out of TMEM first, so that P~V of the next item may start, then to memory
-            if (!ok || !wait_all(&sm->v_empty[(t - 1u) & 3u], ((t - 1u) >> 2) & 1u, sm, P.status)) break;
+            // ---- final normalisation O = A / l: out of TMEM, so that P~V of the next item may start, into the staging
+            if (!ok || !wait_all(&sm->v_empty[(t - 1u) & 3u], ((t - 1u) >> 2) & 1u, sm)) break;
             ptx::tc_fence_after_sync();
             const uint32_t lcol = ptx::tmem_ld1(o_addr + 128);
             ptx::tmem_wait_ld();
             const float l = __uint_as_float(lcol);
             const float inv = l > 0.0f ? 1.0f / l : 0.0f;
-#pragma unroll
+            if (lane == 0) ptx::bulk_wait_read();             // the rows of the item before have left the staging
+            __syncwarp();
+#pragma unroll 1
             for (int c = 0; c < 4; ++c) {
                 uint32_t o[32];
                 ptx::tmem_ld32<0>(o_addr + 32 * c, o);
                 ptx::tmem_wait_ld();
 #pragma unroll
                 for (int i = 0; i < 8; ++i)
-                    *reinterpret_cast<float4*>(stage + lane * kOutRowBytes + 128 * c + 16 * i) =
+                    *reinterpret_cast<float4*>(my_stage + c * (kTile * 128) + ((16 * i) ^ turn)) =
                         make_float4(__uint_as_float(o[4 * i]) * inv, __uint_as_float(o[4 * i + 1]) * inv, __uint_as_float(o[4 * i + 2]) * inv, __uint_as_float(o[4 * i + 3]) * inv);
             }
             ptx::tc_fence_before_sync();
@@ -347,18 +392,40 @@ attention_short_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
             if (lane == 0) ptx::mbar_arrive(&sm->o_ready[t & 3u]);        // first tile of the next item, if there is one
         } else {
             // no visible key for the whole tile: rows are zero
-            for (int i = 0; i < 32; ++i) *reinterpret_cast<float4*>(stage + i * kOutRowBytes + 16 * lane) = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (lane == 0) ptx::bulk_wait_read();
             __syncwarp();
+#pragma unroll 1
+            for (int i = 0; i < 32; ++i) *reinterpret_cast<float4*>(my_stage + (i >> 3) * (kTile * 128) + (i & 7) * 16) = make_float4(0.f, 0.f, 0.f, 0.f);
         }
-        // through shared memory, inside the warp: a lane holds a row, and storing it from registers would touch 32 rows per instruction
-#pragma unroll 8
-        for (int r = 0; r < 32; ++r) {
-            const uint64_t dst = __shfl_sync(0xffffffffu, my_dst, r);
-            const float4 v = *reinterpret_cast<const float4*>(stage + r * kOutRowBytes + 16 * lane);
-            if (dst != 0ull) __stcs(reinterpret_cast<float4*>(dst) + lane, v);
+        // Rows out.  A warp's 32 rows are four boxes of 32 channels, which one lane hands to the copy engine: the warp goes on at
+        // once.  Rows of several heads, and in a packed batch the last rows of a sequence, whose box would reach into the next one,
+        // go the long way.
+        ptx::fence_proxy_async_smem();
+        __syncwarp();
+        const ShortItem w = short_decode<TABLE>(P, walk);
+        const int left = walk.Sq(P) - walk.q0(P) - 32 * quarter;              // rows from the warp's first on
+        if (!walk.packed() && (!TABLE || left >= 32)) {
+            if (left > 0 && lane == 0) {
+#pragma unroll
+                for (int c = 0; c < 4; ++c) ptx::tma_store_3d(&map_o, sm->stage[c] + 4096 * quarter, 32 * c, w.o_y + 32 * quarter, w.o_z);
+                ptx::bulk_commit();
+            }
+        } else if (TABLE) {
+            const int lq = walk.Sq(P), heads = walk.packed() ? P.Hq / P.Hkv : 1;
+#pragma unroll 4
+            for (int i = 0; i < 32; ++i) {
+                const int r = 32 * quarter + i, gq = walk.packed() ? r / lq : 0, token = walk.packed() ? r - gq * lq : walk.q0(P) + r;
+                const float4 v = *reinterpret_cast<const float4*>(sm->stage[lane >> 3] + r * 128 + (((lane ^ r) & 7) * 16));
+                if (gq < heads && token < lq) __stcs(reinterpret_cast<float4*>(P.o + (w.o + gq * P.o_head + token * P.o_row)) + lane, v);
+            }
         }
         __syncwarp();
     }
+    if (lane == 0) {
+        ptx::bulk_wait_read();                                // shared memory ends with the CTA
+        ptx::mbar_arrive(&sm->finished);
+    }
+    __syncwarp();
     } else {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 184;");
     const int quarter = warp & 3;                       // TMEM lane quarter this warp may touch
@@ -367,28 +434,27 @@ attention_short_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
     const uint32_t lane_base = static_cast<uint32_t>(quarter * 32) << 16;
     const ProducerConsts K = P.K;
     if (TABLE) ptx::grid_wait();
-    uint32_t base = 0, idx;                             // tiles of this CTA before the item: buffers and phases count over all items
+    uint32_t base = 0;                                  // tiles of this CTA before the item: buffers and phases count over all items
     bool ok = true;
+    bool in_flight = false;           // the scores of this tile were asked for at the end of the group's previous tile
     float r[128];
     const uint32_t s_addr = tmem + lane_base + kColS + 128 * group;
-    for (uint32_t k = 0; ok && (idx = short_item(k)) < n_items; ++k) {
-        const ShortItem w = short_decode<TABLE>(P, idx);
-        const int n_tiles = w.n_tiles;
+    for (ShortWalk<TABLE> walk(P, n_items); ok && walk.valid(P); walk.advance(P, n_items)) {
+        const int n_tiles = walk.n_tiles(P);
         if (n_tiles <= 0) continue;
-        const int64_t token = TABLE && w.packed ? static_cast<int>(row) % static_cast<int>(w.Sq) : w.q0 + static_cast<int64_t>(row);
-        const int64_t sees = P.causal ? token + w.Sk - w.Sq : w.Sk - 1;
-        const Index limit = static_cast<Index>(sees > w.Sk - 1 ? w.Sk - 1 : sees < -1 ? -1 : sees);   // last visible key of this row
-        bool in_flight = false;           // the scores of this tile were asked for at the end of the group's previous tile
+        const int token = walk.packed() ? static_cast<int>(row) % walk.Sq(P) : walk.q0(P) + static_cast<int>(row);
+        const int sees = P.causal ? token + walk.Sk(P) - walk.Sq(P) : walk.Sk(P) - 1;
+        const int limit = min(max(sees, -1), walk.Sk(P) - 1);   // last visible key of this row
         __syncwarp();
 
-        for (Index j = static_cast<Index>((base & 1u) ^ static_cast<uint32_t>(group)); j < n_tiles; j += 2) {
+        for (int j = static_cast<int>((base & 1u) ^ static_cast<uint32_t>(group)); j < n_tiles; j += 2) {
             const uint32_t t = base + static_cast<uint32_t>(j);
             const int sb = group;                                         // S, P and exchange buffers belong to the group
             const uint32_t ph2 = (t >> 1) & 1u;
 
             // ---- scores of tile j: TMEM -> registers (Algorithm 2, step 1 happened on the tensor core)
             if (!in_flight) {
-                if (!wait_all(&sm->s_full[sb], ph2, sm, P.status)) { ok = false; break; }
+                if (!wait_all(&sm->s_full[sb], ph2, sm)) { ok = false; break; }
                 ptx::tc_fence_after_sync();
                 ptx::tmem_ld32f<0>(s_addr, r);
                 ptx::tmem_ld32f<32>(s_addr + 32, r);
@@ -405,11 +471,16 @@ attention_short_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
                 if (j > 0 && have_prev) m_prev = sm->runmax[sb ^ 1][row];
                 ptx::tmem_wait_ld();
                 ptx::tc_fence_before_sync();          // the S buffer is handed back with the joint publication below
-                const Index last = limit - j * kTile;     // last visible key of the row inside the tile
+                const int last = limit - j * kTile;       // last visible key of the row inside the tile
                 if (__any_sync(0xffffffffu, last < 127)) {     // diagonal or ragged tile: keys past the row's limit are masked in place
 #pragma unroll
-                    for (int i = 0; i < 128; ++i)
-                        if (i > last) r[i] = -INFINITY;
+                    for (int g = 0; g < 4; ++g) {          // a bit per key: predicates come out of a word seven at a time
+                        const int n = last - 32 * g + 1;   // keys of the block that the row sees
+                        const uint32_t bits = n >= 32 ? 0xffffffffu : n <= 0 ? 0u : (1u << n) - 1u;
+#pragma unroll
+                        for (int i = 0; i < 32; ++i)
+                            if ((bits & (1u << i)) == 0u) r[32 * g + i] = -INFINITY;
+                    }
                 }
             }
 #pragma unroll
@@ -417,7 +488,7 @@ attention_short_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
 
             // ---- running row maximum (Eq. rowmax-update): handed over from the group that owns tile j-1
             if (!have_prev) {
-                if (!wait_all(&sm->a_bar[(t - 1u) & 3u][quarter], ((t - 1u) >> 2) & 1u, sm, P.status)) { ok = false; break; }
+                if (!wait_all(&sm->a_bar[(t - 1u) & 3u][quarter], ((t - 1u) >> 2) & 1u, sm)) { ok = false; break; }
                 if (j > 0) m_prev = sm->runmax[sb ^ 1][row];
             }
             float m_new = fmaxf(fmaxf(m_prev, bmax[0]), max3(bmax[1], bmax[2], bmax[3]));
@@ -450,16 +521,16 @@ attention_short_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
                 uint32_t byte;
                 produce32<PRODUCER>(&r[g * 32], bmax[g], m_s, K, codes, byte);
                 if (g == 0 && !have_p) {      // P~V of tile j-2 must have finished: it reads the group's P buffer
-                    if (!wait_all(&sm->p_empty[sb], ph2 ^ 1u, sm, P.status)) { ok = false; break; }
+                    if (!wait_all(&sm->p_empty[sb], ph2 ^ 1u, sm)) { ok = false; break; }
                 }
                 *reinterpret_cast<uint4*>(sm->p[sb] + code_tile_offset(row, g)) = codes;
                 sfword |= byte << (8 * g);
             }
             if (!ok) break;               // the bounded wait inside the block loop gave up
             *reinterpret_cast<uint32_t*>(sm->sf_p[sb] + (row & 31u) * 16u + (row >> 5) * 4u) = sfword;
-            // The registers are free: if S of the group's next tile is there already (it is as a rule, S runs ahead),
-            // its scores set out now and travel while the operand is handed over and the loop turns.
-            in_flight = j + 2 < n_tiles && ptx::mbar_try_wait(&sm->s_full[sb], ph2 ^ 1u);
+            // The registers are free: if S of the group's next tile, of this item or of one after it, is there already (it is as a
+            // rule, S runs ahead), its scores set out now and travel while the operand is handed over and the loop turns.
+            in_flight = ptx::mbar_test_wait(&sm->s_full[sb], ph2 ^ 1u);
             if (in_flight) {
                 ptx::tc_fence_after_sync();
                 ptx::tmem_ld32f<0>(s_addr, r);
@@ -472,8 +543,8 @@ attention_short_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
             if (lane == 0) ptx::mbar_arrive(&sm->p_full[sb]);
         }
         base += static_cast<uint32_t>(n_tiles);
-        ptx::tmem_wait_ld();              // nothing may be in flight when a bounded wait gave up inside the loop
     }
+    ptx::tmem_wait_ld();                  // nothing may be in flight when a bounded wait gave up inside the loop
     }
 
     ptx::tc_fence_before_sync();

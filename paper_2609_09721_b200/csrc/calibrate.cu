@@ -66,7 +66,7 @@ exact_attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
                        float* __restrict__ o, int heads, int Hq, int Hkv, int Sq, int Sk, int causal, float sigma, int inject_skip_loads)
 {
     extern __shared__ uint8_t smem_raw[];
-    ExactSmem* const sm = reinterpret_cast<ExactSmem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
+    ExactSmem* const sm = reinterpret_cast<ExactSmem*>(smem_raw + ptx::smem_round_up(smem_raw, 1024u));
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int bh = static_cast<int>(blockIdx.x % static_cast<unsigned>(heads)), hkv_row = (bh / Hq) * Hkv + (bh % Hq) / (Hq / Hkv);
     const int q0 = static_cast<int>((gridDim.x - 1u - blockIdx.x) / static_cast<unsigned>(heads)) * kTile;      // long rows first

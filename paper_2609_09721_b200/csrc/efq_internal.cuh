@@ -57,7 +57,7 @@ struct QuantJob {
 // The work items of one query tile of one sequence, one per head that owns it, in the order the fused forward takes them.
 // The host lists the tiles (heaviest first); the quantiser's launch spreads them into the item table.
 struct ItemGroup {
-    int32_t first_item, seq, qt;
+    int32_t first_item, seq, qt, n_tiles, Sq, Sk, packed;
 };
 struct ItemDesc;
 
@@ -82,12 +82,16 @@ struct SeqDesc {
     int32_t k_row0, Sk_pad;  // the same for K
     int32_t k_col0;          // first key of the sequence along the key axis of the V^T code matrix (a multiple of 128)
     int32_t packed;          // 1: the query heads of a KV group share one 128-row query tile (few query tokens)
+    int32_t token0, pad;     // its first query token in the batch
 };
-// One work item (CTA) of the fused forward over a packed batch.
-struct ItemDesc {
+// One work item of the fused forward over a packed batch.  What every role needs at once stands here, the rest in the sequence
+// table: a CTA that goes from item to item has the next one's entry loaded in time.
+struct __align__(16) ItemDesc {
     int32_t seq;             // index into the sequence table
     int32_t qt;              // query tile inside the sequence (0 when packed)
     int32_t head;            // query head, or KV head when packed
+    int32_t n_tiles;         // KV tiles that it walks
+    int32_t Sq, Sk, packed;  // of its sequence
     int32_t pad;
 };
 

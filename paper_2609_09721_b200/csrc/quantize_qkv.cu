@@ -153,7 +153,7 @@ __global__ void __launch_bounds__(256) quantize_jobs_kernel(const QuantJob* __re
             if (__ldg(&groups[mid].first_item) <= item) lo = mid; else hi = mid;
         }
         const ItemGroup g = groups[lo];
-        items[item] = ItemDesc{g.seq, g.qt, item - g.first_item, 0};
+        items[item] = ItemDesc{g.seq, g.qt, item - g.first_item, g.n_tiles, g.Sq, g.Sk, g.packed, 0};
         return;
     }
     int lo = 0, hi = n_jobs;                  // first_cta[lo] <= cta < first_cta[hi]
