@@ -272,9 +272,9 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
 
     // Register budget: the probability warpgroups take what the other two give up.  setmaxnreg moves registers
     // inside the CTA's own allocation only (512 threads x 128 at launch = 16 x 128 per lane), so the budgets must
-    // add up to no more than that: 4 x 56 + 8 x 184 + 4 x 88 = 2048.  A role that asks for more waits for good.
+    // add up to no more than that: 4 x 32 + 8 x 184 + 4 x 112 = 2048.  A role that asks for more waits for good.
     if (warp < 4) {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 32;");
     if (run && warp == 0 && lane == 0) {
         // =============================== TMA producer (one thread) ===============================
         // The operands come from the kernel before.  Whatever else this kernel writes or reads follows from the loads.
@@ -377,9 +377,11 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
     // beside the code generation of tile j instead of inside it.  A quarter without growth releases P~V_j at once, so it
     // may run behind P~V_{j-1} without a gap.  Bound: P~V waits for this step, and what takes its time is the latency of
     // the TMEM accesses and the issue slots that the probability warps leave.  So the load of the next 32 columns is on
-    // its way while 32 are multiplied and stored.  S = 16384 (causal, 32 heads): 1589 us with one buffer and 56 registers
-    // (which spilled), 1509 with 88 registers, 1497 with two buffers; 64 columns at a time spills again (1885).
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 88;");
+    // its way while 32 are multiplied and stored (S = 16384, causal, 32 heads, when this form was taken: 1509 -> 1497 us; 64 columns
+    // at a time 1885).  Registers of the three kinds of warp, measured on the persistent form, S = 16384 / S = 32760 not causal / 512 keys:
+    // 56, 184, 88 (which spills) 1339 us / 7491 / 218; 48, 184, 96 1315 / 7340 / 214; 40, 184, 104 1306 / 7327 / 207; 32, 184, 112 1298 /
+    // 7301 / 207; 24, 184, 120 1318 / 7401 / 209; 40, 176, 120 1327 / 7399 / 200; 40, 192, 88 1356 / 7506 / 223.
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 112;");
     const int quarter = warp & 3;
     const uint32_t row = quarter * 32 + lane;
     const uint32_t o_addr = tmem + (static_cast<uint32_t>(quarter * 32) << 16) + kColO;
@@ -795,18 +797,17 @@ cudaError_t launch_one(dim3 grid, size_t smem, cudaStream_t stream, const CUtens
     return launch_overlapped(attention_fwd_kernel<PRODUCER, DEBUG>, grid, kThreads, smem, stream, mq, mk, mv, P);
 }
 
-// Short KV walks and more query tiles than SMs: persistent CTAs (the measurements are in attention_short.cuh).  The line lies where
-// both forms take the same time: 40 KV tiles for the affine rule, 16 for its table form, 64 for the plain exponentials (1, 2); the
-// folded ones gain at every length.  A [B, H, S, d] problem is judged by the mean walk of a query tile, half of a causal square, a
-// packed batch by its longest sequence: nothing up to the line is slower for it, though a batch of short sequences with one long
-// one would gain past it (63 of 64 to 500 tokens and one of 6000, causal: 530 -> 451 us for the affine rule).
+// More query tiles than SMs: persistent CTAs, at every length of the KV walk (the measurements are in attention_short.cuh); with
+// fewer, a CTA has one item and nothing to overlap it with, and the form made for one starts sooner (one head, causal: 1024 tokens
+// 13.4 us against 13.9, 4096 30.5 / 32.5, 16384 97.0 / 100.5).  Only the table form of the rule loses in long walks: 24 heads,
+// 8000 queries, not causal, 4096 keys 497 us with one CTA per tile, 478 persistent, 8192 keys 916 / 924, 12288 keys 1331 / 1368;
+// its line is at a mean walk of 48 tiles.  A packed batch is judged by its longest sequence.
 // P.Sk: the keys of the problem or, with P.Sq = 0, of the longest sequence.
 bool use_short(int producer, bool debug, int64_t items, int sms, const FwdParams& P)
 {
     if (debug || producer == 6 || P.packed || items <= sms) return false;
-    const int64_t tiles = producer == 0 ? 40 : producer == 3 ? 16 : producer <= 2 ? 64 : 1 << 24;
     const int64_t mean = P.causal ? P.Sk - std::min(P.Sq, P.Sk) / 2 : P.Sk;
-    return mean <= tiles * kTile;
+    return producer != 3 || mean <= 48 * kTile;
 }
 
 template <int PRODUCER, bool TABLE>

@@ -1,28 +1,25 @@
-// Fused forward for short KV walks: the kernel of attention_fwd.cu (which includes this file) with persistent CTAs.
+// Fused forward with persistent CTAs: the kernel of attention_fwd.cu (which includes this file) for more query tiles than SMs.
 //
 // A CTA of attention_fwd_kernel spends about 10000 cycles outside its tiles: start, barriers, TMEM, the latency of the first
 // loads and scores, the last P~V, the rows on their way out.  Against 512 keys, 4 tiles of about 1500 cycles, that is more than
 // the work.  Here one CTA per SM walks a list of query tiles and nothing of that stands between two of them: Q is
 // double-buffered and loads run ahead into the next item, S of its first tiles is computed while the last codes of this one
-// are generated, and the rescaling warps write the finished rows while the probability warps are in the next item.  The
+// are generated, and the rescaling warps take the finished rows out while the probability warps are in the next item.  The
 // tile counter t runs over all items of the CTA: it picks buffers and phases, the tile j inside the item picks the keys.
 // Everything else, the arithmetic above all, is that of attention_fwd_kernel, and so is the result, bit for bit.
 //
-// Why not for all shapes: in the steady state the looped form is 3 % slower.  Measured for the affine rule against the other kernel (whole
-// call, 24 heads, 16000 queries, not causal): 128 keys 153 -> 89 us, 256 keys 164 -> 111, 512 keys 195 -> 140, 1024 keys
-// 255 -> 211, 2048 keys 373 -> 342, 3072 keys 487 -> 459, 4096 keys 604 -> 583, 6144 keys 834 -> 827, 8192 keys 1064 -> 1070,
-// 16384 keys 1988 -> 2052.  Causal, 32 heads: 32 x 128 tokens 60 -> 39 us, 4 x 1024 tokens 74 -> 61, 2048 tokens 51 -> 46, 4096
-// tokens 133 -> 129, 8192 tokens 428 -> 421, 16384 tokens 1466 -> 1472.
-// Packed batches, 32 / 8 heads: 64 sequences of 64 to 128 tokens 132 -> 94 us; 16 of 100 to 3000 343 -> 300 causal, 448 -> 420 not;
-// 16 of 500 to 5120 961 -> 884 and 1395 -> 1324; 8 x 5120 1590 -> 1504 and 2517 -> 2426.
-// The table form of the rule loses more in the loop.  24 heads, 8000 queries, not causal: 1024 keys 181 -> 164 us, 1536 238 -> 228, 2048
-// 296 -> 291, 3072 410 -> 416, 4096 524 -> 540; causal: 4096 tokens 205 -> 204, 8192 698 -> 708.  Packed: 8 x 2000 tokens 534 -> 521
-// causal, 797 -> 772 not; 16 of 100 to 2000 286 -> 265, 373 -> 369; 16 of 100 to 3000 448 -> 423 but 626 -> 637.
-// The plain exponentials (scale4; scale6 is the same within 1 %): causal S = 4096 195 -> 187 us, 8192 657 -> 637, 16384 2364 -> 2343,
-// 32768 8871 -> 8985; not causal, 24 heads, 8000 queries: 4096 keys 506 -> 481, 8192 932 -> 922, 12288 1354 -> 1358, 16384 1771 -> 1802.
-// Packed: 6 of 500 to 3000 tokens 340 -> 322 causal, 501 -> 479 not; 4 x 8192 2630 -> 2619, 4693 -> 4659; 4 x 16384 9435 -> 9581.
-// The folded ones gain at every length, their code generation hides what the loop costs: causal S = 4096 157 -> 143, 16384 1859 -> 1765,
-// 131072 103.3 -> 101.9 ms; 4 x 16384 tokens packed 7515 -> 7111 us; with the polynomial 131072 108.1 -> 105.7 ms.
+// What bounds it: the probability warps in long walks; in short ones what stands between the last P~V of an item and the first
+// rescaling of the next, and the size of the code.  The five kinds of warp run different code at the same time and evict one
+// another from the instruction cache: at 75 KB, 40 % of its lookups missed and warps without an instruction were the largest stall
+// (256 keys).  Hence waits of a few instructions, masks from a bit word, loops that are not unrolled, no divisions from item to
+// item.
+//
+// Measured against one CTA per tile, whole call, us.  Affine rule, 24 heads, 16000 queries, not causal: 128 keys 146 -> 65, 256 keys
+// 159 -> 83, 512 191 -> 109, 1024 254 -> 167, 2048 378 -> 288, 4096 619 -> 527, 16384 1998 -> 1897; causal, 32 heads: 32 x 128 tokens
+// 55 -> 32, 2048 tokens 49 -> 37, 4096 129 -> 107, 16384 1436 -> 1300, 32768 5228 -> 4952.  Packed, 32 / 8 heads, causal: 64 of 64 to
+// 128 tokens 128 -> 93, 16 of 100 to 3000 548 -> 383 (not causal 743 -> 580), 4 x 8192 1702 -> 1460, 4 x 16384 5772 -> 5355.
+// Plain exponentials: 4096 keys 500 -> 450, 16384 keys 1738 -> 1696, causal 4096 tokens 187 -> 162, 16384 2300 -> 2158; folded ones
+// 401 -> 355, 1358 -> 1315, 152 -> 129, 1806 -> 1660.
 #pragma once
 
 struct __align__(1024) ShortSmem : Smem {
@@ -190,9 +187,9 @@ attention_short_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
     }
     const uint32_t tmem = warp == 0 ? 0u : sm->tmem_base;
 
-    // 4 x 56 + 8 x 184 + 4 x 88 = 2048 registers per lane, what the launch holds
+    // 4 x 32 + 8 x 184 + 4 x 112 = 2048 registers per lane, what the launch holds
     if (warp < 4) {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 32;");
     if (warp == 0 && lane == 0) {
         // =============================== TMA producer (one thread) ===============================
         // The operands come from the kernel before.  Whatever else this kernel writes or reads follows from the loads.
@@ -314,13 +311,25 @@ attention_short_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
     // =============================== historical rescaling (Eq. alpha), rows out ===============================
     // One warp per TMEM lane quarter: the accumulator rows that grew, as in attention_fwd_kernel, and the finished rows of an
     // item, whose way out takes no time from the probability warps here.
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 88;");
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 112;");
     const int quarter = warp & 3;
     const uint32_t row = quarter * 32 + lane;
     const uint32_t o_addr = tmem + (static_cast<uint32_t>(quarter * 32) << 16) + kColO;
     // this lane's row of the staging: 16-byte pieces, their order turned by the row
     uint8_t* const my_stage = sm->stage[0] + row * 128;
     const uint32_t turn = (row & 7u) * 16u;
+    // The warp's 32 rows of a finished item wait in the staging as four boxes of 32 channels, which one lane hands to the copy
+    // engine.  That takes it some 1500 cycles, in which the first P~V of the next item would wait for its rescaling: so it is done
+    // after that rescaling, while P~V runs (32 heads, causal, 16384 tokens 1393 -> 1328 us; 24 heads, 32760 queries, 512 keys 221 -> 210).
+    int box_y = -1, box_z = 0;
+    auto send_rows = [&]() {
+        if (box_y >= 0 && lane == 0) {
+#pragma unroll
+            for (int c = 0; c < 4; ++c) ptx::tma_store_3d(&map_o, sm->stage[c] + 4096 * quarter, 32 * c, box_y, box_z);
+            ptx::bulk_commit();
+        }
+        box_y = -1;
+    };
     ptx::grid_wait();
     uint32_t t = 0;
     bool ok = true;
@@ -366,6 +375,7 @@ attention_short_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
                 }
                 __syncwarp();
                 if (lane == 0) ptx::mbar_arrive(&sm->o_ready[t & 3u]);
+                send_rows();
                 __syncwarp();
             }
             // ---- final normalisation O = A / l: out of TMEM, so that P~V of the next item may start, into the staging
@@ -375,6 +385,7 @@ attention_short_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
             ptx::tmem_wait_ld();
             const float l = __uint_as_float(lcol);
             const float inv = l > 0.0f ? 1.0f / l : 0.0f;
+            send_rows();
             if (lane == 0) ptx::bulk_wait_read();             // the rows of the item before have left the staging
             __syncwarp();
 #pragma unroll 1
@@ -392,24 +403,21 @@ attention_short_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
             if (lane == 0) ptx::mbar_arrive(&sm->o_ready[t & 3u]);        // first tile of the next item, if there is one
         } else {
             // no visible key for the whole tile: rows are zero
+            send_rows();
             if (lane == 0) ptx::bulk_wait_read();
             __syncwarp();
 #pragma unroll 1
             for (int i = 0; i < 32; ++i) *reinterpret_cast<float4*>(my_stage + (i >> 3) * (kTile * 128) + (i & 7) * 16) = make_float4(0.f, 0.f, 0.f, 0.f);
         }
-        // Rows out.  A warp's 32 rows are four boxes of 32 channels, which one lane hands to the copy engine: the warp goes on at
-        // once.  Rows of several heads, and in a packed batch the last rows of a sequence, whose box would reach into the next one,
-        // go the long way.
+        // Rows out: as boxes (send_rows), later.  Rows of several heads, and in a packed batch the last rows of a sequence, whose
+        // box would reach into the next one, go the long way.
         ptx::fence_proxy_async_smem();
         __syncwarp();
         const ShortItem w = short_decode<TABLE>(P, walk);
         const int left = walk.Sq(P) - walk.q0(P) - 32 * quarter;              // rows from the warp's first on
         if (!walk.packed() && (!TABLE || left >= 32)) {
-            if (left > 0 && lane == 0) {
-#pragma unroll
-                for (int c = 0; c < 4; ++c) ptx::tma_store_3d(&map_o, sm->stage[c] + 4096 * quarter, 32 * c, w.o_y + 32 * quarter, w.o_z);
-                ptx::bulk_commit();
-            }
+            if (left > 0) { box_y = w.o_y + 32 * quarter; box_z = w.o_z; }
+            if (n_tiles <= 1) send_rows();                    // the next item may have no rescaling either
         } else if (TABLE) {
             const int lq = walk.Sq(P), heads = walk.packed() ? P.Hq / P.Hkv : 1;
 #pragma unroll 4
@@ -421,6 +429,7 @@ attention_short_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
         }
         __syncwarp();
     }
+    send_rows();
     if (lane == 0) {
         ptx::bulk_wait_read();                                // shared memory ends with the CTA
         ptx::mbar_arrive(&sm->finished);
