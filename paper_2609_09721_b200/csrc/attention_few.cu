@@ -174,9 +174,18 @@ __global__ void __launch_bounds__(kFewThreads, N <= 8 ? 4 : 3) few_scores_kernel
     few_setup(sm, warp);
     ptx::grid_wait();                // the kernels before: inputs, and the workspace of an earlier call
     ptx::grid_launch_next();
-    const Unit u = find_unit(P, static_cast<int>(blockIdx.x));
+    // A block takes 2^-score_split of a chunk: the scores of a tile need nothing of another, and a few chunks do not fill the chip.
+    Unit u = find_unit(P, static_cast<int>(blockIdx.x) >> P.score_split);
     const int R = P.G * u.Sq;
+    const int per = max(1, few_chunk_tiles(u.Sk_pad / kTile, R) >> P.score_split), part = static_cast<int>(blockIdx.x) & ((1 << P.score_split) - 1);
+    u.j0 = min(u.j0 + part * per, u.j1);
+    u.j1 = min(u.j0 + per, u.j1);
     if (blockIdx.x == 0) P.status[tid] = 0u;
+    if (u.j0 == u.j1) {              // shorter chunks have fewer parts
+        __syncthreads();
+        if (warp == 0) ptx::tmem_dealloc(sm->tmem_base, kFewTmemCols);
+        return;
+    }
     // K: a quad of lanes takes a key, a lane every fourth 16-byte piece of it - a load instruction reads 64 contiguous
     // bytes of every key - and so a quarter of each of the four blocks
     const int quad = tid & 3, key_in_tile = tid >> 2;
@@ -595,7 +604,7 @@ template <int N>
 cudaError_t launch_n(int producer, const FewParams& P, cudaStream_t stream)
 {
     const dim3 grid(static_cast<unsigned>(P.n_units));
-    cudaError_t e = launch_overlapped(few_scores_kernel<N>, grid, kFewThreads, 0, stream, P);
+    cudaError_t e = launch_overlapped(few_scores_kernel<N>, dim3(grid.x << P.score_split), kFewThreads, 0, stream, P);
     if (e != cudaSuccess) return e;
     switch (producer) {
         case 0: e = launch_overlapped(few_values_kernel<N, 0>, grid, kFewThreads, 0, stream, P); break;
@@ -613,9 +622,14 @@ cudaError_t launch_n(int producer, const FewParams& P, cudaStream_t stream)
 
 }  // namespace
 
-cudaError_t launch_few(int producer, const FewParams& P, cudaStream_t stream)
+cudaError_t launch_few(int producer, FewParams& P, cudaStream_t stream)
 {
     if (P.n_units <= 0) return cudaErrorInvalidValue;
+    // Scores in halves, quarters, eighths of a chunk as long as the blocks are all on the chip together (three on each of 148 SMs; four
+    // or eight made no difference).  One head of 60000 keys 33.4 -> 26.7 us, four of 20000 33.4 -> 28.2, 16 rows of 4000 36.9 -> 26.6,
+    // 20 rows of 9000 47.0 -> 37.3, a context of 8191 keys with eight heads 20.9 -> 18.8.
+    P.score_split = 0;
+    while (P.score_split < 3 && (static_cast<int64_t>(P.n_units) << (P.score_split + 1)) <= 3 * 148) ++P.score_split;
     if (P.row_cap <= 8) return launch_n<8>(producer, P, stream);
     if (P.row_cap <= 16) return launch_n<16>(producer, P, stream);
     return launch_n<24>(producer, P, stream);

@@ -148,6 +148,7 @@ struct FewParams {
     int64_t q_seq, q_head, q_row, k_seq, k_head, k_row;    // strides in elements
     int32_t row_cap;                           // query rows the workspace holds per KV head (the most of any sequence)
     int32_t n_units, n_heads;                  // chunks times KV heads, and KV heads, of all sequences
+    int32_t score_split;                       // a chunk's scores are the work of 2^score_split blocks (set by launch_few)
     float rescale_threshold;
     ProducerConsts K;
     float *scores, *block_max, *stats;         // workspace
@@ -162,6 +163,6 @@ struct FewParams {
 struct FewPlan { size_t scores, block_max, stats, total; };   // offsets from a 1024-byte aligned base
 FewPlan plan_few(int64_t units, int64_t keys_padded_all_heads, int rows);
 // Clears the status words.
-cudaError_t launch_few(int producer, const FewParams& P, cudaStream_t stream);
+cudaError_t launch_few(int producer, FewParams& P, cudaStream_t stream);
 
 }  // namespace efq
