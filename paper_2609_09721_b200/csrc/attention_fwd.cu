@@ -302,6 +302,7 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         ptx::grid_wait();
         // an earlier CTA of this launch gave up: the waits of this one end soon instead of after their limit
         if (*reinterpret_cast<volatile uint32_t*>(P.status) != 0u) sm->abort_flag = 1u;
+        ptx::grid_launch_next();
         if (run) wait_watching(&sm->o_done, 0, sm, P.status);
     } else if (run && warp == 1) {
         // =============================== S = Q K^T issuer ===============================

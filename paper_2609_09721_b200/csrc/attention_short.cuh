@@ -226,6 +226,7 @@ attention_short_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
         ptx::grid_wait();
         // an earlier CTA of this launch gave up: the waits of this one end soon instead of after their limit
         if (*reinterpret_cast<volatile uint32_t*>(P.status) != 0u) sm->abort_flag = 1u;
+        ptx::grid_launch_next();
         wait_watching(&sm->finished, 0, sm, P.status);
     } else if (warp == 1) {
         // =============================== S = Q K^T issuer ===============================

@@ -243,6 +243,8 @@ exact_attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
 __global__ void __launch_bounds__(256) error_sums_kernel(const float* __restrict__ a, const float* __restrict__ r,
                                                          int64_t n, double* sums)
 {
+    ptx::grid_wait();
+    ptx::grid_launch_next();
     double d2 = 0.0, r2 = 0.0;
     auto add = [&](float af, float rf) {
         const double x = static_cast<double>(af), y = static_cast<double>(rf);
@@ -340,8 +342,7 @@ static cudaError_t launch_error_sums(const float* a, const float* ref, int64_t n
 {
     int64_t blocks = (n + 2047) / 2048;
     if (blocks > 148 * 8) blocks = 148 * 8;
-    efq::error_sums_kernel<<<static_cast<unsigned>(blocks), 256, 0, s>>>(a, ref, n, sums);
-    return cudaGetLastError();
+    return efq::launch_overlapped(efq::error_sums_kernel, dim3(static_cast<unsigned>(blocks)), 256, 0, s, a, ref, n, sums);
 }
 
 extern "C" efq_status_t efq_relative_error(const float* a, const float* ref, int64_t n, double* sums, void* stream)
