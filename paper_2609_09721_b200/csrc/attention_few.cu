@@ -88,6 +88,21 @@ __device__ __forceinline__ Unit find_unit(const FewParams& P, int id)
     return u;
 }
 
+// 2^-split of a chunk for this block, whose index says which; false if the chunk, as the last of a sequence may be, is too short for it
+__device__ __forceinline__ bool take_part(Unit& u, int rows, int split)
+{
+    const int per = max(1, few_chunk_tiles(u.Sk_pad / kTile, rows) >> split), part = static_cast<int>(blockIdx.x) & ((1 << split) - 1);
+    u.j0 = min(u.j0 + part * per, u.j1);
+    u.j1 = min(u.j0 + per, u.j1);
+    return u.j0 < u.j1;
+}
+
+// The factors of one tile and row, where the values were taken tile by tile
+__device__ __forceinline__ float* tile_stat(const FewParams& P, const Unit& u, int tile, int row)
+{
+    return P.stats + (u.s_off / kTile + static_cast<int64_t>(tile) * P.row_cap + row) * kFewStatFloats;
+}
+
 __device__ __forceinline__ float warp_max(float x)
 {
     float m;
@@ -177,11 +192,9 @@ __global__ void __launch_bounds__(kFewThreads, N <= 8 ? 4 : 3) few_scores_kernel
     // A block takes 2^-score_split of a chunk: the scores of a tile need nothing of another, and a few chunks do not fill the chip.
     Unit u = find_unit(P, static_cast<int>(blockIdx.x) >> P.score_split);
     const int R = P.G * u.Sq;
-    const int per = max(1, few_chunk_tiles(u.Sk_pad / kTile, R) >> P.score_split), part = static_cast<int>(blockIdx.x) & ((1 << P.score_split) - 1);
-    u.j0 = min(u.j0 + part * per, u.j1);
-    u.j1 = min(u.j0 + per, u.j1);
+    const bool work = take_part(u, R, P.score_split);
     if (blockIdx.x == 0) P.status[tid] = 0u;
-    if (u.j0 == u.j1) {              // shorter chunks have fewer parts
+    if (!work) {
         __syncthreads();
         if (warp == 0) ptx::tmem_dealloc(sm->tmem_base, kFewTmemCols);
         return;
@@ -384,15 +397,18 @@ __device__ __forceinline__ void few_row_state(FewSmem* sm, const FewParams& P, i
     }
 }
 
-template <int N, int PRODUCER>
+// TILES: a block takes 2^-value_split of a chunk and leaves the product of every tile by itself, beside its factors, for the merge to
+// add up as the chunk's block would have (same operations, same order, same bits).
+template <int N, int PRODUCER, bool TILES>
 __global__ void __launch_bounds__(kFewThreads, 3) few_values_kernel(const __grid_constant__ FewParams P)
 {
     __shared__ FewSmem smem;
     FewSmem* const sm = &smem;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     ptx::grid_launch_next();
-    const Unit u = find_unit(P, static_cast<int>(blockIdx.x));
+    Unit u = find_unit(P, static_cast<int>(blockIdx.x) >> (TILES ? P.value_split : 0));
     const int R = P.G * u.Sq;
+    if (TILES && !take_part(u, R, P.value_split)) return;
     few_setup(sm, warp);
     const VTileLane L(warp, lane);
     uint4 vv[8];
@@ -443,6 +459,7 @@ __global__ void __launch_bounds__(kFewThreads, 3) few_values_kernel(const __grid
     constexpr int NH = N / 2;
     const int quarter = warp & 3, half = warp >> 2;
     float* s_src = P.scores + u.s_off + few_row_offset(half, n_tiles) + u.j0 * kTile + quarter * 32 + lane;
+    float* const tile_part = s_src;
     float x[NH];
     auto load_scores = [&]() {
 #pragma unroll
@@ -472,7 +489,12 @@ __global__ void __launch_bounds__(kFewThreads, 3) few_values_kernel(const __grid
         ptx::tmem_wait_ld();
         ptx::tc_fence_before_sync();
 #pragma unroll
-        for (int i = 0; i < NH; ++i) acc[i] = fmaf(acc[i], sm->alpha[t % kStateRing][2 * i + half], half ? d[2 * i + 1] : d[2 * i]);
+        for (int i = 0; i < NH; ++i) {
+            const float x = half ? d[2 * i + 1] : d[2 * i];
+            if (!TILES) acc[i] = fmaf(acc[i], sm->alpha[t % kStateRing][2 * i + half], x);
+            // the tile's scores may go, as below
+            else if (2 * i + half < R) tile_part[few_row_offset(2 * i, n_tiles) + t * kTile] = x;
+        }
     };
     const bool dump = P.has_dbg && u.seq == P.dbg.batch && u.head == P.dbg.head / P.G;
     for (int j = u.j0; j < u.j1; ++j) {
@@ -523,7 +545,14 @@ __global__ void __launch_bounds__(kFewThreads, 3) few_values_kernel(const __grid
         if (has_row) {
             sm->sf_b[buf][sf_tile_offset(my_row, quarter)] = static_cast<uint8_t>(byte);
             const float unit = byte != 0u ? __uint_as_float(byte << 23) : __uint_as_float(0x00400000u);
-            l_run = l_run * sm->alpha[slot][my_row] + (PRODUCER == 6 ? psum : static_cast<float>(count) * 0.5f * unit);
+            const float add = PRODUCER == 6 ? psum : __fmul_rn(static_cast<float>(count) * 0.5f, unit), alpha = sm->alpha[slot][my_row];
+            if (!TILES) {
+                l_run = __fmaf_rn(l_run, alpha, add);
+            } else {
+                float* const stat = tile_stat(P, u, j, my_row);
+                stat[quarter] = add;
+                if (quarter == 0) { stat[4] = sm->m_s[slot][my_row]; stat[5] = alpha; }
+            }
         }
         if (j + 1 < u.j1) load_scores();
         // ---- V^T operand of the tile
@@ -545,11 +574,10 @@ __global__ void __launch_bounds__(kFewThreads, 3) few_values_kernel(const __grid
 
     // ---- partial result of the chunk.  Its scores may go: the block's threads used the last of them before the barrier of the last
     // tile, and no other block reads them.
-    float* const part = s_src - (u.j1 - u.j0) * kTile;          // it has gone past the chunk's tiles
 #pragma unroll
     for (int i = 0; i < NH; ++i)
-        if (2 * i + half < R) part[few_row_offset(2 * i, n_tiles)] = acc[i];
-    if (has_row) {
+        if (!TILES && 2 * i + half < R) tile_part[few_row_offset(2 * i, n_tiles)] = acc[i];
+    if (!TILES && has_row) {
         float* const stat = P.stats + (static_cast<size_t>(blockIdx.x) * P.row_cap + my_row) * kFewStatFloats;
         stat[quarter] = l_run;
         if (quarter == 0) stat[4] = sm->m_s[(u.j1 - u.j0 - 1) % kStateRing][my_row];
@@ -559,6 +587,36 @@ __global__ void __launch_bounds__(kFewThreads, 3) few_values_kernel(const __grid
     if (warp == 0) ptx::tmem_dealloc(tmem, kFewTmemCols);
 }
 
+// What the merges share: a chunk's weight against the row's last maximum, and the row's sum over its partial sums.
+__device__ __forceinline__ float chunk_weight(float m, float m_last, const ProducerConsts& K)
+{
+    // equal maxima by comparison: both are infinite where the inputs or a score overflowed
+    return m == -INFINITY ? 0.0f : m == m_last ? 1.0f : ex2_approx(__fmul_rn(__fsub_rn(m, m_last), K.LOG2E));
+}
+__device__ __forceinline__ void add_chunk(float4& a, float& l, const float4& x, const float4& lp, float w)
+{
+    l = fmaf((lp.x + lp.y) + (lp.z + lp.w), w, l);
+    a.x = fmaf(x.x, w, a.x); a.y = fmaf(x.y, w, a.y); a.z = fmaf(x.z, w, a.z); a.w = fmaf(x.w, w, a.w);
+}
+struct MergeRow {
+    Unit u;              // the first chunk, whose length is that of all but the last
+    int first_id, row;
+    __device__ __forceinline__ MergeRow(const FewParams& P) : row(static_cast<int>(blockIdx.y))
+    {
+        const int head = static_cast<int>(blockIdx.x) % P.Hkv, seq = static_cast<int>(blockIdx.x) / P.Hkv;
+        first_id = head + (P.n_seqs == 0 ? seq * P.dense_chunks * P.Hkv : (P.seqs != nullptr ? P.seqs : P.inline_seqs)[seq].first_unit);
+        u = find_unit(P, first_id);
+    }
+    __device__ __forceinline__ void store(const FewParams& P, const float4 (&sum)[4][32], const float (&den)[4]) const
+    {
+        if (threadIdx.x >= 128u) return;
+        const float* s = reinterpret_cast<const float*>(sum) + threadIdx.x;
+        const float t = (s[0] + s[128]) + (s[256] + s[384]), d = (den[0] + den[1]) + (den[2] + den[3]);
+        const int g = row / u.Sq;
+        u.o[g * P.q_head + (row - g * u.Sq) * P.q_row + threadIdx.x] = t * (d > 0.0f ? 1.0f / d : 0.0f);
+    }
+};
+
 // Adds up the chunks of one row (a block per sequence, KV head and row): a warp takes every fourth chunk, a lane four
 // channels, so that all loads of a short list of chunks are in flight together.
 __global__ void __launch_bounds__(128) few_merge_kernel(const __grid_constant__ FewParams P)
@@ -566,16 +624,13 @@ __global__ void __launch_bounds__(128) few_merge_kernel(const __grid_constant__ 
     __shared__ float4 sum[4][32];
     __shared__ float den[4];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int row = static_cast<int>(blockIdx.y);
-    const int head = static_cast<int>(blockIdx.x) % P.Hkv, seq = static_cast<int>(blockIdx.x) / P.Hkv;
-    const int first_id = head + (P.n_seqs == 0 ? seq * P.dense_chunks * P.Hkv : (P.seqs != nullptr ? P.seqs : P.inline_seqs)[seq].first_unit);
-    const Unit u = find_unit(P, first_id);
+    const MergeRow r(P);
+    const Unit& u = r.u;
     ptx::grid_wait();
-    if (row >= P.G * u.Sq) return;
-    // the row's partial results: u is the first chunk, whose length is that of all but the last
-    const float4* const part = reinterpret_cast<const float4*>(P.scores + u.s_off + few_row_offset(row, u.Sk_pad / kTile)) + lane;
+    if (r.row >= P.G * u.Sq) return;
+    const float4* const part = reinterpret_cast<const float4*>(P.scores + u.s_off + few_row_offset(r.row, u.Sk_pad / kTile)) + lane;
     const int part_step = u.j1 * (kTile / 4);
-    const float* const stat = P.stats + (static_cast<size_t>(first_id) * P.row_cap + row) * kFewStatFloats;
+    const float* const stat = P.stats + (static_cast<size_t>(r.first_id) * P.row_cap + r.row) * kFewStatFloats;
     const size_t stat_step = static_cast<size_t>(P.Hkv) * P.row_cap * kFewStatFloats;
     const float m_last = __ldcg(stat + (u.n_chunks - 1) * stat_step + 4);
     float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -585,39 +640,96 @@ __global__ void __launch_bounds__(128) few_merge_kernel(const __grid_constant__ 
         const float m = __ldcg(stat + c * stat_step + 4);
         const float4 x = __ldcg(part + static_cast<int64_t>(c) * part_step);
         const float4 lp = __ldcg(reinterpret_cast<const float4*>(stat + c * stat_step));
-        const float lc = (lp.x + lp.y) + (lp.z + lp.w);
-        // equal maxima by comparison: both are infinite where the inputs or a score overflowed
-        const float w = m == -INFINITY ? 0.0f : m == m_last ? 1.0f : ex2_approx(__fmul_rn(__fsub_rn(m, m_last), P.K.LOG2E));
-        l = fmaf(lc, w, l);
-        a.x = fmaf(x.x, w, a.x); a.y = fmaf(x.y, w, a.y); a.z = fmaf(x.z, w, a.z); a.w = fmaf(x.w, w, a.w);
+        add_chunk(a, l, x, lp, chunk_weight(m, m_last, P.K));
     }
     sum[warp][lane] = a;
     if (lane == 0) den[warp] = l;
     __syncthreads();
-    const float* s = reinterpret_cast<const float*>(sum) + threadIdx.x;
-    const float t = (s[0] + s[128]) + (s[256] + s[384]), d = (den[0] + den[1]) + (den[2] + den[3]);
-    const int g = row / u.Sq;
-    u.o[g * P.q_head + (row - g * u.Sq) * P.q_row + threadIdx.x] = t * (d > 0.0f ? 1.0f / d : 0.0f);
+    r.store(P, sum, den);
+}
+
+// The same where the values were taken tile by tile: sixteen warps first make a chunk each of its tiles, with the operations of the
+// block that would have had it, then four of them add the chunks as above.
+constexpr int kMergeWarps = 16;
+__global__ void __launch_bounds__(32 * kMergeWarps) few_merge_tiles_kernel(const __grid_constant__ FewParams P)
+{
+    __shared__ float4 chunk_sum[kMergeWarps][32], chunk_den[kMergeWarps], sum[4][32];
+    __shared__ float chunk_max[kMergeWarps], den[4];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const MergeRow r(P);
+    const Unit& u = r.u;
+    ptx::grid_wait();
+    if (r.row >= P.G * u.Sq) return;
+    const int n_tiles = u.Sk_pad / kTile, per = u.j1;
+    const float4* const part = reinterpret_cast<const float4*>(P.scores + u.s_off + few_row_offset(r.row, n_tiles)) + lane;
+    const float m_last = __ldcg(tile_stat(P, u, n_tiles - 1, r.row) + 4);
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+    float l = 0.0f;
+    for (int c0 = 0; c0 < u.n_chunks; c0 += kMergeWarps) {
+        const int j0 = (c0 + warp) * per, tiles = min(per, n_tiles - j0);
+        if (tiles > 0) {
+            float4 d[kFewMaxChunk], add[kFewMaxChunk];
+            float2 f[kFewMaxChunk];                  // maximum, factor
+#pragma unroll
+            for (int t = 0; t < kFewMaxChunk; ++t)
+                if (t < tiles) {
+                    const float* const ts = tile_stat(P, u, j0 + t, r.row);
+                    d[t] = __ldcg(part + static_cast<int64_t>(j0 + t) * (kTile / 4));
+                    add[t] = __ldcg(reinterpret_cast<const float4*>(ts));
+                    f[t] = __ldcg(reinterpret_cast<const float2*>(ts + 4));
+                }
+            float4 x = make_float4(0.f, 0.f, 0.f, 0.f), lp = x;
+            float m = -INFINITY;
+#pragma unroll
+            for (int t = 0; t < kFewMaxChunk; ++t)
+                if (t < tiles) {
+                    m = f[t].x;
+                    x.x = fmaf(x.x, f[t].y, d[t].x); x.y = fmaf(x.y, f[t].y, d[t].y); x.z = fmaf(x.z, f[t].y, d[t].z); x.w = fmaf(x.w, f[t].y, d[t].w);
+                    lp.x = __fmaf_rn(lp.x, f[t].y, add[t].x); lp.y = __fmaf_rn(lp.y, f[t].y, add[t].y);
+                    lp.z = __fmaf_rn(lp.z, f[t].y, add[t].z); lp.w = __fmaf_rn(lp.w, f[t].y, add[t].w);
+                }
+            chunk_sum[warp][lane] = x;
+            if (lane == 0) { chunk_den[warp] = lp; chunk_max[warp] = m; }
+        }
+        __syncthreads();
+        if (warp < 4)
+            for (int c = warp; c < min(kMergeWarps, u.n_chunks - c0); c += 4)       // c0 is a multiple of four
+                add_chunk(a, l, chunk_sum[c][lane], chunk_den[c], chunk_weight(chunk_max[c], m_last, P.K));
+        __syncthreads();
+    }
+    if (warp < 4) {
+        sum[warp][lane] = a;
+        if (lane == 0) den[warp] = l;
+    }
+    __syncthreads();
+    r.store(P, sum, den);
+}
+
+template <int N, bool TILES>
+cudaError_t launch_values(int producer, const FewParams& P, cudaStream_t stream)
+{
+    const dim3 grid(static_cast<unsigned>(P.n_units) << P.value_split);
+    switch (producer) {
+        case 0: return launch_overlapped(few_values_kernel<N, 0, TILES>, grid, kFewThreads, 0, stream, P);
+        case 1: return launch_overlapped(few_values_kernel<N, 1, TILES>, grid, kFewThreads, 0, stream, P);
+        case 2: return launch_overlapped(few_values_kernel<N, 2, TILES>, grid, kFewThreads, 0, stream, P);
+        case 3: return launch_overlapped(few_values_kernel<N, 3, TILES>, grid, kFewThreads, 0, stream, P);
+        case 4: return launch_overlapped(few_values_kernel<N, 4, TILES>, grid, kFewThreads, 0, stream, P);
+        case 5: return launch_overlapped(few_values_kernel<N, 5, TILES>, grid, kFewThreads, 0, stream, P);
+        case 6: return launch_overlapped(few_values_kernel<N, 6, TILES>, grid, kFewThreads, 0, stream, P);
+        default: return cudaErrorInvalidValue;
+    }
 }
 
 template <int N>
 cudaError_t launch_n(int producer, const FewParams& P, cudaStream_t stream)
 {
-    const dim3 grid(static_cast<unsigned>(P.n_units));
-    cudaError_t e = launch_overlapped(few_scores_kernel<N>, dim3(grid.x << P.score_split), kFewThreads, 0, stream, P);
+    cudaError_t e = launch_overlapped(few_scores_kernel<N>, dim3(static_cast<unsigned>(P.n_units) << P.score_split), kFewThreads, 0, stream, P);
     if (e != cudaSuccess) return e;
-    switch (producer) {
-        case 0: e = launch_overlapped(few_values_kernel<N, 0>, grid, kFewThreads, 0, stream, P); break;
-        case 1: e = launch_overlapped(few_values_kernel<N, 1>, grid, kFewThreads, 0, stream, P); break;
-        case 2: e = launch_overlapped(few_values_kernel<N, 2>, grid, kFewThreads, 0, stream, P); break;
-        case 3: e = launch_overlapped(few_values_kernel<N, 3>, grid, kFewThreads, 0, stream, P); break;
-        case 4: e = launch_overlapped(few_values_kernel<N, 4>, grid, kFewThreads, 0, stream, P); break;
-        case 5: e = launch_overlapped(few_values_kernel<N, 5>, grid, kFewThreads, 0, stream, P); break;
-        case 6: e = launch_overlapped(few_values_kernel<N, 6>, grid, kFewThreads, 0, stream, P); break;
-        default: return cudaErrorInvalidValue;
-    }
+    e = P.value_split > 0 ? launch_values<N, true>(producer, P, stream) : launch_values<N, false>(producer, P, stream);
     if (e != cudaSuccess) return e;
-    return launch_overlapped(few_merge_kernel, dim3(static_cast<unsigned>(P.n_heads), static_cast<unsigned>(P.row_cap)), 128, 0, stream, P);
+    const dim3 rows(static_cast<unsigned>(P.n_heads), static_cast<unsigned>(P.row_cap));
+    return P.value_split > 0 ? launch_overlapped(few_merge_tiles_kernel, rows, 32 * kMergeWarps, 0, stream, P) : launch_overlapped(few_merge_kernel, rows, 128, 0, stream, P);
 }
 
 }  // namespace
@@ -625,24 +737,26 @@ cudaError_t launch_n(int producer, const FewParams& P, cudaStream_t stream)
 cudaError_t launch_few(int producer, FewParams& P, cudaStream_t stream)
 {
     if (P.n_units <= 0) return cudaErrorInvalidValue;
-    // Scores in halves, quarters, eighths of a chunk as long as the blocks are all on the chip together (three on each of 148 SMs; four
-    // or eight made no difference).  One head of 60000 keys 33.4 -> 26.7 us, four of 20000 33.4 -> 28.2, 16 rows of 4000 36.9 -> 26.6,
-    // 20 rows of 9000 47.0 -> 37.3, a context of 8191 keys with eight heads 20.9 -> 18.8.
+    // Chunks in halves, quarters, eighths as long as the blocks are all on the chip together (three on each of 148 SMs; with four or six
+    // 32 heads of 3000 keys 19.1 -> 19.2 and 22.8 us, 28 / 4 heads of 20000 22.0 -> 22.2 and 24.1).  Whole chunks -> scores in
+    // parts -> values too: one head of 60000 keys 31.2 -> 26.7 -> 22.2 us, 28 / 4 heads of 20000 33.4 -> 28.2 -> 22.0, 16 rows of 4000 36.5
+    // -> 26.6 -> 12.4, 20 rows of 9000 47.3 -> 37.3 -> 15.5, 32 / 8 heads of 8191 20.6 -> 19.7 -> 18.4.
     P.score_split = 0;
     while (P.score_split < 3 && (static_cast<int64_t>(P.n_units) << (P.score_split + 1)) <= 3 * 148) ++P.score_split;
+    P.value_split = P.longest_chunk > 1 ? P.score_split : 0;
     if (P.row_cap <= 8) return launch_n<8>(producer, P, stream);
     if (P.row_cap <= 16) return launch_n<16>(producer, P, stream);
     return launch_n<24>(producer, P, stream);
 }
 
-FewPlan plan_few(int64_t units, int64_t keys_padded_all_heads, int rows)
+FewPlan plan_few(int64_t keys_padded_all_heads, int rows)
 {
     FewPlan w;
     size_t off = 0;
     auto take = [&](size_t bytes) { const size_t at = off; off = (off + bytes + 1023) / 1024 * 1024; return at; };
     w.scores = take(static_cast<size_t>(keys_padded_all_heads) * rows * sizeof(float));
     w.block_max = take(static_cast<size_t>(keys_padded_all_heads / 32) * rows * sizeof(float));
-    w.stats = take(static_cast<size_t>(units) * rows * kFewStatFloats * sizeof(float));
+    w.stats = take(static_cast<size_t>(keys_padded_all_heads / kTile) * rows * kFewStatFloats * sizeof(float));
     w.total = off;
     return w;
 }

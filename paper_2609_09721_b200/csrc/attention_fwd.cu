@@ -763,8 +763,7 @@ size_t workspace_bytes_for(int B, int Hq, int Hkv, int64_t Sq, int64_t Sk)
     size_t total = plan_workspace(B, Hq, Hkv, Sq, Sk).total;
     if (use_few(Hq, Hkv, Sq, Sk)) {
         const int64_t heads = static_cast<int64_t>(B) * Hkv;
-        const size_t few = 1024 + plan_few(heads * few_chunks(Sk, Hq / Hkv * Sq), heads * ((Sk + kTile - 1) / kTile * kTile),
-                                           static_cast<int>(Hq / Hkv * Sq)).total;
+        const size_t few = 1024 + plan_few(heads * ((Sk + kTile - 1) / kTile * kTile), static_cast<int>(Hq / Hkv * Sq)).total;
         if (few > total) total = few;
     }
     return total;
@@ -950,7 +949,8 @@ efq_status_t attention_impl(const void* q, const void* k, const void* v, float* 
         const int64_t units = static_cast<int64_t>(B) * Hkv * F.dense_chunks;
         if (units > 0x7fffffffll) return EFQ_ERR_UNSUPPORTED;
         F.n_units = static_cast<int32_t>(units);
-        const FewPlan fp = plan_few(units, static_cast<int64_t>(B) * Hkv * w.Sk_pad, F.row_cap);
+        F.longest_chunk = few_chunk_tiles(static_cast<int>(w.Sk_pad / kTile), G * static_cast<int>(Sq));
+        const FewPlan fp = plan_few(static_cast<int64_t>(B) * Hkv * w.Sk_pad, F.row_cap);
         F.scores = reinterpret_cast<float*>(ws + 1024 + fp.scores); F.block_max = reinterpret_cast<float*>(ws + 1024 + fp.block_max);
         F.stats = reinterpret_cast<float*>(ws + 1024 + fp.stats);
         F.status = reinterpret_cast<uint32_t*>(ws);
@@ -1079,7 +1079,7 @@ bool plan_varlen(const int64_t* cu_q, const int64_t* cu_k, int n_seqs, int Hq, i
     p.few_table = off;
     if (p.n_few > kFewInlineSeqs) off = align_up(off + sizeof(FewSeq) * p.n_few, 1024);
     p.few = off;
-    if (p.n_few > 0) off += std::max(plan_few(p.few_units, p.few_keys * Hkv, p.few_rows).total, align_up(copies, 1024));
+    if (p.n_few > 0) off += std::max(plan_few(p.few_keys * Hkv, p.few_rows).total, align_up(copies, 1024));
     p.total = off;
     return true;
 }
@@ -1394,6 +1394,7 @@ extern "C" efq_status_t efq_attention_fwd_varlen(const void* q, const void* k, c
             few_seqs[f++] = FewSeq{static_cast<int32_t>(lq), static_cast<int32_t>(lk), static_cast<int32_t>(q0), static_cast<int32_t>(k0),
                                    static_cast<int32_t>(few_key), static_cast<int32_t>(few_unit)};
             few_key += (lk + kTile - 1) / kTile * kTile;
+            F.longest_chunk = std::max(F.longest_chunk, few_chunk_tiles(static_cast<int>((lk + kTile - 1) / kTile), G * static_cast<int>(lq)));
             few_unit += few_chunks(lk, Hq / Hkv * lq) * Hkv;
             continue;
         }
@@ -1448,7 +1449,7 @@ extern "C" efq_status_t efq_attention_fwd_varlen(const void* q, const void* k, c
         F.n_units = static_cast<int32_t>(p.few_units);
         F.rescale_threshold = threshold;
         F.K = producer == 3 ? make_producer_consts_lut(softmax_scale) : make_producer_consts(softmax_scale, tau, h);
-        const FewPlan fp = plan_few(p.few_units, p.few_keys * Hkv, p.few_rows);
+        const FewPlan fp = plan_few(p.few_keys * Hkv, p.few_rows);
         uint8_t* const fw = ws + p.few;
         F.scores = reinterpret_cast<float*>(fw + fp.scores); F.block_max = reinterpret_cast<float*>(fw + fp.block_max);
         F.stats = reinterpret_cast<float*>(fw + fp.stats);

@@ -127,8 +127,9 @@ static_assert(few_row_offset(kFewMaxRows - 2, 100000000 / 128) == 2200000000ll, 
 static_assert(int64_t{kFewMaxRows} * (int64_t{1} << 31) / 32 < int64_t{1} << 31, "block maxima of the longest context");
 // A chunk's partial result: the 128 values of a row's O^T take the place of the row's scores of the chunk's first tile, which
 // nobody reads any more by then; beside them, per row, four parts of the denominator, the maximum they refer to, three unused.
-// So a KV head needs rows * (528 tiles + 32 chunks) bytes, at 24 rows and a tile a chunk 13440 a tile: less than the 17408 of the
-// MXFP4 copies of K and V, and what fits a workspace on the general path fits it here.
+// Where few chunks are taken tile by tile, every tile leaves that, and the factor of its maximum.  So a KV head needs at most
+// rows * (528 + 32) bytes a tile, at 24 rows 13440: less than the 17408 of the MXFP4 copies of K and V, and what fits a workspace
+// on the general path fits it here.
 constexpr int kFewStatFloats = 8;
 constexpr int kFewInlineSeqs = 128;      // sequence tables up to this size travel as kernel parameters
 
@@ -148,7 +149,8 @@ struct FewParams {
     int64_t q_seq, q_head, q_row, k_seq, k_head, k_row;    // strides in elements
     int32_t row_cap;                           // query rows the workspace holds per KV head (the most of any sequence)
     int32_t n_units, n_heads;                  // chunks times KV heads, and KV heads, of all sequences
-    int32_t score_split;                       // a chunk's scores are the work of 2^score_split blocks (set by launch_few)
+    int32_t longest_chunk;                     // tiles
+    int32_t score_split, value_split;          // a chunk is the work of 2^split blocks (set by launch_few)
     float rescale_threshold;
     ProducerConsts K;
     float *scores, *block_max, *stats;         // workspace
@@ -161,7 +163,7 @@ struct FewParams {
 };
 
 struct FewPlan { size_t scores, block_max, stats, total; };   // offsets from a 1024-byte aligned base
-FewPlan plan_few(int64_t units, int64_t keys_padded_all_heads, int rows);
+FewPlan plan_few(int64_t keys_padded_all_heads, int rows);
 // Clears the status words.
 cudaError_t launch_few(int producer, FewParams& P, cudaStream_t stream);
 

@@ -72,6 +72,24 @@ def test_packed_batch_of_few_row_sequences(n_seqs, tokens):
         assert torch.equal(o[a:b].permute(1, 0, 2), alone[0]), f"sequence {n}"
 
 
+@pytest.mark.parametrize("Hq,Hkv,Sq,Sk,B,producer,threshold", [
+    (4, 4, 1, 2049, 8, "efq", 0.0), (4, 4, 1, 3969, 8, "etq4", 0.0),      # chunks of 2 tiles, the last of 1; 31 tiles
+    (32, 8, 1, 8191, 4, "efq", 0.0), (8, 1, 1, 8300, 30, "lut", 0.0),     # 4 tiles, 16 chunks; 17, the last of 1 tile
+    (2, 2, 1, 20000, 12, "efq", 0.0), (1, 1, 1, 16385, 20, "etq0", 0.0),  # 8 tiles; the last chunk of 5 and of 1
+    (1, 1, 9, 4097, 80, "efq", 0.0), (16, 2, 2, 4200, 30, "efq", 1.0),    # 9 and 16 rows: chunks of 8 from 32 tiles on
+    (8, 1, 3, 8193, 40, "efq", 0.0), (8, 2, 5, 9000, 20, "etq2", 0.0),    # 24 and 20 rows
+])
+def test_chunks_in_parts_equal_whole_chunks(Hq, Hkv, Sq, Sk, B, producer, threshold):
+    """Where few chunks do not fill the chip they are taken in parts, tile by tile: a sequence by itself gives the bits that it
+    gives in a batch of B, whose chunks (more than 222) are taken whole."""
+    g = torch.Generator(device="cuda").manual_seed(Sk)
+    q = torch.randn(B, Hq, Sq, 128, generator=g, device="cuda").bfloat16()
+    k, v = (torch.randn(B, Hkv, Sk, 128, generator=g, device="cuda").bfloat16() for _ in range(2))
+    batch = _forward(q, k, v, True, producer, threshold)
+    for b in (0, B - 1):
+        assert torch.equal(_forward(q[b:b + 1].contiguous(), k[b:b + 1].contiguous(), v[b:b + 1].contiguous(), True, producer, threshold)[0], batch[b])
+
+
 @pytest.mark.parametrize("S,Hq,Hkv", [(127, 2, 1), (129, 1, 1), (257, 3, 3)])
 def test_inputs_at_a_16_byte_boundary(S, Hq, Hkv):
     """Operand preparation loads 32 bytes at a time where the input allows it: inputs that start 16 bytes off give the same."""
