@@ -61,6 +61,18 @@ def test_efq_probgen_full_config(oracle):
     assert hist[0] > 0.3 and hist[7] > 0.01
 
 
+@pytest.mark.parametrize("cols", [7, 8, 9, 255, 256, 257, 1016, 1023, 1025, 2047])
+@pytest.mark.parametrize("pad", [0, 4])
+def test_ends_of_rows(oracle, cols, pad):
+    """Where a row does not fill its last 1024 columns it is loaded eight columns at a time, the last few one by one: column counts
+    around those edges, with rows that start on 32 and on 16 bytes."""
+    ld = (cols + 7) // 8 * 8 + pad
+    scores, row_max = inputs.make_score_matrix(19, cols, seed=cols)
+    want_c, want_s = oracle.probgen(scores, row_max, 1.0, *POINTS[0])
+    got_c, got_s = _run_gpu(binding.efq_probgen, scores, row_max, 1.0, POINTS[0], ld=ld)
+    assert np.array_equal(got_s, want_s) and np.array_equal(got_c, want_c)
+
+
 @pytest.mark.parametrize("rows,cols,ld", [(64, 4096, None), (37, 1024 * 3 + 32 * 5, None), (5, 32760, 32768),
                                           (9, 88, 96), (3, 31, 32), (1, 1, 4)])
 def test_efq_lut_probgen_bit_exact(oracle, rows, cols, ld):

@@ -46,6 +46,27 @@ def test_short_walks_equal_one_cta_per_tile(oracle, B, Hq, Hkv, Sq, Sk, causal, 
         assert torch.all(o[:, :, : Sq - Sk] == 0)
 
 
+@pytest.mark.parametrize("Hq,Hkv,Sq,Sk,causal,producer", [
+    (24, 24, 900, 30000, False, "efq"), (32, 8, 20000, 20000, True, "efq"),     # walks of 235 tiles, of 1 to 157
+    (24, 24, 900, 6144, False, "lut"), (24, 24, 900, 6145, False, "lut"),       # the line of the table form, one key past it
+    (24, 24, 900, 20000, False, "etq0"), (24, 24, 900, 20000, False, "etq2"),
+    (1, 1, 148 * 128, 300, False, "efq"), (1, 1, 148 * 128 + 1, 300, False, "efq"),       # as many query tiles as SMs, one more
+])
+def test_long_walks_equal_one_cta_per_tile(Hq, Hkv, Sq, Sk, causal, producer):
+    """Persistent CTAs in long walks, and at the lines of the rule: the bits of the kernel with one CTA per tile, which runs when
+    the operand is dumped."""
+    g = torch.Generator(device="cuda").manual_seed(Sk)
+    q = torch.randn(1, Hq, Sq, 128, generator=g, device="cuda").bfloat16()
+    k, v = (torch.randn(1, Hkv, Sk, 128, generator=g, device="cuda").bfloat16() for _ in range(2))
+
+    def forward(debug=None):
+        if producer.startswith("etq"):
+            return binding.exp_then_quantize_attention_fwd(q, k, v, causal, 0.0, int(producer[3:]), debug=debug)
+        return binding.efq_attention_fwd(q, k, v, causal, 0.0, (MEAN[0], MEAN[1], int(producer == "lut"), 0, 0.0), debug=debug)
+
+    assert torch.equal(forward(), forward(binding.DebugDump(0, Hq - 1, 0, 1, Sk)))
+
+
 @pytest.mark.parametrize("Hq,Hkv,causal,longest,producer", [(8, 2, True, 1000, 0), (6, 6, False, 5120, 0), (8, 4, True, 5121, 0), (8, 2, True, 700, 1), (8, 2, False, 512, 1)])
 def test_short_walks_of_a_packed_batch(Hq, Hkv, causal, longest, producer):
     """Sequences of mixed lengths, up to the longest that the rule takes and one past it: shared query tiles (few tokens), the
