@@ -40,7 +40,7 @@ FALLBACK_HBM_GBS = 6650.0
 # from the ncu capture summarised in the named profile, and valid only for the kernel revision that
 # capture saw (the library's version tag); for any other revision the line carries null.
 NCU_DRAM_BYTES_PER_LAUNCH = {
-    "qwen3_8b_16k": {"bytes": 53545728 + 211486208, "kernel_revision": "fwd.6", "profile": "profiles/attention_fwd_current.md"},
+    "qwen3_8b_16k": {"bytes": 53571840 + 209361664, "kernel_revision": "fwd.7", "profile": "profiles/attention_fwd_current.md"},
 }
 BURST_REGION_S = 1.0   # a timed region shorter than this runs at burst clocks: its roofline uses the burst peak
 
@@ -517,7 +517,7 @@ def run_cuda(args):
                 traffic_source = f"not measured by this run: ncu capture of kernel revision {entry['kernel_revision']}, {entry['profile']}"
             else:
                 traffic_source = f"dropped: the ncu capture in {entry['profile']} saw kernel revision {entry['kernel_revision']}, this library is {binding.version()}"
-        return {"kernel": "attention_fwd_kernel<EFQ>", "bound": "tensor", "achieved": achieved, "peak": peak,
+        return {"kernel": "attention_short_kernel<EFQ>", "bound": "tensor", "achieved": achieved, "peak": peak,
                 "unit": "TFLOP/s", "frac": achieved / peak, "traffic": traffic, "traffic_source": traffic_source,
                 "peak_source": f"{peaks['source']} bf16 {'burst' if burst else 'sustained'} {bf16} TFLOP/s x {NOMINAL_FP4_OVER_BF16} "
                                f"(nominal FP4:bf16 ratio); timed region {region_s:.3f} s",

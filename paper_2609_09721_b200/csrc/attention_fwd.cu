@@ -23,8 +23,8 @@
 // are rescaled by alpha = exp(m_old - m_new) before the next P~V MMA is released (warps 12-15).
 //
 // TMEM columns: S double buffer 2 x 128 | O 144 (128 channels + 16 denominator) | scale factors.
-// Every wait is bounded; on expiry the CTA records EFQ_ERR_DEVICE_TIMEOUT in the workspace status
-// word, all roles drain, TMEM is released and the kernel returns.
+// Every wait is bounded: one thread of warp 3 watches whether P~V goes on, and if it does not the CTA records EFQ_ERR_DEVICE_TIMEOUT
+// in the workspace status word, all roles drain, TMEM is released and the kernel returns.
 #include <cuda.h>
 #include <cuda_runtime.h>
 

@@ -102,12 +102,12 @@ constexpr int kFewMaxRows = 24;
 // The contexts that take it, by the sequence's own shape: up to 16 rows all, 17 to 24 rows from 64 KV tiles on.  Its time grows with
 // the rows (each has its codes made and its scores written for itself), that of the general path does not up to 128; but the
 // general path walks a whole context in one CTA a KV head.  Measured, this path against the general one, us, with 1 / 64 / 256 KV heads:
-//    8 rows: 1000 keys 11.7 / 20.4 / - against 13.5 / 18.7 / -, 4000 keys 19.7 / 43.5 / - against 29.9 / 52.9 / -
-//   16 rows: 1000 keys 15.5 / 23.3 / 58 against 13.3 / 18.8 / 48; 2000 keys 15.7 / 35 / 101 against 19.1 / 29 / 84; 4000 keys 38 / 62 / 159
-//            against 30 / 53 / 155; 8000 keys 39 / 93 / 292 against 51 / 99 / 289; 16000 keys 40 / 154 / 561 against 92 / 189 / 563
-//   24 rows: 1000 keys 19.2 / 29.5 / 75 against 13.5 / 18.9 / 49; 2000 keys 19.8 / 45 / 130 against 19.3 / 29 / 84; 3000 keys 20.2 / 56 / 192
-//            against 24.9 / 41 / 119; 4000 keys 51 / 80 / 218 against 31 / 54 / 155; 8000 keys 52 / 124 / 385 against 52 / 100 / 289;
-//            16000 keys 53 / 214 / 746 against 92 / 189 / 561
+//    8 rows: 2000 keys 11.8 / 27.6 / 80 against 18.8 / 27.2 / 80, 4000 keys 11.6 / 44.1 / 128 against 29.3 / 52.1 / 149; 8100 keys
+//            12.2 / 71 / 246 against 51.0 / 99 / 286
+//   16 rows: 1000 keys 11.9 / 22.6 / 59 against 14.4 / 18.6 / 46; 2000 keys 13.2 / 36 / 107 against 19.5 / 29 / 82; 4000 keys 12.8 / 62 / 159
+//            against 30.9 / 54 / 150; 8100 keys 13.2 / 94 / 290 against 51.9 / 100 / 287; 16000 keys 14.5 / 151 / 550 against 92.8 / 186 / 557
+//   24 rows: 1000 keys 19.2 / 29.5 / 75 against 14.0 / 17.9 / 44; 4000 keys 51 / 80 / 218 against 31.9 / 55 / 152 (both before few chunks
+//            were taken in parts); 8100 keys 15.3 / 128 / 388 against 52.8 / 101 / 289; 16000 keys 16.4 / 210 / 732 against 93.7 / 187 / 559
 // The number of heads and sequences must not matter to the line (a sequence gives the same bits alone and in a batch).  Up to 16
 // rows the gains of a few long contexts outweigh a loss of a fifth in wide batches of short ones; above, the line lies where a few
 // heads begin to gain.
