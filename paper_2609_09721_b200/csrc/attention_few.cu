@@ -228,7 +228,7 @@ __global__ void __launch_bounds__(kFewThreads, N <= 8 ? 4 : 3) few_scores_kernel
         uint32_t w[16];
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            const uint4 x = __ldg(src + i);
+            const uint4 x = __ldca(src + i);
             w[4 * i] = x.x; w[4 * i + 1] = x.y; w[4 * i + 2] = x.z; w[4 * i + 3] = x.w;
         }
         uint4 c;

@@ -239,7 +239,7 @@ exact_attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
 }
 
 // sums[0] += sum (a - r)^2, sums[1] += sum r^2, in double.  Bound by the reads (from L2 where both arrays fit): 16 bytes per
-// load, four loads in flight per thread.
+// load, four loads in flight per thread.  Launched while the kernel that makes the rows still writes them: no read-only loads.
 __global__ void __launch_bounds__(256) error_sums_kernel(const float* __restrict__ a, const float* __restrict__ r,
                                                          int64_t n, double* sums)
 {
@@ -256,16 +256,16 @@ __global__ void __launch_bounds__(256) error_sums_kernel(const float* __restrict
     const int64_t n4 = vec ? n / 4 : 0;
     int64_t i = thread;
     for (; i + threads < n4; i += 2 * threads) {
-        const float4 x0 = __ldg(reinterpret_cast<const float4*>(a) + i), x1 = __ldg(reinterpret_cast<const float4*>(a) + i + threads);
-        const float4 y0 = __ldg(reinterpret_cast<const float4*>(r) + i), y1 = __ldg(reinterpret_cast<const float4*>(r) + i + threads);
+        const float4 x0 = __ldcg(reinterpret_cast<const float4*>(a) + i), x1 = __ldcg(reinterpret_cast<const float4*>(a) + i + threads);
+        const float4 y0 = __ldcg(reinterpret_cast<const float4*>(r) + i), y1 = __ldcg(reinterpret_cast<const float4*>(r) + i + threads);
         add(x0.x, y0.x); add(x0.y, y0.y); add(x0.z, y0.z); add(x0.w, y0.w);
         add(x1.x, y1.x); add(x1.y, y1.y); add(x1.z, y1.z); add(x1.w, y1.w);
     }
     if (i < n4) {
-        const float4 x = __ldg(reinterpret_cast<const float4*>(a) + i), y = __ldg(reinterpret_cast<const float4*>(r) + i);
+        const float4 x = __ldcg(reinterpret_cast<const float4*>(a) + i), y = __ldcg(reinterpret_cast<const float4*>(r) + i);
         add(x.x, y.x); add(x.y, y.y); add(x.z, y.z); add(x.w, y.w);
     }
-    for (int64_t k = 4 * n4 + thread; k < n; k += threads) add(a[k], r[k]);
+    for (int64_t k = 4 * n4 + thread; k < n; k += threads) add(__ldcg(a + k), __ldcg(r + k));
     for (int off = 16; off > 0; off >>= 1) {
         d2 += __shfl_xor_sync(0xffffffffu, d2, off);
         r2 += __shfl_xor_sync(0xffffffffu, r2, off);

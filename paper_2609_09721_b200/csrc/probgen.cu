@@ -157,7 +157,6 @@ __device__ __forceinline__ void probgen_body(const float* __restrict__ scores, i
         const int64_t row = n_tasks <= 0x7fffffff ? static_cast<int64_t>(static_cast<uint32_t>(task) / static_cast<uint32_t>(segs_per_row)) : task / segs_per_row;
         const int64_t c0 = (task - row * segs_per_row) * kSegCols;
         const float* src = scores + row * ld + c0;
-        const float m_s = __ldg(row_max + row);
         uint8_t* crow = codes + row * nblk * (kMxBlock / 2) + c0 / 2;
         uint8_t* srow = scales + row * nblk + c0 / kMxBlock;
         const bool full = c0 + kSegCols <= cols;
@@ -193,6 +192,7 @@ __device__ __forceinline__ void probgen_body(const float* __restrict__ scores, i
                 }
             }
         }
+        const float m_s = __ldca(row_max + row);       // behind the loads of the scores (before them: 51.2 -> 51.9 us)
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             uint32_t code32, byte;

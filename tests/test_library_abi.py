@@ -29,6 +29,16 @@ def test_header_symbols_are_exported():
     assert sorted(binding.EXPORTS) == names
 
 
+def test_no_read_only_loads_of_what_the_kernel_before_writes():
+    """Blocks of an overlapped launch may be there while the kernel before still writes, so its data are not read through the read-only
+    path.  The tables of a packed batch are: a copy from the host writes them, and a copy overlaps no kernel."""
+    tables = ("groups[mid].first_item", "first_cta + ")
+    for name in os.listdir(build.CSRC):
+        for line in open(os.path.join(build.CSRC, name)):
+            if "__ldg(" in line:
+                assert name == "quantize_qkv.cu" and any(t in line for t in tables), (name, line)
+
+
 def test_status_strings_and_version():
     assert binding.version().startswith("efq-b200")
     assert binding.status_string(0) == "ok"

@@ -73,6 +73,27 @@ def test_ends_of_rows(oracle, cols, pad):
     assert np.array_equal(got_s, want_s) and np.array_equal(got_c, want_c)
 
 
+@pytest.mark.parametrize("Sq", [16, 20000])          # the few-row kernels, one CTA per query tile
+def test_stage_straight_behind_a_dumping_forward(Sq):
+    """The stage's blocks may be there while the forward before it still writes the scores and row maxima that it reads: forwards of
+    other queries dump into the same two arrays in turn, and the stage behind each finds that forward's codes and scale bytes."""
+    g = torch.Generator(device="cuda").manual_seed(Sq)
+    k, v = (torch.randn(1, 1, 128, 128, generator=g, device="cuda").bfloat16() for _ in range(2))
+    qs = [torch.randn(1, 1, Sq, 128, generator=g, device="cuda").bfloat16() for _ in range(6)]
+    dumps = [binding.DebugDump(0, 0, 0, Sq, 128) for _ in qs]
+    for d in dumps[1:]:
+        d.c.raw_scores, d.c.row_max = dumps[0].c.raw_scores, dumps[0].c.row_max
+    scores, row_max, sigma = dumps[0].raw_scores, dumps[0].row_max[:, 0], float(np.float32(0.08838834764831845))
+    o, ws = torch.empty(1, 1, Sq, 128, device="cuda"), torch.empty(binding.efq_attention_workspace_bytes(1, 1, 1, Sq, 128, 128), dtype=torch.uint8, device="cuda")
+    codes, scales = (torch.empty(len(qs), Sq, n, dtype=torch.uint8, device="cuda") for n in (64, 4))
+    for i, q in enumerate(qs):
+        binding.efq_attention_fwd(q, k, v, False, 0.0, None, o, ws, dumps[i])
+        binding.efq_probgen(scores, row_max, sigma, None, codes[i], scales[i])
+    for i, d in enumerate(dumps):
+        assert torch.equal(codes[i], d.codes) and torch.equal(scales[i], d.scales), i
+    assert not torch.equal(codes[0], codes[1])
+
+
 @pytest.mark.parametrize("rows,cols,ld", [(64, 4096, None), (37, 1024 * 3 + 32 * 5, None), (5, 32760, 32768),
                                           (9, 88, 96), (3, 31, 32), (1, 1, 4)])
 def test_efq_lut_probgen_bit_exact(oracle, rows, cols, ld):
