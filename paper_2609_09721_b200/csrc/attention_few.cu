@@ -186,19 +186,15 @@ __global__ void __launch_bounds__(kFewThreads, N <= 8 ? 4 : 3) few_scores_kernel
     __shared__ FewSmem smem;
     FewSmem* const sm = &smem;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    // A block takes 2^-split of a chunk: the scores of a tile need nothing of another, and a few chunks do not fill the chip.  The
+    // sequence table was written by a copy, which overlaps no kernel.
+    Unit u = find_unit(P, static_cast<int>(blockIdx.x) >> P.split);
+    const int R = P.G * u.Sq;
+    if (!take_part(u, R, P.split)) return;       // never block 0
     few_setup(sm, warp);
     ptx::grid_wait();                // the kernels before: inputs, and the workspace of an earlier call
     ptx::grid_launch_next();
-    // A block takes 2^-score_split of a chunk: the scores of a tile need nothing of another, and a few chunks do not fill the chip.
-    Unit u = find_unit(P, static_cast<int>(blockIdx.x) >> P.score_split);
-    const int R = P.G * u.Sq;
-    const bool work = take_part(u, R, P.score_split);
     if (blockIdx.x == 0) P.status[tid] = 0u;
-    if (!work) {
-        __syncthreads();
-        if (warp == 0) ptx::tmem_dealloc(sm->tmem_base, kFewTmemCols);
-        return;
-    }
     // K: a quad of lanes takes a key, a lane every fourth 16-byte piece of it - a load instruction reads 64 contiguous
     // bytes of every key - and so a quarter of each of the four blocks
     const int quad = tid & 3, key_in_tile = tid >> 2;
@@ -397,7 +393,7 @@ __device__ __forceinline__ void few_row_state(FewSmem* sm, const FewParams& P, i
     }
 }
 
-// TILES: a block takes 2^-value_split of a chunk and leaves the product of every tile by itself, beside its factors, for the merge to
+// TILES: a block takes 2^-split of a chunk and leaves the product of every tile by itself, beside its factors, for the merge to
 // add up as the chunk's block would have (same operations, same order, same bits).
 template <int N, int PRODUCER, bool TILES>
 __global__ void __launch_bounds__(kFewThreads, 3) few_values_kernel(const __grid_constant__ FewParams P)
@@ -406,9 +402,9 @@ __global__ void __launch_bounds__(kFewThreads, 3) few_values_kernel(const __grid
     FewSmem* const sm = &smem;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     ptx::grid_launch_next();
-    Unit u = find_unit(P, static_cast<int>(blockIdx.x) >> (TILES ? P.value_split : 0));
+    Unit u = find_unit(P, static_cast<int>(blockIdx.x) >> (TILES ? P.split : 0));
     const int R = P.G * u.Sq;
-    if (TILES && !take_part(u, R, P.value_split)) return;
+    if (TILES && !take_part(u, R, P.split)) return;
     few_setup(sm, warp);
     const VTileLane L(warp, lane);
     uint4 vv[8];
@@ -708,7 +704,7 @@ __global__ void __launch_bounds__(32 * kMergeWarps) few_merge_tiles_kernel(const
 template <int N, bool TILES>
 cudaError_t launch_values(int producer, const FewParams& P, cudaStream_t stream)
 {
-    const dim3 grid(static_cast<unsigned>(P.n_units) << P.value_split);
+    const dim3 grid(static_cast<unsigned>(P.n_units) << P.split);
     switch (producer) {
         case 0: return launch_overlapped(few_values_kernel<N, 0, TILES>, grid, kFewThreads, 0, stream, P);
         case 1: return launch_overlapped(few_values_kernel<N, 1, TILES>, grid, kFewThreads, 0, stream, P);
@@ -724,12 +720,12 @@ cudaError_t launch_values(int producer, const FewParams& P, cudaStream_t stream)
 template <int N>
 cudaError_t launch_n(int producer, const FewParams& P, cudaStream_t stream)
 {
-    cudaError_t e = launch_overlapped(few_scores_kernel<N>, dim3(static_cast<unsigned>(P.n_units) << P.score_split), kFewThreads, 0, stream, P);
+    cudaError_t e = launch_overlapped(few_scores_kernel<N>, dim3(static_cast<unsigned>(P.n_units) << P.split), kFewThreads, 0, stream, P);
     if (e != cudaSuccess) return e;
-    e = P.value_split > 0 ? launch_values<N, true>(producer, P, stream) : launch_values<N, false>(producer, P, stream);
+    e = P.split > 0 ? launch_values<N, true>(producer, P, stream) : launch_values<N, false>(producer, P, stream);
     if (e != cudaSuccess) return e;
     const dim3 rows(static_cast<unsigned>(P.n_heads), static_cast<unsigned>(P.row_cap));
-    return P.value_split > 0 ? launch_overlapped(few_merge_tiles_kernel, rows, 32 * kMergeWarps, 0, stream, P) : launch_overlapped(few_merge_kernel, rows, 128, 0, stream, P);
+    return P.split > 0 ? launch_overlapped(few_merge_tiles_kernel, rows, 32 * kMergeWarps, 0, stream, P) : launch_overlapped(few_merge_kernel, rows, 128, 0, stream, P);
 }
 
 }  // namespace
@@ -737,13 +733,15 @@ cudaError_t launch_n(int producer, const FewParams& P, cudaStream_t stream)
 cudaError_t launch_few(int producer, FewParams& P, cudaStream_t stream)
 {
     if (P.n_units <= 0) return cudaErrorInvalidValue;
-    // Chunks in halves, quarters, eighths as long as the blocks are all on the chip together (three on each of 148 SMs; with four or six
-    // 32 heads of 3000 keys 19.1 -> 19.2 and 22.8 us, 28 / 4 heads of 20000 22.0 -> 22.2 and 24.1).  Whole chunks -> scores in
-    // parts -> values too: one head of 60000 keys 31.2 -> 26.7 -> 22.2 us, 28 / 4 heads of 20000 33.4 -> 28.2 -> 22.0, 16 rows of 4000 36.5
-    // -> 26.6 -> 12.4, 20 rows of 9000 47.3 -> 37.3 -> 15.5, 32 / 8 heads of 8191 20.6 -> 19.7 -> 18.4.
-    P.score_split = 0;
-    while (P.score_split < 3 && (static_cast<int64_t>(P.n_units) << (P.score_split + 1)) <= 3 * 148) ++P.score_split;
-    P.value_split = P.longest_chunk > 1 ? P.score_split : 0;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return cudaErrorInvalidDevice;
+    // Chunks in halves, quarters, eighths as long as every part has a tile and the blocks are all on the chip together (three on each
+    // SM; with four or six 32 heads of 3000 keys 19.1 -> 19.2 and 22.8 us, 28 / 4 heads of 20000 22.0 -> 22.2 and 24.1).  Whole
+    // chunks -> parts: one head of 2000 keys 11.9 -> 9.1 us, 32 / 8 heads of 3000 keys 14.2 -> 11.6, of 6000 19.9 -> 14.3, 16 rows of 4000
+    // 35.9 -> 11.1.  Blocks without a tile cost more than they spread: chunks of one tile in eight, 32 / 8 heads of 700 keys
+    // 10.0 -> 11.1 us, of 1500 10.6 -> 12.1, 9.8 and 10.3 with none; chunks of two in eight, four heads of 3000 keys 12.1, 10.0 with none.
+    P.split = 0;
+    while ((2 << P.split) <= P.longest_chunk && (static_cast<int64_t>(P.n_units) << (P.split + 1)) <= 3 * sm_count(dev)) ++P.split;
     if (P.row_cap <= 8) return launch_n<8>(producer, P, stream);
     if (P.row_cap <= 16) return launch_n<16>(producer, P, stream);
     return launch_n<24>(producer, P, stream);

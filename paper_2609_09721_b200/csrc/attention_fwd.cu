@@ -831,15 +831,6 @@ cudaError_t launch_short(unsigned items, unsigned sms, int dev, cudaStream_t str
     return P.items ? launch_short_one<PRODUCER, true>(items, sms, dev, stream, mq, mk, mv, mo, P) : launch_short_one<PRODUCER, false>(items, sms, dev, stream, mq, mk, mv, mo, P);
 }
 
-// SMs of a device, asked for once
-int sm_count(int dev)
-{
-    static std::atomic<int> known[kMaxDevices] = {};
-    int n = known[dev].load(std::memory_order_relaxed);
-    if (n == 0 && cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess) known[dev].store(n, std::memory_order_relaxed);
-    return n;
-}
-
 template <int PRODUCER>
 cudaError_t launch_main(bool debug, dim3 grid, size_t smem, cudaStream_t stream, const CUtensorMap& mq, const CUtensorMap& mk,
                         const CUtensorMap& mv, const FwdParams& P)
@@ -949,7 +940,7 @@ efq_status_t attention_impl(const void* q, const void* k, const void* v, float* 
         const int64_t units = static_cast<int64_t>(B) * Hkv * F.dense_chunks;
         if (units > 0x7fffffffll) return EFQ_ERR_UNSUPPORTED;
         F.n_units = static_cast<int32_t>(units);
-        F.longest_chunk = few_chunk_tiles(static_cast<int>(w.Sk_pad / kTile), G * static_cast<int>(Sq));
+        F.longest_chunk = few_longest_chunk(static_cast<int>(w.Sk_pad / kTile), G * static_cast<int>(Sq));
         const FewPlan fp = plan_few(static_cast<int64_t>(B) * Hkv * w.Sk_pad, F.row_cap);
         F.scores = reinterpret_cast<float*>(ws + 1024 + fp.scores); F.block_max = reinterpret_cast<float*>(ws + 1024 + fp.block_max);
         F.stats = reinterpret_cast<float*>(ws + 1024 + fp.stats);
@@ -1104,6 +1095,14 @@ cudaError_t copy_table(void* dst, std::vector<T>& host, cudaStream_t stream)
 }
 
 }  // namespace
+
+int sm_count(int dev)
+{
+    static std::atomic<int> known[kMaxDevices] = {};
+    int n = dev >= 0 && dev < kMaxDevices ? known[dev].load(std::memory_order_relaxed) : 0;
+    if (n == 0 && cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && dev < kMaxDevices) known[dev].store(n, std::memory_order_relaxed);
+    return n;
+}
 
 bool encode_bf16_map(CUtensorMap* map, const void* base, uint64_t cols, uint64_t rows) { return encode_any(map, base, 2 * cols, rows, kMapBf16); }
 
@@ -1394,7 +1393,7 @@ extern "C" efq_status_t efq_attention_fwd_varlen(const void* q, const void* k, c
             few_seqs[f++] = FewSeq{static_cast<int32_t>(lq), static_cast<int32_t>(lk), static_cast<int32_t>(q0), static_cast<int32_t>(k0),
                                    static_cast<int32_t>(few_key), static_cast<int32_t>(few_unit)};
             few_key += (lk + kTile - 1) / kTile * kTile;
-            F.longest_chunk = std::max(F.longest_chunk, few_chunk_tiles(static_cast<int>((lk + kTile - 1) / kTile), G * static_cast<int>(lq)));
+            F.longest_chunk = std::max(F.longest_chunk, few_longest_chunk(static_cast<int>((lk + kTile - 1) / kTile), G * static_cast<int>(lq)));
             few_unit += few_chunks(lk, Hq / Hkv * lq) * Hkv;
             continue;
         }

@@ -61,6 +61,9 @@ struct ItemGroup {
 };
 struct ItemDesc;
 
+// SMs of a device, asked for once (0: no such device)
+int sm_count(int dev);
+
 // Q, K and V of one [B, H, S, d] problem (or one sequence) in one launch; also clears the 256 status words.
 cudaError_t launch_quantize_qkv(const QuantSeg& q, const QuantSeg& k, const QuantSeg& v, uint32_t* status, cudaStream_t stream);
 // The jobs of a packed batch in one launch: jobs and first_cta (n_jobs + 1 prefix sums of CTAs) live in device memory.
@@ -115,10 +118,20 @@ __host__ __device__ inline bool few_takes(int64_t rows, int64_t n_tiles) { retur
 // Tiles of a chunk of the KV range, by the sequence's own shape: short contexts are cut finely, so that one of them spreads
 // over the chip; with many rows a chunk's partial result (544 bytes a row) has to be small against its 64 KB of K and V a tile.
 constexpr int kFewMaxChunk = 8;
-__host__ __device__ inline int few_chunk_tiles(int n_tiles, int rows)
+__host__ __device__ constexpr int few_chunk_tiles(int n_tiles, int rows)
 {
     return rows <= 8 ? (n_tiles < 16 ? 1 : n_tiles < 32 ? 2 : n_tiles < 128 ? 4 : kFewMaxChunk) : n_tiles < 32 ? 2 : kFewMaxChunk;
 }
+constexpr bool few_chunks_halve()
+{
+    for (int rows = 1; rows <= kFewMaxRows; ++rows)
+        for (int tiles = 1; tiles <= 256; ++tiles)
+            if (const int n = few_chunk_tiles(tiles, rows); n > kFewMaxChunk || (n & (n - 1)) != 0) return false;
+    return true;
+}
+static_assert(few_chunks_halve(), "a chunk is taken in halves, quarters and eighths of it: another length would lose tiles");
+// Tiles that the longest chunk of a context holds
+inline int few_longest_chunk(int n_tiles, int rows) { const int n = few_chunk_tiles(n_tiles, rows); return n < n_tiles ? n : n_tiles; }
 // Start of row `row` of the scores of a KV head, n_tiles of 128 keys: 64-bit, since 24 rows pass 2^31 scores from 97.6 million keys
 // on.  The product of row and tiles fits 32 bits; kept in those, the offsets of a thread's rows take a register each in the loop
 // and not two (9 to 16 rows, 16000 keys: 3 to 5 %).  Block maxima (four a tile) are addressed in 32 bits.
@@ -150,7 +163,7 @@ struct FewParams {
     int32_t row_cap;                           // query rows the workspace holds per KV head (the most of any sequence)
     int32_t n_units, n_heads;                  // chunks times KV heads, and KV heads, of all sequences
     int32_t longest_chunk;                     // tiles
-    int32_t score_split, value_split;          // a chunk is the work of 2^split blocks (set by launch_few)
+    int32_t split;                             // a chunk is the work of 2^split blocks (set by launch_few)
     float rescale_threshold;
     ProducerConsts K;
     float *scores, *block_max, *stats;         // workspace

@@ -1,6 +1,8 @@
 """The path for few query rows (query heads of a KV group times query tokens: at most 24) at its edges, against the CPU
 oracle: 1 row to 24 and the first size past it, key counts around the 128-key tile and around the sizes where the chunk of
 a CTA grows, each producer, and a packed batch too large for the sequence table that travels with the launch."""
+import json
+
 import numpy as np
 import pytest
 import torch
@@ -88,6 +90,26 @@ def test_chunks_in_parts_equal_whole_chunks(Hq, Hkv, Sq, Sk, B, producer, thresh
     batch = _forward(q, k, v, True, producer, threshold)
     for b in (0, B - 1):
         assert torch.equal(_forward(q[b:b + 1].contiguous(), k[b:b + 1].contiguous(), v[b:b + 1].contiguous(), True, producer, threshold)[0], batch[b])
+
+
+@pytest.mark.parametrize("Hq,Hkv,Sq,Sk", [
+    (8, 8, 1, 500), (32, 8, 1, 1000), (1, 1, 1, 1000), (1, 1, 1, 60),        # chunks of one tile
+    (4, 4, 1, 3000), (16, 1, 1, 1000), (16, 4, 4, 1500), (1, 1, 16, 100),    # of two; one tile in a chunk of two
+    (32, 8, 1, 8191), (2, 2, 1, 16384), (1, 1, 16, 4096), (1, 1, 24, 8192),  # of four, eight
+])
+def test_no_block_without_a_tile(tmp_path, Hq, Hkv, Sq, Sk):
+    """A chunk is cut into as many blocks as it has tiles at most: the streaming kernels launch no more blocks than there are tiles."""
+    g = torch.Generator(device="cuda").manual_seed(1)
+    q = torch.randn(1, Hq, Sq, 128, generator=g, device="cuda").bfloat16()
+    k, v = (torch.randn(1, Hkv, Sk, 128, generator=g, device="cuda").bfloat16() for _ in range(2))
+    with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as prof:
+        binding.efq_attention_fwd(q, k, v, True)
+        torch.cuda.synchronize()
+    prof.export_chrome_trace(str(tmp_path / "trace.json"))
+    events = json.load(open(tmp_path / "trace.json"))["traceEvents"]
+    blocks = {n: e["args"]["grid"][0] for e in events for n in ("few_scores", "few_values") if e.get("cat") == "kernel" and n in e["name"]}
+    assert sorted(blocks) == ["few_scores", "few_values"]
+    assert max(blocks.values()) <= Hkv * ((Sk + 127) // 128)
 
 
 @pytest.mark.parametrize("S,Hq,Hkv", [(127, 2, 1), (129, 1, 1), (257, 3, 3)])
