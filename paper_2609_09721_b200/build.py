@@ -29,7 +29,7 @@ def _stale() -> bool:
     if not os.path.exists(LIB) or not os.path.exists(FASTCALL):
         return True
     t = min(os.path.getmtime(LIB), os.path.getmtime(FASTCALL))
-    deps = sources() + [FASTCALL_SRC] + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(ROOT, "include", "*.h"))
+    deps = sources() + [FASTCALL_SRC] + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(ROOT, "include", "*.h"))
     return any(os.path.getmtime(d) > t for d in deps)
 
 

@@ -37,6 +37,7 @@
 #include "efq_common.cuh"
 #include "efq_internal.cuh"
 #include "efq_producers.cuh"
+#include "item_order.h"
 #include "mxfp4.cuh"
 #include "sm100_ptx.cuh"
 
@@ -1006,7 +1007,8 @@ efq_status_t attention_impl(const void* q, const void* k, const void* v, float* 
 // three for all that have few query rows (attention_few.cu).
 // ------------------------------------------------------------------------------------------------
 // Workspace: status words | tables from the host (sequences, quantiser jobs, their CTA prefix sums, query tiles in the order
-// of their weight) | item table (written on the device: it has an entry per head) |
+// of their weight, the places of their items if they are not one after the other) | item table (written on the device: it has an
+// entry per head) |
 // Q codes [rows of all sequences, 64 B] | Q scale tiles | K codes | K scale tiles |
 // V^T codes [Hkv * 128, sum of Sk_pad / 2 B] (the sequences side by side along the keys) | V scale tiles.
 struct VarlenPlan {
@@ -1016,7 +1018,7 @@ struct VarlenPlan {
     int64_t q_rows, k_rows, k_cols;  // rows of the Q and K code matrices, keys along V^T (all padded to 128)
     int64_t items, groups, quant_ctas;
     int64_t longest;                 // keys of the longest sequence of the general path
-    size_t tables, seqs_off, jobs_off, prefix_off, groups_off, items_off, qc, qsf, kc, ksf, vt, vsf, few_table, few, total;
+    size_t tables, seqs_off, jobs_off, prefix_off, groups_off, places_off, items_off, qc, qsf, kc, ksf, vt, vsf, few_table, few, total;
 };
 
 // checks the two prefix arrays and lays the workspace out; false with st set on bad input
@@ -1058,9 +1060,10 @@ bool plan_varlen(const int64_t* cu_q, const int64_t* cu_k, int n_seqs, int Hq, i
     p.seqs_off = off;   off = align_up(off + sizeof(SeqDesc) * p.n_active, 256);
     p.jobs_off = off;   off = align_up(off + sizeof(QuantJob) * 3 * p.n_active, 256);
     p.prefix_off = off; off = align_up(off + sizeof(int32_t) * (3 * p.n_active + 1), 256);
-    p.groups_off = off; off = align_up(off + sizeof(ItemGroup) * static_cast<size_t>(p.groups), 1024);
+    p.groups_off = off; off = align_up(off + sizeof(ItemGroup) * static_cast<size_t>(p.groups), 256);
+    p.places_off = off; off = align_up(off + (p.items <= kOrderMaxItems ? sizeof(int32_t) * static_cast<size_t>(order_places(p.items)) : 0), 1024);
     p.tables = off - 1024;
-    p.items_off = off;  off = align_up(off + sizeof(ItemDesc) * static_cast<size_t>(p.items), 1024);
+    p.items_off = off;  off = align_up(off + sizeof(ItemDesc) * static_cast<size_t>(order_places(p.items)), 1024);
     p.qc = off;  off = align_up(off + static_cast<size_t>(p.q_rows) * 64, 1024);
     p.qsf = off; off = align_up(off + static_cast<size_t>(p.q_rows / kTile) * kSfBytes, 1024);
     p.kc = off;  off = align_up(off + static_cast<size_t>(p.k_rows) * 64, 1024);
@@ -1466,23 +1469,16 @@ extern "C" efq_status_t efq_attention_fwd_varlen(const void* q, const void* k, c
     // The heaviest query tiles of the whole batch first, so that the last CTAs to start are short ones.
     std::stable_sort(order.begin(), order.end(), [](const QueryTile& x, const QueryTile& y) { return x.weight > y.weight; });
     int64_t n_items = 0;
+    std::vector<ItemRun> runs;
     for (size_t i = 0; i < order.size(); ++i) {
         const SeqDesc& sd = seqs[order[i].seq];
         groups[i] = ItemGroup{static_cast<int32_t>(n_items), order[i].seq, order[i].qt, order[i].weight, static_cast<int32_t>(sd.Sq),
                               static_cast<int32_t>(sd.Sk), sd.packed};
-        n_items += sd.packed ? Hkv : Hq;
+        const int heads = sd.packed ? Hkv : Hq;
+        if (i > 0 && order[i].weight == order[i - 1].weight) runs.back().count += heads;
+        else runs.push_back(ItemRun{order[i].weight, heads});
+        n_items += heads;
     }
-
-    if (copy_table(ws + 1024, tables, s) != cudaSuccess) return EFQ_ERR_CUDA;
-    if (launch_quantize_jobs(reinterpret_cast<const QuantJob*>(ws + p.jobs_off), reinterpret_cast<const int32_t*>(ws + p.prefix_off),
-                             3 * p.n_active, ctas, reinterpret_cast<const ItemGroup*>(ws + p.groups_off), static_cast<int>(order.size()), n_items,
-                             reinterpret_cast<ItemDesc*>(ws + p.items_off), p.n_few > 0 ? nullptr : reinterpret_cast<uint32_t*>(ws), s) != cudaSuccess)
-        return EFQ_ERR_CUDA;
-
-    CUtensorMap mq, mk, mv;
-    if (!encode_map(&mq, ws + p.qc, 64, static_cast<uint64_t>(p.q_rows))) return EFQ_ERR_CUDA;
-    if (!encode_map(&mk, ws + p.kc, 64, static_cast<uint64_t>(p.k_rows))) return EFQ_ERR_CUDA;
-    if (!encode_map(&mv, ws + p.vt, static_cast<uint64_t>(p.k_cols / 2), static_cast<uint64_t>(Hkv) * 128)) return EFQ_ERR_CUDA;
 
     FwdParams P{};
     P.B = p.n_active; P.Hq = Hq; P.Hkv = Hkv; P.Sq = 0; P.Sk = p.longest; P.Sq_pad = 0; P.Sk_pad = 0;
@@ -1502,7 +1498,29 @@ extern "C" efq_status_t efq_attention_fwd_varlen(const void* q, const void* k, c
     P.rescale_threshold = threshold;
     P.has_dbg = 0;
     P.dbg = efq_debug_t{};
-    return launch_forward(producer, false, n_items, s, mq, mk, mv, P) == cudaSuccess ? EFQ_OK : EFQ_ERR_CUDA;
+
+    // persistent CTAs: places of the items, if one after the other is not good enough
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return EFQ_ERR_CUDA;
+    const int sms = sm_count(dev);
+    int64_t n_places = 0;
+    if (use_short(producer, false, n_items, sms, P)) n_places = order_items(runs, n_items, sms, reinterpret_cast<int32_t*>(tables.data() + (p.places_off - 1024)));
+    const int32_t* const places = n_places > 0 ? reinterpret_cast<const int32_t*>(ws + p.places_off) : nullptr;
+    tables.resize(p.places_off - 1024 + sizeof(int32_t) * static_cast<size_t>(n_places));
+    if (n_places == 0) n_places = n_items;
+
+    if (copy_table(ws + 1024, tables, s) != cudaSuccess) return EFQ_ERR_CUDA;
+    if (launch_quantize_jobs(reinterpret_cast<const QuantJob*>(ws + p.jobs_off), reinterpret_cast<const int32_t*>(ws + p.prefix_off),
+                             3 * p.n_active, ctas, reinterpret_cast<const ItemGroup*>(ws + p.groups_off), static_cast<int>(order.size()), places, n_places,
+                             reinterpret_cast<ItemDesc*>(ws + p.items_off), p.n_few > 0 ? nullptr : reinterpret_cast<uint32_t*>(ws), s) != cudaSuccess)
+        return EFQ_ERR_CUDA;
+
+    CUtensorMap mq, mk, mv;
+    if (!encode_map(&mq, ws + p.qc, 64, static_cast<uint64_t>(p.q_rows))) return EFQ_ERR_CUDA;
+    if (!encode_map(&mk, ws + p.kc, 64, static_cast<uint64_t>(p.k_rows))) return EFQ_ERR_CUDA;
+    if (!encode_map(&mv, ws + p.vt, static_cast<uint64_t>(p.k_cols / 2), static_cast<uint64_t>(Hkv) * 128)) return EFQ_ERR_CUDA;
+
+    return launch_forward(producer, false, n_places, s, mq, mk, mv, P) == cudaSuccess ? EFQ_OK : EFQ_ERR_CUDA;
 }
 
 extern "C" efq_status_t efq_poll_status(void* workspace, void* stream)

@@ -34,8 +34,8 @@ constexpr uint32_t kColSfQ1 = 440;         // scales of q1: 4 columns behind tho
 // The items of this CTA, one after the other: the CTAs take items in turn, every other round in reverse, so that the heavier items
 // of a round go to those that had the lighter ones before.  Every role walks them for itself, so a step has to be short: it
 // stands between the last tile of an item and the first of the next.  [B, H, S, d] batch (heaviest query tiles first, the heads of a
-// GQA group adjacent): query tile and head by additions.  Packed batch (TABLE; items sorted by weight in memory): the
-// entry of the next item is on its way while this one is worked on.
+// GQA group adjacent): query tile and head by additions.  Packed batch (TABLE; items in the places of a table, item_order.h): the
+// entry of the next item is on its way while this one is worked on; an empty place is the end.
 template <bool TABLE>
 struct ShortWalk {
     uint32_t k;                    // items before this one

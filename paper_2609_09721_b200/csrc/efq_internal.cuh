@@ -67,9 +67,10 @@ int sm_count(int dev);
 // Q, K and V of one [B, H, S, d] problem (or one sequence) in one launch; also clears the 256 status words.
 cudaError_t launch_quantize_qkv(const QuantSeg& q, const QuantSeg& k, const QuantSeg& v, uint32_t* status, cudaStream_t stream);
 // The jobs of a packed batch in one launch: jobs and first_cta (n_jobs + 1 prefix sums of CTAs) live in device memory.
+// places: the item in every place of the table, -1 for an empty place; null: the items one after the other (item_order.h).
 // status: the words to clear, null if an earlier launch of the call has cleared them.
 cudaError_t launch_quantize_jobs(const QuantJob* jobs, const int32_t* first_cta, int n_jobs, int64_t total_ctas, const ItemGroup* groups,
-                                 int n_groups, int64_t n_items, ItemDesc* items, uint32_t* status, cudaStream_t stream);
+                                 int n_groups, const int32_t* places, int64_t n_places, ItemDesc* items, uint32_t* status, cudaStream_t stream);
 // CTAs a job needs (256 threads each)
 int64_t quantize_job_ctas(const QuantJob& job);
 
@@ -93,7 +94,7 @@ struct __align__(16) ItemDesc {
     int32_t seq;             // index into the sequence table
     int32_t qt;              // query tile inside the sequence (0 when packed)
     int32_t head;            // query head, or KV head when packed
-    int32_t n_tiles;         // KV tiles that it walks
+    int32_t n_tiles;         // KV tiles that it walks; -1: an empty place, the CTA is through
     int32_t Sq, Sk, packed;  // of its sequence
     int32_t pad;
 };

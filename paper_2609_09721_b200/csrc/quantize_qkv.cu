@@ -134,10 +134,11 @@ __global__ void __launch_bounds__(256) quantize_qkv_kernel(const __grid_constant
 }
 
 // The jobs of a packed batch in one launch: a CTA finds its job by bisection of the prefix sums.  The CTAs after the last
-// job write the item table of the forward that follows (a thread per item).
+// job write the item table of the forward that follows (a thread per place).
 __global__ void __launch_bounds__(256) quantize_jobs_kernel(const QuantJob* __restrict__ jobs, const int32_t* __restrict__ first_cta,
                                                             int n_jobs, int n_quant, const ItemGroup* __restrict__ groups, int n_groups,
-                                                            int n_items, ItemDesc* __restrict__ items, uint32_t* status)
+                                                            const int32_t* __restrict__ places, int n_places,
+                                                            ItemDesc* __restrict__ items, uint32_t* status)
 {
     __shared__ QuantSmem sm;
     ptx::grid_wait();
@@ -145,15 +146,20 @@ __global__ void __launch_bounds__(256) quantize_jobs_kernel(const QuantJob* __re
     const int cta = blockIdx.x;
     if (cta == 0 && status != nullptr) status[threadIdx.x] = 0u;
     if (cta >= n_quant) {
-        const int item = (cta - n_quant) * 256 + static_cast<int>(threadIdx.x);
-        if (item >= n_items) return;
+        const int place = (cta - n_quant) * 256 + static_cast<int>(threadIdx.x);
+        if (place >= n_places) return;
+        const int item = places != nullptr ? __ldg(places + place) : place;
+        if (item < 0) {
+            items[place] = ItemDesc{0, 0, 0, -1, 0, 0, 0, 0};
+            return;
+        }
         int lo = 0, hi = n_groups;            // groups[lo].first_item <= item < groups[hi].first_item
         while (hi - lo > 1) {
             const int mid = (lo + hi) >> 1;
             if (__ldg(&groups[mid].first_item) <= item) lo = mid; else hi = mid;
         }
         const ItemGroup g = groups[lo];
-        items[item] = ItemDesc{g.seq, g.qt, item - g.first_item, g.n_tiles, g.Sq, g.Sk, g.packed, 0};
+        items[place] = ItemDesc{g.seq, g.qt, item - g.first_item, g.n_tiles, g.Sq, g.Sk, g.packed, 0};
         return;
     }
     int lo = 0, hi = n_jobs;                  // first_cta[lo] <= cta < first_cta[hi]
@@ -182,12 +188,12 @@ cudaError_t launch_quantize_qkv(const QuantSeg& q, const QuantSeg& k, const Quan
 }
 
 cudaError_t launch_quantize_jobs(const QuantJob* jobs, const int32_t* first_cta, int n_jobs, int64_t total_ctas, const ItemGroup* groups,
-                                 int n_groups, int64_t n_items, ItemDesc* items, uint32_t* status, cudaStream_t stream)
+                                 int n_groups, const int32_t* places, int64_t n_places, ItemDesc* items, uint32_t* status, cudaStream_t stream)
 {
-    const int64_t grid = total_ctas + (n_items + 255) / 256;
+    const int64_t grid = total_ctas + (n_places + 255) / 256;
     if (n_jobs <= 0 || total_ctas <= 0 || grid > 0x7fffffffll) return cudaErrorInvalidValue;
     return launch_overlapped(quantize_jobs_kernel, dim3(static_cast<unsigned>(grid)), 256, 0, stream, jobs, first_cta, n_jobs,
-                             static_cast<int>(total_ctas), groups, n_groups, static_cast<int>(n_items), items, status);
+                             static_cast<int>(total_ctas), groups, n_groups, places, static_cast<int>(n_places), items, status);
 }
 
 }  // namespace efq

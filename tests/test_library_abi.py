@@ -32,7 +32,7 @@ def test_header_symbols_are_exported():
 def test_no_read_only_loads_of_what_the_kernel_before_writes():
     """Blocks of an overlapped launch may be there while the kernel before still writes, so its data are not read through the read-only
     path.  The tables of a packed batch are: a copy from the host writes them, and a copy overlaps no kernel."""
-    tables = ("groups[mid].first_item", "first_cta + ")
+    tables = ("groups[mid].first_item", "first_cta + ", "places + ")
     for name in os.listdir(build.CSRC):
         for line in open(os.path.join(build.CSRC, name)):
             if "__ldg(" in line:

@@ -86,3 +86,26 @@ def test_short_walks_of_a_packed_batch(Hq, Hkv, causal, longest, producer):
         one = [t.permute(1, 0, 2)[None].contiguous() for t in (q[cu_q[n]:cu_q[n + 1]], k[cu_k[n]:cu_k[n + 1]], v[cu_k[n]:cu_k[n + 1]])]
         alone = binding.exp_then_quantize_attention_fwd(*one, causal, 0.0, 0) if producer else binding.efq_attention_fwd(*one, causal)
         assert torch.equal(got, alone[0]), f"sequence {n}"
+
+
+@pytest.mark.parametrize("Hq,Hkv,causal,producer,lens", [
+    (8, 2, True, 0, [(20000, 20000), (300, 16000), (5000, 13000), (64, 64)]),         # walks of up to 157 tiles
+    (4, 4, False, 1, [(1500, 13000), (13000, 1500), (400, 400)]), (8, 4, True, 4, [(14000, 14000), (3000, 9000), (129, 129)]),
+    (2, 2, False, 0, [(3000, 3000)] + [(60 + 7 * n, 60 + 7 * n) for n in range(60)]),  # a few long ones among many short: not in turn
+    (4, 4, True, 0, [(6000, 6000)] + [(50 + 7 * n, 50 + 7 * n) for n in range(63)]), (1, 1, True, 2, [(8000, 8000)] * 2 + [(80 + 12 * n, 80 + 12 * n) for n in range(60)]),
+    (28, 4, False, 0, [(5000, 5000)] + [(1 + 5 * n, 1 + 5 * n) for n in range(60)]),   # shared query tiles and few rows beside them
+    (2, 1, True, 0, [(9000, 9000), (4000, 300)] + [(90 + n, 10) for n in range(100)]),  # queries that see nothing, whole tiles of them
+])
+def test_long_walks_of_a_packed_batch(Hq, Hkv, causal, producer, lens):
+    """Walks of a hundred and more KV tiles in a packed batch, and a few long sequences among many short ones, whose items do not go round
+    in turn: each sequence equals its forward alone bit for bit."""
+    g = torch.Generator(device="cuda").manual_seed(14)
+    cu_q = np.concatenate([[0], np.cumsum([a for a, _ in lens])])
+    cu_k = np.concatenate([[0], np.cumsum([b for _, b in lens])])
+    q = torch.randn(int(cu_q[-1]), Hq, 128, generator=g, device="cuda").bfloat16()
+    k, v = (torch.randn(int(cu_k[-1]), Hkv, 128, generator=g, device="cuda").bfloat16() for _ in range(2))
+    o = binding.efq_attention_fwd_varlen(q, k, v, cu_q, cu_k, causal, 0.0, producer)
+    for n in range(len(lens)):
+        one = [t.permute(1, 0, 2)[None].contiguous() for t in (q[cu_q[n]:cu_q[n + 1]], k[cu_k[n]:cu_k[n + 1]], v[cu_k[n]:cu_k[n + 1]])]
+        alone = binding.exp_then_quantize_attention_fwd(*one, causal, 0.0, {1: 0, 2: 1, 4: 2}[producer]) if producer else binding.efq_attention_fwd(*one, causal)
+        assert torch.equal(o[cu_q[n]:cu_q[n + 1]].permute(1, 0, 2), alone[0]), f"sequence {n}"
