@@ -105,16 +105,20 @@ struct __align__(16) ItemDesc {
 constexpr int kFewMaxRows = 24;
 // The contexts that take it, by the sequence's own shape: up to 16 rows all, 17 to 24 rows from 64 KV tiles on.  Its time grows with
 // the rows (each has its codes made and its scores written for itself), that of the general path does not up to 128; but the
-// general path walks a whole context in one CTA a KV head.  Measured, this path against the general one, us, with 1 / 64 / 256 KV heads:
-//    8 rows: 2000 keys 11.8 / 27.6 / 80 against 18.8 / 27.2 / 80, 4000 keys 11.6 / 44.1 / 128 against 29.3 / 52.1 / 149; 8100 keys
-//            12.2 / 71 / 246 against 51.0 / 99 / 286
-//   16 rows: 1000 keys 11.9 / 22.6 / 59 against 14.4 / 18.6 / 46; 2000 keys 13.2 / 36 / 107 against 19.5 / 29 / 82; 4000 keys 12.8 / 62 / 159
-//            against 30.9 / 54 / 150; 8100 keys 13.2 / 94 / 290 against 51.9 / 100 / 287; 16000 keys 14.5 / 151 / 550 against 92.8 / 186 / 557
-//   24 rows: 1000 keys 19.2 / 29.5 / 75 against 14.0 / 17.9 / 44; 4000 keys 51 / 80 / 218 against 31.9 / 55 / 152 (both before few chunks
-//            were taken in parts); 8100 keys 15.3 / 128 / 388 against 52.8 / 101 / 289; 16000 keys 16.4 / 210 / 732 against 93.7 / 187 / 559
-// The number of heads and sequences must not matter to the line (a sequence gives the same bits alone and in a batch).  Up to 16
-// rows the gains of a few long contexts outweigh a loss of a fifth in wide batches of short ones; above, the line lies where a few
-// heads begin to gain.
+// general path walks a whole context in one CTA a KV head.  Measured, this path against the general one, us a call among others
+// with inputs of its own, 1 / 8 / 64 / 256 KV heads:
+//    8 rows:  1000 keys 10.1 / 10.4 / 19.8 /  52 against 13.4 / 12.6 / 17.9 /  43,  2000 keys 10.3 / 11.0 / 27.4 /  77 against 19.7 / 19.0 / 28.3 /  79,
+//             4000 keys 10.3 / 12.8 / 42.0 / 123 against 31.5 / 31.3 / 51.4 / 147,  8100 keys 11.3 / 19.3 / 67.6 / 235 against 51 / 56 / 98 / 285
+//   16 rows:  1000 keys 11.1 / 11.3 / 22.5 /  57 against 13.6 / 13.1 / 18.2 /  43,  2000 keys 11.4 / 12.3 / 34.6 /  98 against 19.8 / 19.8 / 28.7 /  79,
+//             4000 keys 11.6 / 14.2 / 58.6 / 155 against 31.6 / 32.3 / 52.1 / 148,  8100 keys 12.3 / 22.3 / 91.0 / 284 against 53 / 57 /  99 / 287,
+//            16000 keys 13.8 / 36.2 /  148 / 541 against   96 /  102 /  185 / 572
+//   24 rows:  1000 keys 12.9 / 14.4 / 28.5 /  74 against 12.6 / 12.5 / 18.3 /  44,  2000 keys 13.1 / 15.5 / 44.1 / 126 against 18.5 / 19.0 / 29.0 /  80,
+//             4100 keys 13.1 / 19.9 / 76.5 / 213 against 30.7 / 32.7 / 54.2 / 153,  6000 keys 14.1 / 21.3 / 83.3 / 292 against 40 / 44 / 75 / 216,
+//             8100 keys 14.4 / 28.6 /  123 / 378 against 51.4 / 57.2 / 99.5 / 288
+// The number of heads and sequences must not matter to the line (a sequence gives the same bits alone and in a batch), so it weighs a few
+// contexts against wide batches.  Up to 16 rows the gains of the few outweigh a loss of a fifth to a quarter in wide batches of short
+// ones.  At 17 to 24 rows the few gain from 2000 keys on by now, but 64 and more heads lose up to 1.6 times below 32 tiles and 1.4 (128
+// heads: 1.55) from there to 63; at 64 tiles, where the few gain 2 to 3.6 times, the wide still lose 1.25 to 1.4.
 __host__ __device__ inline bool few_takes(int64_t rows, int64_t n_tiles) { return rows <= 16 || (rows <= kFewMaxRows && n_tiles >= 64); }
 // Tiles of a chunk of the KV range, by the sequence's own shape: short contexts are cut finely, so that one of them spreads
 // over the chip; with many rows a chunk's partial result (544 bytes a row) has to be small against its 64 KB of K and V a tile.
