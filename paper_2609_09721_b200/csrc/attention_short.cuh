@@ -1,4 +1,5 @@
-// Fused forward with persistent CTAs: the kernel of attention_fwd.cu (which includes this file) for more query tiles than SMs.
+// Fused forward with persistent CTAs: the kernel of attention_fwd.cu (which includes this file) for more query tiles than SMs, at
+// every length of the KV walk (its name is from the short walks that it was made for).
 //
 // A CTA of attention_fwd_kernel spends about 10000 cycles outside its tiles: start, barriers, TMEM, the latency of the first
 // loads and scores, the last P~V, the rows on their way out.  Against 512 keys, 4 tiles of about 1500 cycles, that is more than
@@ -10,9 +11,9 @@
 //
 // What bounds it: the probability warps in long walks; in short ones what stands between the last P~V of an item and the first
 // rescaling of the next, and the size of the code.  The five kinds of warp run different code at the same time and evict one
-// another from the instruction cache: at 75 KB, 40 % of its lookups missed and warps without an instruction were the largest stall
-// (256 keys).  Hence waits of a few instructions, masks from a bit word, loops that are not unrolled, no divisions from item to
-// item.
+// another from the instruction cache: with 65 KB of code 13 % of its lookups missed against 256 keys and 10 % against 512, with the 51 KB of
+// now 6 % and 5 %; a form of 75 KB, not kept, missed 40 %, and warps without an instruction were its largest stall.  Hence waits of
+// a few instructions, masks from a bit word, loops that are not unrolled, no divisions from item to item.
 //
 // Measured against one CTA per tile, whole call, us.  Affine rule, 24 heads, 16000 queries, not causal: 128 keys 146 -> 65, 256 keys
 // 159 -> 83, 512 191 -> 109, 1024 254 -> 167, 2048 378 -> 288, 4096 619 -> 527, 16384 1998 -> 1897; causal, 32 heads: 32 x 128 tokens

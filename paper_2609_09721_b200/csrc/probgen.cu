@@ -143,7 +143,10 @@ __device__ __forceinline__ void probgen_body(const float* __restrict__ scores, i
                                              int64_t rows, int64_t cols, const ProducerConsts& K, uint8_t* __restrict__ codes,
                                              uint8_t* __restrict__ scales, int aligned32)
 {
-    ptx::grid_wait();                // launched while the kernel before drains, which takes some 2 us off a call among others
+    // Launched while the call before drains: among calls in a stream 11419 x 322 10.3 -> 8.6 us, 4096 x 16384 47.6 -> 45.8; in a graph,
+    // where launches follow closer, 8.7 -> 8.5 and 45.7 -> 45.2.  Behind a kernel that is not of this library it changes nothing or costs
+    // up to 0.2 us.
+    ptx::grid_wait();
     ptx::grid_launch_next();
     const int lane = threadIdx.x & 31;
     const int64_t segs_per_row = (cols + kSegCols - 1) / kSegCols;
@@ -176,8 +179,8 @@ __device__ __forceinline__ void probgen_body(const float* __restrict__ scores, i
                 r[i][4] = b.x; r[i][5] = b.y; r[i][6] = b.z; r[i][7] = b.w;
             }
         } else {
-            // the end of a row, or all of a short one: eight columns at a time as long as there are eight (one at a time: 11419
-            // rows of 322 columns 12.7 -> 9.0 us, 2000 of 3001 8.7 -> 6.6)
+            // the end of a row, or all of a short one: eight columns at a time as long as there are eight (against one at a time, in
+            // a graph, launches not overlapped: 11419 rows of 322 columns 9.7 -> 8.7 us, 2000 of 3001 7.9 -> 7.4)
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const int c = (i * 32 + lane) * 8;
@@ -207,8 +210,8 @@ __device__ __forceinline__ void probgen_body(const float* __restrict__ scores, i
 }
 
 // Four resident CTAs per SM (64 registers): bound by memory, and what counts is how many loads are in flight.  4096 x 16384:
-// 49.8 us with 70 registers and three CTAs, 61.7 with the 104 that the compiler would take, 46.0 with four CTAs, 6.6 TB/s;
-// 16000 x 20000 226 -> 210; exp-then-quantize 49.6 -> 48.0.
+// 49.8 us with 70 registers and three CTAs, 61.7 with the 104 that the compiler would take, 46.0 with four CTAs, 6.6 TB/s (calls one after
+// another; a call by itself on buffers that were not used before takes 51); 16000 x 20000 226 -> 210; exp-then-quantize 49.6 -> 48.0.
 template <int PRODUCER>
 __global__ void __launch_bounds__(kWarpsPerCta * 32, 4)
 probgen_kernel(const float* __restrict__ scores, int64_t ld, const float* __restrict__ row_max, int64_t rows, int64_t cols,
@@ -248,7 +251,7 @@ efq_status_t launch_probgen(int producer, const float* scores, int64_t ld, const
     ProducerConsts K = producer == kEfqLut ? make_producer_consts_lut(sigma) : make_producer_consts(sigma, tau, h);
     const int64_t n_tasks = rows * ((cols + kSegCols - 1) / kSegCols);
     int64_t ctas = (n_tasks + kWarpsPerCta - 1) / kWarpsPerCta;
-    const int64_t cap = static_cast<int64_t>(sms) * 8 * 64;   // whole waves of 8 resident CTAs per SM
+    const int64_t cap = static_cast<int64_t>(sms) * 8 * 64;   // at most 128 waves of four resident CTAs per SM
     if (ctas > cap) ctas = cap;
     const dim3 grid(static_cast<unsigned>(ctas));
     const int a32 = ((reinterpret_cast<uintptr_t>(scores) & 31u) == 0 && (ld & 7) == 0) ? 1 : 0;   // 256-bit loads allowed

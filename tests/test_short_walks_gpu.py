@@ -1,6 +1,6 @@
-"""Persistent CTAs for short KV walks (more query tiles than SMs): every row equals, bit for bit, what the kernel with one
+"""Persistent CTAs (more query tiles than SMs), short KV walks and long ones: every row equals, bit for bit, what the kernel with one
 CTA per query tile returns (it is the one that runs when the operand is dumped), and sampled rows match the CPU oracle.  Key
-counts at the edges of a tile and of the dispatch rule, ragged query tiles, GQA, batches, items without a visible key."""
+counts at the edges of a tile, ragged query tiles, GQA, batches, items without a visible key."""
 import numpy as np
 import pytest
 import torch
@@ -14,14 +14,14 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("B,Hq,Hkv,Sq,Sk,causal,producer,threshold", [
     (1, 24, 24, 1000, 1, False, "efq", 0.0), (1, 8, 2, 2500, 128, False, "efq", 0.0), (2, 8, 8, 1281, 129, False, "efq", 0.0),
     (1, 24, 24, 2100, 512, False, "efq", 0.0), (1, 12, 4, 3000, 1000, False, "efq", 0.0), (1, 8, 4, 2560, 5120, False, "efq", 0.0),
-    (1, 8, 4, 2560, 5121, False, "efq", 0.0),                                # one key past the rule: one CTA per query tile
+    (1, 8, 4, 2560, 5121, False, "efq", 0.0),                                # one key in the last tile
     (100, 4, 2, 127, 127, True, "efq", 0.0), (40, 4, 1, 130, 256, True, "efq", 0.0), (3, 16, 4, 600, 1024, True, "efq", 0.0),
     (5, 8, 2, 900, 200, True, "efq", 0.0),                                   # the first 700 queries see nothing
     (2, 16, 4, 700, 400, False, "efq", 1.0), (2, 16, 4, 700, 400, False, "lut", 0.0),
     (2, 16, 4, 700, 400, False, "etq0", 0.0), (2, 16, 4, 700, 400, False, "etq1", 0.0),
     (2, 16, 4, 700, 400, True, "etq2", 0.0), (2, 16, 4, 700, 400, False, "etq3", 0.0), (2, 16, 4, 700, 400, False, "etq4", 0.0),
     (1, 16, 4, 1300, 4000, True, "etq0", 0.0), (1, 16, 4, 1300, 4000, True, "etq2", 0.0), (2, 16, 4, 700, 400, True, "lut", 0.0), (1, 8, 2, 2600, 6400, True, "efq", 0.0),
-    (1, 8, 4, 2560, 2048, False, "lut", 0.0), (1, 8, 4, 2560, 2049, False, "lut", 0.0),          # at the lines of the other producers
+    (1, 8, 4, 2560, 2048, False, "lut", 0.0), (1, 8, 4, 2560, 2049, False, "lut", 0.0),          # the other producers at the edge of a tile
     (1, 8, 4, 2560, 8192, False, "etq0", 0.0), (1, 8, 4, 2560, 8193, False, "etq1", 0.0), (1, 8, 4, 2560, 9000, False, "etq2", 0.0),
 ])
 def test_short_walks_equal_one_cta_per_tile(oracle, B, Hq, Hkv, Sq, Sk, causal, producer, threshold):
@@ -69,7 +69,7 @@ def test_long_walks_equal_one_cta_per_tile(Hq, Hkv, Sq, Sk, causal, producer):
 
 @pytest.mark.parametrize("Hq,Hkv,causal,longest,producer", [(8, 2, True, 1000, 0), (6, 6, False, 5120, 0), (8, 4, True, 5121, 0), (8, 2, True, 700, 1), (8, 2, False, 512, 1)])
 def test_short_walks_of_a_packed_batch(Hq, Hkv, causal, longest, producer):
-    """Sequences of mixed lengths, up to the longest that the rule takes and one past it: shared query tiles (few tokens), the
+    """Sequences of mixed lengths, whole last tiles and one key more: shared query tiles (few tokens), the
     few-row path beside them, queries that see nothing, none at all.  Each equals its forward alone bit for bit."""
     g = torch.Generator(device="cuda").manual_seed(13)
     lens = [(500, longest), (40, 300), (1, 200), (300, 100), (129, 129), (0, 50), (30, 257), (128, 128), (70, 0), (1300, min(640, longest)), (257, 384), (1000, 512)]
