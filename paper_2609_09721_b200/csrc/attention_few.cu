@@ -186,15 +186,19 @@ __global__ void __launch_bounds__(kFewThreads, N <= 8 ? 4 : 3) few_scores_kernel
     __shared__ FewSmem smem;
     FewSmem* const sm = &smem;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    // A block takes 2^-split of a chunk: the scores of a tile need nothing of another, and a few chunks do not fill the chip.  The
-    // sequence table was written by a copy, which overlaps no kernel.
-    Unit u = find_unit(P, static_cast<int>(blockIdx.x) >> P.split);
-    const int R = P.G * u.Sq;
-    if (!take_part(u, R, P.split)) return;       // never block 0
-    few_setup(sm, warp);
+    few_setup(sm, warp);             // before the search for the unit, which takes longer
     ptx::grid_wait();                // the kernels before: inputs, and the workspace of an earlier call
     ptx::grid_launch_next();
+    // A block takes 2^-split of a chunk: the scores of a tile need nothing of another, and a few chunks do not fill the chip.
+    Unit u = find_unit(P, static_cast<int>(blockIdx.x) >> P.split);
+    const int R = P.G * u.Sq;
+    const bool work = take_part(u, R, P.split);
     if (blockIdx.x == 0) P.status[tid] = 0u;
+    if (!work) {
+        __syncthreads();
+        if (warp == 0) ptx::tmem_dealloc(sm->tmem_base, kFewTmemCols);
+        return;
+    }
     // K: a quad of lanes takes a key, a lane every fourth 16-byte piece of it - a load instruction reads 64 contiguous
     // bytes of every key - and so a quarter of each of the four blocks
     const int quad = tid & 3, key_in_tile = tid >> 2;
