@@ -228,7 +228,7 @@ __global__ void __launch_bounds__(kFewThreads, N <= 8 ? 4 : 3) few_scores_kernel
         uint32_t w[16];
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            const uint4 x = __ldca(src + i);
+            const uint4 x = src[i];
             w[4 * i] = x.x; w[4 * i + 1] = x.y; w[4 * i + 2] = x.z; w[4 * i + 3] = x.w;
         }
         uint4 c;
@@ -741,9 +741,9 @@ cudaError_t launch_few(int producer, FewParams& P, cudaStream_t stream)
     if (cudaGetDevice(&dev) != cudaSuccess) return cudaErrorInvalidDevice;
     // Chunks in halves, quarters, eighths as long as every part has a tile and the blocks are all on the chip together (three on each
     // SM; with four or six 32 heads of 3000 keys 19.1 -> 19.2 and 22.8 us, 28 / 4 heads of 20000 22.0 -> 22.2 and 24.1).  Whole
-    // chunks -> parts: one head of 2000 keys 11.9 -> 9.1 us, 32 / 8 heads of 3000 keys 14.2 -> 11.6, of 6000 19.9 -> 14.3, 16 rows of 4000
-    // 35.9 -> 11.1.  Blocks without a tile cost more than they spread: chunks of one tile in eight, 32 / 8 heads of 700 keys
-    // 10.0 -> 11.1 us, of 1500 10.6 -> 12.1, 9.8 and 10.3 with none; chunks of two in eight, four heads of 3000 keys 12.1, 10.0 with none.
+    // chunks -> parts: one head of 2000 keys 12.0 -> 9.5 us, 32 / 8 heads of 3000 keys 14.3 -> 11.8, of 6000 19.9 -> 14.4, 16 rows of 4000
+    // 35.7 -> 11.2.  Blocks without a tile cost more than they spread: chunks of one tile in eight, 32 / 8 heads of 700 keys
+    // 10.1 -> 11.1 us, of 1500 10.8 -> 12.1, 10.1 and 10.8 with none; chunks of two in eight, four heads of 3000 keys 12.2, 10.1 with none.
     P.split = 0;
     while ((2 << P.split) <= P.longest_chunk && (static_cast<int64_t>(P.n_units) << (P.split + 1)) <= 3 * sm_count(dev)) ++P.split;
     if (P.row_cap <= 8) return launch_n<8>(producer, P, stream);

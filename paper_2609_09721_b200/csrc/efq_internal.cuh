@@ -107,18 +107,18 @@ constexpr int kFewMaxRows = 24;
 // the rows (each has its codes made and its scores written for itself), that of the general path does not up to 128; but the
 // general path walks a whole context in one CTA a KV head.  Measured, this path against the general one, us a call among others
 // with inputs of its own, 1 / 8 / 64 / 256 KV heads:
-//    8 rows:  1000 keys 10.1 / 10.4 / 19.8 /  52 against 13.4 / 12.6 / 17.9 /  43,  2000 keys 10.3 / 11.0 / 27.4 /  77 against 19.7 / 19.0 / 28.3 /  79,
-//             4000 keys 10.3 / 12.8 / 42.0 / 123 against 31.5 / 31.3 / 51.4 / 147,  8100 keys 11.3 / 19.3 / 67.6 / 235 against 51 / 56 / 98 / 285
-//   16 rows:  1000 keys 11.1 / 11.3 / 22.5 /  57 against 13.6 / 13.1 / 18.2 /  43,  2000 keys 11.4 / 12.3 / 34.6 /  98 against 19.8 / 19.8 / 28.7 /  79,
-//             4000 keys 11.6 / 14.2 / 58.6 / 155 against 31.6 / 32.3 / 52.1 / 148,  8100 keys 12.3 / 22.3 / 91.0 / 284 against 53 / 57 /  99 / 287,
-//            16000 keys 13.8 / 36.2 /  148 / 541 against   96 /  102 /  185 / 572
-//   24 rows:  1000 keys 12.9 / 14.4 / 28.5 /  74 against 12.6 / 12.5 / 18.3 /  44,  2000 keys 13.1 / 15.5 / 44.1 / 126 against 18.5 / 19.0 / 29.0 /  80,
-//             4100 keys 13.1 / 19.9 / 76.5 / 213 against 30.7 / 32.7 / 54.2 / 153,  6000 keys 14.1 / 21.3 / 83.3 / 292 against 40 / 44 / 75 / 216,
-//             8100 keys 14.4 / 28.6 /  123 / 378 against 51.4 / 57.2 / 99.5 / 288
+//    8 rows:  1000 keys 10.4 / 10.8 / 20.2 / 55 against 12.4 / 12.3 / 17.9 / 43, 2000 keys 10.5 / 11.5 / 28.2 / 79 against 18.0 / 18.7 / 28.2
+//             / 79, 4000 keys 10.7 / 14.0 / 43 / 127 against 28.8 / 31.0 / 52 / 147, 8100 keys 11.4 / 19.7 / 70 / 246 against 49 / 56 / 98 / 285
+//   16 rows:  1000 keys 11.0 / 11.5 / 23.0 / 58 against 12.5 / 12.6 / 18.1 / 43, 2000 keys 11.8 / 12.4 / 34.9 / 100 against 18.5 / 19.0 / 28.6
+//             / 80, 4000 keys 11.7 / 15.1 / 60 / 155 against 29.4 / 31.5 / 52 / 148, 8100 keys 12.3 / 22.8 / 93 / 289 against 51 / 57 / 99 / 287,
+//             16000 keys 13.9 / 36.7 / 151 / 549 against 92 / 102 / 185 / 556
+//   24 rows:  1000 keys 12.8 / 14.6 / 29.0 / 75 against 12.7 / 12.5 / 18.2 / 44, 2000 keys 13.4 / 15.8 / 45 / 129 against 18.5 / 19.2 / 28.8 / 80,
+//             4100 keys 13.6 / 20.0 / 78 / 217 against 30.7 / 32.7 / 54 / 153, 6000 keys 14.1 / 21.3 / 86 / 299 against 40 / 44 / 75 / 216,
+//             8100 keys 14.3 / 29.0 / 125 / 387 against 51 / 57 / 100 / 288
 // The number of heads and sequences must not matter to the line (a sequence gives the same bits alone and in a batch), so it weighs a few
 // contexts against wide batches.  Up to 16 rows the gains of the few outweigh a loss of a fifth to a quarter in wide batches of short
-// ones.  At 17 to 24 rows the few gain from 2000 keys on by now, but 64 and more heads lose up to 1.6 times below 32 tiles and 1.4 (128
-// heads: 1.55) from there to 63; at 64 tiles, where the few gain 2 to 3.6 times, the wide still lose 1.25 to 1.4.
+// ones.  At 17 to 24 rows the few gain from 2000 keys on by now, but 64 and more heads lose up to 1.7 times below 32 tiles and 1.4 (128
+// heads: 1.6) from there to 63; at 64 tiles, where the few gain 2 to 3.6 times, the wide still lose 1.25 to 1.45.
 __host__ __device__ inline bool few_takes(int64_t rows, int64_t n_tiles) { return rows <= 16 || (rows <= kFewMaxRows && n_tiles >= 64); }
 // Tiles of a chunk of the KV range, by the sequence's own shape: short contexts are cut finely, so that one of them spreads
 // over the chip; with many rows a chunk's partial result (544 bytes a row) has to be small against its 64 KB of K and V a tile.

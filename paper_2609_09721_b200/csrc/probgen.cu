@@ -139,7 +139,7 @@ __device__ __forceinline__ void load8(const float* p, float (&r)[8])
 }
 
 template <int PRODUCER>
-__device__ __forceinline__ void probgen_body(const float* __restrict__ scores, int64_t ld, const float* __restrict__ row_max,
+__device__ __forceinline__ void probgen_body(const float* __restrict__ scores, int64_t ld, const float* row_max,
                                              int64_t rows, int64_t cols, const ProducerConsts& K, uint8_t* __restrict__ codes,
                                              uint8_t* __restrict__ scales, int aligned32)
 {
@@ -160,6 +160,7 @@ __device__ __forceinline__ void probgen_body(const float* __restrict__ scores, i
         const int64_t row = n_tasks <= 0x7fffffff ? static_cast<int64_t>(static_cast<uint32_t>(task) / static_cast<uint32_t>(segs_per_row)) : task / segs_per_row;
         const int64_t c0 = (task - row * segs_per_row) * kSegCols;
         const float* src = scores + row * ld + c0;
+        const float m_s = row_max[row];
         uint8_t* crow = codes + row * nblk * (kMxBlock / 2) + c0 / 2;
         uint8_t* srow = scales + row * nblk + c0 / kMxBlock;
         const bool full = c0 + kSegCols <= cols;
@@ -195,7 +196,6 @@ __device__ __forceinline__ void probgen_body(const float* __restrict__ scores, i
                 }
             }
         }
-        const float m_s = __ldca(row_max + row);       // behind the loads of the scores (before them: 51.2 -> 51.9 us)
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             uint32_t code32, byte;
@@ -214,7 +214,7 @@ __device__ __forceinline__ void probgen_body(const float* __restrict__ scores, i
 // another; a call by itself on buffers that were not used before takes 51); 16000 x 20000 226 -> 210; exp-then-quantize 49.6 -> 48.0.
 template <int PRODUCER>
 __global__ void __launch_bounds__(kWarpsPerCta * 32, 4)
-probgen_kernel(const float* __restrict__ scores, int64_t ld, const float* __restrict__ row_max, int64_t rows, int64_t cols,
+probgen_kernel(const float* __restrict__ scores, int64_t ld, const float* row_max, int64_t rows, int64_t cols,
                ProducerConsts K, uint8_t* __restrict__ codes, uint8_t* __restrict__ scales, int aligned32)
 {
     probgen_body<PRODUCER>(scores, ld, row_max, rows, cols, K, codes, scales, aligned32);
@@ -223,7 +223,7 @@ probgen_kernel(const float* __restrict__ scores, int64_t ld, const float* __rest
 // The LUT producer is issue-bound and register-hungry (one code at a time through a 64-bit shift): it gains more from
 // three resident CTAs per SM than from the registers the compiler would otherwise take (69 -> 54 microseconds).
 __global__ void __launch_bounds__(kWarpsPerCta * 32, 3)
-probgen_lut_kernel(const float* __restrict__ scores, int64_t ld, const float* __restrict__ row_max, int64_t rows,
+probgen_lut_kernel(const float* __restrict__ scores, int64_t ld, const float* row_max, int64_t rows,
                    int64_t cols, ProducerConsts K, uint8_t* __restrict__ codes, uint8_t* __restrict__ scales, int aligned32)
 {
     probgen_body<kEfqLut>(scores, ld, row_max, rows, cols, K, codes, scales, aligned32);

@@ -27,9 +27,9 @@ __device__ __forceinline__ bool elect_one()
 }
 
 // ---------------------------------------------------------------- overlap with the neighbouring kernels of the stream
-// The work before this kernel has finished and is visible.  What it may have written is read behind the wait by loads that keep their
-// place (__ldca, __ldcg, __ldcs, volatile ones): a read-only load (__ldg, or of a const __restrict__ parameter) promises data that nobody
-// writes as long as this kernel is there, and blocks of it may be there while the kernel before still writes.
+// The work before this kernel has finished and is visible.  What it may have written is read behind the wait by plain loads, __ldcg,
+// __ldcs or volatile ones: a read-only load (__ldg, or through a pointer that is const and __restrict__) promises data that nobody writes
+// as long as this kernel is there, and blocks of it may be there while the kernel before still writes.
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // The kernel after this one may start its blocks (it waits by grid_wait() for what it needs).
 __device__ __forceinline__ void grid_launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
