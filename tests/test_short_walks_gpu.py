@@ -105,6 +105,13 @@ def test_long_walks_of_a_packed_batch(Hq, Hkv, causal, producer, lens):
     q = torch.randn(int(cu_q[-1]), Hq, 128, generator=g, device="cuda").bfloat16()
     k, v = (torch.randn(int(cu_k[-1]), Hkv, 128, generator=g, device="cuda").bfloat16() for _ in range(2))
     o = binding.efq_attention_fwd_varlen(q, k, v, cu_q, cu_k, causal, 0.0, producer)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):                    # the table that the host wrote is read at every replay
+        recorded = binding.efq_attention_fwd_varlen(q, k, v, cu_q, cu_k, causal, 0.0, producer)
+    for _ in range(2):
+        recorded.fill_(float("nan"))
+        graph.replay()
+        assert torch.equal(recorded, o)
     for n in range(len(lens)):
         one = [t.permute(1, 0, 2)[None].contiguous() for t in (q[cu_q[n]:cu_q[n + 1]], k[cu_k[n]:cu_k[n + 1]], v[cu_k[n]:cu_k[n + 1]])]
         alone = binding.exp_then_quantize_attention_fwd(*one, causal, 0.0, {1: 0, 2: 1, 4: 2}[producer]) if producer else binding.efq_attention_fwd(*one, causal)
