@@ -1066,7 +1066,7 @@ bool plan_varlen(const int64_t* cu_q, const int64_t* cu_k, int n_seqs, int Hq, i
     p.jobs_off = off;   off = align_up(off + sizeof(QuantJob) * 3 * p.n_active, 256);
     p.prefix_off = off; off = align_up(off + sizeof(int32_t) * (3 * p.n_active + 1), 256);
     p.groups_off = off; off = align_up(off + sizeof(ItemGroup) * static_cast<size_t>(p.groups), 256);
-    p.places_off = off; off = align_up(off + (p.items <= kOrderMaxItems ? sizeof(int32_t) * static_cast<size_t>(order_places(p.items)) : 0), 1024);
+    p.places_off = off; off = align_up(off + sizeof(int32_t) * static_cast<size_t>(order_places(std::min(p.items, kOrderMaxItems))), 1024);
     p.tables = off - 1024;
     p.items_off = off;  off = align_up(off + sizeof(ItemDesc) * static_cast<size_t>(order_places(p.items)), 1024);
     p.qc = off;  off = align_up(off + static_cast<size_t>(p.q_rows) * 64, 1024);

@@ -24,8 +24,9 @@ constexpr int kItemCost = 3;                   // what an item costs beside its 
 constexpr int64_t kOrderMaxItems = 16 * 148;
 // Items for which ordering has to save a tile: they take the host some 0.5 us, a tile 0.7 to 1.3
 constexpr int64_t kOrderItemsPerTile = 64;
-// Places of the item table that n items may take, in order or not
-constexpr int64_t order_places(int64_t n_items) { return n_items <= kOrderMaxItems ? 3 * n_items : n_items; }
+// Places of the item table for n items, in order or not.  More items never take fewer: a workspace that is large enough for a batch
+// stays so for a smaller one, though that may be ordered and the larger one not.
+constexpr int64_t order_places(int64_t n_items) { return n_items + 2 * std::min(n_items, kOrderMaxItems); }
 
 // Place of a CTA's item number k
 constexpr int64_t place_in_turn(int64_t k, int64_t cta, int64_t ctas) { return k * ctas + (k & 1 ? ctas - 1 - cta : cta); }

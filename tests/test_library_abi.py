@@ -130,6 +130,13 @@ def test_few_row_sequences_of_a_packed_batch_take_no_more_than_their_copies(lens
     assert _varlen_bytes(cu_q, cu_k, Hkv, Hkv) <= copies + 1024 * len(lens) + 16384        # a table entry each on the general path
 
 
+def test_workspace_of_a_packed_batch_grows_with_it():
+    """A workspace that is large enough for a batch is so for every smaller one, across the number of items (2368) up to which their
+    order may take more places than they are: a query tile more never needs less."""
+    sizes = [_varlen_bytes([0, 128 * n, 128 * n + 300], [0, 300, 600], 1, 1) for n in range(2340, 2400)]
+    assert all(a <= b for a, b in zip(sizes, sizes[1:]))
+
+
 def test_calls_do_not_hold_the_interpreter_lock(tmp_path):
     """While a call of the extension waits (here in functions that sleep in the place of the library's), other Python threads
     run: the counting thread gets on during each of the six calls."""
