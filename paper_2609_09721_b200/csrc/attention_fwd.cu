@@ -31,7 +31,6 @@
 #include <algorithm>
 #include <atomic>
 #include <mutex>
-#include <type_traits>
 #include <vector>
 
 #include "efq_common.cuh"
@@ -118,7 +117,7 @@ struct FwdParams {
     float rescale_threshold;  // 0: Algorithm 2; > 0: the shifting maximum is kept while the true one is at most this far above
 };
 
-// Waits end with the completion or, false, when the CTA gave up.  That is one warp's business (stalled below): the kernels inline
+// Waits end with the completion or, false, when the CTA gave up.  That is one warp's business (wait_watching): the kernels inline
 // some twenty-five waits, and a clock in each of them made a sixth of the code, which outgrows the instruction cache as it is.
 __device__ __forceinline__ bool wait1(uint64_t* bar, uint32_t parity, Smem* sm)
 {
@@ -739,7 +738,6 @@ struct Workspace {
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 bool use_few(int Hq, int Hkv, int64_t Sq, int64_t Sk);
-int64_t few_chunks(int64_t Sk, int64_t rows);
 
 Workspace plan_workspace(int B, int Hq, int Hkv, int64_t Sq, int64_t Sk)
 {

@@ -46,6 +46,28 @@ def test_short_walks_equal_one_cta_per_tile(oracle, B, Hq, Hkv, Sq, Sk, causal, 
         assert torch.all(o[:, :, : Sq - Sk] == 0)
 
 
+@pytest.mark.parametrize("B,Hq,Hkv,Sq,Sk,producer", [
+    (2, 16, 4, 1087, 470, "efq"), (8, 8, 8, 900, 200, "etq0"), (1, 32, 8, 2000, 1, "lut"),      # most items see nothing, and all but the last
+    (20, 8, 8, 384, 128, "efq"), (20, 8, 8, 384, 129, "etq2"), (20, 8, 8, 384, 257, "efq"),      # whole tiles of zeros: two, one, one
+])
+def test_queries_before_the_first_key(B, Hq, Hkv, Sq, Sk, producer):
+    """Causal with more queries than keys: the rows that see nothing are written as zeros, whole tiles of them by themselves; the others
+    are those of the kernel with one CTA per query tile."""
+    g = torch.Generator(device="cuda").manual_seed(Sq + Sk)
+    q = torch.randn(B, Hq, Sq, 128, generator=g, device="cuda").bfloat16()
+    k, v = (torch.randn(B, Hkv, Sk, 128, generator=g, device="cuda").bfloat16() for _ in range(2))
+
+    def forward(debug=None):
+        o = torch.full((B, Hq, Sq, 128), float("nan"), device="cuda")
+        if producer.startswith("etq"):
+            return binding.exp_then_quantize_attention_fwd(q, k, v, True, 0.0, int(producer[3:]), o, debug=debug)
+        return binding.efq_attention_fwd(q, k, v, True, 0.0, (MEAN[0], MEAN[1], int(producer == "lut"), 0, 0.0), o, debug=debug)
+
+    o = forward()
+    assert torch.all(o[:, :, : Sq - Sk] == 0)
+    assert torch.equal(o, forward(binding.DebugDump(0, Hq - 1, 0, 1, Sk)))
+
+
 @pytest.mark.parametrize("Hq,Hkv,Sq,Sk,causal,producer", [
     (24, 24, 900, 30000, False, "efq"), (32, 8, 20000, 20000, True, "efq"),     # walks of 235 tiles, of 1 to 157
     (24, 24, 900, 6144, False, "lut"), (24, 24, 900, 6145, False, "lut"),       # the line of the table form, one key past it
