@@ -744,8 +744,15 @@ cudaError_t launch_few(int producer, FewParams& P, cudaStream_t stream)
     // chunks -> parts: one head of 2000 keys 12.0 -> 9.5 us, 32 / 8 heads of 3000 keys 14.3 -> 11.8, of 6000 19.9 -> 14.4, 16 rows of 4000
     // 35.7 -> 11.2.  Blocks without a tile cost more than they spread: chunks of one tile in eight, 32 / 8 heads of 700 keys
     // 10.1 -> 11.1 us, of 1500 10.8 -> 12.1, 10.1 and 10.8 with none; chunks of two in eight, four heads of 3000 keys 12.2, 10.1 with none.
+    // The merge of parts has a block of 512 threads for every row, two on an SM at a time.  With more of them than that, parts of short
+    // chunks cost more than they spread: whole -> parts 16 rows of 96 heads, 300 keys 17.0 -> 31.2 us, of 64 heads, 600 keys 16.4 -> 25.8, of
+    // 32 heads, 984 keys 16.0 -> 18.9, 12 rows of 32 heads, 300 keys 13.9 -> 14.3, but of 24 heads 13.7 -> 12.7.  Of eight tiles they gain
+    // with every number of rows that this leaves (16 rows of 32 heads, 4200 keys 39.5 -> 39.3, 6000 keys 48.9 -> 43.2, of 55 heads, 4096 keys
+    // 50.7 -> 47.4).
     P.split = 0;
-    while ((2 << P.split) <= P.longest_chunk && (static_cast<int64_t>(P.n_units) << (P.split + 1)) <= 3 * sm_count(dev)) ++P.split;
+    const int sms = sm_count(dev);
+    if (P.longest_chunk == kFewMaxChunk || static_cast<int64_t>(P.n_heads) * P.row_cap <= 2 * sms)
+        while ((2 << P.split) <= P.longest_chunk && (static_cast<int64_t>(P.n_units) << (P.split + 1)) <= 3 * sms) ++P.split;
     if (P.row_cap <= 8) return launch_n<8>(producer, P, stream);
     if (P.row_cap <= 16) return launch_n<16>(producer, P, stream);
     return launch_n<24>(producer, P, stream);

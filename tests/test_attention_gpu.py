@@ -451,6 +451,18 @@ def test_bounded_wait_expires_and_context_stays_usable(oracle):
     assert np.abs(o.cpu().numpy()[0, 0] - want).max() <= TOL_O
 
 
+def _recorded(call):
+    """The kernels that the call launches, names and blocks, from a graph that it is recorded into and that does not run."""
+    from cuda.bindings import driver
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        call()
+    nodes = driver.cuGraphGetNodes(graph.raw_cuda_graph(), 64)[1]
+    params = [driver.cuGraphKernelNodeGetParams(n) for n in nodes]          # an error for nodes of other kinds
+    name = lambda p: (driver.cuFuncGetName(p.func) if p.func else driver.cuKernelGetName(p.kern))[1].decode()
+    return [(name(p), p.gridDimX) for e, p in params if e == 0]
+
+
 def _kernels(call):
     """Names of the kernels that the call launched."""
     with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as prof:
@@ -459,7 +471,7 @@ def _kernels(call):
     return " ".join(e.key for e in prof.key_averages())
 
 
-@pytest.mark.parametrize("B,Hq,Hkv,Sq,Sk", [(1, 8, 2, 1, 1000), (64, 32, 8, 1, 2000)])      # one wave of CTAs, seven
+@pytest.mark.parametrize("B,Hq,Hkv,Sq,Sk", [(1, 8, 2, 1, 1000), (64, 32, 8, 1, 2000), (1, 8, 2, 1, 5000)])      # one wave of CTAs, seven, parts of chunks
 def test_bounded_wait_expires_in_the_few_row_kernels(B, Hq, Hkv, Sq, Sk):
     """No MMA is issued: both kernels report the expired wait, the CTAs after the first ones do not wait their full second again,
     and the next forward on the same workspace is what it was before."""

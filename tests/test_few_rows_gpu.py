@@ -1,14 +1,12 @@
 """The path for few query rows (query heads of a KV group times query tokens: at most 24) at its edges, against the CPU
 oracle: 1 row to 24 and the first size past it, key counts around the 128-key tile and around the sizes where the chunk of
 a CTA grows, each producer, and a packed batch too large for the sequence table that travels with the launch."""
-import json
-
 import numpy as np
 import pytest
 import torch
 
 from paper_2609_09721_b200 import binding, inputs
-from test_attention_gpu import MEAN, TOL_O, _all_rows, _case_tensors, _check_dump
+from test_attention_gpu import MEAN, TOL_O, _all_rows, _case_tensors, _check_dump, _recorded
 
 pytestmark = pytest.mark.gpu
 
@@ -75,11 +73,13 @@ def test_packed_batch_of_few_row_sequences(n_seqs, tokens):
 
 
 @pytest.mark.parametrize("Hq,Hkv,Sq,Sk,B,producer,threshold", [
-    (4, 4, 1, 2049, 8, "efq", 0.0), (4, 4, 1, 3969, 8, "etq4", 0.0),      # chunks of 2 tiles, the last of 1; 31 tiles
+    (4, 4, 1, 2049, 8, "efq", 0.0), (4, 4, 1, 3968, 8, "etq4", 0.0),      # chunks of 2 tiles, the last of 1; 31 tiles
     (32, 8, 1, 8191, 4, "efq", 0.0), (8, 1, 1, 8300, 30, "lut", 0.0),     # 4 tiles, 16 chunks; 17, the last of 1 tile
     (2, 2, 1, 20000, 12, "efq", 0.0), (1, 1, 1, 16385, 20, "etq0", 0.0),  # 8 tiles; the last chunk of 5 and of 1
     (1, 1, 9, 4097, 80, "efq", 0.0), (16, 2, 2, 4200, 30, "efq", 1.0),    # 9 and 16 rows: chunks of 8 from 32 tiles on
     (8, 1, 3, 8193, 40, "efq", 0.0), (8, 2, 5, 9000, 20, "etq2", 0.0),    # 24 and 20 rows
+    (288, 18, 1, 1000, 4, "efq", 0.0), (296, 37, 1, 2100, 4, "efq", 0.0),   # 288 rows: in parts by itself; 296, but too many chunks
+    (304, 19, 1, 1000, 4, "efq", 0.0), (512, 32, 1, 4200, 2, "efq", 0.0),  # more rows than that: whole; in parts with chunks of 8
 ])
 def test_chunks_in_parts_equal_whole_chunks(Hq, Hkv, Sq, Sk, B, producer, threshold):
     """Where few chunks do not fill the chip they are taken in parts, tile by tile: a sequence by itself gives the bits that it
@@ -92,22 +92,53 @@ def test_chunks_in_parts_equal_whole_chunks(Hq, Hkv, Sq, Sk, B, producer, thresh
         assert torch.equal(_forward(q[b:b + 1].contiguous(), k[b:b + 1].contiguous(), v[b:b + 1].contiguous(), True, producer, threshold)[0], batch[b])
 
 
+@pytest.mark.parametrize("Hq,Hkv,Sq,Sk,parts", [
+    (288, 18, 1, 1000, True), (304, 19, 1, 1000, False),                   # chunks of two: as many rows as the merge takes at once, more
+    (512, 32, 1, 4200, True), (1024, 64, 1, 600, False), (32, 8, 1, 8191, True), (8, 2, 1, 5000, True), (8, 8, 1, 500, False),
+])
+def test_where_chunks_are_taken_in_parts(Hq, Hkv, Sq, Sk, parts):
+    g = torch.Generator(device="cuda").manual_seed(1)
+    q = torch.randn(1, Hq, Sq, 128, generator=g, device="cuda").bfloat16()
+    k, v = (torch.randn(1, Hkv, Sk, 128, generator=g, device="cuda").bfloat16() for _ in range(2))
+    assert any("few_merge_tiles_kernel" in name for name, _ in _recorded(lambda: binding.efq_attention_fwd(q, k, v, True))) == parts
+
+
+@pytest.mark.parametrize("seqs,Hq,Hkv,producer", [
+    ([(1, 700), (1, 2100), (1, 5000), (1, 20000)], 8, 1, 0),               # 1, 2, 4 and 8 tiles a chunk in one launch
+    ([(1, 700), (2, 9000), (3, 8300), (1, 130), (2, 4100)], 8, 1, 0),      # of 8, 16 and 24 rows
+    ([(1, 20000), (4, 3000), (1, 1), (2, 2100)], 8, 2, 4), ([(1, 5000), (1, 300), (1, 16500)], 4, 2, 1),
+])
+def test_packed_sequences_in_parts(seqs, Hq, Hkv, producer):
+    """A packed batch of few contexts is taken tile by tile, whatever the lengths of their chunks and their rows: each sequence gives
+    the bits of its forward in a dense batch large enough to be taken in whole chunks."""
+    g = torch.Generator(device="cuda").manual_seed(11)
+    cu_q = np.concatenate([[0], np.cumsum([a for a, _ in seqs])])
+    cu_k = np.concatenate([[0], np.cumsum([b for _, b in seqs])])
+    q = torch.randn(int(cu_q[-1]), Hq, 128, generator=g, device="cuda").bfloat16()
+    k, v = (torch.randn(int(cu_k[-1]), Hkv, 128, generator=g, device="cuda").bfloat16() for _ in range(2))
+    call = lambda: binding.efq_attention_fwd_varlen(q, k, v, cu_q, cu_k, True, 0.0, producer)
+    assert any("few_merge_tiles_kernel" in kernel for kernel, _ in _recorded(call))
+    o = call()
+    name = {0: "efq", 1: "etq0", 4: "etq2"}[producer]
+    for n, (lq, lk) in enumerate(seqs):
+        a, b, c, d = cu_q[n], cu_q[n + 1], cu_k[n], cu_k[n + 1]
+        copies = 300 if lk < 8192 else 160                     # more than 222 chunks
+        dense = [t.permute(1, 0, 2)[None].expand(copies, -1, -1, -1).contiguous() for t in (q[a:b], k[c:d], v[c:d])]
+        assert torch.equal(o[a:b].permute(1, 0, 2), _forward(*dense, True, name)[copies - 1]), f"sequence {n}"
+
+
 @pytest.mark.parametrize("Hq,Hkv,Sq,Sk", [
     (8, 8, 1, 500), (32, 8, 1, 1000), (1, 1, 1, 1000), (1, 1, 1, 60),        # chunks of one tile
     (4, 4, 1, 3000), (16, 1, 1, 1000), (16, 4, 4, 1500), (1, 1, 16, 100),    # of two; one tile in a chunk of two
     (32, 8, 1, 8191), (2, 2, 1, 16384), (1, 1, 16, 4096), (1, 1, 24, 8192),  # of four, eight
 ])
-def test_no_block_without_a_tile(tmp_path, Hq, Hkv, Sq, Sk):
+def test_no_block_without_a_tile(Hq, Hkv, Sq, Sk):
     """A chunk is cut into as many blocks as it has tiles at most: the streaming kernels launch no more blocks than there are tiles."""
     g = torch.Generator(device="cuda").manual_seed(1)
     q = torch.randn(1, Hq, Sq, 128, generator=g, device="cuda").bfloat16()
     k, v = (torch.randn(1, Hkv, Sk, 128, generator=g, device="cuda").bfloat16() for _ in range(2))
-    with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as prof:
-        binding.efq_attention_fwd(q, k, v, True)
-        torch.cuda.synchronize()
-    prof.export_chrome_trace(str(tmp_path / "trace.json"))
-    events = json.load(open(tmp_path / "trace.json"))["traceEvents"]
-    blocks = {n: e["args"]["grid"][0] for e in events for n in ("few_scores", "few_values") if e.get("cat") == "kernel" and n in e["name"]}
+    launched = _recorded(lambda: binding.efq_attention_fwd(q, k, v, True))
+    blocks = {n: grid for name, grid in launched for n in ("few_scores", "few_values") if n in name}
     assert sorted(blocks) == ["few_scores", "few_values"]
     assert max(blocks.values()) <= Hkv * ((Sk + 127) // 128)
 
