@@ -6,7 +6,7 @@ import pytest
 import torch
 
 from paper_2609_09721_b200 import binding, inputs
-from test_attention_gpu import MEAN, TOL_O, _case_tensors
+from test_attention_gpu import MEAN, TOL_O, _case_tensors, _recorded
 
 pytestmark = pytest.mark.gpu
 
@@ -68,15 +68,15 @@ def test_queries_before_the_first_key(B, Hq, Hkv, Sq, Sk, producer):
     assert torch.equal(o, forward(binding.DebugDump(0, Hq - 1, 0, 1, Sk)))
 
 
-@pytest.mark.parametrize("Hq,Hkv,Sq,Sk,causal,producer", [
-    (24, 24, 900, 30000, False, "efq"), (32, 8, 20000, 20000, True, "efq"),     # walks of 235 tiles, of 1 to 157
-    (24, 24, 900, 6144, False, "lut"), (24, 24, 900, 6145, False, "lut"),       # the line of the table form, one key past it
-    (24, 24, 900, 20000, False, "etq0"), (24, 24, 900, 20000, False, "etq2"),
-    (1, 1, 148 * 128, 300, False, "efq"), (1, 1, 148 * 128 + 1, 300, False, "efq"),       # as many query tiles as SMs, one more
+@pytest.mark.parametrize("Hq,Hkv,Sq,Sk,causal,producer,persistent", [
+    (24, 24, 900, 30000, False, "efq", True), (32, 8, 20000, 20000, True, "efq", True),     # walks of 235 tiles, of 1 to 157
+    (24, 24, 900, 6144, False, "lut", True), (24, 24, 900, 6145, False, "lut", False),      # the line of the table form, one key past it
+    (24, 24, 900, 20000, False, "etq0", True), (24, 24, 900, 20000, False, "etq2", True), (24, 24, 900, 20000, False, "etq4", False),
+    (1, 1, 148 * 128, 300, False, "efq", False), (1, 1, 148 * 128 + 1, 300, False, "efq", True),       # as many query tiles as SMs, one more
 ])
-def test_long_walks_equal_one_cta_per_tile(Hq, Hkv, Sq, Sk, causal, producer):
-    """Persistent CTAs in long walks, and at the lines of the rule: the bits of the kernel with one CTA per tile, which runs when
-    the operand is dumped."""
+def test_long_walks_equal_one_cta_per_tile(Hq, Hkv, Sq, Sk, causal, producer, persistent):
+    """Persistent CTAs in long walks, and which kernel runs at the lines of the rule: the bits of the kernel with one CTA per tile, which
+    runs when the operand is dumped."""
     g = torch.Generator(device="cuda").manual_seed(Sk)
     q = torch.randn(1, Hq, Sq, 128, generator=g, device="cuda").bfloat16()
     k, v = (torch.randn(1, Hkv, Sk, 128, generator=g, device="cuda").bfloat16() for _ in range(2))
@@ -86,7 +86,28 @@ def test_long_walks_equal_one_cta_per_tile(Hq, Hkv, Sq, Sk, causal, producer):
             return binding.exp_then_quantize_attention_fwd(q, k, v, causal, 0.0, int(producer[3:]), debug=debug)
         return binding.efq_attention_fwd(q, k, v, causal, 0.0, (MEAN[0], MEAN[1], int(producer == "lut"), 0, 0.0), debug=debug)
 
+    kernels = [name for name, _ in _recorded(forward)]
+    assert any(("attention_short_kernel" if persistent else "attention_fwd_kernel") in name for name in kernels)
     assert torch.equal(forward(), forward(binding.DebugDump(0, Hq - 1, 0, 1, Sk)))
+
+
+def test_a_forward_longer_than_the_limit_of_a_wait():
+    """The limit (1.5e9 cycles, 0.76 s) is one on the time without another tile, not on that of a CTA: a forward of a second, all of it in
+    the same CTAs, reports no problem, and its rows are those of short ones."""
+    g = torch.Generator(device="cuda").manual_seed(9)
+    q = torch.randn(1, 32, 340000, 128, generator=g, device="cuda", dtype=torch.bfloat16)
+    k, v = (torch.randn(1, 1, 340000, 128, generator=g, device="cuda", dtype=torch.bfloat16) for _ in range(2))
+    ws = torch.empty(binding.efq_attention_workspace_bytes(1, 32, 1, 340000, 340000, 128), dtype=torch.uint8, device="cuda")
+    start, end = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+    o = torch.empty(1, 32, 340000, 128, device="cuda")
+    start.record()
+    binding.efq_attention_fwd(q, k, v, False, 0.0, None, o, ws)
+    end.record()
+    assert binding.efq_poll_status(ws) == 0
+    assert start.elapsed_time(end) > 850.0
+    for head, row in ((0, 0), (31, 339800)):
+        few = q[:, head:head + 1, row:row + 200].contiguous()
+        assert torch.equal(o[0, head, row:row + 200], binding.efq_attention_fwd(few, k, v)[0, 0])
 
 
 @pytest.mark.parametrize("Hq,Hkv,causal,longest,producer", [(8, 2, True, 1000, 0), (6, 6, False, 5120, 0), (8, 4, True, 5121, 0), (8, 2, True, 700, 1), (8, 2, False, 512, 1)])
