@@ -501,7 +501,9 @@ def run_cuda(args):
     value = whole_job_tflops(flops, ms_step, world)
     mma_only = micro["fp4_mma_only_tflops"] if micro else None
 
-    def roofline_of(flops_per_launch, ms_launch, region_s, workload_name):
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+
+    def roofline_of(flops_per_launch, ms_launch, region_s, workload_name, c):
         """Roofline object of the fused kernel: achieved = algorithmic FLOPs of a launch / its CUDA-event duration; the
         peak is the measured cuBLAS bf16 rate x 4 (nominal FP4 : bf16), the burst figure for a timed region under
         BURST_REGION_S and the sustained one above it; the other denominators are given beside it."""
@@ -517,7 +519,9 @@ def run_cuda(args):
                 traffic_source = f"not measured by this run: ncu capture of kernel revision {entry['kernel_revision']}, {entry['profile']}"
             else:
                 traffic_source = f"dropped: the ncu capture in {entry['profile']} saw kernel revision {entry['kernel_revision']}, this library is {binding.version()}"
-        return {"kernel": "attention_short_kernel<EFQ>", "bound": "tensor", "achieved": achieved, "peak": peak,
+        # persistent CTAs for more query tiles than SMs
+        kernel = "attention_short_kernel<EFQ>" if c.B * c.Hq * ((c.Sq + 127) // 128) > sms else "attention_fwd_kernel<EFQ>"
+        return {"kernel": kernel, "bound": "tensor", "achieved": achieved, "peak": peak,
                 "unit": "TFLOP/s", "frac": achieved / peak, "traffic": traffic, "traffic_source": traffic_source,
                 "peak_source": f"{peaks['source']} bf16 {'burst' if burst else 'sustained'} {bf16} TFLOP/s x {NOMINAL_FP4_OVER_BF16} "
                                f"(nominal FP4:bf16 ratio); timed region {region_s:.3f} s",
@@ -527,7 +531,7 @@ def run_cuda(args):
                 "frac_of_fp4_mma_only_probe": achieved / mma_only if mma_only else None,
                 "frac_of_nominal_9pflops": achieved / 9000.0}
 
-    roofline = roofline_of(flops, ms_main, ms_step * args.steps * 1e-3, args.workload)
+    roofline = roofline_of(flops, ms_main, ms_step * args.steps * 1e-3, args.workload, case)
 
     # the other two attention shapes of the metric, a few steps each (EFQ and the strongest exponential baseline),
     # with their own step time, roofline fraction and clocks
@@ -543,7 +547,7 @@ def run_cuda(args):
             others[name] = {"config": {"workload": c2.name, "B": c2.B, "Hq": c2.Hq, "Hkv": c2.Hkv, "S": c2.Sq, "d": c2.d,
                                        "causal": c2.causal, "kv_tile": 128},
                             "steps": n2, "warmup": 3, "ms_per_step": ms2, "value": c2.flops / (ms2 * 1e-3) / 1e12, "unit": UNIT,
-                            "roofline": roofline_of(c2.flops, main2, ms2 * n2 * 1e-3, name), "clocks": clk2,
+                            "roofline": roofline_of(c2.flops, main2, ms2 * n2 * 1e-3, name, c2), "clocks": clk2,
                             "exp_then_quantize_folded": {"value": c2.flops / (f_ms2 * 1e-3) / 1e12, "ms_per_step": f_ms2,
                                                          "main_kernel_ms": f_main2, "efq_speedup": f_ms2 / ms2}}
             del w2

@@ -14,7 +14,8 @@
 // its neighbours.  The shifted scores use the running maximum over all keys up to the tile (Algorithm 2), which the first
 // kernel makes available to every chunk: the codes are those of the one-pass forward, bit for bit.
 //
-// A block takes one chunk; several blocks per SM hide the latencies of one another's tiles (load, quantise, MMA,
+// A block takes one chunk, or where few chunks do not fill the chip a half to an eighth of one, whose tiles the merge then adds up
+// in the chunk's order (few_merge_tiles_kernel).  Several blocks per SM hide the latencies of one another's tiles (load, quantise, MMA,
 // accumulator).  Loads by TMA with a role per warp (two blocks of 16 warps) were built too and are no faster: the short
 // dependent sequences of the code warps then wait behind the quantisers of their scheduler.
 #include <cuda_bf16.h>
