@@ -227,7 +227,8 @@ attention_short_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
         ptx::grid_wait();
         // an earlier CTA of this launch gave up: the waits of this one end soon instead of after their limit
         if (*reinterpret_cast<volatile uint32_t*>(P.status) != 0u) sm->abort_flag = 1u;
-        ptx::grid_launch_next();
+        // No early launch of what follows, as there (2 x 16 heads, causal, 1087 queries of 470 keys 13.2 us, with it 14.4; 2048 tokens 35.3 and
+        // 35.4; the 16 forwards of a calibration 794 and 796).
         wait_watching(&sm->finished, 0, sm, P.status);
     } else if (warp == 1) {
         // =============================== S = Q K^T issuer ===============================
@@ -431,7 +432,7 @@ attention_short_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
     // Rows without a visible key: zeros, which need no staging, in a loop of their own.  The lightest items come last, so they are what
     // is left of a packed batch; the other form walks again (the faster way in each).  With the boxes that the other rows take, and the
     // code for it in the loop above, two batches of 16 heads, causal, 1087 queries of 470 keys took 16.7 us (scale4: 19.3), 32 heads, 16384
-    // queries of 2000 keys 146; now 14.5 (16.2) and 104.
+    // queries of 2000 keys 146; without 14.4 (16.3) and 104.
     auto zero_rows = [&](const ShortWalk<TABLE>& at) {
         const ShortItem w = short_decode<TABLE>(P, at);
         const int lq = at.Sq(P), heads = at.packed() ? P.Hq / P.Hkv : 1;

@@ -239,7 +239,7 @@ exact_attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
 }
 
 // sums[0] += sum (a - r)^2, sums[1] += sum r^2, in double.  Bound by the reads (from L2 where both arrays fit): 16 bytes per
-// load, four loads in flight per thread.  Launched while the kernel that makes the rows still writes them: no read-only loads.
+// load, four loads in flight per thread.  Its blocks may be there before the kernel that makes the rows is done: no read-only loads.
 __global__ void __launch_bounds__(256) error_sums_kernel(const float* __restrict__ a, const float* __restrict__ r,
                                                          int64_t n, double* sums)
 {
