@@ -40,7 +40,7 @@ FALLBACK_HBM_GBS = 6650.0
 # from the ncu capture summarised in the named profile, and valid only for the kernel revision that
 # capture saw (the library's version tag); for any other revision the line carries null.
 NCU_DRAM_BYTES_PER_LAUNCH = {
-    "qwen3_8b_16k": {"bytes": 53571840 + 209361664, "kernel_revision": "fwd.7", "profile": "profiles/attention_fwd_current.md"},
+    "qwen3_8b_16k": {"bytes": 53661952 + 210900480, "kernel_revision": "fwd.8", "profile": "profiles/attention_fwd_current.md"},
 }
 BURST_REGION_S = 1.0   # a timed region shorter than this runs at burst clocks: its roofline uses the burst peak
 
