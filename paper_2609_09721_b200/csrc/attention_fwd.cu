@@ -798,15 +798,15 @@ cudaError_t launch_one(dim3 grid, size_t smem, cudaStream_t stream, const CUtens
 }
 
 // More query tiles than SMs: persistent CTAs, at every length of the KV walk (the measurements are in attention_short.cuh); with
-// fewer, a CTA has one item and nothing to overlap it with, and the form made for one starts sooner (one head, causal: 1024 tokens
-// 13.4 us against 13.9, 4096 30.5 / 32.5, 16384 97.0 / 100.5).  The table form of the rule loses in long walks: 24 heads,
-// 8000 queries, not causal, 4096 keys 497 us with one CTA per tile, 478 persistent, 8192 keys 916 / 924, 12288 keys 1331 / 1368;
-// its line is at a mean walk of 48 tiles.  A packed batch is judged by its longest sequence.
+// fewer, a CTA has one item and nothing to overlap it with, and the form made for one starts sooner (causal: one head, 1024 tokens
+// 12.1 us against 12.4, 4096 28.7 / 29.0, 16384 94.3 / 93.6; 36 heads, 512 tokens 10.2 / 10.5).  The table form of the rule loses in long
+// walks: 24 heads, 8000 queries, not causal, 4096 keys 495 us with one CTA per tile, 471 persistent, 8192 keys 914 / 911, 12288 keys
+// 1329 / 1349; its line is at a mean walk of 48 tiles.  A packed batch is judged by its longest sequence.
 // Little more tiles than SMs and the heaviest of them outlasting the rest: both forms end with that tile, and the line is not drawn for
-// it.  One CTA per tile / persistent, causal, affine rule 8 heads of 2600 tokens 25.1 / 24.9 us, 8 of 2432 23.7 / 24.2, 5 of 4000
-// 32.8 / 32.5; plain exponentials 16 of 1400 23.7 / 24.9, 8 of 2600 35.3 / 35.3; table 16 of 1280 22.4 / 24.0, 8 of 2600 35.4 / 36.6.  A packed
-// batch whose heaviest tile takes 1.2 times the mean of a CTA is slower by 2 % persistent, at most 6 (one head, causal, one
-// sequence of 3000 tokens and 30 of up to 1500: 35.5 / 37.4).
+// it.  One CTA per tile / persistent, causal, affine rule 8 heads of 2600 tokens 22.3 / 21.8 us, 8 of 2432 20.9 / 20.8, 16 of 1400 17.0 /
+// 15.4, 40 of 512 14.8 / 11.0; plain exponentials 16 of 1400 20.8 / 21.1, 8 of 2600 32.5 / 32.1, 40 of 512 16.3 / 12.5; table 16 of 1280
+// 19.5 / 20.0, 8 of 2600 33.1 / 33.5, 40 of 512 16.4 / 12.6.  A packed batch whose heaviest tile takes 1.2 times the mean of a CTA is slower
+// by 1 to 5 % persistent (one head, causal, one sequence of 3000 tokens and 30 of up to 1500: 34.9 / 36.5).
 // P.Sk: the keys of the problem or, with P.Sq = 0, of the longest sequence.
 bool use_short(int producer, bool debug, int64_t items, int sms, const FwdParams& P)
 {
